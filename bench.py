@@ -45,30 +45,31 @@ KERNEL_MODEL = {
     "eos_coef": (16, 33, "f64"),
     "mg_coarsen": (17, 18, "f64"),
     "H": (17, 44, "f64"),
-    "helm_rhs": (15, 51, "f64"),
-    "mg_down": (5.25, 11.5, "f64"),
-    "mg_coarse": (7, 6.5, "f64"),
-    "mg_up": (7.25, 15, "f64"),
-    "mg_single": (6, 15, "f64"),
-    "cg_pspmv": (7, 13.5, "f64"),
-    "cg_update_single": (11, 22, "f64"),
-    "cg_update_down": (10.25, 18, "f64"),
-    "correct": (16, 38, "f64"),
+    "helm_rhs": (13, 51, "f64"),
+    "mg_down": (4.25, 9, "f64"),
+    "mg_coarse": (5, 9.5, "f64"),
+    "mg_up": (5.25, 10, "f64"),
+    "rb_start": (5, 6, "f64"),
+    "rb_up": (3.75, 5.5, "f64"),
+    "cg_pspmv": (5, 10.5, "f64"),
+    "cg_update_single": (4, 4.5, "f64"),
+    "cg_update_down": (5.75, 7.5, "f64"),
+    "correct": (20.5, 43.5, "f64"),
     "mx_pred": (23.5, 104, "f64"),
     "mx_mom": (8, 46, "f32"),
     "mx_enth_rhs": (23.5, 70, "f64"),
     "mx_enth": (6.5, 31, "f32"),
     "mx_eos": (18, 33, "f64"),
     "mx_coarsen": (8.5, 18, "f32"),
-    "mx_helm_rhs": (14.5, 51, "f64"),
-    "mx_mg_down": (2.625, 11.5, "f32"),
-    "mx_mg_coarse": (3.5, 6.5, "f32"),
-    "mx_mg_up": (3.625, 15, "f32"),
-    "mx_mg_single": (3, 15, "f32"),
-    "mx_pspmv": (3.5, 13.5, "f32"),
-    "mx_update_single": (5.5, 22, "f32"),
-    "mx_update_down": (5.125, 18, "f32"),
-    "mx_p_apply": (2.5, 1, "f64"),
+    "mx_helm_rhs": (12.5, 51, "f64"),
+    "mx_mg_down": (2.125, 9, "f32"),
+    "mx_mg_coarse": (2.5, 9.5, "f32"),
+    "mx_mg_up": (2.625, 10, "f32"),
+    "mx_rb_start": (2.5, 6, "f32"),
+    "mx_rb_up": (1.875, 5.5, "f32"),
+    "mx_pspmv": (2.5, 10.5, "f32"),
+    "mx_update_single": (2, 4.5, "f32"),
+    "mx_update_down": (2.875, 7.5, "f32"),
 }
 
 

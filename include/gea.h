@@ -282,12 +282,12 @@ int gea_attach_net(gea_ctx *ctx, struct gea_net *net, int32_t mode);
  * outside 0..16). */
 int gea_set_tiles_per_block(gea_ctx *ctx, int32_t n);
 
-/* Weight omega of the Jacobi sweeps of the pressure solve's preconditioner:
- * the smoother of the multigrid V-cycle (default 0.8), or the two sweeps of
- * a one-level preconditioner (default 1, undamped). Takes effect from the
- * next step (the operator's omega/d is formed in every step's EOS phase);
- * the converged pressure does not depend on it, the CG iterations do.
- * Synchronises the stream; the step graphs are recorded anew. Errors:
+/* Weight omega of the relaxations of the black cells in the red-black
+ * Gauss-Seidel smoother of the pressure solve's multigrid V-cycle (default 1;
+ * the red cells are always relaxed exactly). A one-level preconditioner only
+ * scales by it, which conjugate gradients do not see. Takes effect from the
+ * next step; the converged pressure does not depend on it, the CG iterations
+ * do. Synchronises the stream; the step graphs are recorded anew. Errors:
  * GEA_ERR_INVAL (omega outside (0, 2)). */
 int gea_set_smoother_weight(gea_ctx *ctx, double omega);
 
@@ -340,9 +340,11 @@ int gea_set_trace(gea_ctx *ctx, uint64_t *trace, int32_t max_barriers, int64_t c
 int gea_get_field(gea_ctx *ctx, int32_t which, double *host);
 
 /* Apply the pressure solve's preconditioner to r: z = M r with M one
- * V(1,1)-cycle of the Galerkin multigrid hierarchy of the last completed step
+ * V(1,1)-cycle of the multigrid hierarchy of the last completed step, with a
+ * red-black Gauss-Seidel smoother (red then black before the coarse
+ * correction, black then red after it)
  * (the operator of eq. p_prime_sd in its Helmholtz form, as the CG of Step 3
- * uses it; two undamped Jacobi sweeps when the hierarchy has one level). r, z:
+ * uses it; one symmetric red-black sweep when the hierarchy has one level). r, z:
  * nz*nx doubles, host or device. Lets a caller check what CG needs of M: it
  * is linear, symmetric and positive definite. FP64 contexts only.
  * Synchronises. Errors: GEA_ERR_INVAL (null pointers, a mixed-precision

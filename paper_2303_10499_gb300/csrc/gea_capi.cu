@@ -146,8 +146,6 @@ StepArgs step_args(gea_ctx *c, int from)
     return a;
 }
 
-constexpr int kCoarseSweeps = 2;   // damped Jacobi sweeps on the coarsest level (even)
-constexpr double kOmega = 0.8;     // smoother weight
 // The multigrid hierarchy stops once the Laplacian part of the Helmholtz
 // operator is small against its diagonal psi/dt: with D ~ dt and psi ~ 1/(RT),
 // sum_f a_f / c ~ 2 dt^2 R T (1/dx^2 + 1/dz^2), and every coarsening divides
@@ -301,9 +299,8 @@ int record_step(gea_ctx *ctx, int from, cudaStream_t s, bool graph, Tracer *tr)
     });
     if (rc) return rc;
     launch_eos_coef(a, L[0], s, tr); ++fixed;
-    for (int l = 0; l + 1 < nlev; ++l) { launch_mg_coarsen(L[l], L[l + 1], ctx->F.omega, s, tr); ++fixed; }
+    for (int l = 0; l + 1 < nlev; ++l) { launch_mg_coarsen<double>(L[l], L[l + 1], s, tr); ++fixed; }
     // Step 3: PISO correctors
-    const int body_cg = (nlev == 1 ? 2 : 2 + (nlev - 2) + kCoarseSweeps + (nlev - 1)) + 1;
     for (int c = 0; c < ctx->C.n_corr; ++c) {
         const double *U = c == 0 ? a.ua : a.N.u;
         const double *W = c == 0 ? a.wa : a.N.w;
@@ -312,11 +309,14 @@ int record_step(gea_ctx *ctx, int from, cudaStream_t s, bool graph, Tracer *tr)
         // recorded as external
         CK(graph ? cudaEventRecordWithFlags(ctx->ev[2 * c], s, cudaEventRecordExternal)
                  : cudaEventRecord(ctx->ev[2 * c], s));
-        launch_helm_rhs(a, L[0], c == 0 ? a.S.pp : a.N.pp, a.N.pp, c, s, tr); ++fixed;
+        // a learned network works on x itself: a copy of the solve's start
+        const double *x0 = pp_in(a, c, ctx->C.n_corr);
+        double *xnet = ctx->net ? a.bh : nullptr;
+        launch_helm_rhs(a, L[0], x0, xnet, c, s, tr); ++fixed;
         if (ctx->r0keep && c == 0)
             CK(cudaMemcpyAsync(ctx->r0keep, L[0].r, arr_bytes(ctx->G, ctx->G.nz), cudaMemcpyDeviceToDevice, s));
         if (ctx->net && (ctx->net_mode & 1)) {
-            const int k = record_guess<double>(ctx, a, L[0], a.q, a.N.pp, a.cg_rtol2, s, graph, tr);
+            const int k = record_guess<double>(ctx, a, L[0], a.q, xnet, a.cg_rtol2, s, graph, tr);
             if (k < 0) return fail(ctx, GEA_ERR_CUDA, "learned initial guess failed");
             fixed += k;
         }
@@ -327,8 +327,7 @@ int record_step(gea_ctx *ctx, int from, cudaStream_t s, bool graph, Tracer *tr)
             // already converged runs no network pass
             int bad = 0;
             auto body = [&](cudaStream_t bs, cudaGraphConditionalHandle h, bool g) {
-                const int nb = launch_fcg_iter(a, L, nlev, kCoarseSweeps, a.N.pp, ctx->net, ctx->net_r,
-                                               ctx->net_e, ctx->net_s, bs, tr);
+                const int nb = launch_fcg_iter(a, L, nlev, xnet, ctx->net, ctx->net_r, ctx->net_e, ctx->net_s, bs, tr);
                 if (nb < 0) bad = 1;
                 launch_loop_ctl(a.sc, h, g, LOOP_CG, ctx->C.cg_maxit, nb < 0 ? 0 : nb + 1, bs, tr);
             };
@@ -338,16 +337,18 @@ int record_step(gea_ctx *ctx, int from, cudaStream_t s, bool graph, Tracer *tr)
             if (rc) return rc;
             if (bad) return fail(ctx, GEA_ERR_CUDA, "network preconditioner failed");
         } else {
-            fixed += launch_vcycle(a, L, nlev, kCoarseSweeps, s, tr);   // z = M^-1 r_0
+            fixed += launch_cg_start<double>(a, L, nlev, s, tr);
             rc = loop(LOOP_CG, ctx->C.cg_maxit, [&](cudaStream_t bs, cudaGraphConditionalHandle h, bool g) {
-                launch_cg_iter(a, L, nlev, kCoarseSweeps, a.N.pp, bs, tr);
-                launch_loop_ctl(a.sc, h, g, LOOP_CG, ctx->C.cg_maxit, body_cg, bs, tr);
+                const int nb = launch_cg_iter<double>(a, L, nlev, cg_vecs(a), a.cg_rtol2, bs, tr);
+                launch_loop_ctl(a.sc, h, g, LOOP_CG, ctx->C.cg_maxit, nb + 1, bs, tr);
             });
             if (rc) return rc;
         }
         CK(graph ? cudaEventRecordWithFlags(ctx->ev[2 * c + 1], s, cudaEventRecordExternal)
                  : cudaEventRecord(ctx->ev[2 * c + 1], s));
-        launch_correct(a, s, tr); ++fixed;
+        launch_correct<double>(a, L[0],
+                               SolveT<double>{xnet ? xnet : x0, nullptr, xnet && (ctx->net_mode & 2) ? nullptr : cg_vecs(a).x},
+                               pp_out(a, c, ctx->C.n_corr), s, tr); ++fixed;
     }
     ++fixed;
     launch_step_end(ctx->sc, fixed, s, tr);
@@ -357,8 +358,8 @@ int record_step(gea_ctx *ctx, int from, cudaStream_t s, bool graph, Tracer *tr)
 // The mixed-precision step: the same phases, with the three linear solves
 // done as FP64 residual + FP32 solve for the increment + FP64 update. The
 // increments du, dw (Step 1) and dh (Step 2) run their Jacobi sweeps in
-// pairs that end in du[0], dw[0], dh[0]; the pressure increment accumulates
-// in mx.x and is added to p' before the correction.
+// pairs that end in du[0], dw[0], dh[0]; the pressure increment is added to p'
+// in the correction.
 int record_step_mixed(gea_ctx *ctx, int from, cudaStream_t s, bool graph, Tracer *tr)
 {
     StepArgs a = step_args(ctx, from);
@@ -390,30 +391,30 @@ int record_step_mixed(gea_ctx *ctx, int from, cudaStream_t s, bool graph, Tracer
     });
     if (rc) return rc;
     launch_mx_eos(a, L0, Lf[0], m.dh[0], s, tr); ++fixed;
-    for (int l = 0; l + 1 < nlev; ++l) { launch_mx_coarsen(Lf[l], Lf[l + 1], ctx->F.omega, s, tr); ++fixed; }
-    const int body_cg = (nlev == 1 ? 2 : 2 + (nlev - 2) + kCoarseSweeps + (nlev - 1)) + 1;
+    for (int l = 0; l + 1 < nlev; ++l) { launch_mg_coarsen<float>(Lf[l], Lf[l + 1], s, tr); ++fixed; }
     for (int c = 0; c < ctx->C.n_corr; ++c) {
         const double *U = c == 0 ? a.ua : a.N.u;
         const double *W = c == 0 ? a.wa : a.N.w;
         launch_H(a, U, W, s, tr); ++fixed;
         CK(graph ? cudaEventRecordWithFlags(ctx->ev[2 * c], s, cudaEventRecordExternal)
                  : cudaEventRecord(ctx->ev[2 * c], s));
-        launch_mx_helm_rhs(a, L0, Lf[0], m, c == 0 ? a.S.pp : a.N.pp, a.N.pp, c, s, tr); ++fixed;
+        const double *x0 = pp_in(a, c, ctx->C.n_corr);
+        launch_mx_helm_rhs(a, L0, Lf[0], m, x0, ctx->net != nullptr, c, s, tr); ++fixed;
         if (ctx->net && (ctx->net_mode & 1)) {
             const int k = record_guess<float>(ctx, a, Lf[0], m.q, m.x, m.tol2, s, graph, tr);
             if (k < 0) return fail(ctx, GEA_ERR_CUDA, "learned initial guess failed");
             fixed += k;
         }
-        fixed += launch_mx_vcycle(a, Lf, nlev, kCoarseSweeps, s, tr);
+        fixed += launch_cg_start<float>(a, Lf, nlev, s, tr);
         rc = loop(LOOP_CG, ctx->C.cg_maxit, [&](cudaStream_t bs, cudaGraphConditionalHandle h, bool g) {
-            launch_mx_cg_iter(a, m, Lf, nlev, kCoarseSweeps, bs, tr);
-            launch_loop_ctl(a.sc, h, g, LOOP_CG, ctx->C.cg_maxit, body_cg, bs, tr);
+            const int nb = launch_cg_iter<float>(a, Lf, nlev, cg_vecs(m), m.tol2, bs, tr);
+            launch_loop_ctl(a.sc, h, g, LOOP_CG, ctx->C.cg_maxit, nb + 1, bs, tr);
         });
         if (rc) return rc;
-        launch_mx_p_apply(a, m, s, tr); ++fixed;
         CK(graph ? cudaEventRecordWithFlags(ctx->ev[2 * c + 1], s, cudaEventRecordExternal)
                  : cudaEventRecord(ctx->ev[2 * c + 1], s));
-        launch_correct(a, s, tr); ++fixed;
+        launch_correct<float>(a, Lf[0], SolveT<float>{x0, ctx->net ? m.x : nullptr, cg_vecs(m).x},
+                              pp_out(a, c, ctx->C.n_corr), s, tr); ++fixed;
     }
     ++fixed;
     launch_step_end(ctx->sc, fixed, s, tr);
@@ -472,9 +473,9 @@ struct EventTracer : Tracer {
     // the loop whose finished flag makes the kernel return, or -1
     static int gate(const char *name)
     {
-        static const char *cg[] = {"mg_down", "mg_coarse", "mg_up", "mg_single", "cg_pspmv", "cg_update_single",
-                                   "cg_update_down", "mx_mg_down", "mx_mg_coarse", "mx_mg_up", "mx_mg_single",
-                                   "mx_pspmv", "mx_update_single", "mx_update_down"};
+        static const char *cg[] = {"mg_down", "mg_coarse", "mg_up", "rb_start", "rb_up", "cg_pspmv",
+                                   "cg_update_single", "cg_update_down", "mx_mg_down", "mx_mg_coarse", "mx_mg_up",
+                                   "mx_rb_start", "mx_rb_up", "mx_pspmv", "mx_update_single", "mx_update_down"};
         for (const char *c : cg)
             if (!strcmp(name, c)) return LOOP_CG;
         if (!strcmp(name, "mom_jacobi") || !strcmp(name, "mx_mom")) return LOOP_MOM;
@@ -608,15 +609,8 @@ int gea_create(const gea_grid *grid, const gea_constants *c, gea_ctx **out)
         lg.push_back(make_geom(f.nx / 2, f.nz / 2, f.nx * f.dx, f.nz * f.dz));
         ratio *= 0.25;
     }
-    // Jacobi weight: omega damps the smoother of a multigrid hierarchy; a
-    // one-level preconditioner is two undamped sweeps (omega = 1), whose
-    // preconditioned operator lambda (2 - lambda) on the spectrum of D^-1 A
-    // (inside its Gershgorin interval [1 - rho, 1 + rho], rho < 1) is the
-    // degree-2 Chebyshev polynomial of that interval up to a factor, which
-    // CG does not see: condition number 1 / (1 - rho^2) for any rho, against
-    // (1 - (1 - omega (1 + rho))^2) / (1 - (1 - omega (1 - rho))^2) for two
-    // damped sweeps (1.28 against 1.50 at rho = 0.47, omega = 0.8)
-    ctx->F.omega = lg.size() == 1 ? 1.0 : kOmega;
+    ctx->F.omega = 1.0;   // undamped red-black Gauss-Seidel
+    ctx->F.om_ne1 = 0;
 
     // one allocation for everything
     const Geom &G = ctx->G;
@@ -909,11 +903,10 @@ int gea_step_async(gea_ctx *ctx, int32_t n)
         const int first = (int)((ctx->base + ctx->steps_at_sync) & 1);
         const PersistOps &o = persist_ops(ctx->shape);
         if (ctx->mixed)
-            CK(o.launch_mixed(a, ctx->L[0], ctx->mx, ctx->Lf.data(), (int)ctx->Lf.size(), kCoarseSweeps,
-                                       ctx->C.n_corr, ctx->C.jac_maxit, ctx->C.cg_maxit, first, n,
+            CK(o.launch_mixed(a, ctx->L[0], ctx->mx, ctx->Lf.data(), (int)ctx->Lf.size(), ctx->C.n_corr, ctx->C.jac_maxit, ctx->C.cg_maxit, first, n,
                                        ctx->pers_blocks, ctx->wait_polls, ctx->stream));
         else
-            CK(o.launch(a, ctx->L.data(), (int)ctx->L.size(), kCoarseSweeps, ctx->C.n_corr,
+            CK(o.launch(a, ctx->L.data(), (int)ctx->L.size(), ctx->C.n_corr,
                                  ctx->C.jac_maxit, ctx->C.cg_maxit, first, n, ctx->pers_blocks,
                                  ctx->wait_polls, ctx->stream));
         ctx->steps_at_sync += n;
@@ -1251,6 +1244,7 @@ int gea_set_smoother_weight(gea_ctx *ctx, double omega)
         ctx->graph[f] = nullptr;
     }
     ctx->F.omega = omega;
+    ctx->F.om_ne1 = omega != 1.0 ? 1 : 0;
     return GEA_OK;
 }
 
@@ -1274,7 +1268,7 @@ int gea_apply_precond(gea_ctx *ctx, const double *r, double *z)
     rc = copy_in(ctx, L[0].r, r, ctx->G.nx, ctx->G.nz);
     if (!rc) {
         StepArgs a = step_args(ctx, 0);
-        launch_vcycle(a, L, (int)ctx->L.size(), kCoarseSweeps, ctx->stream, nullptr);
+        launch_vcycle<double>(a, L, (int)ctx->L.size(), ctx->stream, nullptr);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = fail(ctx, GEA_ERR_CUDA, "V-cycle launch: %s", cudaGetErrorString(e));
     }
@@ -1425,11 +1419,10 @@ void ensemble_fill(gea_ensemble *e, int n, int parity)
         const int first = parity >= 0 ? parity : (int)((c->base + c->steps_at_sync) & 1);
         if (e->mixed)
             persist_args_fill_mixed(e->hargs + i * e->argb, a, c->L[0], c->mx, c->Lf.data(), (int)c->Lf.size(),
-                                    kCoarseSweeps, c->C.n_corr, c->C.jac_maxit, c->C.cg_maxit, first, n,
+                                    c->C.n_corr, c->C.jac_maxit, c->C.cg_maxit, first, n,
                                     c->wait_polls);
         else
-            persist_args_fill(e->hargs + i * e->argb, a, c->L.data(), (int)c->L.size(), kCoarseSweeps,
-                              c->C.n_corr, c->C.jac_maxit, c->C.cg_maxit, first, n, c->wait_polls);
+            persist_args_fill(e->hargs + i * e->argb, a, c->L.data(), (int)c->L.size(), c->C.n_corr, c->C.jac_maxit, c->C.cg_maxit, first, n, c->wait_polls);
     }
 }
 

@@ -39,12 +39,13 @@ struct Geom {
 
 struct Phys {
     double R, cp, g, p0, mu, nuh, dt, idt;   // nuh = mu / Pr
-    double omega;                            // damped-Jacobi weight of the smoother
+    double omega;                            // weight of the smoother's black relaxations
     double les_d2;                           // Smagorinsky (cs Delta)^2; 0: constant viscosity
     int k_lagged;                            // GEA_READING_K_LAGGED: K^{n-1} in eq. step3_sd
     // uniform branch flags as integers (an FP64 compare issues on the FP64 pipe)
     int les;                                 // les_d2 > 0
     int pr_ne1;                              // nuh != mu (Pr != 1): the enthalpy stencil differs
+    int om_ne1;                              // omega != 1
 };
 
 // Persistent state of one time level (Section 3's solution tuple plus the
@@ -56,25 +57,39 @@ struct State {
 
 // One multigrid level of the Helmholtz operator
 //   (A x)_i = c_i x_i + sum_f a_f (x_i - x_N) = d_i x_i - sum_f a_f x_N,
-// d_i = c_i + sum_f a_f, kept as d and wd = omega / d.
+// d_i = c_i + sum_f a_f, kept as d and wd = 1 / d.
 // R is the value type: double on the FP64 path, float for the inner solves
 // of the mixed-precision path.
 template <class R>
 struct LevelT {
     Geom G;
-    R *c, *d, *wd, *ax, *az;  // reaction, diagonal, omega/diagonal, face coefficients
-    R *r, *e, *e2;            // residual, pre-smoothed correction, post-smoothed
-    R *r_alt;                 // finest level: second residual buffer (CG iterations
-                              // alternate r and r_alt; the update reads one, writes the other)
+    R *c, *d, *wd, *ax, *az;  // reaction, diagonal, 1 / diagonal, face coefficients
+    R *r, *e, *e2;            // residual, scratch, correction
+    R *r_alt;                 // finest level: second residual buffer of the flexible CG
+                              // (iterations alternate r and r_alt)
 };
 using Level = LevelT<double>;
 using LevelF = LevelT<float>;
 
-// Finest-level residual after `it` CG updates.
+// Finest-level residual of the flexible CG after `it` updates.
 template <class R>
 __host__ __device__ __forceinline__ R *res_of(const LevelT<R> &L, int it)
 {
     return (it & 1) ? L.r_alt : L.r;
+}
+
+// The vectors of a red-black pressure solve (black halves, gea_tiles_body.cuh)
+// besides the residual at its start (L.r, all cells): the black residual
+// alternates between the finest level's e and r_alt, the preconditioned one is in
+// e2, x is the increment, and the directions alternate between p0 and p1.
+template <class R>
+struct CgVecT {
+    R *x, *p0, *p1, *q;
+};
+template <class R>
+__host__ __device__ __forceinline__ R *black_res(const LevelT<R> &L, int it)
+{
+    return (it & 1) ? L.r_alt : L.e;
 }
 
 // The implicit transport operator of Steps 1-2,
@@ -96,7 +111,7 @@ struct MixedArgs {
     float *dinvu, *dinvh;          // Jacobi reciprocals
     float *r0u, *r0w, *r0h;        // FP64 residuals of the predictors, rounded to FP32
     float *du[2], *dw[2], *dh[2];  // increments (Jacobi ping-pong)
-    float *x, *p0, *p1, *q;        // pressure increment, CG directions, A p
+    float *x, *p0, *p1, *q;        // increment of the learned guess, CG directions, A p
     double tol2;                   // inner tolerance^2, relative to the initial residual
 };
 
@@ -332,6 +347,13 @@ inline dim3 grid_tiles(const Geom &G, int tpb)
     if (tpb <= 0) tpb = (long long)tx * tz >= kMultiTileMin ? kTilesPerBlock : 1;
     return dim3(tx, (tz + tpb - 1) / tpb);
 }
+// Same for the red-black phases, whose tiles are BX pairs of cells wide.
+inline dim3 grid_pair_tiles(const Geom &G, int tpb)
+{
+    Geom H = G;
+    H.nx = (G.nx + 1) / 2;
+    return grid_tiles(H, tpb);
+}
 // f(bx, bz) for the block's tiles (block-uniform loop; each f ends with a
 // block barrier).
 template <class F>
@@ -344,6 +366,39 @@ __device__ __forceinline__ void block_tiles(const Geom &G, F f)
         if (bz >= tz) break;
         f((int)blockIdx.x, bz);
     }
+}
+
+// The vectors of the pressure solve. The increment lies in a right-hand side
+// of the momentum predictor (or, mixed, its FP32 residual), which nothing
+// reads once the predictor is done.
+__host__ __device__ __forceinline__ CgVecT<double> cg_vecs(const StepArgs &a)
+{
+    return CgVecT<double>{a.bu, a.p0, a.p1, a.q};
+}
+__host__ __device__ __forceinline__ CgVecT<float> cg_vecs(const MixedArgs &m)
+{
+    return CgVecT<float>{m.r0u, m.p0, m.p1, m.q};
+}
+// What a pressure solve left: p' = x + dx with x the solve's start and, once
+// an iteration ran, dx = xb on the black cells and (r + sum a dx) / d on the
+// red ones, r the residual at the start (a null xb: dx = 0). inc (mixed
+// precision with a learned guess): an FP32 increment of x.
+template <class R>
+struct SolveT {
+    const double *x;
+    const float *inc;
+    const R *xb;
+};
+// p' after corrector c: N.pp after the last one, before it alternating with
+// another free right-hand side (a corrector reads its start's halo while it
+// writes).
+__host__ __device__ __forceinline__ double *pp_out(const StepArgs &a, int c, int n_corr)
+{
+    return ((n_corr - 1 - c) & 1) ? a.bw : a.N.pp;
+}
+__host__ __device__ __forceinline__ const double *pp_in(const StepArgs &a, int c, int n_corr)
+{
+    return c == 0 ? a.S.pp : pp_out(a, c - 1, n_corr);
 }
 
 // ---- host-side launchers (gea_kernels.cu); tr may be null ----
@@ -362,16 +417,25 @@ void launch_enth_rhs(const StepArgs &a, cudaStream_t st, Tracer *tr);
 void launch_enth_jacobi(const StepArgs &a, const double *hin, double *hout, int second,
                         cudaStream_t st, Tracer *tr);
 void launch_eos_coef(const StepArgs &a, const Level &L0, cudaStream_t st, Tracer *tr);
-void launch_mg_coarsen(const Level &f, const Level &c, double omega, cudaStream_t st, Tracer *tr);
+template <class R>
+void launch_mg_coarsen(const LevelT<R> &f, const LevelT<R> &c, cudaStream_t st, Tracer *tr);
 void launch_H(const StepArgs &a, const double *U, const double *W, cudaStream_t st, Tracer *tr);
 void launch_helm_rhs(const StepArgs &a, const Level &L0, const double *xin, double *xout,
                      int corr, cudaStream_t st, Tracer *tr);
-// returns the number of kernels launched
-int launch_vcycle(const StepArgs &a, Level *levels, int nlev, int ncoarse, cudaStream_t st,
-                  Tracer *tr);
-int launch_cg_iter(const StepArgs &a, Level *levels, int nlev, int ncoarse, double *x,
-                   cudaStream_t st, Tracer *tr);
-void launch_correct(const StepArgs &a, cudaStream_t st, Tracer *tr);
+// One V-cycle on L[0].r into L[0].e2 with r.z (all cells; the preconditioner of
+// gea_apply_precond and of the flexible CG), the start of a red-black CG solve,
+// and one of its iterations to the relative residual tol2 (squared). Each
+// returns the number of kernels launched.
+template <class R>
+int launch_vcycle(const StepArgs &a, const LevelT<R> *L, int nlev, cudaStream_t st, Tracer *tr);
+template <class R>
+int launch_cg_start(const StepArgs &a, const LevelT<R> *L, int nlev, cudaStream_t st, Tracer *tr);
+template <class R>
+int launch_cg_iter(const StepArgs &a, const LevelT<R> *L, int nlev, const CgVecT<R> &v, double tol2, cudaStream_t st,
+                   Tracer *tr);
+template <class R>
+void launch_correct(const StepArgs &a, const LevelT<R> &L, const SolveT<R> &v, double *ppout, cudaStream_t st,
+                    Tracer *tr);
 // graph: set the WHILE condition through h; otherwise bookkeeping only
 void launch_loop_ctl(Scal *sc, cudaGraphConditionalHandle h, bool graph, int which,
                      int maxtrips, int body_launches, cudaStream_t st, Tracer *tr);
@@ -399,8 +463,8 @@ int launch_net_guess(const StepArgs &a, const LevelT<R> &L, R *r, R *q, R *x, do
 // levels L): z = g N(r) + M(r - g A N(r)) with the network N and one
 // V-cycle M (s_buf: a field for r - g A N(r)), the direction update, q = A p,
 // x and r. Returns the number of launches, or -1.
-int launch_fcg_iter(const StepArgs &a, Level *L, int nlev, int ncoarse, double *x, gea_net *net,
-                    float *dense_r, float *dense_e, double *s_buf, cudaStream_t st, Tracer *tr);
+int launch_fcg_iter(const StepArgs &a, Level *L, int nlev, double *x, gea_net *net, float *dense_r,
+                    float *dense_e, double *s_buf, cudaStream_t st, Tracer *tr);
 // mixed-precision step (gea_mixed.cu)
 void launch_mx_pred(const StepArgs &a, const MixedArgs &m, cudaStream_t st, Tracer *tr);
 void launch_mx_mom(const StepArgs &a, const MixedArgs &m, const float *ui, const float *wi, float *uo,
@@ -410,13 +474,8 @@ void launch_mx_enth(const StepArgs &a, const MixedArgs &m, const float *hi, floa
                     cudaStream_t st, Tracer *tr);
 void launch_mx_eos(const StepArgs &a, const Level &L0, const LevelF &L32, const float *dh, cudaStream_t st,
                    Tracer *tr);
-void launch_mx_coarsen(const LevelF &f, const LevelF &c, double omega, cudaStream_t st, Tracer *tr);
 void launch_mx_helm_rhs(const StepArgs &a, const Level &L0, const LevelF &L32, const MixedArgs &m,
-                        const double *xin, double *xout, int corr, cudaStream_t st, Tracer *tr);
-int launch_mx_vcycle(const StepArgs &a, LevelF *L, int nlev, int ncoarse, cudaStream_t st, Tracer *tr);
-int launch_mx_cg_iter(const StepArgs &a, const MixedArgs &m, LevelF *L, int nlev, int ncoarse,
-                      cudaStream_t st, Tracer *tr);
-void launch_mx_p_apply(const StepArgs &a, const MixedArgs &m, cudaStream_t st, Tracer *tr);
+                        const double *xin, bool guess, int corr, cudaStream_t st, Tracer *tr);
 // ---- persistent cooperative step kernels (gea_persistent_body.cuh) ----
 
 // Arguments of one context's persistent launch (or of one member of an
@@ -424,7 +483,7 @@ void launch_mx_p_apply(const StepArgs &a, const MixedArgs &m, cudaStream_t st, T
 struct PersistArgs {
     StepArgs a[2];          // a[s] reads state slot s and writes slot s ^ 1
     Level L[kMaxLevels];
-    int nlev, ncoarse, nsteps, first_slot, n_corr, jac_maxit, cg_maxit;
+    int nlev, nsteps, first_slot, n_corr, jac_maxit, cg_maxit;
     unsigned long long spin_limit;   // polls of a grid barrier before giving up
 };
 
@@ -465,11 +524,11 @@ struct PersistOps {
     int (*max_blocks)();
     int (*mixed_max_blocks)();
     int (*ensemble_max_blocks)(int mixed);
-    cudaError_t (*launch)(const StepArgs a[2], const Level *L, int nlev, int ncoarse, int n_corr, int jac_maxit,
+    cudaError_t (*launch)(const StepArgs a[2], const Level *L, int nlev, int n_corr, int jac_maxit,
                           int cg_maxit, int first_slot, int nsteps, int blocks, long long wait_polls,
                           cudaStream_t st);
     cudaError_t (*launch_mixed)(const StepArgs a[2], const Level &L0, const MixedArgs &m, const LevelF *Lf,
-                                int nlev, int ncoarse, int n_corr, int jac_maxit, int cg_maxit, int first_slot,
+                                int nlev, int n_corr, int jac_maxit, int cg_maxit, int first_slot,
                                 int nsteps, int blocks, long long wait_polls, cudaStream_t st);
     cudaError_t (*launch_ensemble)(const void *Pm, int mixed, const int *groups, int ngroups, int blocks,
                                    cudaStream_t st);
@@ -483,12 +542,12 @@ inline long long shape_tiles(const Geom &G, int bx, int bz)
 }
 // bytes of one member's argument block of an ensemble launch
 size_t persist_args_bytes(int mixed);
-void persist_args_fill(void *dst, const StepArgs a[2], const Level *L, int nlev, int ncoarse, int n_corr,
+void persist_args_fill(void *dst, const StepArgs a[2], const Level *L, int nlev, int n_corr,
                        int jac_maxit, int cg_maxit, int first_slot, int nsteps, long long wait_polls);
 // the mixed-precision member's block: PersistArgs (the FP64 finest level
 // L0) followed by MixedPersist (m, the FP32 hierarchy Lf[0 .. nlev-1])
 void persist_args_fill_mixed(void *dst, const StepArgs a[2], const Level &L0, const MixedArgs &m,
-                             const LevelF *Lf, int nlev, int ncoarse, int n_corr, int jac_maxit, int cg_maxit,
+                             const LevelF *Lf, int nlev, int n_corr, int jac_maxit, int cg_maxit,
                              int first_slot, int nsteps, long long wait_polls);
 
 }  // namespace gea

@@ -139,13 +139,14 @@ __global__ void k_enth_jacobi(StepArgs a, const double *hin, double *hout, int s
 __global__ void k_eos_coef(StepArgs a, Level L)
 {
     if (a.sc->status) return;
-    __shared__ double sm[2 * kT1 + BZ * (BX + 1) + (BZ + 1) * BX];
+    __shared__ double sm[2 * kT1 + kFaces];
     ph_eos(a, L, a.ha, sm, blockIdx.x, blockIdx.y);
 }
 
-__global__ void k_mg_coarsen(Level f, Level c, double omega)
+template <class R>
+__global__ void k_mg_coarsen(LevelT<R> f, LevelT<R> c)
 {
-    ph_coarsen(f, c, omega, blockIdx.x, blockIdx.y);
+    ph_coarsen<R>(f, c, blockIdx.x, blockIdx.y);
 }
 
 // ---- Step 3 ----
@@ -168,99 +169,123 @@ __global__ void k_helm_rhs(StepArgs a, Level L, const double *xin, double *xout,
         fin_helm(a.sc, tot, a.cg_rtol2, corr);
 }
 
-__global__ void k_mg_down(Level f, Level c, double omega, Scal *sc)
+// ---- the pressure solve (R: double, or float for the mixed-precision step) ----
+
+template <class R>
+__global__ void k_rb_start(LevelT<R> L, Scal *sc, double *partials)
 {
     if (loop_over(sc, LOOP_CG)) return;
-    __shared__ double sm[kT1 + BZ * BX];
-    ph_mg_down(f, c, omega, sm, blockIdx.x, blockIdx.y);
-}
-
-__global__ void k_mg_coarse_sweep(Level L, const double *ein, double *eout, int first, Scal *sc)
-{
-    if (loop_over(sc, LOOP_CG)) return;
-    __shared__ double sm[kT1];
-    ph_mg_coarse(L, ein, eout, first, sm, blockIdx.x, blockIdx.y);
-}
-
-__global__ void k_mg_up(Level f, const double *ec, int Pc, double *out, int finest, StepArgs a)
-{
-    if (loop_over(a.sc, LOOP_CG)) return;
-    __shared__ double sm[kT1];
+    __shared__ R sm[kPH1];
     __shared__ double red[NTHREADS];
-    double acc[1] = {0.0}, tot[1];
-    // the finest level's residual alternates between two buffers
-    const double *res = finest ? res_of(f, a.sc->cg_it) : f.r;
-    block_tiles(f.G, [&](int bx, int bz) { ph_mg_up(f, res, ec, Pc, out, sm, bx, bz, acc); });
+    R acc[1] = {(R)0};
+    double tot[1];
+    block_tiles(L.G, [&](int bx, int bz) {
+        ph_rb_start<R>(L, black_res(L, 0), L.e2, reinterpret_cast<double *>(sm), bx, bz, acc);
+    });
+    if (grid_sum<1, R>(acc, red, partials, &sc->counters[CNT_RZ], tot)) fin_rz(sc, tot);
+}
+
+template <bool FINE, class R>
+__global__ void k_mg_down(LevelT<R> f, LevelT<R> c, Phys F, Scal *sc)
+{
+    if (loop_over(sc, LOOP_CG)) return;
+    __shared__ R sm[kPH2 + kPH1 + BZ * BX];
+    ph_mg_down<FINE, R>(f, c, FINE ? black_res(f, 0) : nullptr, F, reinterpret_cast<double *>(sm), blockIdx.x,
+                        blockIdx.y);
+}
+
+// finest: also r.z
+template <class R>
+__global__ void k_mg_up(LevelT<R> f, const R *ec, int Pc, int finest, Phys F, Scal *sc, double *partials)
+{
+    if (loop_over(sc, LOOP_CG)) return;
+    __shared__ R sm[kPH2 + kPH1];
+    __shared__ double red[NTHREADS];
+    R acc[1] = {(R)0};
+    double tot[1];
+    block_tiles(f.G, [&](int bx, int bz) {
+        ph_mg_up<R>(f, f.r, ec, Pc, f.e2, F, reinterpret_cast<double *>(sm), bx, bz, acc);
+    });
     if (!finest) return;
-    if (grid_sum<1>(acc, red, a.partials, &a.sc->counters[CNT_RZ], tot)) fin_rz(a.sc, tot);
+    if (grid_sum<1, R>(acc, red, partials, &sc->counters[CNT_RZ], tot)) fin_rz(sc, tot);
 }
 
-__global__ void k_mg_single(Level f, double *out, StepArgs a)
+template <class R>
+__global__ void k_rb_up(LevelT<R> f, const R *ec, int Pc, Phys F, Scal *sc, double *partials)
 {
-    if (loop_over(a.sc, LOOP_CG)) return;
-    __shared__ double sm[kT1];
+    if (loop_over(sc, LOOP_CG)) return;
     __shared__ double red[NTHREADS];
-    double acc[1] = {0.0}, tot[1];
-    block_tiles(f.G, [&](int bx, int bz) { ph_mg_single(f, out, sm, bx, bz, acc); });
-    if (grid_sum<1>(acc, red, a.partials, &a.sc->counters[CNT_RZ], tot)) fin_rz(a.sc, tot);
+    R acc[1] = {(R)0};
+    double tot[1];
+    const R *rb = black_res(f, sc->cg_it);
+    block_tiles(f.G, [&](int bx, int bz) { ph_rb_up<R>(f, rb, ec, Pc, f.e2, F, bx, bz, acc); });
+    if (grid_sum<1, R>(acc, red, partials, &sc->counters[CNT_RZ], tot)) fin_rz(sc, tot);
 }
 
 // The directions alternate between p0 and p1 by iteration parity: iteration
 // it reads p[it & 1] and writes p[(it + 1) & 1].
-__global__ void k_cg_pspmv(StepArgs a, Level L)
+template <class R>
+__global__ void k_cg_pspmv(LevelT<R> L, CgVecT<R> v, Scal *sc, double *partials)
 {
-    Scal *sc = a.sc;
     if (loop_over(sc, LOOP_CG)) return;
-    __shared__ double sm[kT1];
+    __shared__ R sm[kPH2 + kPH1];
     __shared__ double red[NTHREADS];
     const int it = sc->cg_it;
-    const double *pold = (it & 1) ? a.p1 : a.p0;
-    double *pnew = (it & 1) ? a.p0 : a.p1;
-    double acc[1] = {0.0}, tot[1];
-    block_tiles(L.G, [&](int bx, int bz) { ph_pspmv<double>(L, pold, pnew, a.q, sc->beta, sm, bx, bz, acc); });
-    if (grid_sum<1>(acc, red, a.partials, &sc->counters[CNT_PQ], tot)) fin_pq(sc, tot);
+    const R *pold = (it & 1) ? v.p1 : v.p0;
+    R *pnew = (it & 1) ? v.p0 : v.p1;
+    const double beta = sc->beta;
+    R acc[1] = {(R)0};
+    double tot[1];
+    block_tiles(L.G, [&](int bx, int bz) {
+        ph_pspmv<R>(L, L.e2, pold, pnew, v.q, beta, it == 0, reinterpret_cast<double *>(sm), bx, bz, acc);
+    });
+    if (grid_sum<1, R>(acc, red, partials, &sc->counters[CNT_PQ], tot)) fin_pq(sc, tot);
 }
 
-__global__ void k_cg_update_single(StepArgs a, Level L, double *x)
+template <class R>
+__global__ void k_cg_update_single(LevelT<R> L, CgVecT<R> v, Scal *sc, double *partials, double tol2)
 {
-    Scal *sc = a.sc;
     if (loop_over(sc, LOOP_CG)) return;
-    __shared__ double sm[2 * kT1];
     __shared__ double red[2 * NTHREADS];
     const int it = sc->cg_it;
-    const double *p = (it & 1) ? a.p0 : a.p1;
-    double acc[2] = {0.0, 0.0}, tot[2];
+    const R *p = (it & 1) ? v.p0 : v.p1;
+    const double alpha = sc->alpha;
+    R acc[2] = {(R)0, (R)0};
+    double tot[2];
     block_tiles(L.G, [&](int bx, int bz) {
-        ph_update_single<double>(L, a.q, res_of(L, it), res_of(L, it + 1), x, p, sc->alpha, sm, bx, bz, acc);
+        ph_update_single<R>(L, v.q, black_res(L, 0), L.e2, v.x, p, alpha, it == 0, bx, bz, acc);
     });
-    if (grid_sum<2>(acc, red, a.partials, &sc->counters[CNT_UPD], tot)) {
+    if (grid_sum<2, R>(acc, red, partials, &sc->counters[CNT_UPD], tot)) {
         const double t0[1] = {tot[0]}, t1[1] = {tot[1]};
-        fin_update(sc, t0, a.cg_rtol2);
+        fin_update(sc, t0, tol2);
         fin_rz(sc, t1);
     }
 }
 
-__global__ void k_cg_update_down(StepArgs a, Level f, Level c, double *x)
+template <class R>
+__global__ void k_cg_update_down(LevelT<R> f, LevelT<R> c, CgVecT<R> v, Phys F, Scal *sc, double *partials, double tol2)
 {
-    Scal *sc = a.sc;
     if (loop_over(sc, LOOP_CG)) return;
-    __shared__ double sm[2 * kT1 + BZ * BX];
+    __shared__ R sm[kPH1 + BZ * BX];
     __shared__ double red[NTHREADS];
     const int it = sc->cg_it;
-    const double *p = (it & 1) ? a.p0 : a.p1;
-    double acc[1] = {0.0}, tot[1];
+    const R *p = (it & 1) ? v.p0 : v.p1;
+    const double alpha = sc->alpha;
+    R acc[1] = {(R)0};
+    double tot[1];
     block_tiles(f.G, [&](int bx, int bz) {
-        ph_update_down<double>(f, c, a.q, res_of(f, it), res_of(f, it + 1), x, p, sc->alpha, a.F.omega, sm,
-                               bx, bz, acc);
+        ph_update_down<R>(f, c, v.q, black_res(f, it), black_res(f, it + 1), v.x, p, alpha, it == 0, F,
+                          reinterpret_cast<double *>(sm), bx, bz, acc);
     });
-    if (grid_sum<1>(acc, red, a.partials, &sc->counters[CNT_UPD], tot)) fin_update(sc, tot, a.cg_rtol2);
+    if (grid_sum<1, R>(acc, red, partials, &sc->counters[CNT_UPD], tot)) fin_update(sc, tot, tol2);
 }
 
-__global__ void k_correct(StepArgs a)
+template <class R>
+__global__ void k_correct(StepArgs a, LevelT<R> L, SolveT<R> v, double *ppout)
 {
     if (a.sc->status) return;
-    __shared__ double sm[2 * kT1 + BZ * (BX + 1) + (BZ + 1) * BX];
-    ph_correct(a, sm, blockIdx.x, blockIdx.y);
+    __shared__ double sm[kCorrectSmem];
+    ph_correct<R>(a, L, v, v.xb && a.sc->cg_it > 0, ppout, sm, blockIdx.x, blockIdx.y);
 }
 
 // ---- loop control and step bookkeeping (one thread) ----
@@ -331,6 +356,7 @@ __global__ void k_diag(Geom G, Phys F, State S, const double *__restrict__ thbar
 }
 
 inline dim3 grid_of(const Geom &G) { return dim3((G.nx + BX - 1) / BX, (G.nz + BZ - 1) / BZ); }
+inline dim3 grid_pairs(const Geom &G) { return grid_pair_tiles(G, 1); }
 const dim3 kBlock(BX, BZ);
 
 }  // namespace
@@ -398,9 +424,18 @@ void launch_eos_coef(const StepArgs &a, const Level &L0, cudaStream_t st, Tracer
     TRACED(tr, "eos_coef", ncell(a.G), (k_eos_coef<<<grid_of(a.G), kBlock, 0, st>>>(a, L0)));
 }
 
-void launch_mg_coarsen(const Level &f, const Level &c, double omega, cudaStream_t st, Tracer *tr)
+// launch names: the FP32 kernels of the mixed-precision step carry "mx_"
+template <class R>
+const char *name_of(const char *f64, const char *f32)
 {
-    TRACED(tr, "mg_coarsen", ncell(c.G), (k_mg_coarsen<<<grid_of(c.G), kBlock, 0, st>>>(f, c, omega)));
+    return sizeof(R) == sizeof(double) ? f64 : f32;
+}
+
+template <class R>
+void launch_mg_coarsen(const LevelT<R> &f, const LevelT<R> &c, cudaStream_t st, Tracer *tr)
+{
+    TRACED(tr, name_of<R>("mg_coarsen", "mx_coarsen"), ncell(c.G),
+           (k_mg_coarsen<R><<<grid_of(c.G), kBlock, 0, st>>>(f, c)));
 }
 
 void launch_H(const StepArgs &a, const double *U, const double *W, cudaStream_t st, Tracer *tr)
@@ -415,74 +450,106 @@ void launch_helm_rhs(const StepArgs &a, const Level &L0, const double *xin, doub
            (k_helm_rhs<<<grid_of(a.G), kBlock, 0, st>>>(a, L0, xin, xout, corr)));
 }
 
-// z = M^-1 r into levels[0].e2 (one V(1,1)-cycle; ncoarse sweeps on the
-// coarsest level). Returns the number of kernels launched.
-int launch_vcycle(const StepArgs &a, Level *L, int nlev, int ncoarse, cudaStream_t st, Tracer *tr)
-{
-    if (nlev == 1) {
-        TRACED(tr, "mg_single", ncell(L[0].G),
-               (k_mg_single<<<grid_tiles(L[0].G, a.tiles_per_block), kBlock, 0, st>>>(L[0], L[0].e2, a)));
-        return 1;
-    }
-    int n = 0;
-    for (int l = 0; l + 1 < nlev; ++l, ++n)
-        TRACED(tr, "mg_down", ncell(L[l].G),
-               (k_mg_down<<<grid_of(L[l].G), kBlock, 0, st>>>(L[l], L[l + 1], a.F.omega, a.sc)));
-    Level &C = L[nlev - 1];
-    // sweep s writes e2 when ncoarse-1-s is even, so the last sweep ends in e2
-    for (int s = 0; s < ncoarse; ++s, ++n) {
-        double *out = ((ncoarse - 1 - s) % 2 == 0) ? C.e2 : C.e;
-        const double *in = (out == C.e2) ? C.e : C.e2;
-        TRACED(tr, "mg_coarse", ncell(C.G),
-               (k_mg_coarse_sweep<<<grid_of(C.G), kBlock, 0, st>>>(C, in, out, s == 0, a.sc)));
-    }
-    for (int l = nlev - 2; l >= 0; --l, ++n)
-        TRACED(tr, "mg_up", ncell(L[l].G),
-               (k_mg_up<<<grid_tiles(L[l].G, a.tiles_per_block), kBlock, 0, st>>>(L[l], L[l + 1].e2, L[l + 1].G.P, L[l].e2,
-                                                             l == 0, a)));
-    return n;
-}
+namespace {
 
-// V-cycle levels below the finest: restriction steps of levels 1..nlev-2,
-// the coarsest sweeps and the prolongation steps down to the finest (which
-// yields z and r.z). Returns the number of kernels launched.
-static int launch_vcycle_rest(const StepArgs &a, Level *L, int nlev, int ncoarse, cudaStream_t st,
-                              Tracer *tr)
+// V-cycle levels below the finest: down halves of levels 1 .. nlev-2, the
+// coarsest sweep, up halves to level 1.
+template <class R>
+int vcycle_below(const StepArgs &a, const LevelT<R> *L, int nlev, cudaStream_t st, Tracer *tr)
 {
     int n = 0;
     for (int l = 1; l + 1 < nlev; ++l, ++n)
-        TRACED(tr, "mg_down", ncell(L[l].G),
-               (k_mg_down<<<grid_of(L[l].G), kBlock, 0, st>>>(L[l], L[l + 1], a.F.omega, a.sc)));
-    Level &C = L[nlev - 1];
-    for (int s = 0; s < ncoarse; ++s, ++n) {
-        double *out = ((ncoarse - 1 - s) % 2 == 0) ? C.e2 : C.e;
-        const double *in = (out == C.e2) ? C.e : C.e2;
-        TRACED(tr, "mg_coarse", ncell(C.G),
-               (k_mg_coarse_sweep<<<grid_of(C.G), kBlock, 0, st>>>(C, in, out, s == 0, a.sc)));
+        TRACED(tr, name_of<R>("mg_down", "mx_mg_down"), ncell(L[l].G),
+               (k_mg_down<false, R><<<grid_pairs(L[l].G), kBlock, 0, st>>>(L[l], L[l + 1], a.F, a.sc)));
+    for (int l = nlev - 1; l >= 1; --l, ++n) {
+        const bool last = l == nlev - 1;
+        const R *ec = last ? nullptr : L[l + 1].e2;
+        TRACED(tr, last ? name_of<R>("mg_coarse", "mx_mg_coarse") : name_of<R>("mg_up", "mx_mg_up"), ncell(L[l].G),
+               (k_mg_up<R><<<grid_pairs(L[l].G), kBlock, 0, st>>>(L[l], ec, last ? 0 : L[l + 1].G.P, 0, a.F, a.sc,
+                                                                  a.partials)));
     }
-    for (int l = nlev - 2; l >= 0; --l, ++n)
-        TRACED(tr, "mg_up", ncell(L[l].G),
-               (k_mg_up<<<grid_tiles(L[l].G, a.tiles_per_block), kBlock, 0, st>>>(L[l], L[l + 1].e2, L[l + 1].G.P, L[l].e2,
-                                                             l == 0, a)));
     return n;
 }
 
-// One CG iteration after the first preconditioning: p = z + beta p and q = A p;
-// x, r updated together with the first step of the next V-cycle; the rest of
-// the V-cycle. Returns the number of kernels launched.
-int launch_cg_iter(const StepArgs &a, Level *L, int nlev, int ncoarse, double *x, cudaStream_t st,
+// the finest level's up half of the red-black iteration
+template <class R>
+void rb_up(const StepArgs &a, const LevelT<R> *L, cudaStream_t st, Tracer *tr)
+{
+    TRACED(tr, name_of<R>("rb_up", "mx_rb_up"), ncell(L[0].G),
+           (k_rb_up<R><<<grid_pair_tiles(L[0].G, a.tiles_per_block), kBlock, 0, st>>>(L[0], L[1].e2, L[1].G.P, a.F,
+                                                                                      a.sc, a.partials)));
+}
+
+}  // namespace
+
+template <class R>
+int launch_vcycle(const StepArgs &a, const LevelT<R> *L, int nlev, cudaStream_t st, Tracer *tr)
+{
+    int n = 0;
+    if (nlev > 1) {
+        TRACED(tr, name_of<R>("mg_down", "mx_mg_down"), ncell(L[0].G),
+               (k_mg_down<false, R><<<grid_pairs(L[0].G), kBlock, 0, st>>>(L[0], L[1], a.F, a.sc)));
+        n = 1 + vcycle_below<R>(a, L, nlev, st, tr);
+    }
+    const R *ec = nlev > 1 ? L[1].e2 : nullptr;
+    TRACED(tr, name_of<R>("mg_up", "mx_mg_up"), ncell(L[0].G),
+           (k_mg_up<R><<<grid_pair_tiles(L[0].G, a.tiles_per_block), kBlock, 0, st>>>(
+               L[0], ec, nlev > 1 ? L[1].G.P : 0, 1, a.F, a.sc, a.partials)));
+    return n + 1;
+}
+
+template <class R>
+int launch_cg_start(const StepArgs &a, const LevelT<R> *L, int nlev, cudaStream_t st, Tracer *tr)
+{
+    if (nlev == 1) {
+        TRACED(tr, name_of<R>("rb_start", "mx_rb_start"), ncell(a.G),
+               (k_rb_start<R><<<grid_pair_tiles(a.G, a.tiles_per_block), kBlock, 0, st>>>(L[0], a.sc, a.partials)));
+        return 1;
+    }
+    TRACED(tr, name_of<R>("mg_down", "mx_mg_down"), ncell(a.G),
+           (k_mg_down<true, R><<<grid_pairs(a.G), kBlock, 0, st>>>(L[0], L[1], a.F, a.sc)));
+    const int n = vcycle_below<R>(a, L, nlev, st, tr);
+    rb_up<R>(a, L, st, tr);
+    return n + 2;
+}
+
+template <class R>
+int launch_cg_iter(const StepArgs &a, const LevelT<R> *L, int nlev, const CgVecT<R> &v, double tol2, cudaStream_t st,
                    Tracer *tr)
 {
-    TRACED(tr, "cg_pspmv", ncell(a.G), (k_cg_pspmv<<<grid_tiles(a.G, a.tiles_per_block), kBlock, 0, st>>>(a, L[0])));
+    const dim3 grid = grid_pair_tiles(a.G, a.tiles_per_block);
+    TRACED(tr, name_of<R>("cg_pspmv", "mx_pspmv"), ncell(a.G),
+           (k_cg_pspmv<R><<<grid, kBlock, 0, st>>>(L[0], v, a.sc, a.partials)));
     if (nlev == 1) {
-        TRACED(tr, "cg_update_single", ncell(a.G),
-               (k_cg_update_single<<<grid_tiles(a.G, a.tiles_per_block), kBlock, 0, st>>>(a, L[0], x)));
+        TRACED(tr, name_of<R>("cg_update_single", "mx_update_single"), ncell(a.G),
+               (k_cg_update_single<R><<<grid, kBlock, 0, st>>>(L[0], v, a.sc, a.partials, tol2)));
         return 2;
     }
-    TRACED(tr, "cg_update_down", ncell(a.G),
-           (k_cg_update_down<<<grid_tiles(a.G, a.tiles_per_block), kBlock, 0, st>>>(a, L[0], L[1], x)));
-    return 2 + launch_vcycle_rest(a, L, nlev, ncoarse, st, tr);
+    TRACED(tr, name_of<R>("cg_update_down", "mx_update_down"), ncell(a.G),
+           (k_cg_update_down<R><<<grid, kBlock, 0, st>>>(L[0], L[1], v, a.F, a.sc, a.partials, tol2)));
+    const int n = vcycle_below<R>(a, L, nlev, st, tr);
+    rb_up<R>(a, L, st, tr);
+    return n + 3;
 }
+
+template <class R>
+void launch_correct(const StepArgs &a, const LevelT<R> &L, const SolveT<R> &v, double *ppout, cudaStream_t st,
+                    Tracer *tr)
+{
+    TRACED(tr, "correct", ncell(a.G), (k_correct<R><<<grid_of(a.G), kBlock, 0, st>>>(a, L, v, ppout)));
+}
+
+#define INSTANTIATE(R)                                                                                              \
+    template void launch_mg_coarsen<R>(const LevelT<R> &, const LevelT<R> &, cudaStream_t, Tracer *);               \
+    template int launch_vcycle<R>(const StepArgs &, const LevelT<R> *, int, cudaStream_t, Tracer *);                \
+    template int launch_cg_start<R>(const StepArgs &, const LevelT<R> *, int, cudaStream_t, Tracer *);              \
+    template int launch_cg_iter<R>(const StepArgs &, const LevelT<R> *, int, const CgVecT<R> &, double,             \
+                                   cudaStream_t, Tracer *);                                                         \
+    template void launch_correct<R>(const StepArgs &, const LevelT<R> &, const SolveT<R> &, double *, cudaStream_t, \
+                                    Tracer *);
+INSTANTIATE(double)
+INSTANTIATE(float)
+#undef INSTANTIATE
 
 namespace {
 
@@ -642,7 +709,10 @@ __global__ void k_fcg_pspmv(StepArgs a, Level L)
     const double beta = sc->beta;
     const int bx = blockIdx.x, bz = blockIdx.y;
     Tile<1> &sp = tile_at<1>(sm, 0);
-    load_tile_fn<1, double>(sp, G, bx, bz, [&](int q, int, int) { return fma(beta, ld(&pold[q]), ld(&L.e2[q])); });
+    if (it == 0)
+        load_tile_fn<1, double>(sp, G, bx, bz, [&](int q, int, int) { return ld(&L.e2[q]); });
+    else
+        load_tile_fn<1, double>(sp, G, bx, bz, [&](int q, int, int) { return fma(beta, ld(&pold[q]), ld(&L.e2[q])); });
     __syncthreads();
     double acc[2] = {0.0, 0.0}, tot[2];
     int i, k;
@@ -715,8 +785,8 @@ int launch_net_guess(const StepArgs &a, const LevelT<R> &L, R *r, R *q, R *x, do
     return 2 + nk;
 }
 
-int launch_fcg_iter(const StepArgs &a, Level *L, int nlev, int ncoarse, double *x, gea_net *net,
-                    float *dense_r, float *dense_e, double *s_buf, cudaStream_t st, Tracer *tr)
+int launch_fcg_iter(const StepArgs &a, Level *L, int nlev, double *x, gea_net *net, float *dense_r,
+                    float *dense_e, double *s_buf, cudaStream_t st, Tracer *tr)
 {
     const Geom &G = L[0].G;
     TRACED(tr, "fcg_stage_in", ncell(G), (k_fcg_stage_in<<<grid_of(G), kBlock, 0, st>>>(L[0], dense_r, a.sc)));
@@ -732,7 +802,7 @@ int launch_fcg_iter(const StepArgs &a, Level *L, int nlev, int ncoarse, double *
     Level M[kMaxLevels];
     for (int l = 0; l < nlev; ++l) M[l] = L[l];
     M[0].r = M[0].r_alt = s_buf;
-    const int nv = launch_vcycle(a, M, nlev, ncoarse, st, tr);
+    const int nv = launch_vcycle<double>(a, M, nlev, st, tr);
     TRACED(tr, "fcg_out", ncell(G),
            (k_fcg_out<<<grid_of(G), kBlock, 0, st>>>(L[0], dense_e, a.q, a.sc, a.partials)));
     TRACED(tr, "fcg_pspmv", ncell(G), (k_fcg_pspmv<<<grid_of(G), kBlock, 0, st>>>(a, L[0])));
@@ -748,11 +818,6 @@ template int launch_net_guess<double>(const StepArgs &, const LevelT<double> &, 
                                       double, gea_net *, float *, float *, cudaStream_t, Tracer *);
 template int launch_net_guess<float>(const StepArgs &, const LevelT<float> &, float *, float *, float *, double,
                                      gea_net *, float *, float *, cudaStream_t, Tracer *);
-
-void launch_correct(const StepArgs &a, cudaStream_t st, Tracer *tr)
-{
-    TRACED(tr, "correct", ncell(a.G), (k_correct<<<grid_of(a.G), kBlock, 0, st>>>(a)));
-}
 
 void launch_loop_ctl(Scal *sc, cudaGraphConditionalHandle h, bool graph, int which,
                      int maxtrips, int body_launches, cudaStream_t st, Tracer *tr)

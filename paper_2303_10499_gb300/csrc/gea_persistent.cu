@@ -33,10 +33,10 @@ const PersistOps &persist_ops(int shape)
 size_t persist_args_bytes(int mixed) { return mixed ? sizeof(PersistArgs) + sizeof(MixedPersist) : sizeof(PersistArgs); }
 
 void persist_args_fill_mixed(void *dst, const StepArgs a[2], const Level &L0, const MixedArgs &m,
-                             const LevelF *Lf, int nlev, int ncoarse, int n_corr, int jac_maxit, int cg_maxit,
+                             const LevelF *Lf, int nlev, int n_corr, int jac_maxit, int cg_maxit,
                              int first_slot, int nsteps, long long wait_polls)
 {
-    persist_args_fill(dst, a, &L0, 1, ncoarse, n_corr, jac_maxit, cg_maxit, first_slot, nsteps, wait_polls);
+    persist_args_fill(dst, a, &L0, 1, n_corr, jac_maxit, cg_maxit, first_slot, nsteps, wait_polls);
     MixedPersist X;
     memset(&X, 0, sizeof(X));
     X.m = m;
@@ -45,7 +45,7 @@ void persist_args_fill_mixed(void *dst, const StepArgs a[2], const Level &L0, co
     memcpy(static_cast<char *>(dst) + sizeof(PersistArgs), &X, sizeof(X));
 }
 
-void persist_args_fill(void *dst, const StepArgs a[2], const Level *L, int nlev, int ncoarse, int n_corr,
+void persist_args_fill(void *dst, const StepArgs a[2], const Level *L, int nlev, int n_corr,
                        int jac_maxit, int cg_maxit, int first_slot, int nsteps, long long wait_polls)
 {
     PersistArgs P;
@@ -54,7 +54,6 @@ void persist_args_fill(void *dst, const StepArgs a[2], const Level *L, int nlev,
     P.a[1] = a[1];
     for (int l = 0; l < nlev && l < kMaxLevels; ++l) P.L[l] = L[l];
     P.nlev = nlev;
-    P.ncoarse = ncoarse;
     P.nsteps = nsteps;
     P.first_slot = first_slot;
     P.n_corr = n_corr;

@@ -203,6 +203,15 @@ __device__ __forceinline__ void for_tiles(const Grp &g, const Geom &G, F f)
     for (int t = g.rank; t < nt; t += g.nb) f(t % tx, t / tx);
 }
 
+// the tiles of the red-black phases: BX pairs of cells wide
+template <class F>
+__device__ __forceinline__ void for_pair_tiles(const Grp &g, const Geom &G, F f)
+{
+    const int tx = (pairs_of(G) + BX - 1) / BX, tz = (G.nz + BZ - 1) / BZ;
+    const int nt = tx * tz;
+    for (int t = g.rank; t < nt; t += g.nb) f(t % tx, t / tx);
+}
+
 __device__ __forceinline__ bool stop(const Scal *) { return s_stop != 0; }
 
 // End of a step: its counters into the block's copy and, from block rank 0,
@@ -231,6 +240,94 @@ __device__ __forceinline__ void end_step(const Grp &g)
             }
             gs->last_status = 0;
             gs->press_ns = c.press_ns;
+        }
+    }
+}
+
+// The pressure solve from the residual L[0].r (gea_tiles_body.cuh: red-black
+// multigrid CG) to the relative residual tol2 (squared), after fin_helm; the
+// increment is left in v.x.
+template <class R>
+__device__ __forceinline__ void pressure_solve(const Grp &g, const LevelT<R> *L, int nlev, const CgVecT<R> &v,
+                                               const Phys &F, double tol2, int cg_maxit, double *partials, double *sm,
+                                               double *red)
+{
+    Scal *sc = &s_ctl;
+    const Geom &G = L[0].G;
+    auto go = [&] { return s_stop == 0 && !sc->done[LOOP_CG]; };
+    auto to_rz = [&](const double (&t)[1]) { fin_rz(sc, t); };
+    // the V-cycle below the finest level's down half, then its up half
+    auto vcycle = [&] {
+        R none[1] = {(R)0};
+        for (int l = 1; l + 1 < nlev; ++l) {
+            for_pair_tiles(g, L[l].G, [&](int bx, int bz) {
+                ph_mg_down<false, R>(L[l], L[l + 1], nullptr, F, sm, bx, bz);
+            });
+            gbar(g);
+        }
+        for (int l = nlev - 1; l >= 1; --l) {
+            const R *ec = l == nlev - 1 ? nullptr : L[l + 1].e2;
+            const int Pc = l == nlev - 1 ? 0 : L[l + 1].G.P;
+            for_pair_tiles(g, L[l].G, [&](int bx, int bz) {
+                ph_mg_up<R>(L[l], L[l].r, ec, Pc, L[l].e2, F, sm, bx, bz, none);
+            });
+            gbar(g);
+        }
+        R acc[1] = {(R)0};
+        const R *rb = black_res(L[0], sc->cg_it);
+        for_pair_tiles(g, G, [&](int bx, int bz) { ph_rb_up<R>(L[0], rb, L[1].e2, L[1].G.P, L[0].e2, F, bx, bz, acc); });
+        rbar<1>(g, acc, red, partials, to_rz);
+    };
+    if (!go()) return;
+    if (nlev == 1) {
+        R acc[1] = {(R)0};
+        for_pair_tiles(g, G, [&](int bx, int bz) { ph_rb_start<R>(L[0], black_res(L[0], 0), L[0].e2, sm, bx, bz, acc); });
+        rbar<1>(g, acc, red, partials, to_rz);
+    } else {
+        for_pair_tiles(g, G, [&](int bx, int bz) {
+            ph_mg_down<true, R>(L[0], L[1], black_res(L[0], 0), F, sm, bx, bz);
+        });
+        gbar(g);
+        vcycle();
+    }
+    while (go()) {
+        const int it = sc->cg_it;
+        const R *pold = (it & 1) ? v.p1 : v.p0;
+        R *pnew = (it & 1) ? v.p0 : v.p1;
+        {
+            const double beta = sc->beta;
+            R acc[1] = {(R)0};
+            for_pair_tiles(g, G, [&](int bx, int bz) {
+                ph_pspmv<R>(L[0], L[0].e2, pold, pnew, v.q, beta, it == 0, sm, bx, bz, acc);
+            });
+            rbar<1>(g, acc, red, partials, [&](const double (&t)[1]) { fin_pq(sc, t); });
+        }
+        const double alpha = sc->alpha;
+        auto cap = [&] {
+            if (!sc->done[LOOP_CG] && !sc->status && sc->cg_it >= cg_maxit) sc->status = GEA_ERR_NOCONV;
+        };
+        if (nlev == 1) {
+            R acc[2] = {(R)0, (R)0};
+            for_pair_tiles(g, G, [&](int bx, int bz) {
+                ph_update_single<R>(L[0], v.q, black_res(L[0], 0), L[0].e2, v.x, pnew, alpha, it == 0, bx, bz, acc);
+            });
+            rbar<2>(g, acc, red, partials, [&](const double (&t)[2]) {
+                const double t0[1] = {t[0]}, t1[1] = {t[1]};
+                fin_update(sc, t0, tol2);
+                fin_rz(sc, t1);
+                cap();
+            });
+        } else {
+            R acc[1] = {(R)0};
+            for_pair_tiles(g, G, [&](int bx, int bz) {
+                ph_update_down<R>(L[0], L[1], v.q, black_res(L[0], it), black_res(L[0], it + 1), v.x, pnew, alpha,
+                                  it == 0, F, sm, bx, bz, acc);
+            });
+            rbar<1>(g, acc, red, partials, [&](const double (&t)[1]) {
+                fin_update(sc, t, tol2);
+                cap();
+            });
+            if (go()) vcycle();
         }
     }
 }
@@ -321,7 +418,7 @@ __device__ bool run_step(const PersistArgs &P, const StepArgs &a, const Grp &g, 
     for_tiles(g, G, [&](int bx, int bz) { ph_H(a, u1, w1, sm, bx, bz); });
     gbar(g);
     for (int l = 0; l + 1 < nlev; ++l) {
-        for_tiles(g, L[l + 1].G, [&](int bx, int bz) { ph_coarsen(L[l], L[l + 1], a.F.omega, bx, bz); });
+        for_tiles(g, L[l + 1].G, [&](int bx, int bz) { ph_coarsen(L[l], L[l + 1], bx, bz); });
         gbar(g);
     }
     if (stop(sc)) return false;
@@ -336,91 +433,22 @@ __device__ bool run_step(const PersistArgs &P, const StepArgs &a, const Grp &g, 
             for_tiles(g, G, [&](int bx, int bz) { ph_H(a, a.N.u, a.N.w, sm, bx, bz); });
             gbar(g);
         }
+        const double *x0 = pp_in(a, c, P.n_corr);
         unsigned long long t0 = 0;
         if (g.rank == 0 && tid_of() == 0) t0 = globaltimer();
         {
             double acc[2] = {0.0, 0.0};
-            const double *xin = c == 0 ? a.S.pp : a.N.pp;
-            for_tiles(g, G, [&](int bx, int bz) { ph_helm_rhs(a, L[0], xin, a.N.pp, sm, bx, bz, acc); });
+            for_tiles(g, G, [&](int bx, int bz) { ph_helm_rhs(a, L[0], x0, nullptr, sm, bx, bz, acc); });
             rbar<2>(g, acc, red, a.partials, [&](const double (&t)[2]) { fin_helm(sc, t, a.cg_rtol2, c); });
         }
-        // z = M^-1 r_0 (one V(1,1)-cycle), then the iterations
-        auto vcycle_levels = [&](int lfirst) {
-            for (int l = lfirst; l + 1 < nlev; ++l) {
-                for_tiles(g, L[l].G, [&](int bx, int bz) { ph_mg_down(L[l], L[l + 1], a.F.omega, sm, bx, bz); });
-                gbar(g);
-            }
-            const Level &C = L[nlev - 1];
-            for (int s = 0; s < P.ncoarse; ++s) {
-                double *out = ((P.ncoarse - 1 - s) % 2 == 0) ? C.e2 : C.e;
-                const double *in = (out == C.e2) ? C.e : C.e2;
-                for_tiles(g, C.G, [&](int bx, int bz) { ph_mg_coarse(C, in, out, s == 0, sm, bx, bz); });
-                gbar(g);
-            }
-            const double *res0 = res_of(L[0], sc->cg_it);
-            for (int l = nlev - 2; l >= 0; --l) {
-                double acc[1] = {0.0};
-                const double *res = l == 0 ? res0 : L[l].r;
-                for_tiles(g, L[l].G, [&](int bx, int bz) {
-                    ph_mg_up(L[l], res, L[l + 1].e2, L[l + 1].G.P, L[l].e2, sm, bx, bz, acc);
-                });
-                if (l > 0) gbar(g);
-                else rbar<1>(g, acc, red, a.partials, [&](const double (&t)[1]) { fin_rz(sc, t); });
-            }
-        };
-        if (!stop(sc) && !sc->done[LOOP_CG]) {
-            if (nlev == 1) {
-                double acc[1] = {0.0};
-                for_tiles(g, G, [&](int bx, int bz) { ph_mg_single(L[0], L[0].e2, sm, bx, bz, acc); });
-                rbar<1>(g, acc, red, a.partials, [&](const double (&t)[1]) { fin_rz(sc, t); });
-            } else {
-                vcycle_levels(0);
-            }
-        }
-        while (!stop(sc) && !sc->done[LOOP_CG]) {
-            // p = z + beta p, q = A p
-            const int it = sc->cg_it;
-            const double *pold = (it & 1) ? a.p1 : a.p0;
-            double *pnew = (it & 1) ? a.p0 : a.p1;
-            {
-                const double beta = sc->beta;
-                double acc[1] = {0.0};
-                for_tiles(g, G, [&](int bx, int bz) { ph_pspmv<double>(L[0], pold, pnew, a.q, beta, sm, bx, bz, acc); });
-                rbar<1>(g, acc, red, a.partials, [&](const double (&t)[1]) { fin_pq(sc, t); });
-            }
-            // x += alpha p, r -= alpha q, with the first step of the next V-cycle
-            const double alpha = sc->alpha;
-            auto cap = [&] {
-                if (!sc->done[LOOP_CG] && !sc->status && sc->cg_it >= P.cg_maxit) sc->status = GEA_ERR_NOCONV;
-            };
-            if (nlev == 1) {
-                double acc[2] = {0.0, 0.0};
-                for_tiles(g, G, [&](int bx, int bz) {
-                    ph_update_single<double>(L[0], a.q, res_of(L[0], it), res_of(L[0], it + 1), a.N.pp,
-                                             pnew, alpha, sm, bx, bz, acc);
-                });
-                rbar<2>(g, acc, red, a.partials, [&](const double (&t)[2]) {
-                    const double t0[1] = {t[0]}, t1[1] = {t[1]};
-                    fin_update(sc, t0, a.cg_rtol2);
-                    fin_rz(sc, t1);
-                    cap();
-                });
-            } else {
-                double acc[1] = {0.0};
-                for_tiles(g, G, [&](int bx, int bz) {
-                    ph_update_down<double>(L[0], L[1], a.q, res_of(L[0], it), res_of(L[0], it + 1), a.N.pp,
-                                           pnew, alpha, a.F.omega, sm, bx, bz, acc);
-                });
-                rbar<1>(g, acc, red, a.partials, [&](const double (&t)[1]) {
-                    fin_update(sc, t, a.cg_rtol2);
-                    cap();
-                });
-                if (!stop(sc) && !sc->done[LOOP_CG]) vcycle_levels(1);
-            }
-        }
+        pressure_solve<double>(g, L, nlev, cg_vecs(a), a.F, a.cg_rtol2, P.cg_maxit, a.partials, sm, red);
         if (stop(sc)) return false;
         if (g.rank == 0 && tid_of() == 0) sc->press_ns += globaltimer() - t0;
-        for_tiles(g, G, [&](int bx, int bz) { ph_correct(a, sm, bx, bz); });
+        {
+            const SolveT<double> v{x0, nullptr, cg_vecs(a).x};
+            const bool dx = sc->cg_it > 0;
+            for_tiles(g, G, [&](int bx, int bz) { ph_correct<double>(a, L[0], v, dx, pp_out(a, c, P.n_corr), sm, bx, bz); });
+        }
         if (c + 1 < P.n_corr) gbar(g);
     }
     end_step(g);
@@ -514,7 +542,7 @@ __device__ bool run_step_mixed(const PersistArgs &P, const MixedPersist &X, cons
     for_tiles(g, G, [&](int bx, int bz) { ph_H(a, a.ua, a.wa, sm, bx, bz); });
     gbar(g);
     for (int l = 0; l + 1 < nlev; ++l) {
-        for_tiles(g, L[l + 1].G, [&](int bx, int bz) { ph_coarsen<float>(L[l], L[l + 1], a.F.omega, bx, bz); });
+        for_tiles(g, L[l + 1].G, [&](int bx, int bz) { ph_coarsen<float>(L[l], L[l + 1], bx, bz); });
         gbar(g);
     }
     if (stop(sc)) return false;
@@ -525,99 +553,27 @@ __device__ bool run_step_mixed(const PersistArgs &P, const MixedPersist &X, cons
             for_tiles(g, G, [&](int bx, int bz) { ph_H(a, a.N.u, a.N.w, sm, bx, bz); });
             gbar(g);
         }
+        const double *x0 = pp_in(a, c, P.n_corr);
         unsigned long long t0 = 0;
         if (g.rank == 0 && tid_of() == 0) t0 = globaltimer();
         {
             double acc[2] = {0.0, 0.0};
-            const double *xin = c == 0 ? a.S.pp : a.N.pp;
             for_tiles(g, G, [&](int bx, int bz) {
-                ph_helm_rhs_t<true>(a, L0, L[0], m, xin, a.N.pp, sm, bx, bz, acc);
+                ph_helm_rhs_t<true>(a, L0, L[0], m, x0, nullptr, false, sm, bx, bz, acc);
             });
             rbar<2>(g, acc, red, a.partials, [&](const double (&t)[2]) {
                 fin_helm_mixed(sc, t, a.cg_rtol2, c);
             });
         }
-        auto vcycle_levels = [&](int lfirst) {
-            for (int l = lfirst; l + 1 < nlev; ++l) {
-                for_tiles(g, L[l].G, [&](int bx, int bz) {
-                    ph_mg_down<float>(L[l], L[l + 1], a.F.omega, sm, bx, bz);
-                });
-                gbar(g);
-            }
-            const LevelF &C = L[nlev - 1];
-            for (int s = 0; s < P.ncoarse; ++s) {
-                float *out = ((P.ncoarse - 1 - s) % 2 == 0) ? C.e2 : C.e;
-                const float *in = (out == C.e2) ? C.e : C.e2;
-                for_tiles(g, C.G, [&](int bx, int bz) { ph_mg_coarse<float>(C, in, out, s == 0, sm, bx, bz); });
-                gbar(g);
-            }
-            const float *res0 = res_of(L[0], sc->cg_it);
-            for (int l = nlev - 2; l >= 0; --l) {
-                float acc[1] = {0.0f};
-                const float *res = l == 0 ? res0 : L[l].r;
-                for_tiles(g, L[l].G, [&](int bx, int bz) {
-                    ph_mg_up<float>(L[l], res, L[l + 1].e2, L[l + 1].G.P, L[l].e2, sm, bx, bz, acc);
-                });
-                if (l > 0) gbar(g);
-                else rbar<1>(g, acc, red, a.partials, [&](const double (&t)[1]) { fin_rz(sc, t); });
-            }
-        };
-        if (!stop(sc) && !sc->done[LOOP_CG]) {
-            if (nlev == 1) {
-                float acc[1] = {0.0f};
-                for_tiles(g, G, [&](int bx, int bz) { ph_mg_single<float>(L[0], L[0].e2, sm, bx, bz, acc); });
-                rbar<1>(g, acc, red, a.partials, [&](const double (&t)[1]) { fin_rz(sc, t); });
-            } else {
-                vcycle_levels(0);
-            }
-        }
-        while (!stop(sc) && !sc->done[LOOP_CG]) {
-            const int it = sc->cg_it;
-            const float *pold = (it & 1) ? m.p1 : m.p0;
-            float *pnew = (it & 1) ? m.p0 : m.p1;
-            {
-                const double beta = sc->beta;
-                float acc[1] = {0.0f};
-                for_tiles(g, G, [&](int bx, int bz) {
-                    ph_pspmv<float>(L[0], pold, pnew, m.q, beta, sm, bx, bz, acc);
-                });
-                rbar<1>(g, acc, red, a.partials, [&](const double (&t)[1]) { fin_pq(sc, t); });
-            }
-            const double alpha = sc->alpha;
-            auto cap = [&] {
-                if (!sc->done[LOOP_CG] && !sc->status && sc->cg_it >= P.cg_maxit) sc->status = GEA_ERR_NOCONV;
-            };
-            if (nlev == 1) {
-                float acc[2] = {0.0f, 0.0f};
-                for_tiles(g, G, [&](int bx, int bz) {
-                    ph_update_single<float>(L[0], m.q, res_of(L[0], it), res_of(L[0], it + 1), m.x, pnew, alpha,
-                                            sm, bx, bz, acc);
-                });
-                rbar<2>(g, acc, red, a.partials, [&](const double (&t)[2]) {
-                    const double t0[1] = {t[0]}, t1[1] = {t[1]};
-                    fin_update(sc, t0, m.tol2);
-                    fin_rz(sc, t1);
-                    cap();
-                });
-            } else {
-                float acc[1] = {0.0f};
-                for_tiles(g, G, [&](int bx, int bz) {
-                    ph_update_down<float>(L[0], L[1], m.q, res_of(L[0], it), res_of(L[0], it + 1), m.x, pnew,
-                                          alpha, a.F.omega, sm, bx, bz, acc);
-                });
-                rbar<1>(g, acc, red, a.partials, [&](const double (&t)[1]) {
-                    fin_update(sc, t, m.tol2);
-                    cap();
-                });
-                if (!stop(sc) && !sc->done[LOOP_CG]) vcycle_levels(1);
-            }
-        }
+        pressure_solve<float>(g, L, nlev, cg_vecs(m), a.F, m.tol2, P.cg_maxit, a.partials, sm, red);
         if (stop(sc)) return false;
-        // p' += dp, then the FP64 correction
-        for_tiles(g, G, [&](int bx, int bz) { ph_p_apply(a, m, bx, bz); });
-        gbar(g);
         if (g.rank == 0 && tid_of() == 0) sc->press_ns += globaltimer() - t0;
-        for_tiles(g, G, [&](int bx, int bz) { ph_correct(a, sm, bx, bz); });
+        {
+            // p' += dp, and the FP64 correction
+            const SolveT<float> v{x0, nullptr, cg_vecs(m).x};
+            const bool dx = sc->cg_it > 0;
+            for_tiles(g, G, [&](int bx, int bz) { ph_correct<float>(a, L[0], v, dx, pp_out(a, c, P.n_corr), sm, bx, bz); });
+        }
         if (c + 1 < P.n_corr) gbar(g);
     }
     end_step(g);
@@ -784,7 +740,7 @@ int persistent_max_blocks()
     return per_sm * sms;
 }
 
-cudaError_t launch_persistent(const StepArgs a[2], const Level *L, int nlev, int ncoarse, int n_corr,
+cudaError_t launch_persistent(const StepArgs a[2], const Level *L, int nlev, int n_corr,
                               int jac_maxit, int cg_maxit, int first_slot, int nsteps, int blocks,
                               long long wait_polls, cudaStream_t st)
 {
@@ -795,7 +751,6 @@ cudaError_t launch_persistent(const StepArgs a[2], const Level *L, int nlev, int
     P.a[1] = a[1];
     for (int l = 0; l < nlev; ++l) P.L[l] = L[l];
     P.nlev = nlev;
-    P.ncoarse = ncoarse;
     P.nsteps = nsteps;
     P.first_slot = first_slot;
     P.n_corr = n_corr;
@@ -822,7 +777,7 @@ int persistent_mixed_max_blocks()
 }
 
 cudaError_t launch_persistent_mixed(const StepArgs a[2], const Level &L0, const MixedArgs &m, const LevelF *Lf,
-                                    int nlev, int ncoarse, int n_corr, int jac_maxit, int cg_maxit,
+                                    int nlev, int n_corr, int jac_maxit, int cg_maxit,
                                     int first_slot, int nsteps, int blocks, long long wait_polls,
                                     cudaStream_t st)
 {
@@ -833,7 +788,6 @@ cudaError_t launch_persistent_mixed(const StepArgs a[2], const Level &L0, const 
     P.a[1] = a[1];
     P.L[0] = L0;
     P.nlev = 1;
-    P.ncoarse = ncoarse;
     P.nsteps = nsteps;
     P.first_slot = first_slot;
     P.n_corr = n_corr;

@@ -41,11 +41,17 @@ using Tile = R[BZ + 2 * H][BX + 2 * H];
 constexpr int kT1 = (BZ + 2) * (BX + 2);   // doubles of a halo-1 tile
 constexpr int kT2 = (BZ + 4) * (BX + 4);   // doubles of a halo-2 tile
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
+constexpr int kPW = BX + 2;                // columns of a pair tile (red-black phases)
+constexpr int kPH2 = (BZ + 4) * kPW;       // doubles of a pair tile with two halo rows
+constexpr int kPH1 = (BZ + 2) * kPW;       // with one
+constexpr int kFaces = BZ * (BX + 1) + (BZ + 1) * BX;   // x- and z-face values of a tile
+constexpr int kCorrectSmem = 2 * kT1 + cmax(kFaces, kT2);   // of the correction
 // the largest phase footprint: four halo-1 tiles (pressure right-hand
 // side), three halo-2 tiles (enthalpy right-hand side), two halo-1 tiles and
-// the x- and z-face rows (EOS, correction) or a tile of residuals (restriction)
+// the face values or a halo-2 tile (EOS, correction), or two pair tiles and
+// a tile of residuals (V-cycle)
 constexpr int kTileSmem =
-    cmax(cmax(4 * kT1, 3 * kT2), 2 * kT1 + cmax(BZ * (BX + 1) + (BZ + 1) * BX, BZ * BX));
+    cmax(cmax(4 * kT1, 3 * kT2), cmax(kCorrectSmem, kPH2 + kPH1 + BZ * BX));
 
 template <int H, class R = double>
 __device__ __forceinline__ Tile<H, R> &tile_at(double *sm, int slot)
@@ -654,7 +660,7 @@ __device__ __forceinline__ void ph_enth(const StepArgs &a, const double *hin, do
 // T^{n+1} = T^n + (h^{n+1} - h^n)/cp; psi = 1/(R T^{n+1}); rho^{n+2/3} = p^n/(R T^{n+1})
 // (eq. step3_3sd); face coefficients D_f = dt rho2_f / rho1_f (linear face
 // averages); the fine Helmholtz operator c = psi/dt, a_f = D_f |A_f|/(V Delta_f),
-// d = c + sum a_f and omega/d. h1 holds h^{n+1}.
+// d = c + sum a_f and 1/d. h1 holds h^{n+1}.
 // MX: h^{n+1} = h^n + dh, and FP32 copies of the fine operator into L32.
 template <bool MX>
 __device__ __forceinline__ void ph_eos_t(const StepArgs &a, const Level &L, const LevelF &L32,
@@ -711,11 +717,12 @@ __device__ __forceinline__ void ph_eos_t(const StepArgs &a, const Level &L, cons
         const double d = c + (Dw + De) * ix2 + (Ds + Dn) * iz2;
         L.c[q] = c;
         L.d[q] = d;
-        L.wd[q] = F.omega / d;
+        const double id = 1.0 / d;
+        L.wd[q] = id;
         if (MX) {
             L32.c[q] = (float)c;
             L32.d[q] = (float)d;
-            L32.wd[q] = (float)(F.omega / d);
+            L32.wd[q] = (float)id;
             L32.ax[k * G.P + i] = (float)(Dw * ix2);
             L32.az[k * G.P + i] = (float)(Ds * iz2);
             if (i == G.nx - 1) L32.ax[k * G.P + G.nx] = 0.0f;
@@ -731,12 +738,16 @@ __device__ __forceinline__ void ph_eos(const StepArgs &a, const Level &L, const 
     ph_eos_t<false>(a, L, LevelF{}, h1, nullptr, sm, bx, bz);
 }
 
-// Galerkin coarsening with piecewise-constant transfer: the coarse reaction
-// term averages the four fine ones, a coarse face coefficient is a quarter
-// of the sum of its two fine faces. (bx, bz) is a tile of the coarse level.
+// Coarse operator for piecewise-constant transfer: the coarse reaction term
+// averages the four fine ones; a coarse face coefficient is an eighth of the
+// sum of its two fine faces. The Galerkin product would give a quarter,
+// which makes the coarse Laplacian twice too stiff on every level (the jump
+// of a piecewise-constant function over one fine spacing stands for a slope
+// over a coarse one) and the coarse correction too small; an eighth is the
+// operator discretised on the coarse grid. (bx, bz) is a tile of the coarse
+// level.
 template <class R>
-__device__ __forceinline__ void ph_coarsen(const LevelT<R> &f, const LevelT<R> &c, double omega, int bx,
-                                           int bz)
+__device__ __forceinline__ void ph_coarsen(const LevelT<R> &f, const LevelT<R> &c, int bx, int bz)
 {
     const Geom &G = c.G;
     int I, K;
@@ -744,12 +755,12 @@ __device__ __forceinline__ void ph_coarsen(const LevelT<R> &f, const LevelT<R> &
     const int Pf = f.G.P;
     const int q00 = (2 * K) * Pf + 2 * I;
     const int Q = cidx(G, I, K);
-    const R q4 = (R)0.25;
+    const R q4 = (R)0.25, q8 = (R)0.125;
     const R cc = q4 * (ld(&f.c[q00]) + ld(&f.c[q00 + 1]) + ld(&f.c[q00 + Pf]) + ld(&f.c[q00 + Pf + 1]));
-    const R aw = q4 * (ld(&f.ax[q00]) + ld(&f.ax[q00 + Pf]));
-    const R ae = q4 * (ld(&f.ax[q00 + 2]) + ld(&f.ax[q00 + Pf + 2]));
-    const R as = q4 * (ld(&f.az[q00]) + ld(&f.az[q00 + 1]));
-    const R an = q4 * (ld(&f.az[q00 + 2 * Pf]) + ld(&f.az[q00 + 2 * Pf + 1]));
+    const R aw = q8 * (ld(&f.ax[q00]) + ld(&f.ax[q00 + Pf]));
+    const R ae = q8 * (ld(&f.ax[q00 + 2]) + ld(&f.ax[q00 + Pf + 2]));
+    const R as = q8 * (ld(&f.az[q00]) + ld(&f.az[q00 + 1]));
+    const R an = q8 * (ld(&f.az[q00 + 2 * Pf]) + ld(&f.az[q00 + 2 * Pf + 1]));
     c.c[Q] = cc;
     c.ax[K * G.P + I] = aw;
     c.az[K * G.P + I] = as;
@@ -757,7 +768,7 @@ __device__ __forceinline__ void ph_coarsen(const LevelT<R> &f, const LevelT<R> &
     if (K == G.nz - 1) c.az[G.nz * G.P + I] = an;
     const R d = cc + aw + ae + as + an;
     c.d[Q] = d;
-    c.wd[Q] = (R)omega / d;
+    c.wd[Q] = (R)1 / d;
 }
 
 // ---------------------------------------------------------------------------
@@ -802,13 +813,13 @@ __device__ __forceinline__ void ph_H(const StepArgs &a, const double *U, const d
 // Right-hand side of the pressure equation,
 //   b_i = (rho^n_i + psi_i rho2_i g z_i)/dt
 //         - (1/V) sum_f D_f |A_f| [H_f . n + g z_f (rho2_N - rho2_i)/Delta_f],
-// the initial residual r = b - A x (x = xin, copied to xout) and p0 = 0.
+// and the initial residual r = b - A x (x = xin, copied to xout unless null).
 // acc += (b^2, r^2).
-// MX: r0 rounded to FP32 into L32.r (instead of L.r), and a zero pressure
-// increment and first CG direction of the FP32 solve.
+// MX: r0 rounded to FP32 into L32.r (instead of L.r), and with a learned guess
+// its increment m.x set to zero.
 template <bool MX>
 __device__ __forceinline__ void ph_helm_rhs_t(const StepArgs &a, const Level &L, const LevelF &L32,
-                                              const MixedArgs &m, const double *xin, double *xout,
+                                              const MixedArgs &m, const double *xin, double *xout, bool guess,
                                               double *sm, int bx, int bz, double (&acc)[2])
 {
     const Geom &G = a.G;
@@ -850,14 +861,12 @@ __device__ __forceinline__ void ph_helm_rhs_t(const StepArgs &a, const Level &L,
         const double b = fma(ld(&a.psi[q]) * r2q, gz, ld(&a.S.rho[q])) * F.idt - flux * G.iV;
         const double r = b - helm_apply<1>(hc, sx, y, x);
         a.b[q] = b;
-        xout[q] = sx[y][x];
         if (!MX) {
             L.r[q] = r;
-            a.p0[q] = 0.0;
+            if (xout) xout[q] = sx[y][x];
         } else {
             L32.r[q] = (float)r;
-            m.x[q] = 0.0f;
-            m.p0[q] = 0.0f;
+            if (guess) m.x[q] = 0.0f;
         }
         acc[0] = fma(b, b, acc[0]);
         acc[1] = fma(r, r, acc[1]);
@@ -869,307 +878,358 @@ __device__ __forceinline__ void ph_helm_rhs(const StepArgs &a, const Level &L, c
                                             double *xout, double *sm, int bx, int bz,
                                             double (&acc)[2])
 {
-    ph_helm_rhs_t<false>(a, L, LevelF{}, MixedArgs{}, xin, xout, sm, bx, bz, acc);
+    ph_helm_rhs_t<false>(a, L, LevelF{}, MixedArgs{}, xin, xout, false, sm, bx, bz, acc);
 }
 
-// p' <- p' + dp (mixed-precision path: the FP32 solve's increment).
-__device__ __forceinline__ void ph_p_apply(const StepArgs &a, const MixedArgs &m, int bx, int bz)
+// ---- pressure solve: red-black multigrid CG ----
+//
+// A cell (i, k) is black if i + k is even, red otherwise; the four neighbours
+// of a cell have the other colour, so either colour is relaxed exactly in
+// one pass. The solve is the conjugate gradient method preconditioned by a
+// V(1,1)-cycle whose smoother is red-black Gauss-Seidel: before the coarse
+// correction red then black, after it black then red (symmetric). On the
+// finest level the red cells are relaxed before the first iteration. Every
+// direction the cycle yields then leaves them relaxed, (A p)_red = 0, so the
+// iteration runs on the black half of the vectors alone, with the Schur
+// complement S = A_bb - A_br A_rr^-1 A_rb as its operator: the red part of a
+// direction is A_rr^-1 A_rb p_b on the fly, the red residual stays zero, and
+// the red part of the solution follows at the end from the black one.
+//
+// Why: FP64 issue bounds these phases. Against full vectors and a damped
+// Jacobi smoother (pspmv 7.3, update with pre-smoothing 12, post-smoothing 9
+// FP64 instructions per cell and iteration) the black half takes 7.1, 4.8
+// and 3, and red-black smoothing contracts better: with the halved coarse
+// faces (ph_coarsen) CG takes 9-11 iterations per ten decades where it took
+// 14 (4096 x 2048) to 38 (400 x 400 at 2.5 m).
+//
+// Layout: a black-half array keeps black cell (2 j + (k & 1), k) at k P + j, a
+// pair (j, k) being the cells 2 j and 2 j + 1 of row k. With s = k & 1 the
+// black cell j of row k has the red neighbours j - 1 + s (west), j + s (east)
+// and j (south, north), the red cell j the black ones j - s, j + 1 - s, j and
+// j: four-point stencils on the pair grid, without strided access. A tile is
+// BX pairs x BZ rows, one pair per thread. A cell beyond an odd nx is zero.
+
+// Pairs of a row.
+__host__ __device__ __forceinline__ int pairs_of(const Geom &G) { return (G.nx + 1) >> 1; }
+
+template <int H, class R>
+using PairTile = R[BZ + 2 * H][kPW];
+
+template <int H, class R>
+__device__ __forceinline__ PairTile<H, R> &pair_tile(double *sm, int at)
 {
-    int i, k;
-    if (!cell_of(a.G, bx, bz, i, k)) return;
-    const int q = cidx(a.G, i, k);
-    a.N.pp[q] = ld(&a.N.pp[q]) + (double)ld(&m.x[q]);
+    return *reinterpret_cast<PairTile<H, R> *>(reinterpret_cast<R *>(sm) + at);
 }
 
-// ---- V-cycle ----
+// The thread's pair (j, k); false outside the rows and pairs of the level.
+__device__ __forceinline__ bool pair_of(const Geom &G, int bx, int bz, int &j, int &k)
+{
+    j = bx * BX + threadIdx.x;
+    k = bz * BZ + threadIdx.y;
+    return j < pairs_of(G) && k < G.nz;
+}
 
-// Restriction step of a level: pre-smooth with one damped Jacobi sweep from
-// zero, e = (omega/d) r, and restrict the new residual r - A e (= (1-omega) r +
-// sum a e_N) by averaging the four fine cells of each coarse cell. (bx, bz)
-// is a tile of the fine level, whose sizes are even.
+// sum of the face coefficients of cell q times its four neighbours' values
 template <class R>
-__device__ __forceinline__ void ph_mg_down(const LevelT<R> &f, const LevelT<R> &c, double omega,
-                                           double *sm, int bx, int bz)
+__device__ __forceinline__ R faces4(const LevelT<R> &L, int q, R w, R e, R s, R n)
 {
-    const Geom &G = f.G;
-    Tile<1, R> &se = tile_at<1, R>(sm, 0);
-    R(*sres)[BX] = reinterpret_cast<R(*)[BX]>(reinterpret_cast<R *>(sm) + kT1);
-    int i, k;
+    R t = ld(&L.ax[q]) * w;
+    t = fma(ld(&L.ax[q + 1]), e, t);
+    t = fma(ld(&L.az[q]), s, t);
+    return fma(ld(&L.az[q + L.G.P]), n, t);
+}
+
+// Fills rows -H .. BZ + H - 1 and pairs -1 .. BX of a pair tile with
+// f(q, c) at the cells of one colour (RED: the red ones) inside the box
+// (q: cell index, c: pair index), zero elsewhere.
+template <int H, bool RED, class R, class Fn>
+__device__ __forceinline__ void fill_pairs(PairTile<H, R> &t, const Geom &G, int bx, int bz, Fn f)
+{
+    const int tid = threadIdx.x + threadIdx.y * BX;
+    for (int e = tid; e < (BZ + 2 * H) * kPW; e += NTHREADS) {
+        const int tk = e / kPW, tj = e - tk * kPW;
+        const int j = bx * BX - 1 + tj, k = bz * BZ - H + tk;
+        const int i = 2 * j + (RED ? 1 - (k & 1) : (k & 1));
+        t[tk][tj] = (j >= 0 && i < G.nx && k >= 0 && k < G.nz) ? (R)f(k * G.P + i, k * G.P + j, j, k) : (R)0;
+    }
+}
+
+// Same for values f(q, c, tk, tj) that combine the other colour's tile: only
+// the BX + 1 pairs of each row that the own cells' stencils reach. The red
+// pairs next to the black pairs 0 .. BX - 1 of a row are -1 + s .. BX - 1 + s,
+// the black ones next to the red pairs -s .. BX - s (tile columns one more).
+template <bool RED, class R, class Fn>
+__device__ __forceinline__ void fill_next(PairTile<1, R> &t, const Geom &G, int bx, int bz, Fn f)
+{
+    const int tid = threadIdx.x + threadIdx.y * BX;
+    for (int e = tid; e < (BZ + 2) * (BX + 1); e += NTHREADS) {
+        const int tk = e / (BX + 1);
+        const int k = bz * BZ - 1 + tk, s = k & 1;
+        const int tj = e - tk * (BX + 1) + (RED ? s : 1 - s);
+        const int j = bx * BX - 1 + tj;
+        const int i = 2 * j + (RED ? 1 - s : s);
+        t[tk][tj] = (j >= 0 && i < G.nx && k >= 0 && k < G.nz) ? (R)f(k * G.P + i, k * G.P + j, tk, tj, s) : (R)0;
+    }
+}
+
+// Coarse residual of the tile's rows from the threads' contributions v (the
+// residual of the pair's two cells after pre-smoothing): a quarter of the sum
+// over the two pairs of a coarse cell, which has the pair's index.
+template <class R>
+__device__ __forceinline__ void restrict_pairs(const LevelT<R> &c, R v, R *sres, int bx, int bz)
+{
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const bool in = cell_of(G, bx, bz, i, k);
-    const int q0 = in ? cidx(G, i, k) : 0;
-    HelmCoef<R> hc{};
-    R rq = 0;
-    auto fetch = [&] {   // ahead of the tile barrier
-        hc = helm_coef(f, q0, i, k);
-        rq = ld(&f.r[q0]);
-    };
-    if (kPrefetch && in) fetch();
-    load_tile_fn<1, R>(se, G, bx, bz, [&](int q, int, int) { return ld(&f.wd[q]) * ld(&f.r[q]); });
+    sres[ty * BX + tx] = v;
     __syncthreads();
-    if (in) {
-        if (!kPrefetch) fetch();
-        const int y = ty + 1, x = tx + 1;
-        R t = (R)(1.0 - omega) * rq;
-        t = fma(hc.aw, se[y][x - 1], t);
-        t = fma(hc.ae, se[y][x + 1], t);
-        t = fma(hc.as, se[y - 1][x], t);
-        t = fma(hc.an, se[y + 1][x], t);
-        f.e[q0] = se[y][x];
-        sres[ty][tx] = t;
-    }
-    __syncthreads();
-    // one thread per coarse cell: all four of its fine cells are inside the
-    // box or all outside
-    if (tx < BX / 2 && ty < BZ / 2) {
-        const int I = bx * (BX / 2) + tx, K = bz * (BZ / 2) + ty;
+    if (ty < BZ / 2) {
+        const int I = bx * BX + tx, K = bz * (BZ / 2) + ty;
         if (I < c.G.nx && K < c.G.nz)
-            c.r[cidx(c.G, I, K)] = (R)0.25 * ((sres[2 * ty][2 * tx] + sres[2 * ty][2 * tx + 1]) +
-                                              (sres[2 * ty + 1][2 * tx] + sres[2 * ty + 1][2 * tx + 1]));
+            c.r[cidx(c.G, I, K)] = (R)0.25 * (sres[2 * ty * BX + tx] + sres[(2 * ty + 1) * BX + tx]);
     }
-    __syncthreads();
 }
 
-// Coarsest level: one damped Jacobi sweep (first = starts from zero).
+// Start of a solve on the finest level of a one-level hierarchy: the red
+// cells relaxed, the black residual that leaves, rb = r_b + sum a (r / d)_red,
+// and z = rb / d; acc += rb z.
 template <class R>
-__device__ __forceinline__ void ph_mg_coarse(const LevelT<R> &L, const R *ein, R *eout, int first,
-                                             double *sm, int bx, int bz)
+__device__ __forceinline__ void ph_rb_start(const LevelT<R> &L, R *rb, R *z, double *sm, int bx, int bz, R (&acc)[1])
 {
     const Geom &G = L.G;
-    int i, k;
-    if (first) {
-        if (cell_of(G, bx, bz, i, k)) {
-            const int q = cidx(G, i, k);
-            eout[q] = ld(&L.wd[q]) * ld(&L.r[q]);
-        }
-        return;
-    }
-    Tile<1, R> &se = tile_at<1, R>(sm, 0);
-    load_tile_fn<1, R>(se, G, bx, bz, [&](int q, int, int) { return ld(&ein[q]); });
+    PairTile<1, R> &st = pair_tile<1, R>(sm, 0);
+    fill_pairs<1, true, R>(st, G, bx, bz, [&](int q, int, int, int) { return ld(&L.wd[q]) * ld(&L.r[q]); });
     __syncthreads();
-    if (cell_of(G, bx, bz, i, k)) {
-        const int q = cidx(G, i, k);
-        const int y = threadIdx.y + 1, x = threadIdx.x + 1;
-        eout[q] = fma(ld(&L.wd[q]), ld(&L.r[q]) - helm_tile<1, R>(L, q, i, k, se, y, x), se[y][x]);
+    int j, k;
+    if (pair_of(G, bx, bz, j, k)) {
+        const int s = k & 1, i = 2 * j + s;
+        if (i < G.nx) {
+            const int q = cidx(G, i, k), c = cidx(G, j, k);
+            const int y = threadIdx.y + 1, x = threadIdx.x + 1;
+            const R g = ld(&L.r[q]) + faces4<R>(L, q, st[y][x - 1 + s], st[y][x + s], st[y - 1][x], st[y + 1][x]);
+            const R zv = ld(&L.wd[q]) * g;
+            rb[c] = g;
+            z[c] = zv;
+            acc[0] = fma(g, zv, acc[0]);
+        }
     }
     __syncthreads();
 }
 
-// Prolongation step of a level: e' = e + P e_c (piecewise constant), then one
-// damped Jacobi post-smoothing sweep e'' = e' + (omega/d)(r - A e'). At the
-// finest level the result is z = M^-1 r; acc += r.z.
+// Down half of a level's V-cycle: e_r = r / d on red, e_b = w (r + sum a e_r) / d
+// on black (w = omega), and the residual that leaves, sum a e_b on red and
+// (1 - w) (r + sum a e_r) on black, restricted to level c. FINE (the start of
+// a solve on the finest level): the black residual r + sum a e_r goes to rb.
+// With w != 1, e_b is kept in f.e for the up half (on the finest level of the
+// iteration it follows from rb).
+template <bool FINE, class R>
+__device__ __forceinline__ void ph_mg_down(const LevelT<R> &f, const LevelT<R> &c, R *rb, const Phys &F, double *sm,
+                                           int bx, int bz)
+{
+    const Geom &G = f.G;
+    PairTile<2, R> &st = pair_tile<2, R>(sm, 0);
+    PairTile<1, R> &se = pair_tile<1, R>(sm, kPH2);
+    R *sres = reinterpret_cast<R *>(sm) + kPH2 + kPH1;
+    const R om = (R)F.omega;
+    fill_pairs<2, true, R>(st, G, bx, bz, [&](int q, int, int, int) { return ld(&f.wd[q]) * ld(&f.r[q]); });
+    __syncthreads();
+    fill_next<false, R>(se, G, bx, bz, [&](int q, int cc, int tk, int tj, int s) {
+        const R g = ld(&f.r[q]) + faces4<R>(f, q, st[tk + 1][tj - 1 + s], st[tk + 1][tj + s], st[tk][tj], st[tk + 2][tj]);
+        R e = ld(&f.wd[q]) * g;
+        if (F.om_ne1) e *= om;
+        if (tk >= 1 && tk <= BZ && tj >= 1 && tj <= BX) {
+            if (FINE) rb[cc] = g;
+            if (F.om_ne1 && !FINE) f.e[q] = e;
+        }
+        return e;
+    });
+    __syncthreads();
+    int j, k;
+    R v = 0;
+    if (pair_of(G, bx, bz, j, k)) {
+        const int s = k & 1, q = cidx(G, 2 * j + 1 - s, k);
+        const int y = threadIdx.y + 1, x = threadIdx.x + 1;
+        v = faces4<R>(f, q, se[y][x - s], se[y][x + 1 - s], se[y - 1][x], se[y + 1][x]);
+        if (F.om_ne1) {
+            const R gb = ld(&f.d[cidx(G, 2 * j + s, k)]) * se[y][x];   // omega times the black residual
+            v = fma((R)(1.0 - F.omega) / om, gb, v);
+        }
+    }
+    restrict_pairs<R>(c, v, sres, bx, bz);
+    __syncthreads();
+}
+
+// Up half of a level's V-cycle with the coarse correction ec (row pitch Pc;
+// null on the coarsest level, whose solve is one symmetric red-black sweep):
+// red e = r / d + P ec, black z = (1 - w) (e_b + P ec) + w (r + sum a e) / d with
+// e_b of the down half, then red z = (r + sum a z) / d. Writes the whole correction;
+// acc += r z (used on the finest level).
 template <class R>
-__device__ __forceinline__ void ph_mg_up(const LevelT<R> &f, const R *res, const R *ec, int Pc, R *out,
+__device__ __forceinline__ void ph_mg_up(const LevelT<R> &f, const R *res, const R *ec, int Pc, R *out, const Phys &F,
                                          double *sm, int bx, int bz, R (&acc)[1])
 {
     const Geom &G = f.G;
-    Tile<1, R> &se = tile_at<1, R>(sm, 0);
-    int i, k;
-    const bool in = cell_of(G, bx, bz, i, k);
-    const int q0 = in ? cidx(G, i, k) : 0;
-    HelmCoef<R> hc{};
-    R rq = 0, wq = 0;
-    auto fetch = [&] {   // ahead of the tile barrier
-        hc = helm_coef(f, q0, i, k);
-        rq = ld(&res[q0]);
-        wq = ld(&f.wd[q0]);
-    };
-    if (kPrefetch && in) fetch();
-    load_tile_fn<1, R>(se, G, bx, bz, [&](int q, int ii, int kk) {
-        return ld(&f.e[q]) + ld(&ec[(kk >> 1) * Pc + (ii >> 1)]);
+    PairTile<2, R> &st = pair_tile<2, R>(sm, 0);
+    PairTile<1, R> &sz = pair_tile<1, R>(sm, kPH2);
+    fill_pairs<2, true, R>(st, G, bx, bz, [&](int q, int, int jj, int kk) {
+        const R r = ld(&res[q]), w = ld(&f.wd[q]);
+        return ec ? fma(w, r, ld(&ec[(kk >> 1) * Pc + jj])) : w * r;
+    });
+    __syncthreads();
+    fill_next<false, R>(sz, G, bx, bz, [&](int q, int, int tk, int tj, int s) {
+        const R r = ld(&res[q]);
+        R z = ld(&f.wd[q]) *
+              (r + faces4<R>(f, q, st[tk + 1][tj - 1 + s], st[tk + 1][tj + s], st[tk][tj], st[tk + 2][tj]));
+        // the coarsest level keeps no down half: its one sweep is undamped
+        if (F.om_ne1 && ec)
+            z = fma((R)F.omega, z,
+                    (R)(1.0 - F.omega) * (ld(&f.e[q]) + ld(&ec[((bz * BZ - 1 + tk) >> 1) * Pc + bx * BX - 1 + tj])));
+        if (tk >= 1 && tk <= BZ && tj >= 1 && tj <= BX) {
+            out[q] = z;
+            acc[0] = fma(r, z, acc[0]);
+        }
+        return z;
+    });
+    __syncthreads();
+    int j, k;
+    if (pair_of(G, bx, bz, j, k)) {
+        const int s = k & 1, i = 2 * j + 1 - s;
+        if (i < G.nx) {
+            const int q = cidx(G, i, k);
+            const int y = threadIdx.y + 1, x = threadIdx.x + 1;
+            const R r = ld(&res[q]);
+            const R z = ld(&f.wd[q]) * (r + faces4<R>(f, q, sz[y][x - s], sz[y][x + 1 - s], sz[y - 1][x], sz[y + 1][x]));
+            out[q] = z;
+            acc[0] = fma(r, z, acc[0]);
+        }
+    }
+    __syncthreads();
+}
+
+// Up half on the finest level of the black-half iteration (red residual
+// zero): z = (1 - w) (w rb / d + P ec) + w (rb + sum a P ec) / d, pair by pair;
+// acc += rb z.
+template <class R>
+__device__ __forceinline__ void ph_rb_up(const LevelT<R> &f, const R *rb, const R *ec, int Pc, R *z, const Phys &F,
+                                         int bx, int bz, R (&acc)[1])
+{
+    const Geom &G = f.G;
+    int j, k;
+    if (!pair_of(G, bx, bz, j, k)) return;
+    const int s = k & 1, q = cidx(G, 2 * j + s, k), c = cidx(G, j, k);
+    // coarse values of the red neighbours; a neighbour beyond a wall meets a
+    // zero coefficient, its index only stays inside the level
+    const int jw = max(j - 1 + s, 0), je = min(j + s, pairs_of(G) - 1);
+    const R *row = ec + (k >> 1) * Pc;
+    const R *rs = ec + (max(k - 1, 0) >> 1) * Pc, *rn = ec + (min(k + 1, G.nz - 1) >> 1) * Pc;
+    const R r = ld(&rb[c]), w = ld(&f.wd[q]);
+    R zv = w * (r + faces4<R>(f, q, ld(&row[jw]), ld(&row[je]), ld(&rs[j]), ld(&rn[j])));
+    if (F.om_ne1) zv = fma((R)F.omega, zv, (R)(1.0 - F.omega) * fma((R)F.omega * w, r, ld(&row[j])));
+    z[c] = zv;
+    acc[0] = fma(r, zv, acc[0]);
+}
+
+// ---- CG vector steps (black halves) ----
+
+// p_new = z + beta p_old (first: z) and q = S p_new, with the red part of the
+// direction formed on the tile; acc += p.q.
+template <class R>
+__device__ __forceinline__ void ph_pspmv(const LevelT<R> &L, const R *z, const R *pold, R *pnew, R *qv, double beta,
+                                         bool first, double *sm, int bx, int bz, R (&acc)[1])
+{
+    const Geom &G = L.G;
+    const R b = (R)beta;
+    PairTile<2, R> &sp = pair_tile<2, R>(sm, 0);
+    PairTile<1, R> &sw = pair_tile<1, R>(sm, kPH2);
+    int j, k;
+    const bool own = pair_of(G, bx, bz, j, k);
+    const int s = k & 1, i = 2 * j + s;
+    const bool in = own && i < G.nx;
+    const int q = in ? cidx(G, i, k) : 0;
+    HelmCoef<R> h{};
+    if (kPrefetchSpmv && in) h = helm_coef(L, q, i, k);
+    if (first)
+        fill_pairs<2, false, R>(sp, G, bx, bz, [&](int, int c, int, int) { return ld(&z[c]); });
+    else
+        fill_pairs<2, false, R>(sp, G, bx, bz, [&](int, int c, int, int) { return fma(b, ld(&pold[c]), ld(&z[c])); });
+    __syncthreads();
+    fill_next<true, R>(sw, G, bx, bz, [&](int qr, int, int tk, int tj, int sr) {
+        return ld(&L.wd[qr]) *
+               faces4<R>(L, qr, sp[tk + 1][tj - sr], sp[tk + 1][tj + 1 - sr], sp[tk][tj], sp[tk + 2][tj]);
     });
     __syncthreads();
     if (in) {
-        if (!kPrefetch) fetch();
-        const int y = threadIdx.y + 1, x = threadIdx.x + 1;
-        const R z = fma(wq, rq - helm_apply<1, R>(hc, se, y, x), se[y][x]);
-        out[q0] = z;
-        acc[0] = fma(rq, z, acc[0]);
+        if (!kPrefetchSpmv) h = helm_coef(L, q, i, k);
+        const int y = threadIdx.y + 1, x = threadIdx.x + 1, c = cidx(G, j, k);
+        const R p = sp[y + 1][x];
+        R t = h.d * p;
+        t = fma(-h.aw, sw[y][x - 1 + s], t);
+        t = fma(-h.ae, sw[y][x + s], t);
+        t = fma(-h.as, sw[y - 1][x], t);
+        t = fma(-h.an, sw[y + 1][x], t);
+        pnew[c] = p;
+        qv[c] = t;
+        acc[0] = fma(p, t, acc[0]);
     }
     __syncthreads();
 }
 
-// Single-level preconditioner: two Jacobi sweeps from zero,
-// z = e + (omega/d)(r - A e) with e = (omega/d) r (omega = 1 unless the
-// caller set another weight: then M^-1 A has the eigenvalues l (2 - l) of
-// the Chebyshev-optimal degree-2 form); acc += r.z.
+// One-level hierarchy: x += alpha p, rb -= alpha q and z = rb / d, cell by
+// cell; acc += (rb^2, rb z).
 template <class R>
-__device__ __forceinline__ void ph_mg_single(const LevelT<R> &f, R *out, double *sm, int bx, int bz,
-                                             R (&acc)[1])
+__device__ __forceinline__ void ph_update_single(const LevelT<R> &L, const R *qv, R *rb, R *z, R *x, const R *p,
+                                                 double alpha_d, bool first, int bx, int bz, R (&acc)[2])
+{
+    const Geom &G = L.G;
+    const R alpha = (R)alpha_d;
+    int j, k;
+    if (!pair_of(G, bx, bz, j, k)) return;
+    const int i = 2 * j + (k & 1);
+    if (i >= G.nx) return;
+    const int c = cidx(G, j, k);
+    const R pq = ld(&p[c]);
+    x[c] = first ? alpha * pq : fma(alpha, pq, ld(&x[c]));
+    const R rn = fma(-alpha, ld(&qv[c]), ld(&rb[c]));
+    rb[c] = rn;
+    const R zv = ld(&L.wd[cidx(G, i, k)]) * rn;
+    z[c] = zv;
+    acc[0] = fma(rn, rn, acc[0]);
+    acc[1] = fma(rn, zv, acc[1]);
+}
+
+// Multigrid: x += alpha p and rb -= alpha q, fused with the down half of the
+// finest level (a CG iteration then needs one grid-wide synchronisation
+// less): e = w rb / d on the black cells and the residual that leaves, sum a e on
+// red (and (1 - w) rb on black), restricted to level c. The residual is read
+// from rin (halo included) and written to rout: other blocks still read the
+// old one. acc += rb^2.
+template <class R>
+__device__ __forceinline__ void ph_update_down(const LevelT<R> &f, const LevelT<R> &c, const R *qv, const R *rin,
+                                               R *rout, R *x, const R *p, double alpha_d, bool first, const Phys &F,
+                                               double *sm, int bx, int bz, R (&acc)[1])
 {
     const Geom &G = f.G;
-    Tile<1, R> &se = tile_at<1, R>(sm, 0);
-    int i, k;
-    const bool in = cell_of(G, bx, bz, i, k);
-    const int q = in ? cidx(G, i, k) : 0;
-    HelmCoef<R> c{};
-    R rq = 0, wq = 0;
-    auto fetch = [&] {
-        c = helm_coef(f, q, i, k);
-        rq = ld(&f.r[q]);
-        wq = ld(&f.wd[q]);
-    };
-    if (kPrefetch && in) fetch();
-    load_tile_fn<1, R>(se, G, bx, bz, [&](int qq, int, int) { return ld(&f.wd[qq]) * ld(&f.r[qq]); });
-    __syncthreads();
-    if (in) {
-        if (!kPrefetch) fetch();
-        const int y = threadIdx.y + 1, x = threadIdx.x + 1;
-        const R z = fma(wq, rq - helm_apply<1, R>(c, se, y, x), se[y][x]);
-        out[q] = z;
-        acc[0] = fma(rq, z, acc[0]);
-    }
-    __syncthreads();
-}
-
-// ---- CG vector steps ----
-
-// p_new = z + beta p_old (computed once per tile cell) and q = A p_new;
-// acc += p.q.
-template <class R>
-__device__ __forceinline__ void ph_pspmv(const LevelT<R> &L, const R *pold, R *pnew, R *qv, double beta,
-                                         double *sm, int bx, int bz, R (&acc)[1])
-{
-    const Geom &G = L.G;
-    const R *z = L.e2;
-    const R b = (R)beta;
-    Tile<1, R> &sp = tile_at<1, R>(sm, 0);
-    int i, k;
-    const bool in = cell_of(G, bx, bz, i, k);
-    const int q = in ? cidx(G, i, k) : 0;
-    HelmCoef<R> c{};
-    if (kPrefetchSpmv && in) c = helm_coef(L, q, i, k);
-    load_tile_fn<1, R>(sp, G, bx, bz, [&](int qq, int, int) { return fma(b, ld(&pold[qq]), ld(&z[qq])); });
-    __syncthreads();
-    if (in) {
-        if (!kPrefetchSpmv) c = helm_coef(L, q, i, k);
-        const int y = threadIdx.y + 1, x = threadIdx.x + 1;
-        const R pq = sp[y][x];
-        const R Ap = helm_apply<1, R>(c, sp, y, x);
-        pnew[q] = pq;
-        qv[q] = Ap;
-        acc[0] = fma(pq, Ap, acc[0]);
-    }
-    __syncthreads();
-}
-
-// x += alpha p and r -= alpha q, fused with the first step of the next
-// V-cycle on the new residual (a CG iteration then needs one grid-wide
-// synchronisation less): the new residual and e = (omega/d) r_new are formed
-// on the tile and its halo from the old r and q in one pass.
-template <class R>
-__device__ __forceinline__ void update_tiles(const LevelT<R> &L, const R *qv, const R *rin, R alpha,
-                                             Tile<1, R> &sr, Tile<1, R> &se, int bx, int bz)
-{
-    const Geom &G = L.G;
-    const int i0 = bx * BX - 1, k0 = bz * BZ - 1;
-    const int tid = threadIdx.x + threadIdx.y * BX;
-    constexpr int W = BX + 2, NE = (BZ + 2) * (BX + 2);
-    for (int e = tid; e < NE; e += NTHREADS) {
-        const int tk = e / W, ti = e - tk * W;
-        const int i = i0 + ti, k = k0 + tk;
-        R rn = 0, ev = 0;
-        if (i >= 0 && i < G.nx && k >= 0 && k < G.nz) {
-            const int q = k * G.P + i;
-            rn = fma(-alpha, ld(&qv[q]), ld(&rin[q]));
-            ev = ld(&L.wd[q]) * rn;
+    const R alpha = (R)alpha_d;
+    PairTile<1, R> &se = pair_tile<1, R>(sm, 0);
+    R *sres = reinterpret_cast<R *>(sm) + kPH1;
+    fill_next<false, R>(se, G, bx, bz, [&](int q, int cc, int tk, int tj, int) {
+        const R rn = fma(-alpha, ld(&qv[cc]), ld(&rin[cc]));
+        if (tk >= 1 && tk <= BZ && tj >= 1 && tj <= BX) {
+            rout[cc] = rn;
+            const R pq = ld(&p[cc]);
+            x[cc] = first ? alpha * pq : fma(alpha, pq, ld(&x[cc]));
+            acc[0] = fma(rn, rn, acc[0]);
         }
-        sr[tk][ti] = rn;
-        se[tk][ti] = ev;
-    }
-}
-
-// The residual is read from rin (halo included) and written to rout: other
-// blocks still read the old residual while this one writes the new.
-// Single-level preconditioner: then z = e + (omega/d)(r_new - A e);
-// acc += (r_new^2, r_new . z).
-template <class R>
-__device__ __forceinline__ void ph_update_single(const LevelT<R> &L, const R *qv, const R *rin, R *rout,
-                                                 R *x, const R *p, double alpha_d, double *sm, int bx,
-                                                 int bz, R (&acc)[2])
-{
-    const Geom &G = L.G;
-    const R alpha = (R)alpha_d;
-    Tile<1, R> &sr = tile_at<1, R>(sm, 0), &se = tile_at<1, R>(sm, 1);
-    int i, k;
-    const bool in = cell_of(G, bx, bz, i, k);
-    const int q = in ? cidx(G, i, k) : 0;
-    HelmCoef<R> c{};
-    R wq = 0, xq = 0, pq = 0;
-    auto fetch = [&] {
-        c = helm_coef(L, q, i, k);
-        wq = ld(&L.wd[q]);
-        xq = ld(&x[q]);
-        pq = ld(&p[q]);
-    };
-    if (kPrefetch && in) fetch();
-    update_tiles<R>(L, qv, rin, alpha, sr, se, bx, bz);
+        return ld(&f.wd[q]) * rn;
+    });
     __syncthreads();
-    if (in) {
-        if (!kPrefetch) fetch();
+    int j, k;
+    R v = 0;
+    if (pair_of(G, bx, bz, j, k)) {
+        const int s = k & 1, q = cidx(G, 2 * j + 1 - s, k);
         const int y = threadIdx.y + 1, xx = threadIdx.x + 1;
-        const R rn = sr[y][xx];
-        x[q] = fma(alpha, pq, xq);
-        rout[q] = rn;
-        const R z = fma(wq, rn - helm_apply<1, R>(c, se, y, xx), se[y][xx]);
-        L.e2[q] = z;
-        acc[0] = fma(rn, rn, acc[0]);
-        acc[1] = fma(rn, z, acc[1]);
+        v = faces4<R>(f, q, se[y][xx - s], se[y][xx + 1 - s], se[y - 1][xx], se[y + 1][xx]);
+        if (F.om_ne1) v = fma((R)F.omega, v, (R)(1.0 - F.omega) * ld(&f.d[cidx(G, 2 * j + s, k)]) * se[y][xx]);
     }
-    __syncthreads();
-}
-
-// Multigrid preconditioner: then the restriction step of the finest level
-// (pre-smoothed e and the averaged residual (1-omega) r_new + sum a e_N into
-// the next level); acc += r_new^2.
-template <class R>
-__device__ __forceinline__ void ph_update_down(const LevelT<R> &f, const LevelT<R> &c, const R *qv,
-                                               const R *rin, R *rout, R *x, const R *p, double alpha_d,
-                                               double omega, double *sm, int bx, int bz, R (&acc)[1])
-{
-    const Geom &G = f.G;
-    const R alpha = (R)alpha_d;
-    Tile<1, R> &sr = tile_at<1, R>(sm, 0), &se = tile_at<1, R>(sm, 1);
-    R(*sres)[BX] = reinterpret_cast<R(*)[BX]>(reinterpret_cast<R *>(sm) + 2 * kT1);
-    int i, k;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const bool in = cell_of(G, bx, bz, i, k);
-    const int q0 = in ? cidx(G, i, k) : 0;
-    R aw = 0, ae = 0, as = 0, an = 0, xq = 0, pq = 0;
-    auto fetch = [&] {   // ahead of the tile barrier
-        aw = ld(&f.ax[k * G.P + i]);
-        ae = ld(&f.ax[k * G.P + i + 1]);
-        as = ld(&f.az[k * G.P + i]);
-        an = ld(&f.az[(k + 1) * G.P + i]);
-        xq = ld(&x[q0]);
-        pq = ld(&p[q0]);
-    };
-    if (kPrefetch && in) fetch();
-    update_tiles<R>(f, qv, rin, alpha, sr, se, bx, bz);
-    __syncthreads();
-    if (in) {
-        if (!kPrefetch) fetch();
-        const int q = q0;
-        const int y = ty + 1, xx = tx + 1;
-        const R rn = sr[y][xx];
-        x[q] = fma(alpha, pq, xq);
-        rout[q] = rn;
-        R t = (R)(1.0 - omega) * rn;
-        t = fma(aw, se[y][xx - 1], t);
-        t = fma(ae, se[y][xx + 1], t);
-        t = fma(as, se[y - 1][xx], t);
-        t = fma(an, se[y + 1][xx], t);
-        f.e[q] = se[y][xx];
-        sres[ty][tx] = t;
-        acc[0] = fma(rn, rn, acc[0]);
-    }
-    __syncthreads();
-    if (tx < BX / 2 && ty < BZ / 2) {
-        const int I = bx * (BX / 2) + tx, K = bz * (BZ / 2) + ty;
-        if (I < c.G.nx && K < c.G.nz)
-            c.r[cidx(c.G, I, K)] = (R)0.25 * ((sres[2 * ty][2 * tx] + sres[2 * ty][2 * tx + 1]) +
-                                              (sres[2 * ty + 1][2 * tx] + sres[2 * ty + 1][2 * tx + 1]));
-    }
+    restrict_pairs<R>(c, v, sres, bx, bz);
     __syncthreads();
 }
 
@@ -1212,11 +1272,58 @@ __device__ __forceinline__ void ph_guess_apply(const LevelT<R> &L, const float *
     acc[0] = fma(rn, rn, acc[0]);
 }
 
-// Flux and velocity correction: F_f = D_f (H_f - G_f) with
+// p' on the tile and its one-cell halo. sd: scratch of a halo-2 tile.
+template <class R>
+__device__ __forceinline__ void load_solution(Tile<1> &sx, Tile<2, R> &sd, const LevelT<R> &L, const SolveT<R> &v,
+                                              bool dx, int bx, int bz)
+{
+    const Geom &G = L.G;
+    const int i0 = bx * BX, k0 = bz * BZ;
+    auto start = [&](int q) {
+        double x = ld(&v.x[q]);
+        if (v.inc) x += (double)ld(&v.inc[q]);
+        return x;
+    };
+    if (!dx) {
+        load_tile_fn<1>(sx, G, bx, bz, [&](int q, int, int) { return start(q); });
+        return;
+    }
+    const int tid = threadIdx.x + threadIdx.y * BX;
+    constexpr int NJ = BX / 2 + 2;   // pairs that cover the halo: tile columns -2 .. BX + 1
+    for (int e = tid; e < (BZ + 4) * NJ; e += NTHREADS) {
+        const int tk = e / NJ, tj = e - tk * NJ;
+        const int j = i0 / 2 - 1 + tj, k = k0 - 2 + tk, s = k & 1, i = 2 * j + s;
+        sd[tk][2 * tj + s] = (j >= 0 && i < G.nx && k >= 0 && k < G.nz) ? ld(&v.xb[k * G.P + j]) : (R)0;
+    }
+    __syncthreads();
+    for (int e = tid; e < (BZ + 2) * NJ; e += NTHREADS) {
+        const int tk = e / NJ, tj = e - tk * NJ;
+        const int j = i0 / 2 - 1 + tj, k = k0 - 1 + tk, s = k & 1;
+        const bool zin = k >= 0 && k < G.nz && j >= 0;
+        const int cb = 2 * tj + s, cr = 2 * tj + 1 - s;   // halo-2 tile columns of the pair's cells
+        if (cb >= 1 && cb <= BX + 2)
+            sx[tk][cb - 1] = zin && 2 * j + s < G.nx ? start(k * G.P + 2 * j + s) + (double)sd[tk + 1][cb] : 0.0;
+        if (cr >= 1 && cr <= BX + 2) {
+            double xv = 0.0;
+            if (zin && 2 * j + 1 - s < G.nx) {
+                const int q = k * G.P + 2 * j + 1 - s;
+                const R t = ld(&L.r[q]) + faces4<R>(L, q, sd[tk + 1][cr - 1], sd[tk + 1][cr + 1], sd[tk][cr], sd[tk + 2][cr]);
+                xv = start(q) + (double)(ld(&L.wd[q]) * t);
+            }
+            sx[tk][cr - 1] = xv;
+        }
+    }
+}
+
+// The solution of the pressure solve, and the flux and velocity correction:
+// F_f = D_f (H_f - G_f) with
 // G_f = (p'_b - p'_a)/Delta - g z_f (rho2_b - rho2_a)/Delta; u = (dt/rho1)(H - G_cell);
 // p = p' - rho2 g z; rho = p / (R T^{n+1}) = p psi; phi = F |A|; p^{n-1} <- p^n
-// (and K^{n-1} <- K^n in the literal reading of eq. step3_sd).
-__device__ __forceinline__ void ph_correct(const StepArgs &a, double *sm, int bx, int bz)
+// (and K^{n-1} <- K^n in the literal reading of eq. step3_sd). p' goes to ppout
+// (not the solve's start, which other blocks still read).
+template <class R>
+__device__ __forceinline__ void ph_correct(const StepArgs &a, const LevelT<R> &L, const SolveT<R> &v, bool dx,
+                                           double *ppout, double *sm, int bx, int bz)
 {
     const Geom &G = a.G;
     const Phys &F = a.F;
@@ -1247,8 +1354,9 @@ __device__ __forceinline__ void ph_correct(const StepArgs &a, double *sm, int bx
         pnq = ld(&a.S.p[q0]);
     };
     if (kPrefetch && in) fetch();
-    load_tile_fn<1>(sx, G, bx, bz, [&](int q, int, int) { return ld(&N.pp[q]); });
     load_tile_fn<1>(s2, G, bx, bz, [&](int q, int, int) { return ld(&a.rho2[q]); });
+    // the scratch lies where the face forces go after the barrier
+    load_solution<R>(sx, tile_at<2, R>(sm + 2 * kT1, 0), L, v, dx, bx, bz);
     __syncthreads();
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int y = ty + 1, x = tx + 1;
@@ -1278,6 +1386,7 @@ __device__ __forceinline__ void ph_correct(const StepArgs &a, double *sm, int bx
         if (k == G.nz - 1) N.phiz[G.nz * G.P + i] = 0.0;
         N.u[q] = dtr1 * (hxq - 0.5 * (gxw + gxe));
         N.w[q] = dtr1 * (hzq - 0.5 * (gzs + gzn));
+        ppout[q] = sx[y][x];
         const double pn = fma(-s2[y][x], gzk, sx[y][x]);
         N.p[q] = pn;
         N.rho[q] = pn * psq;
