@@ -5,9 +5,9 @@
 // The 3x3 layers with 16-64 channels run on the tensor cores (gea_conv.cu):
 // forward, and the data gradient as the same correlation with the taps
 // mirrored and the channel roles swapped. The first layer (one input
-// channel), the 1x1 output layer, the weight gradients (a reduction over all
-// pixels into at most 64 x 64 x 9 values per layer, which does not fill a
-// 128-row MMA tile) and the elementwise parts run on the CUDA cores in FP32.
+// channel), the 1x1 output layer, the weight gradients (FP32 gradients times
+// bfloat16 inputs, summed over all pixels) and the elementwise parts run on
+// the CUDA cores in FP32.
 // Every reduction is deterministic: per-block partial sums added in a fixed
 // order.
 #include "../../include/gea.h"
@@ -19,6 +19,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 cudaError_t gea_conv3x3_launch(int n, int h, int w, int cin, int cout, int mode, int flags, const uint16_t *x0,
@@ -55,9 +56,7 @@ constexpr LayerDef kL[L] = {
 };
 constexpr int kOut = L - 1;
 constexpr int kThreads = 256;
-constexpr int kWgThreads = 128;
-constexpr int kWgTile = 128;     // pixels per weight-gradient tile (one row segment)
-constexpr int kMaxSlices = 96;   // weight-gradient CTAs per tap
+constexpr int kWgPix = 64;       // pixels of a weight-gradient row segment at most
 
 __device__ __forceinline__ float bf2f(uint16_t u) { return __uint_as_float((uint32_t)u << 16); }
 __device__ __forceinline__ uint16_t f2bf(float f)
@@ -243,163 +242,380 @@ __global__ void k_out_backward(long long npix, const float *dy, const uint16_t *
     if (threadIdx.x < 17) part[(size_t)blockIdx.x * 17 + threadIdx.x] = red[threadIdx.x][0];
 }
 
-// out[j] = sum over s < ns of part[s * stride + j], j < nout
-__global__ void k_sum_partials(const float *part, int ns, int stride, int nout, float *out)
+// out[j] = sum over s < ns of part[s * stride + j], one block per output: thread
+// t adds partials t, t + kThreads, ..., then a fixed-order tree
+__global__ void k_sum_partials(const float *part, int ns, int stride, float *out)
 {
-    const int j = blockIdx.x * kThreads + threadIdx.x;
-    if (j >= nout) return;
+    __shared__ float red[kThreads];
+    const int j = blockIdx.x;
     float s = 0.0f;
-    for (int i = 0; i < ns; ++i) s += part[(size_t)i * stride + j];
-    out[j] = s;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < ns; i += kThreads) s += part[(size_t)i * stride + j];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = kThreads / 2; o > 0; o >>= 1) {
+        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[j] = red[0];
 }
 
 // ---- backward elementwise parts ----
 
-// g *= (act > 0) when relu; gb = bfloat16(g)
-__global__ void k_mask(long long cnt, float *g, const uint16_t *act, int relu, uint16_t *gb)
+// Four values a thread (channel counts are multiples of 16): one 16-byte
+// access of FP32 data, 8 bytes of bfloat16.
+__device__ __forceinline__ uint2 pack4(float4 v)
 {
-    const long long i = blockIdx.x * (long long)kThreads + threadIdx.x;
-    if (i >= cnt) return;
-    float v = g[i];
-    if (relu && !(bf2f(act[i]) > 0.0f)) v = 0.0f;
-    g[i] = v;
-    if (gb) gb[i] = f2bf(v);
+    return make_uint2((uint32_t)f2bf(v.x) | ((uint32_t)f2bf(v.y) << 16),
+                      (uint32_t)f2bf(v.z) | ((uint32_t)f2bf(v.w) << 16));
+}
+__device__ __forceinline__ float4 unpack4(uint2 u)
+{
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                       __uint_as_float(u.y & 0xFFFF0000u));
 }
 
-__global__ void k_add(long long cnt, float *dst, const float *src)
+// g *= (act > 0) when relu; gb = bfloat16(g) (may be null)
+__global__ void k_mask(long long quads, float4 *g, const uint2 *act, int relu, uint2 *gb)
 {
     const long long i = blockIdx.x * (long long)kThreads + threadIdx.x;
-    if (i < cnt) dst[i] += src[i];
+    if (i >= quads) return;
+    float4 v = g[i];
+    if (relu) {
+        const float4 a = unpack4(act[i]);
+        if (!(a.x > 0.0f)) v.x = 0.0f;
+        if (!(a.y > 0.0f)) v.y = 0.0f;
+        if (!(a.z > 0.0f)) v.z = 0.0f;
+        if (!(a.w > 0.0f)) v.w = 0.0f;
+        g[i] = v;
+    }
+    if (gb) gb[i] = pack4(v);
 }
 
-// the gradient of a 2x2 average: dst (n x 2h x 2w x c) += gin(n x h x w x c) / 4
-__global__ void k_pool_backward(int n, int h, int w, int c, float *dst, const float *gin)
+// the gradient of a 2x2 average: dst (n x 2h x 2w x 4 c4) += gin(n x h x w x 4 c4) / 4
+__global__ void k_pool_backward(int n, int h, int w, int c4, float4 *dst, const float4 *gin)
 {
     const long long i = blockIdx.x * (long long)kThreads + threadIdx.x;
-    const long long tot = (long long)n * 4 * h * w * c;
+    const long long tot = (long long)n * 4 * h * w * c4;
     if (i >= tot) return;
-    const int ch = (int)(i % c);
-    const long long pix = i / c;
+    const int ch = (int)(i % c4);
+    const long long pix = i / c4;
     const int W2 = 2 * w, H2 = 2 * h;
     const int x = (int)(pix % W2), y = (int)((pix / W2) % H2);
     const long long b = pix / ((long long)W2 * H2);
-    dst[i] += 0.25f * gin[(((size_t)b * h + y / 2) * w + x / 2) * c + ch];
+    const float4 s = gin[(((size_t)b * h + y / 2) * w + x / 2) * c4 + ch];
+    float4 d = dst[i];
+    d.x += 0.25f * s.x;
+    d.y += 0.25f * s.y;
+    d.z += 0.25f * s.z;
+    d.w += 0.25f * s.w;
+    dst[i] = d;
 }
 
-// the gradient of a nearest-neighbour prolongation: dst (n x h/2 x w/2 x c)
-// += sum of the 2x2 children in gin (n x h x w x c)
-__global__ void k_up_backward(int n, int h, int w, int c, float *dst, const float *gin)
+// the gradient of a nearest-neighbour prolongation: dst (n x h/2 x w/2 x 4 c4)
+// = sum of the 2x2 children in gin (n x h x w x 4 c4)
+__global__ void k_up_backward(int n, int h, int w, int c4, float4 *dst, const float4 *gin)
 {
     const int hc = h / 2, wc = w / 2;
     const long long i = blockIdx.x * (long long)kThreads + threadIdx.x;
-    const long long tot = (long long)n * hc * wc * c;
+    const long long tot = (long long)n * hc * wc * c4;
     if (i >= tot) return;
-    const int ch = (int)(i % c);
-    const long long pix = i / c;
+    const int ch = (int)(i % c4);
+    const long long pix = i / c4;
     const int x = (int)(pix % wc), y = (int)((pix / wc) % hc);
     const long long b = pix / ((long long)wc * hc);
-    const float *g = gin + (((size_t)b * h + 2 * y) * w + 2 * x) * c + ch;
-    dst[i] += (g[0] + g[c]) + (g[(size_t)w * c] + g[(size_t)w * c + c]);
+    const float4 *g = gin + (((size_t)b * h + 2 * y) * w + 2 * x) * c4 + ch;
+    const float4 p = g[0], q = g[c4], r = g[(size_t)w * c4], s = g[(size_t)w * c4 + c4];
+    dst[i] = make_float4((p.x + q.x) + (r.x + s.x), (p.y + q.y) + (r.y + s.y), (p.z + q.z) + (r.z + s.z),
+                         (p.w + q.w) + (r.w + s.w));
+}
+
+// The input of a layer that reads an average (POOL: x0 n x 2h x 2w x 4 c4) or a
+// sum with a prolonged coarser tensor (x1 n x h/2 x w/2), in bfloat16, formed
+// as the forward pass forms it.
+template <int MODE>
+__global__ void k_form_input(int n, int h, int w, int c4, const uint2 *x0, const uint2 *x1, uint2 *out)
+{
+    const long long i = blockIdx.x * (long long)kThreads + threadIdx.x;
+    const long long tot = (long long)n * h * w * c4;
+    if (i >= tot) return;
+    const int ch = (int)(i % c4);
+    const long long pix = i / c4;
+    const int x = (int)(pix % w), y = (int)((pix / w) % h);
+    const long long b = pix / ((long long)w * h);
+    if (MODE == GEA_CONV_POOL) {
+        const size_t W2 = (size_t)2 * w * c4;
+        const uint2 *s = x0 + ((size_t)b * 2 * h + 2 * y) * W2 + (size_t)2 * x * c4 + ch;
+        const float4 p = unpack4(s[0]), q = unpack4(s[c4]), r = unpack4(s[W2]), t = unpack4(s[W2 + c4]);
+        out[i] = pack4(make_float4(0.25f * ((p.x + q.x) + (r.x + t.x)), 0.25f * ((p.y + q.y) + (r.y + t.y)),
+                                   0.25f * ((p.z + q.z) + (r.z + t.z)), 0.25f * ((p.w + q.w) + (r.w + t.w))));
+    } else {
+        const float4 p = unpack4(x0[i]);
+        const float4 q = unpack4(x1[(((size_t)b * (h / 2) + y / 2) * (w / 2) + x / 2) * c4 + ch]);
+        out[i] = pack4(make_float4(p.x + q.x, p.y + q.y, p.z + q.z, p.w + q.w));
+    }
 }
 
 // ---- weight gradients (FP32, CUDA cores) ----
 
+//
+// dW[tap][co][ci] = sum over pixels p of g[p][co] x[p + off(tap)][ci], db = sum g.
+//
+// Bound: FP32 FMA issue (2 x 9 x cin x cout flops per pixel; 23 GFLOP for a
+// batch of 8 x 256 x 256, 0.3 ms at the FP32 rate). A thread keeps a 4 x 4
+// block of (co, ci) for the three taps of one row offset in registers and
+// walks along a row with a sliding window of three input pixels: per pixel
+// one 16-byte read of g and one 8-byte read of x from shared memory feed 48
+// FMAs. Rows arrive by 16-byte asynchronous copies one row ahead, each input
+// row once per block for its three uses. Against one accumulator per thread
+// and tap with two shared-memory reads per FMA, a layer of that batch went
+// from 461 to 73 us (16 -> 16 channels, full size) and from 490 to 44 us
+// (64 -> 64, a quarter of the size), 33 TFLOP/s; with the sums over the blocks
+// in parallel and first gradients written in place the backward pass went
+// from 6.46 to 1.2 ms.
+
 struct WgArgs {
-    int n, h, w;            // the layer's (output) size; POOL sources are 2h x 2w
-    const uint16_t *x0, *x1;
+    int n, h, w;            // the layer's size
+    const uint16_t *x;      // its input, n x h x w x cin
     const float *g;         // masked output gradient, n x h x w x cout
-    float *part;            // [slice][tap][cout * cin]
-    float *partb;           // [slice][cout]
-    int ntiles, tiles_per_row, nslices;
+    float *part;            // [block][tap][cout][cin]
+    float *partb;           // [block][cout]
+    int strips, pt;         // row segments per row and their pixels
+    int rb, chunks;         // rows of a work item and items per column of segments
+    int items;              // n x strips x chunks
 };
 
-// The input value of the layer (fused as the forward pass forms it) at
-// pixel (b, yy, xx), channel c; zero outside the image.
-template <int CIN, int MODE>
-__device__ __forceinline__ float wg_input(const WgArgs &a, int b, int yy, int xx, int c)
+// First pixel, rows and sample of item t.
+__device__ __forceinline__ void wg_item(const WgArgs &a, int t, int &b, int &x0, int &y0, int &y1)
 {
-    if (yy < 0 || yy >= a.h || xx < 0 || xx >= a.w) return 0.0f;
-    if (MODE == GEA_CONV_PLAIN) return bf2f(a.x0[(((size_t)b * a.h + yy) * a.w + xx) * CIN + c]);
-    if (MODE == GEA_CONV_POOL) {
-        const size_t W2 = (size_t)2 * a.w;
-        const uint16_t *s = a.x0 + (((size_t)b * 2 * a.h + 2 * yy) * W2 + 2 * xx) * CIN + c;
-        return round_bf(0.25f * ((bf2f(s[0]) + bf2f(s[CIN])) + (bf2f(s[W2 * CIN]) + bf2f(s[W2 * CIN + CIN]))));
-    }
-    const int hc = a.h / 2, wc = a.w / 2;
-    return round_bf(bf2f(a.x0[(((size_t)b * a.h + yy) * a.w + xx) * CIN + c]) +
-                    bf2f(a.x1[(((size_t)b * hc + yy / 2) * wc + xx / 2) * CIN + c]));
+    const int c = t % a.chunks, s = (t / a.chunks) % a.strips;
+    b = t / (a.chunks * a.strips);
+    x0 = s * a.pt;
+    y0 = c * a.rb;
+    y1 = min(y0 + a.rb, a.h);
 }
 
-// Block (tap, slice): dW[tap][co][ci] += sum over the slice's tiles of
-// g[p][co] x[p + off(tap)][ci]; the centre tap's blocks also sum db.
-template <int CIN, int COUT, int MODE>
-__global__ void __launch_bounds__(kWgThreads) k_wgrad(WgArgs a)
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool valid)
 {
-    constexpr int NOUT = CIN * COUT;
-    constexpr int PER = (NOUT + kWgThreads - 1) / kWgThreads;
-    constexpr int XS = CIN + (CIN > 1 ? 1 : 0);       // padded row of the input tile
-    extern __shared__ float wsm[];
-    float *gs = wsm;                                  // [kWgTile][COUT]
-    float *xs = wsm + kWgTile * COUT;                 // [kWgTile][XS]
-    const int tap = blockIdx.x, ntap = gridDim.x;
-    const int dy = ntap == 9 ? tap / 3 - 1 : 0, dx = ntap == 9 ? tap % 3 - 1 : 0;
-    const bool centre = (ntap == 9 && tap == 4) || ntap == 1;
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0));
+}
+
+// Threads: 3 row offsets x cout/4 x cin/4 blocks of outputs x GR groups that
+// split a segment's pixels (so that small layers fill a block).
+template <int CIN, int COUT, int GR>
+struct WgShape {
+    static constexpr int TI = CIN / 4, TC = COUT / 4, OUT = 3 * TI * TC, THREADS = OUT * GR;
+    static constexpr int GF = kWgPix * COUT;               // floats of a gradient row
+    static constexpr int XH = (kWgPix + 2) * CIN;          // bfloat16s of an input row
+    static constexpr int STAGE = 2 * GF * 4 + 4 * XH * 2;  // bytes: two gradient rows, four input rows
+    static constexpr int RED = (GR - 1) * OUT * 52 * 4;    // bytes of the groups' sums
+    static constexpr int SMEM = STAGE > RED ? STAGE : RED;
+};
+
+template <int CIN, int COUT, int GR>
+__global__ void __launch_bounds__(WgShape<CIN, COUT, GR>::THREADS, 768 / WgShape<CIN, COUT, GR>::THREADS) k_wgrad(WgArgs a)
+{
+    using S = WgShape<CIN, COUT, GR>;
+    extern __shared__ __align__(16) unsigned char wsm[];
+    float *gs = reinterpret_cast<float *>(wsm);                              // [2][kWgPix][COUT]
+    uint16_t *xs = reinterpret_cast<uint16_t *>(wsm + 2 * S::GF * 4);        // [4][kWgPix + 2][CIN]
     const int tid = threadIdx.x;
-    float acc[PER];
+    const int ci = (tid % S::TI) * 4, co = (tid / S::TI % S::TC) * 4;
+    const int dy = tid / (S::TI * S::TC) % 3, gr = tid / S::OUT;
+    const bool bias = dy == 1 && ci == 0;
+    const int pg = (a.pt + GR - 1) / GR, p0 = gr * pg, p1 = min(p0 + pg, a.pt);
+    float acc[3][4][4], accb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int q = 0; q < PER; ++q) acc[q] = 0.0f;
-    float accb = 0.0f;
-    for (int t = blockIdx.y; t < a.ntiles; t += a.nslices) {
-        const int tx = t % a.tiles_per_row, row = t / a.tiles_per_row;
-        const int y = row % a.h, b = row / a.h;
-        const int x0 = tx * kWgTile;
-        for (int e = tid; e < kWgTile * COUT; e += kWgThreads) {
-            const int p = e / COUT, c = e % COUT;
-            const int xx = x0 + p;
-            gs[e] = xx < a.w ? a.g[(((size_t)b * a.h + y) * a.w + xx) * COUT + c] : 0.0f;
+    for (int t = 0; t < 3; ++t)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[t][c][i] = 0.0f;
+    for (int t = blockIdx.x; t < a.items; t += gridDim.x) {
+        int b, x0, y0, y1;
+        wg_item(a, t, b, x0, y0, y1);
+        // input row y into slot (y - y0 + 1) & 3, pixels x0 - 1 .. x0 + pt, zero outside the image
+        auto load_x = [&](int y) {
+            uint16_t *dst = xs + ((y - y0 + 1) & 3) * S::XH;
+            const bool yin = y >= 0 && y < a.h;
+            for (int e = tid; e < (a.pt + 2) * (CIN / 8); e += S::THREADS) {
+                const int p = e / (CIN / 8), c = e % (CIN / 8) * 8, xx = x0 - 1 + p;
+                const bool in = yin && xx >= 0 && xx < a.w;
+                cp_async16(dst + p * CIN + c, in ? a.x + (((size_t)b * a.h + y) * a.w + xx) * CIN + c : a.x, in);
+            }
+        };
+        auto load_g = [&](int y) {
+            float *dst = gs + ((y - y0) & 1) * S::GF;
+            for (int e = tid; e < a.pt * (COUT / 4); e += S::THREADS) {
+                const int p = e / (COUT / 4), c = e % (COUT / 4) * 4;
+                const bool in = x0 + p < a.w;
+                cp_async16(dst + p * COUT + c, in ? a.g + (((size_t)b * a.h + y) * a.w + x0 + p) * COUT + c : a.g, in);
+            }
+        };
+        load_x(y0 - 1);
+        load_x(y0);
+        load_x(y0 + 1);
+        load_g(y0);
+        asm volatile("cp.async.commit_group;");
+        for (int y = y0; y < y1; ++y) {
+            if (y + 1 < y1) {
+                load_x(y + 2);
+                load_g(y + 1);
+            }
+            asm volatile("cp.async.commit_group;");
+            asm volatile("cp.async.wait_group 1;");
+            __syncthreads();
+            const float *gp = gs + ((y - y0) & 1) * S::GF + co;
+            const uint16_t *xp = xs + ((y - y0 + dy) & 3) * S::XH + ci;
+            auto ldx = [&](int p) { return unpack4(*reinterpret_cast<const uint2 *>(xp + p * CIN)); };
+            float4 xl = ldx(min(p0, a.pt)), xc = ldx(min(p0, a.pt) + 1);
+#pragma unroll 3
+            for (int p = p0; p < p1; ++p) {
+                const float4 xr = ldx(p + 2);
+                const float4 gv = *reinterpret_cast<const float4 *>(gp + p * COUT);
+                const float g4[4] = {gv.x, gv.y, gv.z, gv.w};
+                const float xv[3][4] = {{xl.x, xl.y, xl.z, xl.w}, {xc.x, xc.y, xc.z, xc.w}, {xr.x, xr.y, xr.z, xr.w}};
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) acc[k][c][i] = fmaf(g4[c], xv[k][i], acc[k][c][i]);
+                if (bias) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) accb[c] += g4[c];
+                }
+                xl = xc;
+                xc = xr;
+            }
+            __syncthreads();
         }
-        for (int e = tid; e < kWgTile * CIN; e += kWgThreads) {
-            const int p = e / CIN, c = e % CIN;
-            xs[p * XS + c] = (x0 + p < a.w) ? wg_input<CIN, MODE>(a, b, y + dy, x0 + p + dx, c) : 0.0f;
+    }
+    // the groups' sums in group order, then the block's partials
+    asm volatile("cp.async.wait_group 0;");
+    if (GR > 1) {
+        float *red = reinterpret_cast<float *>(wsm);
+        const int o = tid % S::OUT;
+        __syncthreads();
+        if (gr > 0) {
+            float *r = red + (size_t)(gr - 1) * 52 * S::OUT + o;
+#pragma unroll
+            for (int k = 0; k < 48; ++k) r[k * S::OUT] = acc[k / 16][k / 4 % 4][k % 4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) r[(48 + c) * S::OUT] = accb[c];
         }
         __syncthreads();
+        if (gr > 0) return;
+        for (int q = 0; q < GR - 1; ++q) {
+            const float *r = red + (size_t)q * 52 * S::OUT + o;
 #pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            const int j = tid + q * kWgThreads;
-            if (j < NOUT) {
-                const int co = j / CIN, ci = j % CIN;
-                float s = 0.0f;
-#pragma unroll 8
-                for (int p = 0; p < kWgTile; ++p) s = fmaf(gs[p * COUT + co], xs[p * XS + ci], s);
-                acc[q] += s;
+            for (int k = 0; k < 48; ++k) acc[k / 16][k / 4 % 4][k % 4] += r[k * S::OUT];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) accb[c] += r[(48 + c) * S::OUT];
+        }
+    }
+    float *out = a.part + (size_t)blockIdx.x * 9 * CIN * COUT;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            *reinterpret_cast<float4 *>(out + ((size_t)(dy * 3 + k) * COUT + co + c) * CIN + ci) =
+                make_float4(acc[k][c][0], acc[k][c][1], acc[k][c][2], acc[k][c][3]);
+    if (bias)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) a.partb[(size_t)blockIdx.x * COUT + co + c] = accb[c];
+}
+
+// The first layer (one input channel, 16 outputs): a thread keeps the 9 taps
+// of four outputs for one pixel column of a segment and walks down its rows
+// with a 3 x 3 window of the input; the 64 columns of a block are added in a
+// fixed order (lanes, then warps).
+__global__ void __launch_bounds__(kThreads) k_wgrad_first(WgArgs a)
+{
+    __shared__ float red[kThreads / 32][160];
+    const int cg = threadIdx.x & 3, px = threadIdx.x >> 2;
+    float acc[40];   // 9 taps x 4 outputs, then db
+#pragma unroll
+    for (int k = 0; k < 40; ++k) acc[k] = 0.0f;
+    for (int t = blockIdx.x; t < a.items; t += gridDim.x) {
+        int b, x0, y0, y1;
+        wg_item(a, t, b, x0, y0, y1);
+        const int xx = x0 + px;
+        if (px >= a.pt || xx >= a.w) continue;
+        auto row = [&](int y, float (&v)[3]) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int c = xx + d - 1;
+                v[d] = (y >= 0 && y < a.h && c >= 0 && c < a.w) ? bf2f(a.x[((size_t)b * a.h + y) * a.w + c]) : 0.0f;
+            }
+        };
+        float v[3][3];
+        row(y0 - 1, v[0]);
+        row(y0, v[1]);
+#pragma unroll 3
+        for (int y = y0; y < y1; ++y) {
+            row(y + 1, v[2]);
+            const float4 gv =
+                *reinterpret_cast<const float4 *>(a.g + (((size_t)b * a.h + y) * a.w + xx) * 16 + 4 * cg);
+            const float g4[4] = {gv.x, gv.y, gv.z, gv.w};
+#pragma unroll
+            for (int k = 0; k < 9; ++k)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[4 * k + c] = fmaf(g4[c], v[k / 3][k % 3], acc[4 * k + c]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[36 + c] += g4[c];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                v[0][d] = v[1][d];
+                v[1][d] = v[2][d];
             }
         }
-        if (centre && tid < COUT) {
-            float s = 0.0f;
-            for (int p = 0; p < kWgTile; ++p) s += gs[p * COUT + tid];
-            accb += s;
-        }
-        __syncthreads();
     }
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int j = tid + q * kWgThreads;
-        if (j < NOUT) a.part[((size_t)blockIdx.y * ntap + tap) * NOUT + j] = acc[q];
+    for (int k = 0; k < 40; ++k)
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+    if ((threadIdx.x & 31) < 4)
+#pragma unroll
+        for (int k = 0; k < 40; ++k) red[threadIdx.x / 32][k / 4 * 16 + 4 * cg + k % 4] = acc[k];
+    __syncthreads();
+    const int j = threadIdx.x;
+    if (j < 160) {
+        float s = 0.0f;
+        for (int q = 0; q < kThreads / 32; ++q) s += red[q][j];
+        if (j < 144) a.part[(size_t)blockIdx.x * 144 + j] = s;
+        else a.partb[(size_t)blockIdx.x * 16 + j - 144] = s;
     }
-    if (centre && tid < COUT) a.partb[(size_t)blockIdx.y * COUT + tid] = accb;
 }
 
-// dW[co][tap][ci] (parameter order) from the slice partials
-__global__ void k_wgrad_reduce(const float *part, int nslices, int ntap, int cin, int cout, float *dw)
+// dW[co][tap][ci] (parameter order) and db from the block partials: 32 outputs
+// x 8 lanes per block; lane q adds partials q, q + 8, ..., the lanes are added
+// in order.
+__global__ void k_wgrad_reduce(const float *part, const float *partb, int ns, int cin, int cout, float *dw, float *db)
 {
-    const int nout = cin * cout;
-    const int j = blockIdx.x * kThreads + threadIdx.x;
-    if (j >= ntap * nout) return;
-    const int tap = j / nout, r = j % nout;
-    const int co = r / cin, ci = r % cin;
+    __shared__ float red[8][32];
+    const int nout = cin * cout, nw = 9 * nout;
+    const int j = blockIdx.x * 32 + threadIdx.x, q = threadIdx.y;
     float s = 0.0f;
-    for (int i = 0; i < nslices; ++i) s += part[((size_t)i * ntap + tap) * nout + r];
-    dw[((size_t)co * ntap + tap) * cin + ci] = s;
+    if (j < nw + cout) {
+        const float *p = j < nw ? part + j : partb + (j - nw);
+        const size_t stride = j < nw ? nw : cout;
+#pragma unroll 8
+        for (int i = q; i < ns; i += 8) s += p[i * stride];
+    }
+    red[q][threadIdx.x] = s;
+    __syncthreads();
+    if (q || j >= nw + cout) return;
+    s = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += red[k][threadIdx.x];
+    if (j < nw) {
+        const int tap = j / nout, r = j % nout, co = r / cin, ci = r % cin;
+        dw[((size_t)co * 9 + tap) * cin + ci] = s;
+    } else {
+        db[j - nw] = s;
+    }
 }
 
 // ---- parameters: bfloat16 weight copies and Adam ----
@@ -464,51 +680,47 @@ __global__ void k_energy(int n, int h, int w, const float *y, const float *x, co
     if (threadIdx.x == 0) part[(size_t)b * gridDim.x + blockIdx.x] = red[0];
 }
 
+// mean over the samples of each one's loss sum / per; one block
 __global__ void k_energy_finish(const double *part, int nblk, int n, long long per, double *out)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double tot = 0.0;
-    for (int b = 0; b < n; ++b) {
-        double s = 0.0;
-        for (int i = 0; i < nblk; ++i) s += part[(size_t)b * nblk + i];
-        tot += s / (double)per;
+    __shared__ double red[kThreads];
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n * nblk; i += kThreads) s += part[i];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = kThreads / 2; o > 0; o >>= 1) {
+        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
     }
-    *out = tot / n;
+    if (threadIdx.x == 0) *out = red[0] / (double)per / n;
 }
 
 inline unsigned blocks(long long cnt) { return (unsigned)((cnt + kThreads - 1) / kThreads); }
 
-template <int CIN, int COUT>
-cudaError_t wgrad_mode(const WgArgs &a, int mode, int ntap, cudaStream_t st)
+// Weight-gradient kernel of a layer: its function, threads and shared memory.
+struct WgKernel {
+    void (*f)(WgArgs);
+    int threads, smem;
+};
+template <int CIN, int COUT, int GR>
+constexpr WgKernel wg_of()
 {
-    const int smem = (kWgTile * COUT + kWgTile * (CIN + (CIN > 1 ? 1 : 0))) * (int)sizeof(float);
-    dim3 grid(ntap, a.nslices);
-    cudaError_t e = cudaSuccess;
-    switch (mode) {
-    case GEA_CONV_PLAIN:
-        e = cudaFuncSetAttribute(k_wgrad<CIN, COUT, GEA_CONV_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) k_wgrad<CIN, COUT, GEA_CONV_PLAIN><<<grid, kWgThreads, smem, st>>>(a);
-        break;
-    case GEA_CONV_POOL:
-        e = cudaFuncSetAttribute(k_wgrad<CIN, COUT, GEA_CONV_POOL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) k_wgrad<CIN, COUT, GEA_CONV_POOL><<<grid, kWgThreads, smem, st>>>(a);
-        break;
-    default:
-        e = cudaFuncSetAttribute(k_wgrad<CIN, COUT, GEA_CONV_UPADD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) k_wgrad<CIN, COUT, GEA_CONV_UPADD><<<grid, kWgThreads, smem, st>>>(a);
-        break;
-    }
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return WgKernel{k_wgrad<CIN, COUT, GR>, WgShape<CIN, COUT, GR>::THREADS, WgShape<CIN, COUT, GR>::SMEM};
 }
-
-cudaError_t wgrad_launch(const WgArgs &a, int cin, int cout, int mode, int ntap, cudaStream_t st)
+// Pixel groups: a block of 192 threads (48 or 96 per group) keeps several
+// blocks on an SM; from 32 x 32 on one group fills it.
+inline WgKernel wg_kernel(int cin, int cout)
 {
-#define GEA_WG(CI, CO) \
-    if (cin == CI && cout == CO) return wgrad_mode<CI, CO>(a, mode, ntap, st);
-    GEA_WG(1, 16) GEA_WG(16, 16) GEA_WG(16, 32) GEA_WG(32, 32) GEA_WG(32, 64) GEA_WG(64, 64) GEA_WG(64, 32)
-    GEA_WG(32, 16)
-#undef GEA_WG
-    return cudaErrorInvalidValue;
+    switch (cin * 100 + cout) {
+    case 1616: return wg_of<16, 16, 4>();
+    case 1632: return wg_of<16, 32, 2>();
+    case 3216: return wg_of<32, 16, 2>();
+    case 3232: return wg_of<32, 32, 1>();
+    case 3264: return wg_of<32, 64, 1>();
+    case 6432: return wg_of<64, 32, 1>();
+    case 6464: return wg_of<64, 64, 1>();
+    default: return WgKernel{k_wgrad_first, kThreads, 0};
+    }
 }
 
 }  // namespace gea_net_impl
@@ -527,6 +739,7 @@ struct gea_net {
     uint16_t *gbf = nullptr, *xbf = nullptr;
     float *gin = nullptr, *xh = nullptr, *rms = nullptr, *cmean = nullptr;
     float *part = nullptr, *partb = nullptr;
+    int wg_blocks[L] = {};   // resident blocks of each layer's weight-gradient kernel
     double *dpart = nullptr, *loss = nullptr;
     int *status = nullptr;
     int n = 0, h = 0, w = 0;
@@ -584,10 +797,12 @@ int pack_all(gea_net *net)
 // per-sample reduction of x (n samples of `per` values) into out[b]
 void sample_stat(gea_net *net, const float *x, int n, long long per, int mode, float *out)
 {
-    dim3 g(kStatBlocks, n);
+    // one pass of the threads over a small sample, several over a large one
+    const int nb = (int)std::min<long long>(kStatBlocks, (per / 4 + kThreads - 1) / kThreads);
+    dim3 g(nb, n);
     const int vec = (reinterpret_cast<uintptr_t>(x) & 15u) == 0;
     k_sample_partials<<<g, kThreads, 0, net->st>>>(x, per, mode == 0 ? 1 : 0, vec, net->dpart);
-    k_sample_finish<<<n, kThreads, 0, net->st>>>(net->dpart, kStatBlocks, per, mode, out);
+    k_sample_finish<<<n, kThreads, 0, net->st>>>(net->dpart, nb, per, mode, out);
 }
 
 int forward(gea_net *net, int n, int h, int w, const float *r, float *y)
@@ -620,61 +835,90 @@ int forward(gea_net *net, int n, int h, int w, const float *r, float *y)
     return GEA_OK;
 }
 
+// Split of a weight gradient over `slots` resident blocks: row segments of at
+// most kWgPix pixels, and as many rows per work item as make the longest
+// block's rows (plus the item's two extra input rows) fewest. Returns the
+// blocks to launch.
+int wgrad_split(WgArgs &a, int n, int h, int w, int slots)
+{
+    a.n = n; a.h = h; a.w = w;
+    a.strips = (w + kWgPix - 1) / kWgPix;
+    a.pt = (w + a.strips - 1) / a.strips;
+    long long best = -1;
+    for (int rb = 1; rb <= h; ++rb) {
+        const int chunks = (h + rb - 1) / rb;
+        const long long items = (long long)n * a.strips * chunks;
+        const long long cost = (items + slots - 1) / slots * (rb + 1);
+        if (best < 0 || cost < best) {
+            best = cost;
+            a.rb = rb;
+            a.chunks = chunks;
+            a.items = (int)items;
+        }
+    }
+    return a.items < slots ? a.items : slots;
+}
+
 int backward(gea_net *net, const float *dy, float *grad)
 {
     cudaStream_t st = net->st;
     const int n = net->n, h = net->h, w = net->w;
     const long long tot = (long long)n * h * w;
-    for (int l = 0; l < kOut; ++l)
-        if (cudaMemsetAsync(net->gact[l], 0, (size_t)level_pix(n, h, w, kL[l].level) * kL[l].cout * sizeof(float),
-                            st) != cudaSuccess)
-            return GEA_ERR_CUDA;
     // output layer
     {
         const unsigned nb = blocks(tot);
         k_out_backward<<<nb, kThreads, 0, st>>>(tot, dy, net->act[kOut - 1], net->theta + net->offw[kOut],
                                                 net->gact[kOut - 1], net->part);
-        k_sum_partials<<<1, kThreads, 0, st>>>(net->part, (int)nb, 17, 17, grad + net->offw[kOut]);
+        k_sum_partials<<<17, kThreads, 0, st>>>(net->part, (int)nb, 17, grad + net->offw[kOut]);
     }
     for (int l = kOut - 1; l >= 0; --l) {
         const LayerDef &d = kL[l];
         const int hl = h >> d.level, wl = w >> d.level;
-        const long long cnt = level_pix(n, h, w, d.level) * d.cout;
-        k_mask<<<blocks(cnt), kThreads, 0, st>>>(cnt, net->gact[l], net->act[l], net->relu && d.act,
-                                                 l > 0 ? net->gbf : nullptr);
-        // weight gradient
+        const long long pix = level_pix(n, h, w, d.level), quads = pix * d.cout / 4;
+        const int relu = net->relu && d.act;
+        if (relu || l > 0)
+            k_mask<<<blocks(quads), kThreads, 0, st>>>(quads, reinterpret_cast<float4 *>(net->gact[l]),
+                                                       reinterpret_cast<const uint2 *>(net->act[l]), relu,
+                                                       l > 0 ? reinterpret_cast<uint2 *>(net->gbf) : nullptr);
+        // the layer's input: an averaged or summed one is formed again, in the
+        // buffer that the data gradient overwrites afterwards
         WgArgs a{};
-        a.n = n; a.h = hl; a.w = wl;
+        uint2 *xin = reinterpret_cast<uint2 *>(net->gin);
+        const int c4 = d.cin / 4;
+        if (d.kind == SRC_X) a.x = net->xbf;
+        else if (d.kind == SRC_PREV) a.x = net->act[d.a];
+        else {
+            a.x = reinterpret_cast<const uint16_t *>(xin);
+            if (d.kind == SRC_POOL)
+                k_form_input<GEA_CONV_POOL><<<blocks(pix * c4), kThreads, 0, st>>>(
+                    n, hl, wl, c4, reinterpret_cast<const uint2 *>(net->act[d.a]), nullptr, xin);
+            else
+                k_form_input<GEA_CONV_UPADD><<<blocks(pix * c4), kThreads, 0, st>>>(
+                    n, hl, wl, c4, reinterpret_cast<const uint2 *>(net->act[d.b]),
+                    reinterpret_cast<const uint2 *>(net->act[d.a]), xin);
+        }
         a.g = net->gact[l];
         a.part = net->part; a.partb = net->partb;
-        a.tiles_per_row = (wl + kWgTile - 1) / kWgTile;
-        a.ntiles = n * hl * a.tiles_per_row;
-        a.nslices = a.ntiles < kMaxSlices ? a.ntiles : kMaxSlices;
-        int mode = GEA_CONV_PLAIN;
-        if (d.kind == SRC_X) a.x0 = net->xbf;
-        else if (d.kind == SRC_PREV) a.x0 = net->act[d.a];
-        else if (d.kind == SRC_POOL) { a.x0 = net->act[d.a]; mode = GEA_CONV_POOL; }
-        else { a.x0 = net->act[d.b]; a.x1 = net->act[d.a]; mode = GEA_CONV_UPADD; }
-        if (wgrad_launch(a, d.cin, d.cout, mode, 9, st) != cudaSuccess) return GEA_ERR_CUDA;
-        const int nw = 9 * d.cin * d.cout;
-        k_wgrad_reduce<<<blocks(nw), kThreads, 0, st>>>(net->part, a.nslices, 9, d.cin, d.cout, grad + net->offw[l]);
-        k_sum_partials<<<blocks(d.cout), kThreads, 0, st>>>(net->partb, a.nslices, d.cout, d.cout,
-                                                            grad + net->offb[l]);
+        const int ns = wgrad_split(a, n, hl, wl, net->wg_blocks[l]);
+        const WgKernel k = wg_kernel(d.cin, d.cout);
+        k.f<<<ns, k.threads, k.smem, st>>>(a);
+        k_wgrad_reduce<<<(9 * d.cin * d.cout + d.cout + 31) / 32, dim3(32, 8), 0, st>>>(
+            net->part, net->partb, ns, d.cin, d.cout, grad + net->offw[l], grad + net->offb[l]);
         if (l == 0) break;
         // data gradient on the tensor cores: correlation of bf16(g) with the
-        // mirrored, transposed weights
+        // mirrored, transposed weights. A tensor's first gradient is written
+        // in place (the layers run last to first: a skip tensor's comes from
+        // the way up), the averaging's is added to it.
+        float *dst = d.kind == SRC_POOL ? net->gin : net->gact[d.kind == SRC_UPADD ? d.b : d.a];
         if (gea_conv3x3_launch(n, hl, wl, d.cout, d.cin, GEA_CONV_PLAIN, GEA_CONV_OUT_F32, net->gbf, nullptr,
-                               net->wb[l], nullptr, net->gin, net->status, st) != cudaSuccess)
+                               net->wb[l], nullptr, dst, net->status, st) != cudaSuccess)
             return GEA_ERR_CUDA;
-        const long long icnt = level_pix(n, h, w, d.level) * d.cin;
-        if (d.kind == SRC_PREV) {
-            k_add<<<blocks(icnt), kThreads, 0, st>>>(icnt, net->gact[d.a], net->gin);
-        } else if (d.kind == SRC_POOL) {
-            k_pool_backward<<<blocks(icnt * 4), kThreads, 0, st>>>(n, hl, wl, d.cin, net->gact[d.a], net->gin);
-        } else {
-            k_add<<<blocks(icnt), kThreads, 0, st>>>(icnt, net->gact[d.b], net->gin);
-            k_up_backward<<<blocks(icnt / 4), kThreads, 0, st>>>(n, hl, wl, d.cin, net->gact[d.a], net->gin);
-        }
+        const float4 *dst4 = reinterpret_cast<const float4 *>(dst);
+        float4 *ga = reinterpret_cast<float4 *>(net->gact[d.a]);
+        if (d.kind == SRC_POOL)
+            k_pool_backward<<<blocks(pix * c4 * 4), kThreads, 0, st>>>(n, hl, wl, c4, ga, dst4);
+        else if (d.kind == SRC_UPADD)
+            k_up_backward<<<blocks(pix * c4 / 4), kThreads, 0, st>>>(n, hl, wl, c4, ga, dst4);
     }
     return cudaGetLastError() == cudaSuccess ? GEA_OK : GEA_ERR_CUDA;
 }
@@ -688,7 +932,7 @@ int energy(gea_net *net, const float *c, const float *ax, const float *az, float
     sample_stat(net, c, n, per, 1, net->cmean);
     dim3 g(kSampleBlocks, n);
     k_energy<<<g, kThreads, 0, st>>>(n, h, w, net->last_y, net->xh, c, ax, az, net->cmean, dy, net->dpart);
-    k_energy_finish<<<1, 32, 0, st>>>(net->dpart, kSampleBlocks, n, per, net->loss);
+    k_energy_finish<<<1, kThreads, 0, st>>>(net->dpart, kSampleBlocks, n, per, net->loss);
     double hl = 0.0;
     if (cudaMemcpyAsync(&hl, net->loss, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
@@ -786,11 +1030,22 @@ int gea_net_create(int32_t n_max, int32_t h_max, int32_t w_max, int32_t flags, g
     net->xh = take<float>(net, pix, ok);
     net->rms = take<float>(net, n_max, ok);
     net->cmean = take<float>(net, n_max, ok);
-    const long long ns = kMaxSlices;
-    long long pcount = ns * 9 * 64 * 64;
-    if (17 * ((pix + kThreads - 1) / kThreads) > pcount) pcount = 17 * ((pix + kThreads - 1) / kThreads);
+    // block partials of the weight gradients: one set per resident block
+    int dev = 0, sms = 0;
+    long long pcount = 17 * ((pix + kThreads - 1) / kThreads), bcount = 0;
+    ok = ok && cudaGetDevice(&dev) == cudaSuccess &&
+         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+    for (int l = 0; l < kOut && ok; ++l) {
+        const WgKernel k = wg_kernel(kL[l].cin, kL[l].cout);
+        int per_sm = 0;
+        ok = cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem) == cudaSuccess &&
+             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.f, k.threads, k.smem) == cudaSuccess && per_sm > 0;
+        net->wg_blocks[l] = per_sm * sms;
+        pcount = std::max(pcount, (long long)net->wg_blocks[l] * 9 * kL[l].cin * kL[l].cout);
+        bcount = std::max(bcount, (long long)net->wg_blocks[l] * kL[l].cout);
+    }
     net->part = take<float>(net, pcount, ok);
-    net->partb = take<float>(net, ns * 64, ok);
+    net->partb = take<float>(net, bcount, ok);
     net->dpart = take<double>(net, (size_t)n_max * (kStatBlocks > kSampleBlocks ? kStatBlocks : kSampleBlocks), ok);
     net->loss = take<double>(net, 1, ok);
     net->status = take<int>(net, 1, ok);
