@@ -553,6 +553,43 @@ int copy_out(gea_ctx *ctx, double *dst, const double *src, int ncols, int rows)
     return GEA_OK;
 }
 
+// A full view's arrays in field order (the first nf fields).
+DenseFields dense_fields(const gea_state_view *v, int nf)
+{
+    DenseFields d = {{v->rho, v->u, v->w, v->T, v->h, v->p, v->pp, v->pold, v->phix, v->phiz, v->Kold}};
+    for (int f = nf; f < NFIELDS; ++f) d.p[f] = nullptr;
+    return d;
+}
+
+// Whether the non-null pointers are plain device memory of the context's
+// device, which a kernel may access directly (managed and host pointers, and
+// another device's, go through the runtime's copies whatever the caller's mem).
+bool on_device(const gea_ctx *ctx, double *const *p, int n)
+{
+    for (int f = 0; f < n; ++f) {
+        if (!p[f]) continue;
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, p[f]) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (at.type != cudaMemoryTypeDevice || at.device != ctx->device ||
+            reinterpret_cast<uintptr_t>(p[f]) % sizeof(double))
+            return false;
+    }
+    return true;
+}
+
+// Whether no two of the arrays (count[f] values each) overlap: one kernel
+// writes them in no particular order.
+bool disjoint(double *const *p, const size_t *count, int n)
+{
+    for (int f = 0; f < n; ++f)
+        for (int g = 0; g < f; ++g)
+            if (p[f] && p[g] && p[f] < p[g] + count[g] && p[g] < p[f] + count[f]) return false;
+    return true;
+}
+
 }  // namespace
 
 extern "C" {
@@ -847,14 +884,20 @@ int gea_set_state(gea_ctx *ctx, const gea_state_view *v)
     // reset the device scalars: status, counters, step count
     CK(cudaMemsetAsync(ctx->sc, 0, sizeof(Scal), ctx->stream));
     if (v->kind == GEA_STATE_CONSERVATIVE) {
+        double *const in[4] = {v->rho, v->rhou, v->rhow, v->rhoe};
         const size_t cellw = ctx->stage_stride;
         double *st = ctx->stage;
         int rc;
-        if ((rc = copy_in(ctx, st, v->rho, nx, nz)) || (rc = copy_in(ctx, st + cellw, v->rhou, nx, nz)) ||
-            (rc = copy_in(ctx, st + 2 * cellw, v->rhow, nx, nz)) ||
-            (rc = copy_in(ctx, st + 3 * cellw, v->rhoe, nx, nz)))
-            return rc;
-        launch_derive(G, ctx->F, st, st + cellw, st + 2 * cellw, st + 3 * cellw, S, ctx->sc, ctx->stream);
+        if (v->mem == GEA_MEM_DEVICE && on_device(ctx, in, 4)) {
+            launch_derive(G, ctx->F, v->rho, v->rhou, v->rhow, v->rhoe, nx, S, ctx->sc, ctx->stream);
+        } else {
+            for (int f = 0; f < 4; ++f)
+                if ((rc = copy_in(ctx, st + f * cellw, in[f], nx, nz))) return rc;
+            launch_derive(G, ctx->F, st, st + cellw, st + 2 * cellw, st + 3 * cellw, G.P, S, ctx->sc, ctx->stream);
+        }
+        CK(cudaGetLastError());
+    } else if (DenseFields d = dense_fields(v, nf); v->mem == GEA_MEM_DEVICE && on_device(ctx, d.p, nf)) {
+        launch_fields_in(G, S, d, ctx->stream);
         CK(cudaGetLastError());
     } else {
         for (int f = 0; f < nf; ++f) {
@@ -950,34 +993,47 @@ int gea_get_state(gea_ctx *ctx, gea_state_view *v)
 {
     if (!ctx || !v) return GEA_ERR_INVAL;
     if (!ctx->have_state) return fail(ctx, GEA_ERR_STATE, "no state set");
-    Scal h;
-    int rc = read_scal(ctx, &h);
-    if (rc) return rc;
+    if (v->kind != GEA_STATE_FULL && v->kind != GEA_STATE_CONSERVATIVE)
+        return fail(ctx, GEA_ERR_INVAL, "unknown state kind %d", v->kind);
     const Geom &G = ctx->G;
     const int nx = G.nx, nz = G.nz;
-    const State &S = ctx->S[current_slot(ctx, h)];
+    int rc;
     if (v->kind == GEA_STATE_FULL) {
-        double *dst[11] = {v->rho, v->u, v->w, v->T, v->h, v->p, v->pp, v->pold, v->phix, v->phiz, v->Kold};
-        const double *src[11] = {S.rho, S.u, S.w, S.T, S.h, S.p, S.pp, S.pold, S.phix, S.phiz, S.Kold};
         const int nf = ctx->F.k_lagged ? 11 : 10;
+        const DenseFields d = dense_fields(v, nf);
+        int cols[NFIELDS], rows[NFIELDS];
+        size_t count[NFIELDS];
         for (int f = 0; f < nf; ++f) {
-            if (!dst[f]) continue;
-            const int cols = f == 8 ? nx + 1 : nx, rows = f == 9 ? nz + 1 : nz;
-            if ((rc = copy_out(ctx, dst[f], src[f], cols, rows))) return rc;
+            cols[f] = f == FIELD_PHIX ? nx + 1 : nx;
+            rows[f] = f == FIELD_PHIZ ? nz + 1 : nz;
+            count[f] = (size_t)cols[f] * rows[f];
         }
-    } else if (v->kind == GEA_STATE_CONSERVATIVE) {
-        // computed on the device into the staging area, then copied out
-        const size_t cellw = ctx->stage_stride;
-        double *st = ctx->stage;
-        launch_conserve(G, ctx->F, S, st, st + cellw, st + 2 * cellw, st + 3 * cellw, ctx->stream);
-        CK(cudaGetLastError());
-        double *dst[4] = {v->rho, v->rhou, v->rhow, v->rhoe};
-        for (int f = 0; f < 4; ++f) {
-            if (!dst[f]) continue;
-            if ((rc = copy_out(ctx, dst[f], st + f * cellw, nx, nz))) return rc;
+        if (v->mem == GEA_MEM_DEVICE && on_device(ctx, d.p, nf) && disjoint(d.p, count, nf)) {
+            launch_fields_out(G, ctx->S, ctx->base, ctx->sc, d, ctx->stream);
+            CK(cudaGetLastError());
+        } else {
+            Scal h;
+            if ((rc = read_scal(ctx, &h))) return rc;
+            const FieldPtrs src = state_fields(ctx->S[current_slot(ctx, h)]);
+            for (int f = 0; f < nf; ++f)
+                if (d.p[f] && (rc = copy_out(ctx, d.p[f], src.p[f], cols[f], rows[f]))) return rc;
         }
     } else {
-        return fail(ctx, GEA_ERR_INVAL, "unknown state kind %d", v->kind);
+        double *const dst[4] = {v->rho, v->rhou, v->rhow, v->rhoe};
+        const size_t cells = (size_t)nx * nz, count[4] = {cells, cells, cells, cells};
+        if (v->mem == GEA_MEM_DEVICE && on_device(ctx, dst, 4) && disjoint(dst, count, 4)) {
+            launch_conserve(G, ctx->F, ctx->S, ctx->base, ctx->sc, v->rho, v->rhou, v->rhow, v->rhoe, nx, ctx->stream);
+            CK(cudaGetLastError());
+        } else {
+            // computed on the device into the staging area, then copied out
+            const size_t cellw = ctx->stage_stride;
+            double *st = ctx->stage;
+            launch_conserve(G, ctx->F, ctx->S, ctx->base, ctx->sc, st, st + cellw, st + 2 * cellw, st + 3 * cellw, G.P,
+                            ctx->stream);
+            CK(cudaGetLastError());
+            for (int f = 0; f < 4; ++f)
+                if (dst[f] && (rc = copy_out(ctx, dst[f], st + f * cellw, nx, nz))) return rc;
+        }
     }
     CK(cudaStreamSynchronize(ctx->stream));
     return GEA_OK;

@@ -55,6 +55,20 @@ struct State {
     double *rho, *u, *w, *T, *h, *p, *pp, *pold, *phix, *phiz, *Kold;
 };
 
+// A state's fields in the order of gea_state_view, and a caller's arrays for
+// them (dense rows).
+enum { FIELD_PHIX = 8, FIELD_PHIZ = 9, NFIELDS = 11 };
+struct FieldPtrs {
+    double *p[NFIELDS];
+};
+struct DenseFields {
+    double *p[NFIELDS];   // only read when they are the source
+};
+inline FieldPtrs state_fields(const State &S)
+{
+    return FieldPtrs{{S.rho, S.u, S.w, S.T, S.h, S.p, S.pp, S.pold, S.phix, S.phiz, S.Kold}};
+}
+
 // One multigrid level of the Helmholtz operator
 //   (A x)_i = c_i x_i + sum_f a_f (x_i - x_N) = d_i x_i - sum_f a_f x_N,
 // d_i = c_i + sum_f a_f, kept as d and wd = 1 / d.
@@ -402,12 +416,17 @@ __host__ __device__ __forceinline__ const double *pp_in(const StepArgs &a, int c
 }
 
 // ---- host-side launchers (gea_kernels.cu); tr may be null ----
+// conservative variables (rows of `pitch` values) to a state, and of the state
+// in slot (base + steps done) & 1 (null arrays are left out)
 void launch_derive(const Geom &G, const Phys &F, const double *rho, const double *rhou,
-                   const double *rhow, const double *rhoe, const State &S, Scal *sc,
+                   const double *rhow, const double *rhoe, int pitch, const State &S, Scal *sc,
                    cudaStream_t st);
-// conservative variables rho, rho u, rho w, rho e of state S (pitched arrays)
-void launch_conserve(const Geom &G, const Phys &F, const State &S, double *rho, double *rhou, double *rhow,
-                     double *rhoe, cudaStream_t st);
+void launch_conserve(const Geom &G, const Phys &F, const State S[2], int base, const Scal *sc, double *rho,
+                     double *rhou, double *rhow, double *rhoe, int pitch, cudaStream_t st);
+// all fields between a state and a caller's dense device arrays (null: left out)
+void launch_fields_in(const Geom &G, const State &S, const DenseFields &src, cudaStream_t st);
+void launch_fields_out(const Geom &G, const State S[2], int base, const Scal *sc, const DenseFields &dst,
+                       cudaStream_t st);
 void launch_les(const StepArgs &a, cudaStream_t st, Tracer *tr);
 void launch_pred_setup(const StepArgs &a, cudaStream_t st, Tracer *tr);
 // second = 1: the second sweep of a pair (copies instead once converged)
