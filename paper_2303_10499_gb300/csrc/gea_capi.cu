@@ -41,6 +41,7 @@ struct gea_ctx {
     double *rho1, *dinvu, *dinvh, *bu, *bw, *ua, *wa, *ub, *wb, *bh, *ha, *hb, *rho2, *psi, *Dx,
         *Dz, *Hx, *Hz, *b, *p0, *p1, *q, *dtr1;
     double *gzc, *gzf;                     // g z of cell-centre rows (nz) and z-face rows (nz + 1)
+    double *gx2, *gz2;                     // 2 g z / dx and 2 g z / dz of them
     double *stage;                         // staging for conservative set/get (4 fields)
     size_t stage_stride = 0;               // elements from one staging field to the next
     double *thbar;                         // nz values
@@ -136,6 +137,8 @@ StepArgs step_args(gea_ctx *c, int from)
     a.dtr1 = c->dtr1;
     a.gzc = c->gzc;
     a.gzf = c->gzf;
+    a.gx2 = c->gx2;
+    a.gz2 = c->gz2;
     a.sc = c->sc;
     a.partials = c->partials;
     a.jac_rtol2 = c->C.jac_rtol * c->C.jac_rtol;
@@ -622,6 +625,16 @@ int gea_create(const gea_grid *grid, const gea_constants *c, gea_ctx **out)
     ctx->F.les_d2 = c->cs * c->cs * ctx->G.dx * ctx->G.dz;
     ctx->F.R = c->R; ctx->F.cp = c->cp; ctx->F.g = c->g; ctx->F.p0 = c->p0;
     ctx->F.mu = c->mu; ctx->F.nuh = c->mu / c->Pr; ctx->F.dt = c->dt; ctx->F.idt = 1.0 / c->dt;
+    {
+        const Geom &g = ctx->G;
+        Phys &F = ctx->F;
+        F.ix2 = g.idx * g.idx; F.iz2 = g.idz * g.idz; F.hix2 = 0.5 * F.ix2; F.hiz2 = 0.5 * F.iz2;
+        F.mux = F.mu * F.ix2; F.muz = F.mu * F.iz2; F.mud = 2.0 * (F.mux + F.muz);
+        F.hix = 0.5 * g.idx; F.hiz = 0.5 * g.idz; F.tix = 2.0 * g.idx; F.tiz = 2.0 * g.idz;
+        F.hdx = 0.5 * g.dx; F.hdz = 0.5 * g.dz;
+        F.s12 = g.iV / 12.0; F.s24 = g.iV / 24.0;
+        F.icp = 1.0 / c->cp;
+    }
     ctx->F.k_lagged = (c->reading_flags & GEA_READING_K_LAGGED) ? 1 : 0;
     ctx->F.les = ctx->F.les_d2 > 0.0 ? 1 : 0;
     ctx->F.pr_ne1 = ctx->F.nuh != ctx->F.mu ? 1 : 0;
@@ -655,7 +668,7 @@ int gea_create(const gea_grid *grid, const gea_constants *c, gea_ctx **out)
     size_t total = 0;
     total += 2 * (10 * cell + fz);                 // two states (phiz has nz+1 rows)
     total += 34 * cell + 2 * fz;                   // scratch (Dz has nz+1 rows)
-    total += round_up((2 * (size_t)G.nz + 1) * sizeof(double), 256);   // height tables
+    total += 2 * round_up((2 * (size_t)G.nz + 1) * sizeof(double), 256);   // height tables
     total += 4 * cell;                             // staging for conservative fields
     total += 2 * cell + round_up(G.nz * sizeof(double), 256);   // theta_bar, theta'
     if (c->flags & GEA_FLAG_KEEP_R0) total += cell;
@@ -744,6 +757,8 @@ int gea_create(const gea_grid *grid, const gea_constants *c, gea_ctx **out)
     ctx->dtr1 = cellA("dtr1", 0);
     ctx->gzc = vec(2 * (size_t)nz + 1, "gz");
     ctx->gzf = ctx->gzc + nz;
+    ctx->gx2 = vec(2 * (size_t)nz + 1, "gz2");
+    ctx->gz2 = ctx->gx2 + nz;
     ctx->stage = cellA("stage%d", 0);
     for (int j = 1; j < 4; ++j) cellA("stage%d", j);
     ctx->stage_stride = (arr_bytes(G, nz) + guard) / sizeof(double);
@@ -805,7 +820,11 @@ int gea_create(const gea_grid *grid, const gea_constants *c, gea_ctx **out)
         std::vector<double> h(2 * (size_t)G.nz + 1);
         for (int k = 0; k < G.nz; ++k) h[k] = ctx->F.g * ((k + 0.5) * G.dz);
         for (int k = 0; k <= G.nz; ++k) h[G.nz + k] = ctx->F.g * (k * G.dz);
-        if (cudaMemcpy(ctx->gzc, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) {
+        std::vector<double> h2(h);
+        for (int k = 0; k < G.nz; ++k) h2[k] *= ctx->F.tix;
+        for (int k = 0; k <= G.nz; ++k) h2[G.nz + k] *= ctx->F.tiz;
+        if (cudaMemcpy(ctx->gzc, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaMemcpy(ctx->gx2, h2.data(), h2.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) {
             gea_destroy(ctx);
             return GEA_ERR_CUDA;
         }

@@ -42,6 +42,14 @@ struct Phys {
     double omega;                            // weight of the smoother's black relaxations
     double les_d2;                           // Smagorinsky (cs Delta)^2; 0: constant viscosity
     int k_lagged;                            // GEA_READING_K_LAGGED: K^{n-1} in eq. step3_sd
+    // products of the constants above and the spacings, formed once on the host:
+    // in a kernel each would be an FP64 instruction of every thread
+    double mux, muz, mud;                    // mu / dx^2, mu / dz^2, twice their sum
+    double ix2, iz2, hix2, hiz2;             // 1 / dx^2, 1 / dz^2 and their halves
+    double hix, hiz, tix, tiz;               // 1 / (2 dx), 1 / (2 dz), 2 / dx, 2 / dz
+    double hdx, hdz;                         // dx / 2, dz / 2
+    double s12, s24;                         // 1 / (12 dx dz), 1 / (24 dx dz)
+    double icp;                              // 1 / cp
     // uniform branch flags as integers (an FP64 compare issues on the FP64 pipe)
     int les;                                 // les_d2 > 0
     int pr_ne1;                              // nuh != mu (Pr != 1): the enthalpy stencil differs
@@ -191,6 +199,7 @@ struct StepArgs {
     double *rho2, *psi, *Dx, *Dz, *Hx, *Hz, *b;          // Step 3
     double *dtr1;                                        // dt / rho^{n+1/3} (Step 1, used by Step 3)
     const double *gzc, *gzf;   // g z of the cell centres of row k (nz values) and of z-face k (nz + 1)
+    const double *gx2, *gz2;   // 2 g z / dx of the cell centres and 2 g z / dz of the z-faces
     double *p0, *p1, *q;                                 // CG directions (ping-pong) and A p
     Scal *sc;
     double *partials;
@@ -234,6 +243,24 @@ __device__ __forceinline__ double ldc(const Geom &G, const Phys &F, const double
         return v;
     }
     return X[k * G.P + i];
+}
+
+// 1 / a for a normal a (densities, temperatures, diagonals) by one step of
+// Chebyshev's third-order iteration for the reciprocal, x0 (1 + e + e^2) with
+// e = 1 - a x0, from the hardware's seed (about 20 bits, so e^3 is below the
+// last bit): three FP64 instructions, the result within an ulp. The division
+// operator takes about three times as many, with a test for the cases that
+// cannot occur here (0, infinities and subnormals give NaN, which the residual
+// norms report). With the constants' products formed on the host and each
+// residual one chain of FMAs it took the 4096 x 2048 step from 17.1 to 15.5 ms
+// (mixed 11.3 to 9.5): eos_coef 79 -> about 40 FP64 instructions per cell,
+// pred_setup 72 -> 44, helm_rhs 42 -> 31, correct 34 -> 28.
+__device__ __forceinline__ double recip(double a)
+{
+    double x;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(a));
+    const double e = fma(-a, x, 1.0);
+    return fma(x, fma(e, e, e), x);
 }
 
 template <class T>

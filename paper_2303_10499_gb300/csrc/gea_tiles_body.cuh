@@ -169,29 +169,12 @@ __device__ __forceinline__ void ph_copy(const Geom &G, const R *X, R *Y, int bx,
     if (cell_of(G, bx, bz, i, k)) Y[cidx(G, i, k)] = ld(&X[cidx(G, i, k)]);
 }
 
-// 9-point cross stencil sum_o c_o X_o at tile position (y, x).
-template <int H, class R>
-__device__ __forceinline__ R apply9(const Stencil9T<R> &T, int q, const Tile<H, R> &s, int y, int x)
-{
-    R acc = ld(&T.cC[q]) * s[y][x];
-    acc = fma(ld(&T.cE1[q]), s[y][x + 1], acc);
-    acc = fma(ld(&T.cW1[q]), s[y][x - 1], acc);
-    acc = fma(ld(&T.cN1[q]), s[y + 1][x], acc);
-    acc = fma(ld(&T.cS1[q]), s[y - 1][x], acc);
-    acc = fma(ld(&T.cE2[q]), s[y][x + 2], acc);
-    acc = fma(ld(&T.cW2[q]), s[y][x - 2], acc);
-    acc = fma(ld(&T.cN2[q]), s[y + 2][x], acc);
-    acc = fma(ld(&T.cS2[q]), s[y - 2][x], acc);
-    return acc;
-}
-
 // 5-point Laplacian (X_E + X_W - 2 X_C)/dx^2 + (X_N + X_S - 2 X_C)/dz^2.
 template <int H, class R>
-__device__ __forceinline__ R lap5(const Geom &G, const Tile<H, R> &s, int y, int x)
+__device__ __forceinline__ R lap5(const Phys &F, const Tile<H, R> &s, int y, int x)
 {
     const R c2 = (R)2 * s[y][x];
-    return (s[y][x + 1] + s[y][x - 1] - c2) * (R)(G.idx * G.idx) +
-           (s[y + 1][x] + s[y - 1][x] - c2) * (R)(G.idz * G.idz);
+    return (s[y][x + 1] + s[y][x - 1] - c2) * (R)F.ix2 + (s[y + 1][x] + s[y - 1][x] - c2) * (R)F.iz2;
 }
 
 // A x = d x - sum a x_N at tile position (y, x) of cell (i, k) (zero tile
@@ -262,20 +245,19 @@ __device__ __forceinline__ Coef9<R> coef9(const Stencil9T<R> &T, int q)
                     ld(&T.cE2[q]), ld(&T.cW2[q]), ld(&T.cN2[q]), ld(&T.cS2[q])};
 }
 
-// sum_o c_o X_o in apply9's order.
+// b - sum_o c_o X_o as one chain of nine FMAs.
 template <int H, class R>
-__device__ __forceinline__ R apply9c(const Coef9<R> &c, const Tile<H, R> &s, int y, int x)
+__device__ __forceinline__ R sub9c(R b, const Coef9<R> &c, const Tile<H, R> &s, int y, int x)
 {
-    R acc = c.cC * s[y][x];
-    acc = fma(c.cE1, s[y][x + 1], acc);
-    acc = fma(c.cW1, s[y][x - 1], acc);
-    acc = fma(c.cN1, s[y + 1][x], acc);
-    acc = fma(c.cS1, s[y - 1][x], acc);
-    acc = fma(c.cE2, s[y][x + 2], acc);
-    acc = fma(c.cW2, s[y][x - 2], acc);
-    acc = fma(c.cN2, s[y + 2][x], acc);
-    acc = fma(c.cS2, s[y - 2][x], acc);
-    return acc;
+    R acc = fma(-c.cC, s[y][x], b);
+    acc = fma(-c.cE1, s[y][x + 1], acc);
+    acc = fma(-c.cW1, s[y][x - 1], acc);
+    acc = fma(-c.cN1, s[y + 1][x], acc);
+    acc = fma(-c.cS1, s[y - 1][x], acc);
+    acc = fma(-c.cE2, s[y][x + 2], acc);
+    acc = fma(-c.cW2, s[y][x - 2], acc);
+    acc = fma(-c.cN2, s[y + 2][x], acc);
+    return fma(-c.cS2, s[y - 2][x], acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -347,24 +329,24 @@ __device__ __forceinline__ void ph_pred_t(const StepArgs &a, const MixedArgs &m,
         const double pw = ld(&S.phix[q]), pe = ld(&S.phix[q + 1]), ps = ld(&S.phiz[q]), pn = ld(&S.phiz[q + G.P]);
         const double div = (pe - pw + pn - ps) * G.iV;
         const double rq = ld(&S.rho[q]);
-        const double rho1 = rq - F.dt * div;
-        const double s12 = G.iV * (1.0 / 12.0);
-        const double fe = pe * s12, fw = pw * s12, fn = pn * s12, fs = ps * s12;
+        const double rho1 = fma(-F.dt, div, rq);
+        const double fe = pe * F.s12, fw = pw * F.s12, fn = pn * F.s12, fs = ps * F.s12;
         // diffusion: mu/dx^2 per face, or with LES the face mean of mu_eff
         // (a wall face takes the cell's own)
-        double me, mw, mn, ms;
+        double me, mw, mn, ms, md;
         if (F.les) {
             const double mc = ld(&a.mueff[q]);
-            const double ix2 = 0.5 * G.idx * G.idx, iz2 = 0.5 * G.idz * G.idz;
-            me = (mc + (i + 1 < G.nx ? ld(&a.mueff[q + 1]) : mc)) * ix2;
-            mw = (mc + (i > 0 ? ld(&a.mueff[q - 1]) : mc)) * ix2;
-            mn = (mc + (k + 1 < G.nz ? ld(&a.mueff[q + G.P]) : mc)) * iz2;
-            ms = (mc + (k > 0 ? ld(&a.mueff[q - G.P]) : mc)) * iz2;
+            me = (mc + (i + 1 < G.nx ? ld(&a.mueff[q + 1]) : mc)) * F.hix2;
+            mw = (mc + (i > 0 ? ld(&a.mueff[q - 1]) : mc)) * F.hix2;
+            mn = (mc + (k + 1 < G.nz ? ld(&a.mueff[q + G.P]) : mc)) * F.hiz2;
+            ms = (mc + (k > 0 ? ld(&a.mueff[q - G.P]) : mc)) * F.hiz2;
+            md = (me + mw) + (mn + ms);
         } else {
-            me = mw = F.mu * G.idx * G.idx;
-            mn = ms = F.mu * G.idz * G.idz;
+            me = mw = F.mux;
+            mn = ms = F.muz;
+            md = F.mud;
         }
-        const double cC = rho1 * F.idt + (7.0 / 12.0) * div + ((me + mw) + (mn + ms));
+        const double cC = fma(rho1, F.idt, fma(7.0 / 12.0, div, md));
         const double cE1 = fma(7.0, fe, fw) - me, cW1 = -fma(7.0, fw, fe) - mw;
         const double cN1 = fma(7.0, fn, fs) - mn, cS1 = -fma(7.0, fs, fn) - ms;
         const double cE2 = -fe, cW2 = fw, cN2 = -fn, cS2 = fs;
@@ -377,49 +359,37 @@ __device__ __forceinline__ void ph_pred_t(const StepArgs &a, const MixedArgs &m,
         a.T.cS1[q] = cS1;
         a.T.cN2[q] = cN2;
         a.T.cS2[q] = cS2;
-        const double diu = 1.0 / cC;
-        const double dih =
-            F.pr_ne1 ? 1.0 / (cC + 2.0 * (F.nuh - F.mu) * (G.idx * G.idx + G.idz * G.idz)) : diu;
+        const double diu = recip(cC);
+        const double dih = F.pr_ne1 ? recip(fma(2.0 * (F.nuh - F.mu), F.ix2 + F.iz2, cC)) : diu;
         if (!MX) {
             a.dinvu[q] = diu;
             a.dinvh[q] = dih;
         }
-        // face forces (p'_b - p'_a - g z_f (rho_b - rho_a)) / Delta; the cell
-        // and face heights g z come from per-row tables
-        const double gz = ld(&a.gzc[k]);
-        const double pq = ld(&S.pp[q]);
-        double gxw = 0.0, gxe = 0.0, gzs = 0.0, gzn = 0.0;
-        if (i > 0) gxw = fma(-gz, rq - ld(&S.rho[q - 1]), pq - ld(&S.pp[q - 1])) * G.idx;
-        if (i + 1 < G.nx) gxe = fma(-gz, ld(&S.rho[q + 1]) - rq, ld(&S.pp[q + 1]) - pq) * G.idx;
-        if (k > 0) gzs = fma(-ld(&a.gzf[k]), rq - ld(&S.rho[q - G.P]), pq - ld(&S.pp[q - G.P])) * G.idz;
-        if (k + 1 < G.nz)
-            gzn = fma(-ld(&a.gzf[k + 1]), ld(&S.rho[q + G.P]) - rq, ld(&S.pp[q + G.P]) - pq) * G.idz;
+        // the sum of the two face forces p'_b - p'_a - g z_f (rho_b - rho_a) of each
+        // direction (over the spacing): in x both faces have the cell's height;
+        // a wall face carries none, which the cell's own values in the place of
+        // the missing neighbour's give
+        const int qe = i + 1 < G.nx ? q + 1 : q, qw = i > 0 ? q - 1 : q;
+        const int qn = k + 1 < G.nz ? q + G.P : q, qs = k > 0 ? q - G.P : q;
+        const double sx = fma(-ld(&a.gzc[k]), ld(&S.rho[qe]) - ld(&S.rho[qw]), ld(&S.pp[qe]) - ld(&S.pp[qw]));
+        const double sz = fma(-ld(&a.gzf[k + 1]), ld(&S.rho[qn]) - rq,
+                              fma(-ld(&a.gzf[k]), rq - ld(&S.rho[qs]), ld(&S.pp[qn]) - ld(&S.pp[qs])));
         const double u = ld(&S.u[q]), w = ld(&S.w[q]);
-        const double bu = rq * u * F.idt - 0.5 * (gxw + gxe);
-        const double bw = rq * w * F.idt - 0.5 * (gzs + gzn);
+        const double rdt = rq * F.idt;
+        const double bu = fma(-F.hix, sx, rdt * u);
+        const double bw = fma(-F.hiz, sz, rdt * w);
         a.rho1[q] = rho1;
-        a.dtr1[q] = F.dt / rho1;
+        a.dtr1[q] = F.dt * recip(rho1);
         const int y = threadIdx.y + 2, x = threadIdx.x + 2;
-        // T(X) at the cell from a halo-2 tile, in apply9's order
-        auto t9 = [&](const Tile<2> &t) {
-            double v = cC * t[y][x];
-            v = fma(cE1, t[y][x + 1], v);
-            v = fma(cW1, t[y][x - 1], v);
-            v = fma(cN1, t[y + 1][x], v);
-            v = fma(cS1, t[y - 1][x], v);
-            v = fma(cE2, t[y][x + 2], v);
-            v = fma(cW2, t[y][x - 2], v);
-            v = fma(cN2, t[y + 2][x], v);
-            v = fma(cS2, t[y - 2][x], v);
-            return v;
-        };
+        // b - T(X) at the cell from a halo-2 tile
+        const Coef9<double> c9{cC, cE1, cW1, cN1, cS1, cE2, cW2, cN2, cS2};
         if (!MX) {
             a.bu[q] = bu;
             a.bw[q] = bw;
             acc[0] = fma(bu, bu, acc[0]);
             acc[1] = fma(bw, bw, acc[1]);
             if (SW1) {
-                const double r0u = bu - t9(tile_at<2>(sm, 0)), r0w = bw - t9(tile_at<2>(sm, 1));
+                const double r0u = sub9c<2>(bu, c9, tile_at<2>(sm, 0), y, x), r0w = sub9c<2>(bw, c9, tile_at<2>(sm, 1), y, x);
                 a.ua[q] = fma(r0u, diu, u);
                 a.wa[q] = fma(r0w, diu, w);
                 acc[SW1 ? 2 : 0] = fma(r0u, r0u, acc[SW1 ? 2 : 0]);
@@ -429,7 +399,7 @@ __device__ __forceinline__ void ph_pred_t(const StepArgs &a, const MixedArgs &m,
                 a.wa[q] = w;
             }
         } else {
-            const double r0u = bu - t9(tile_at<2>(sm, 0)), r0w = bw - t9(tile_at<2>(sm, 1));
+            const double r0u = sub9c<2>(bu, c9, tile_at<2>(sm, 0), y, x), r0w = sub9c<2>(bw, c9, tile_at<2>(sm, 1), y, x);
             m.T.cC[q] = (float)cC;
             m.T.cE1[q] = (float)cE1;
             m.T.cW1[q] = (float)cW1;
@@ -491,8 +461,8 @@ __device__ __forceinline__ void ph_sweep2(const Geom &G, const Phys &F, const St
     if (in) {
         if (!kPrefetch) fetch();
         const int y = threadIdx.y + 2, x = threadIdx.x + 2;
-        const R ra = bva - apply9c<2, R>(c, sa, y, x);
-        const R rb = bvb - apply9c<2, R>(c, sb, y, x);
+        const R ra = sub9c<2, R>(bva, c, sa, y, x);
+        const R rb = sub9c<2, R>(bvb, c, sb, y, x);
         ya[q] = fma(ra, di, sa[y][x]);
         yb[q] = fma(rb, di, sb[y][x]);
         acc[0] = fma(ra, ra, acc[0]);
@@ -527,9 +497,8 @@ __device__ __forceinline__ void ph_sweep1(const Geom &G, const Phys &F, const St
     if (in) {
         if (!kPrefetchSweep1) fetch();
         const int y = threadIdx.y + 2, x = threadIdx.x + 2;
-        R t = apply9c<2, R>(c, sh, y, x);
-        if (F.pr_ne1) t = fma(lc, lap5<2, R>(G, sh, y, x), t);
-        const R r = bq - t;
+        R r = sub9c<2, R>(bq, c, sh, y, x);
+        if (F.pr_ne1) r = fma(-lc, lap5<2, R>(F, sh, y, x), r);
         xout[q] = fma(r, di, sh[y][x]);
         acc[0] = fma(r, r, acc[0]);
     }
@@ -577,7 +546,7 @@ __device__ __forceinline__ void ph_enth_rhs_t(const StepArgs &a, const MixedArgs
         if (SW1) load_tile<BC_H, 2>(tile_at<2>(sm, 2), G, F, S.h, bx, bz);
     }
     __syncthreads();
-    // K1 in place of u (ghost velocities give the mirrored cell's K); u1 and
+    // 2 K1 in place of u (ghost velocities give the mirrored cell's K); u1 and
     // w1 at the cell centre are kept aside first
     const double u1c = su[threadIdx.y + 2][threadIdx.x + 2], w1c = sw[threadIdx.y + 2][threadIdx.x + 2];
     __syncthreads();
@@ -585,7 +554,7 @@ __device__ __forceinline__ void ph_enth_rhs_t(const StepArgs &a, const MixedArgs
         const int tid = threadIdx.x + threadIdx.y * BX;
         for (int e = tid; e < kT2; e += NTHREADS) {
             const int tk = e / (BX + 4), ti = e - tk * (BX + 4);
-            su[tk][ti] = 0.5 * (su[tk][ti] * su[tk][ti] + sw[tk][ti] * sw[tk][ti]);
+            su[tk][ti] = fma(su[tk][ti], su[tk][ti], sw[tk][ti] * sw[tk][ti]);
         }
     }
     __syncthreads();
@@ -600,21 +569,20 @@ __device__ __forceinline__ void ph_enth_rhs_t(const StepArgs &a, const MixedArgs
         c -= ld(&S.phix[q]) * (7.0 * (K[y][x - 1] + K[y][x]) - (K[y][x - 2] + K[y][x + 1]));
         c += ld(&S.phiz[q + G.P]) * (7.0 * (K[y][x] + K[y + 1][x]) - (K[y - 1][x] + K[y + 2][x]));
         c -= ld(&S.phiz[q]) * (7.0 * (K[y - 1][x] + K[y][x]) - (K[y - 2][x] + K[y + 1][x]));
-        c *= G.iV * (1.0 / 12.0);
         const double rq = ld(&S.rho[q]), u = ld(&S.u[q]), w = ld(&S.w[q]), h = ld(&S.h[q]);
         // b~_e carries rho^n K^n, or rho^n K^{n-1} in the literal reading
         const double Kn = F.k_lagged ? ld(&S.Kold[q]) : 0.5 * (u * u + w * w);
         const double rho1 = ld(&a.rho1[q]);
-        const double be = (rq * h + rq * Kn - ld(&S.pold[q])) * F.idt;
-        const double bh = be - rho1 * K[y][x] * F.idt - c + ld(&S.p[q]) * F.idt - rho1 * F.g * w1c;
+        const double te = fma(rq, h + Kn, -ld(&S.pold[q])) + ld(&S.p[q]);
+        const double bh =
+            fma(-rho1 * F.g, w1c, fma(F.idt, fma(-0.5 * rho1, K[y][x], te), -(F.s24 * c)));
         if (!MX) {
             a.bh[q] = bh;
             acc[0] = fma(bh, bh, acc[0]);
             if (SW1) {
                 const Tile<2> &sh = tile_at<2>(sm, 2);
-                double t = apply9<2>(a.T, q, sh, y, x);
-                if (F.pr_ne1) t = fma(F.mu - F.nuh, lap5<2>(G, sh, y, x), t);
-                const double r0 = bh - t;
+                double r0 = sub9c<2>(bh, coef9(a.T, q), sh, y, x);
+                if (F.pr_ne1) r0 = fma(F.nuh - F.mu, lap5<2>(F, sh, y, x), r0);
                 h0[q] = fma(r0, ld(&a.dinvh[q]), sh[y][x]);
                 acc[SW1 ? 1 : 0] = fma(r0, r0, acc[SW1 ? 1 : 0]);
             } else {
@@ -624,9 +592,8 @@ __device__ __forceinline__ void ph_enth_rhs_t(const StepArgs &a, const MixedArgs
             a.ua[q] = u1c;
             a.wa[q] = w1c;
             const Tile<2> &sh = tile_at<2>(sm, 2);
-            double t = apply9<2>(a.T, q, sh, y, x);
-            if (F.pr_ne1) t = fma(F.mu - F.nuh, lap5<2>(G, sh, y, x), t);
-            const double r0 = bh - t;
+            double r0 = sub9c<2>(bh, coef9(a.T, q), sh, y, x);
+            if (F.pr_ne1) r0 = fma(F.nuh - F.mu, lap5<2>(F, sh, y, x), r0);
             const float fr = (float)r0;
             m.r0h[q] = fr;
             m.dh[0][q] = fr * ld(&m.dinvh[q]);
@@ -668,27 +635,48 @@ __device__ __forceinline__ void ph_eos_t(const StepArgs &a, const Level &L, cons
 {
     const Geom &G = a.G;
     const Phys &F = a.F;
-    Tile<1> &s2 = tile_at<1>(sm, 0), &s1 = tile_at<1>(sm, 1);
+    Tile<1> &s2 = tile_at<1>(sm, 0), &s1 = tile_at<1>(sm, 1);   // dt rho^{n+2/3}, rho^{n+1/3}
     double(*fx)[BX + 1] = reinterpret_cast<double(*)[BX + 1]>(sm + 2 * kT1);
     double(*fz)[BX] = reinterpret_cast<double(*)[BX]>(sm + 2 * kT1 + BZ * (BX + 1));
     const State &S = a.S;
-    const double icp = 1.0 / F.cp;
     auto h1_of = [&](int q) { return MX ? ld(&S.h[q]) + (double)ld(&dh[q]) : ld(&h1[q]); };
-    load_tile_fn<1>(s2, G, bx, bz, [&](int q, int, int) {
-        const double T1 = fma(h1_of(q) - ld(&S.h[q]), icp, ld(&S.T[q]));
-        return ld(&S.p[q]) / (F.R * T1);
-    });
-    load_tile_fn<1>(s1, G, bx, bz, [&](int q, int, int) { return ld(&a.rho1[q]); });
-    __syncthreads();
     int i, k;
     const bool in = cell_of(G, bx, bz, i, k);
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int y = ty + 1, x = tx + 1;
-    const double ix2 = G.idx * G.idx, iz2 = G.idz * G.idz;
+    const int q = in ? cidx(G, i, k) : 0;
+    // the cell's own update in registers, and its share of the tile; the ring
+    // of halo cells (corners are not used) repeats the density alone
+    double h1q = 0.0, T1 = 0.0, psi = 0.0, rho2 = 0.0;
+    auto eos = [&](int c, double &hv, double &Tv, double &ps) {
+        hv = h1_of(c);
+        Tv = fma(hv - ld(&S.h[c]), F.icp, ld(&S.T[c]));
+        ps = recip(F.R * Tv);
+        return ld(&S.p[c]) * ps;
+    };
+    if (in) rho2 = eos(q, h1q, T1, psi);
+    s2[y][x] = F.dt * rho2;
+    s1[y][x] = in ? ld(&a.rho1[q]) : 0.0;
+    for (int e = tx + ty * BX; e < 2 * (BX + BZ); e += NTHREADS) {
+        const bool row = e < 2 * BX;
+        const int tk = row ? (e < BX ? 0 : BZ + 1) : 1 + ((e - 2 * BX) >> 1);
+        const int ti = row ? 1 + (e < BX ? e : e - BX) : ((e & 1) ? BX + 1 : 0);
+        const int ii = bx * BX - 1 + ti, kk = bz * BZ - 1 + tk;
+        double v2 = 0.0, v1 = 0.0;
+        if (ii >= 0 && ii < G.nx && kk >= 0 && kk < G.nz) {
+            const int c = cidx(G, ii, kk);
+            double hv, Tv, ps;
+            v2 = F.dt * eos(c, hv, Tv, ps);
+            v1 = ld(&a.rho1[c]);
+        }
+        s2[tk][ti] = v2;
+        s1[tk][ti] = v1;
+    }
+    __syncthreads();
     // dt rho2_f / rho1_f with linear face averages (the two halves cancel
     // exactly in binary)
     auto dface = [&](int ya, int xa, int yb, int xb) {
-        return F.dt * (s2[ya][xa] + s2[yb][xb]) / (s1[ya][xa] + s1[yb][xb]);
+        return (s2[ya][xa] + s2[yb][xb]) * recip(s1[ya][xa] + s1[yb][xb]);
     };
     if (in) {
         fx[ty][tx] = i > 0 ? dface(y, x - 1, y, x) : 0.0;
@@ -698,33 +686,30 @@ __device__ __forceinline__ void ph_eos_t(const StepArgs &a, const Level &L, cons
     }
     __syncthreads();
     if (in) {
-        const int q = cidx(G, i, k);
-        const double h1q = h1_of(q);
-        const double T1 = fma(h1q - ld(&S.h[q]), icp, ld(&S.T[q]));
-        const double psi = 1.0 / (F.R * T1);
         a.N.T[q] = T1;
         a.N.h[q] = h1q;
-        a.rho2[q] = s2[y][x];
+        a.rho2[q] = rho2;
         a.psi[q] = psi;
         const double Dw = fx[ty][tx], De = fx[ty][tx + 1], Ds = fz[ty][tx], Dn = fz[ty + 1][tx];
         a.Dx[k * G.P + i] = Dw;
         a.Dz[k * G.P + i] = Ds;
-        L.ax[k * G.P + i] = Dw * ix2;
-        L.az[k * G.P + i] = Ds * iz2;
+        const double aw = Dw * F.ix2, as = Ds * F.iz2;
+        L.ax[k * G.P + i] = aw;
+        L.az[k * G.P + i] = as;
         if (i == G.nx - 1) { a.Dx[k * G.P + G.nx] = 0.0; L.ax[k * G.P + G.nx] = 0.0; }
         if (k == G.nz - 1) { a.Dz[G.nz * G.P + i] = 0.0; L.az[G.nz * G.P + i] = 0.0; }
         const double c = psi * F.idt;
-        const double d = c + (Dw + De) * ix2 + (Ds + Dn) * iz2;
+        const double d = fma(Ds + Dn, F.iz2, fma(Dw + De, F.ix2, c));
         L.c[q] = c;
         L.d[q] = d;
-        const double id = 1.0 / d;
+        const double id = recip(d);
         L.wd[q] = id;
         if (MX) {
             L32.c[q] = (float)c;
             L32.d[q] = (float)d;
             L32.wd[q] = (float)id;
-            L32.ax[k * G.P + i] = (float)(Dw * ix2);
-            L32.az[k * G.P + i] = (float)(Ds * iz2);
+            L32.ax[k * G.P + i] = (float)aw;
+            L32.az[k * G.P + i] = (float)as;
             if (i == G.nx - 1) L32.ax[k * G.P + G.nx] = 0.0f;
             if (k == G.nz - 1) L32.az[G.nz * G.P + i] = 0.0f;
         }
@@ -789,13 +774,13 @@ __device__ __forceinline__ void ph_H(const StepArgs &a, const double *U, const d
     // the cell's stencil weights (shared by both components) and state,
     // loaded ahead of the tile barrier
     Coef9<double> c{};
-    double ru = 0.0, rw = 0.0, r1dt = 0.0;
+    double ru = 0.0, rw = 0.0;
     auto fetch = [&] {
         c = coef9(a.T, q);
         const double rdt = ld(&a.S.rho[q]) * F.idt;
         ru = rdt * ld(&a.S.u[q]);
         rw = rdt * ld(&a.S.w[q]);
-        r1dt = ld(&a.rho1[q]) * F.idt;
+        c.cC = fma(-ld(&a.rho1[q]), F.idt, c.cC);   // the stencil without its time term
     };
     if (kPrefetch && in) fetch();
     load_tile<BC_U, 2>(su, G, F, U, bx, bz);
@@ -804,8 +789,8 @@ __device__ __forceinline__ void ph_H(const StepArgs &a, const double *U, const d
     if (in) {
         if (!kPrefetch) fetch();
         const int y = threadIdx.y + 2, x = threadIdx.x + 2;
-        a.Hx[q] = fma(r1dt, su[y][x], ru - apply9c<2>(c, su, y, x));
-        a.Hz[q] = fma(r1dt, sw[y][x], rw - apply9c<2>(c, sw, y, x));
+        a.Hx[q] = sub9c<2>(ru, c, su, y, x);
+        a.Hz[q] = sub9c<2>(rw, c, sw, y, x);
     }
     __syncthreads();
 }
@@ -850,16 +835,22 @@ __device__ __forceinline__ void ph_helm_rhs_t(const StepArgs &a, const Level &L,
         if (!kPrefetch) fetch();
         const int q = q0;
         const int y = threadIdx.y + 1, x = threadIdx.x + 1;
-        const double gz = ld(&a.gzc[k]);
-        const double gzx = gz * G.idx, gzs = ld(&a.gzf[k]) * G.idz, gzn = ld(&a.gzf[k + 1]) * G.idz;
-        const double r2q = s2[y][x];
-        // wall faces have D = 0 and zero tile entries beyond the box
-        double flux = De * G.dz * fma(0.5, shx[y][x] + shx[y][x + 1], gzx * (s2[y][x + 1] - r2q));
-        flux += Dw * G.dz * fma(-0.5, shx[y][x] + shx[y][x - 1], gzx * (s2[y][x - 1] - r2q));
-        flux += Dn * G.dx * fma(0.5, shz[y][x] + shz[y + 1][x], gzn * (s2[y + 1][x] - r2q));
-        flux += Ds * G.dx * fma(-0.5, shz[y][x] + shz[y - 1][x], gzs * (s2[y - 1][x] - r2q));
-        const double b = fma(ld(&a.psi[q]) * r2q, gz, ld(&a.S.rho[q])) * F.idt - flux * G.iV;
-        const double r = b - helm_apply<1>(hc, sx, y, x);
+        const double gx2 = ld(&a.gx2[k]);
+        const double r2q = s2[y][x], hxq = shx[y][x], hzq = shz[y][x];
+        // twice the face flux over D and the spacing, H_a + H_b + 2 g z_f
+        // (rho2_b - rho2_a) / Delta; wall faces have D = 0 and zero tile entries
+        // beyond the box
+        double fx = De * fma(gx2, s2[y][x + 1] - r2q, hxq + shx[y][x + 1]);
+        fx = fma(-Dw, fma(gx2, r2q - s2[y][x - 1], hxq + shx[y][x - 1]), fx);
+        double fz = Dn * fma(ld(&a.gz2[k + 1]), s2[y + 1][x] - r2q, hzq + shz[y + 1][x]);
+        fz = fma(-Ds, fma(ld(&a.gz2[k]), r2q - s2[y - 1][x], hzq + shz[y - 1][x]), fz);
+        const double flux = fma(F.hiz, fz, F.hix * fx);
+        const double b = fma(fma(ld(&a.psi[q]) * r2q, ld(&a.gzc[k]), ld(&a.S.rho[q])), F.idt, -flux);
+        double r = fma(-hc.d, sx[y][x], b);
+        r = fma(hc.aw, sx[y][x - 1], r);
+        r = fma(hc.ae, sx[y][x + 1], r);
+        r = fma(hc.as, sx[y - 1][x], r);
+        r = fma(hc.an, sx[y + 1][x], r);
         a.b[q] = b;
         if (!MX) {
             L.r[q] = r;
@@ -1361,11 +1352,12 @@ __device__ __forceinline__ void ph_correct(const StepArgs &a, const LevelT<R> &L
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int y = ty + 1, x = tx + 1;
     const double gzk = in ? ld(&a.gzc[k]) : 0.0;
+    // Delta G_f
     auto gxf = [&](int xa) {   // x-face between tile columns xa and xa+1 of row y
-        return fma(-gzk, s2[y][xa + 1] - s2[y][xa], sx[y][xa + 1] - sx[y][xa]) * G.idx;
+        return fma(-gzk, s2[y][xa + 1] - s2[y][xa], sx[y][xa + 1] - sx[y][xa]);
     };
     auto gzf = [&](int ya, int kf) {   // z-face between tile rows ya and ya+1, face index kf
-        return fma(-ld(&a.gzf[kf]), s2[ya + 1][x] - s2[ya][x], sx[ya + 1][x] - sx[ya][x]) * G.idz;
+        return fma(-ld(&a.gzf[kf]), s2[ya + 1][x] - s2[ya][x], sx[ya + 1][x] - sx[ya][x]);
     };
     if (in) {
         gx[ty][tx] = i > 0 ? gxf(x - 1) : 0.0;
@@ -1378,14 +1370,13 @@ __device__ __forceinline__ void ph_correct(const StepArgs &a, const LevelT<R> &L
         if (!kPrefetch) fetch();
         const int q = q0;
         const double gxw = gx[ty][tx], gxe = gx[ty][tx + 1], gzs = gz[ty][tx], gzn = gz[ty + 1][tx];
-        const double Fw = i > 0 ? Dw * (0.5 * (hxw + hxq) - gxw) : 0.0;   // wall faces carry zero
-        const double Fs = k > 0 ? Ds * (0.5 * (hzs + hzq) - gzs) : 0.0;
-        N.phix[k * G.P + i] = Fw * G.dz;
-        N.phiz[k * G.P + i] = Fs * G.dx;
+        // F |A| = D (|A| / 2) (H_a + H_b - 2 G); wall faces have D = 0 here
+        N.phix[k * G.P + i] = (Dw * F.hdz) * fma(-F.tix, gxw, hxw + hxq);
+        N.phiz[k * G.P + i] = (Ds * F.hdx) * fma(-F.tiz, gzs, hzs + hzq);
         if (i == G.nx - 1) N.phix[k * G.P + G.nx] = 0.0;
         if (k == G.nz - 1) N.phiz[G.nz * G.P + i] = 0.0;
-        N.u[q] = dtr1 * (hxq - 0.5 * (gxw + gxe));
-        N.w[q] = dtr1 * (hzq - 0.5 * (gzs + gzn));
+        N.u[q] = dtr1 * fma(-F.hix, gxw + gxe, hxq);
+        N.w[q] = dtr1 * fma(-F.hiz, gzs + gzn, hzq);
         ppout[q] = sx[y][x];
         const double pn = fma(-s2[y][x], gzk, sx[y][x]);
         N.p[q] = pn;
