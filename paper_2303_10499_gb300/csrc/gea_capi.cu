@@ -634,6 +634,7 @@ int gea_create(const gea_grid *grid, const gea_constants *c, gea_ctx **out)
         F.hdx = 0.5 * g.dx; F.hdz = 0.5 * g.dz;
         F.s12 = g.iV / 12.0; F.s24 = g.iV / 24.0;
         F.icp = 1.0 / c->cp;
+        F.icv = 1.0 / (c->cp - c->R);
     }
     ctx->F.k_lagged = (c->reading_flags & GEA_READING_K_LAGGED) ? 1 : 0;
     ctx->F.les = ctx->F.les_d2 > 0.0 ? 1 : 0;
@@ -908,11 +909,11 @@ int gea_set_state(gea_ctx *ctx, const gea_state_view *v)
         double *st = ctx->stage;
         int rc;
         if (v->mem == GEA_MEM_DEVICE && on_device(ctx, in, 4)) {
-            launch_derive(G, ctx->F, v->rho, v->rhou, v->rhow, v->rhoe, nx, S, ctx->sc, ctx->stream);
+            launch_derive(G, ctx->F, v->rho, v->rhou, v->rhow, v->rhoe, nx, ctx->gzc, S, ctx->sc, ctx->stream);
         } else {
             for (int f = 0; f < 4; ++f)
                 if ((rc = copy_in(ctx, st + f * cellw, in[f], nx, nz))) return rc;
-            launch_derive(G, ctx->F, st, st + cellw, st + 2 * cellw, st + 3 * cellw, G.P, S, ctx->sc, ctx->stream);
+            launch_derive(G, ctx->F, st, st + cellw, st + 2 * cellw, st + 3 * cellw, G.P, ctx->gzc, S, ctx->sc, ctx->stream);
         }
         CK(cudaGetLastError());
     } else if (DenseFields d = dense_fields(v, nf); v->mem == GEA_MEM_DEVICE && on_device(ctx, d.p, nf)) {

@@ -49,7 +49,7 @@ struct Phys {
     double hix, hiz, tix, tiz;               // 1 / (2 dx), 1 / (2 dz), 2 / dx, 2 / dz
     double hdx, hdz;                         // dx / 2, dz / 2
     double s12, s24;                         // 1 / (12 dx dz), 1 / (24 dx dz)
-    double icp;                              // 1 / cp
+    double icp, icv;                         // 1 / cp, 1 / cv
     // uniform branch flags as integers (an FP64 compare issues on the FP64 pipe)
     int les;                                 // les_d2 > 0
     int pr_ne1;                              // nuh != mu (Pr != 1): the enthalpy stencil differs
@@ -263,6 +263,18 @@ __device__ __forceinline__ double recip(double a)
     return fma(x, fma(e, e, e), x);
 }
 
+// f() if flag (0 or 1, the same in every thread), as a branch that stays one: a
+// short conditional body is otherwise predicated, and predicated-off FP64
+// instructions issue all the same (the options below cost the default path 5
+// of 12 instructions in the finest prolongation, 1.7 ms of the 4096 x 2048 step
+// in all). The trip count of a loop is not known to be 0 or 1.
+template <class F>
+__device__ __forceinline__ void rarely(int flag, F f)
+{
+#pragma unroll 1
+    for (int t = 0; t < flag; ++t) f();
+}
+
 template <class T>
 __device__ __forceinline__ T warp_sum(T v)
 {
@@ -446,7 +458,7 @@ __host__ __device__ __forceinline__ const double *pp_in(const StepArgs &a, int c
 // conservative variables (rows of `pitch` values) to a state, and of the state
 // in slot (base + steps done) & 1 (null arrays are left out)
 void launch_derive(const Geom &G, const Phys &F, const double *rho, const double *rhou,
-                   const double *rhow, const double *rhoe, int pitch, const State &S, Scal *sc,
+                   const double *rhow, const double *rhoe, int pitch, const double *gzc, const State &S, Scal *sc,
                    cudaStream_t st);
 void launch_conserve(const Geom &G, const Phys &F, const State S[2], int base, const Scal *sc, double *rho,
                      double *rhou, double *rhow, double *rhoe, int pitch, cudaStream_t st);

@@ -28,18 +28,21 @@ __device__ __forceinline__ bool loop_over(const Scal *sc, int which)
 // dense device arrays, read in place).
 __global__ void k_derive(Geom G, Phys F, const double *__restrict__ rho,
                          const double *__restrict__ rhou, const double *__restrict__ rhow,
-                         const double *__restrict__ rhoe, int pitch, State S, Scal *sc)
+                         const double *__restrict__ rhoe, int pitch, const double *__restrict__ gzc, State S, Scal *sc)
 {
     int i, k;
     if (!cell_of(G, blockIdx.x, blockIdx.y, i, k)) return;
     const int q = cidx(G, i, k);
     const size_t d = (size_t)k * pitch + i;
-    const double cv = F.cp - F.R;
-    const double z = (k + 0.5) * G.dz;
-    const double r = rho[d];
-    const double u = rhou[d] / r, w = rhow[d] / r;
-    const double K = 0.5 * (u * u + w * w);
-    const double T = (rhoe[d] / r - K - F.g * z) / cv;
+    const double gz = gzc[k];
+    const double r = rho[d], ir = recip(r);
+    const double ru = rhou[d], rw = rhow[d], re = rhoe[d];
+    const double u = ru * ir, w = rw * ir;
+    const double K = 0.5 * fma(u, u, w * w);
+    // e = re / r rounded as a division would: T and with it p = rho R T carry the
+    // hydrostatic balance
+    const double e0 = re * ir, e = fma(fma(-r, e0, re), ir, e0);
+    const double T = ((e - K) - gz) * F.icv;
     if (!(r > 0.0) || !(T > 0.0)) atomicAdd(&sc->bad_cells, 1);
     S.rho[q] = r;
     S.u[q] = u;
@@ -48,12 +51,12 @@ __global__ void k_derive(Geom G, Phys F, const double *__restrict__ rho,
     S.h[q] = F.cp * T;
     const double p = r * F.R * T;
     S.p[q] = p;
-    S.pp[q] = p + r * F.g * z;
+    S.pp[q] = fma(r, gz, p);
     S.pold[q] = p;
     S.Kold[q] = K;   // K^{-1} := K^0
-    S.phix[k * G.P + i] = i > 0 ? 0.5 * (rhou[d - 1] + rhou[d]) * G.dz : 0.0;
+    S.phix[k * G.P + i] = i > 0 ? F.hdz * (rhou[d - 1] + ru) : 0.0;
     if (i == G.nx - 1) S.phix[k * G.P + G.nx] = 0.0;
-    S.phiz[k * G.P + i] = k > 0 ? 0.5 * (rhow[d - pitch] + rhow[d]) * G.dx : 0.0;
+    S.phiz[k * G.P + i] = k > 0 ? F.hdx * (rhow[d - pitch] + rw) : 0.0;
     if (k == G.nz - 1) S.phiz[G.nz * G.P + i] = 0.0;
 }
 
@@ -235,9 +238,9 @@ __global__ void k_mg_down(LevelT<R> f, LevelT<R> c, Phys F, Scal *sc)
                         blockIdx.y);
 }
 
-// finest: also r.z
-template <class R>
-__global__ void k_mg_up(LevelT<R> f, const R *ec, int Pc, int finest, Phys F, Scal *sc, double *partials)
+// FINEST: also r.z
+template <bool FINEST, class R>
+__global__ void k_mg_up(LevelT<R> f, const R *ec, int Pc, Phys F, Scal *sc, double *partials)
 {
     if (loop_over(sc, LOOP_CG)) return;
     __shared__ R sm[kPH2 + kPH1];
@@ -245,9 +248,9 @@ __global__ void k_mg_up(LevelT<R> f, const R *ec, int Pc, int finest, Phys F, Sc
     R acc[1] = {(R)0};
     double tot[1];
     block_tiles(f.G, [&](int bx, int bz) {
-        ph_mg_up<R>(f, f.r, ec, Pc, f.e2, F, reinterpret_cast<double *>(sm), bx, bz, acc);
+        ph_mg_up<FINEST, R>(f, f.r, ec, Pc, f.e2, F, reinterpret_cast<double *>(sm), bx, bz, acc);
     });
-    if (!finest) return;
+    if (!FINEST) return;
     if (grid_sum<1, R>(acc, red, partials, &sc->counters[CNT_RZ], tot)) fin_rz(sc, tot);
 }
 
@@ -409,10 +412,10 @@ int max_blocks(const Geom &G)
 }
 
 void launch_derive(const Geom &G, const Phys &F, const double *rho, const double *rhou,
-                   const double *rhow, const double *rhoe, int pitch, const State &S, Scal *sc,
+                   const double *rhow, const double *rhoe, int pitch, const double *gzc, const State &S, Scal *sc,
                    cudaStream_t st)
 {
-    k_derive<<<grid_of(G), kBlock, 0, st>>>(G, F, rho, rhou, rhow, rhoe, pitch, S, sc);
+    k_derive<<<grid_of(G), kBlock, 0, st>>>(G, F, rho, rhou, rhow, rhoe, pitch, gzc, S, sc);
 }
 
 void launch_conserve(const Geom &G, const Phys &F, const State S[2], int base, const Scal *sc, double *rho,
@@ -520,8 +523,8 @@ int vcycle_below(const StepArgs &a, const LevelT<R> *L, int nlev, cudaStream_t s
         const bool last = l == nlev - 1;
         const R *ec = last ? nullptr : L[l + 1].e2;
         TRACED(tr, last ? name_of<R>("mg_coarse", "mx_mg_coarse") : name_of<R>("mg_up", "mx_mg_up"), ncell(L[l].G),
-               (k_mg_up<R><<<grid_pairs(L[l].G), kBlock, 0, st>>>(L[l], ec, last ? 0 : L[l + 1].G.P, 0, a.F, a.sc,
-                                                                  a.partials)));
+               (k_mg_up<false, R><<<grid_pairs(L[l].G), kBlock, 0, st>>>(L[l], ec, last ? 0 : L[l + 1].G.P, a.F, a.sc,
+                                                                         a.partials)));
     }
     return n;
 }
@@ -548,8 +551,8 @@ int launch_vcycle(const StepArgs &a, const LevelT<R> *L, int nlev, cudaStream_t 
     }
     const R *ec = nlev > 1 ? L[1].e2 : nullptr;
     TRACED(tr, name_of<R>("mg_up", "mx_mg_up"), ncell(L[0].G),
-           (k_mg_up<R><<<grid_pair_tiles(L[0].G, a.tiles_per_block), kBlock, 0, st>>>(
-               L[0], ec, nlev > 1 ? L[1].G.P : 0, 1, a.F, a.sc, a.partials)));
+           (k_mg_up<true, R><<<grid_pair_tiles(L[0].G, a.tiles_per_block), kBlock, 0, st>>>(
+               L[0], ec, nlev > 1 ? L[1].G.P : 0, a.F, a.sc, a.partials)));
     return n + 1;
 }
 

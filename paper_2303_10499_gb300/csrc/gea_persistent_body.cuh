@@ -269,7 +269,7 @@ __device__ __forceinline__ void pressure_solve(const Grp &g, const LevelT<R> *L,
             const R *ec = l == nlev - 1 ? nullptr : L[l + 1].e2;
             const int Pc = l == nlev - 1 ? 0 : L[l + 1].G.P;
             for_pair_tiles(g, L[l].G, [&](int bx, int bz) {
-                ph_mg_up<R>(L[l], L[l].r, ec, Pc, L[l].e2, F, sm, bx, bz, none);
+                ph_mg_up<false, R>(L[l], L[l].r, ec, Pc, L[l].e2, F, sm, bx, bz, none);
             });
             gbar(g);
         }

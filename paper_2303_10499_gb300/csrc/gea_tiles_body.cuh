@@ -360,7 +360,8 @@ __device__ __forceinline__ void ph_pred_t(const StepArgs &a, const MixedArgs &m,
         a.T.cN2[q] = cN2;
         a.T.cS2[q] = cS2;
         const double diu = recip(cC);
-        const double dih = F.pr_ne1 ? recip(fma(2.0 * (F.nuh - F.mu), F.ix2 + F.iz2, cC)) : diu;
+        double dih = diu;
+        rarely(F.pr_ne1, [&] { dih = recip(fma(2.0 * (F.nuh - F.mu), F.ix2 + F.iz2, cC)); });
         if (!MX) {
             a.dinvu[q] = diu;
             a.dinvh[q] = dih;
@@ -498,7 +499,7 @@ __device__ __forceinline__ void ph_sweep1(const Geom &G, const Phys &F, const St
         if (!kPrefetchSweep1) fetch();
         const int y = threadIdx.y + 2, x = threadIdx.x + 2;
         R r = sub9c<2, R>(bq, c, sh, y, x);
-        if (F.pr_ne1) r = fma(-lc, lap5<2, R>(F, sh, y, x), r);
+        rarely(F.pr_ne1, [&] { r = fma(-lc, lap5<2, R>(F, sh, y, x), r); });
         xout[q] = fma(r, di, sh[y][x]);
         acc[0] = fma(r, r, acc[0]);
     }
@@ -571,7 +572,8 @@ __device__ __forceinline__ void ph_enth_rhs_t(const StepArgs &a, const MixedArgs
         c -= ld(&S.phiz[q]) * (7.0 * (K[y - 1][x] + K[y][x]) - (K[y - 2][x] + K[y + 1][x]));
         const double rq = ld(&S.rho[q]), u = ld(&S.u[q]), w = ld(&S.w[q]), h = ld(&S.h[q]);
         // b~_e carries rho^n K^n, or rho^n K^{n-1} in the literal reading
-        const double Kn = F.k_lagged ? ld(&S.Kold[q]) : 0.5 * (u * u + w * w);
+        double Kn = 0.5 * fma(u, u, w * w);
+        rarely(F.k_lagged, [&] { Kn = ld(&S.Kold[q]); });
         const double rho1 = ld(&a.rho1[q]);
         const double te = fma(rq, h + Kn, -ld(&S.pold[q])) + ld(&S.p[q]);
         const double bh =
@@ -582,7 +584,7 @@ __device__ __forceinline__ void ph_enth_rhs_t(const StepArgs &a, const MixedArgs
             if (SW1) {
                 const Tile<2> &sh = tile_at<2>(sm, 2);
                 double r0 = sub9c<2>(bh, coef9(a.T, q), sh, y, x);
-                if (F.pr_ne1) r0 = fma(F.nuh - F.mu, lap5<2>(F, sh, y, x), r0);
+                rarely(F.pr_ne1, [&] { r0 = fma(F.nuh - F.mu, lap5<2>(F, sh, y, x), r0); });
                 h0[q] = fma(r0, ld(&a.dinvh[q]), sh[y][x]);
                 acc[SW1 ? 1 : 0] = fma(r0, r0, acc[SW1 ? 1 : 0]);
             } else {
@@ -593,7 +595,7 @@ __device__ __forceinline__ void ph_enth_rhs_t(const StepArgs &a, const MixedArgs
             a.wa[q] = w1c;
             const Tile<2> &sh = tile_at<2>(sm, 2);
             double r0 = sub9c<2>(bh, coef9(a.T, q), sh, y, x);
-            if (F.pr_ne1) r0 = fma(F.nuh - F.mu, lap5<2>(F, sh, y, x), r0);
+            rarely(F.pr_ne1, [&] { r0 = fma(F.nuh - F.mu, lap5<2>(F, sh, y, x), r0); });
             const float fr = (float)r0;
             m.r0h[q] = fr;
             m.dh[0][q] = fr * ld(&m.dinvh[q]);
@@ -1019,17 +1021,17 @@ __device__ __forceinline__ void ph_mg_down(const LevelT<R> &f, const LevelT<R> &
     PairTile<2, R> &st = pair_tile<2, R>(sm, 0);
     PairTile<1, R> &se = pair_tile<1, R>(sm, kPH2);
     R *sres = reinterpret_cast<R *>(sm) + kPH2 + kPH1;
-    const R om = (R)F.omega;
     fill_pairs<2, true, R>(st, G, bx, bz, [&](int q, int, int, int) { return ld(&f.wd[q]) * ld(&f.r[q]); });
     __syncthreads();
     fill_next<false, R>(se, G, bx, bz, [&](int q, int cc, int tk, int tj, int s) {
         const R g = ld(&f.r[q]) + faces4<R>(f, q, st[tk + 1][tj - 1 + s], st[tk + 1][tj + s], st[tk][tj], st[tk + 2][tj]);
         R e = ld(&f.wd[q]) * g;
-        if (F.om_ne1) e *= om;
-        if (tk >= 1 && tk <= BZ && tj >= 1 && tj <= BX) {
-            if (FINE) rb[cc] = g;
-            if (F.om_ne1 && !FINE) f.e[q] = e;
-        }
+        const bool own = tk >= 1 && tk <= BZ && tj >= 1 && tj <= BX;
+        if (FINE && own) rb[cc] = g;
+        rarely(F.om_ne1, [&] {
+            e *= (R)F.omega;
+            if (own && !FINE) f.e[q] = e;
+        });
         return e;
     });
     __syncthreads();
@@ -1039,10 +1041,10 @@ __device__ __forceinline__ void ph_mg_down(const LevelT<R> &f, const LevelT<R> &
         const int s = k & 1, q = cidx(G, 2 * j + 1 - s, k);
         const int y = threadIdx.y + 1, x = threadIdx.x + 1;
         v = faces4<R>(f, q, se[y][x - s], se[y][x + 1 - s], se[y - 1][x], se[y + 1][x]);
-        if (F.om_ne1) {
+        rarely(F.om_ne1, [&] {
             const R gb = ld(&f.d[cidx(G, 2 * j + s, k)]) * se[y][x];   // omega times the black residual
-            v = fma((R)(1.0 - F.omega) / om, gb, v);
-        }
+            v = fma((R)((1.0 - F.omega) / F.omega), gb, v);
+        });
     }
     restrict_pairs<R>(c, v, sres, bx, bz);
     __syncthreads();
@@ -1051,9 +1053,9 @@ __device__ __forceinline__ void ph_mg_down(const LevelT<R> &f, const LevelT<R> &
 // Up half of a level's V-cycle with the coarse correction ec (row pitch Pc;
 // null on the coarsest level, whose solve is one symmetric red-black sweep):
 // red e = r / d + P ec, black z = (1 - w) (e_b + P ec) + w (r + sum a e) / d with
-// e_b of the down half, then red z = (r + sum a z) / d. Writes the whole correction;
-// acc += r z (used on the finest level).
-template <class R>
+// e_b of the down half, then red z = (r + sum a z) / d. Writes the whole
+// correction. DOT (on the finest level): acc += r z.
+template <bool DOT, class R>
 __device__ __forceinline__ void ph_mg_up(const LevelT<R> &f, const R *res, const R *ec, int Pc, R *out, const Phys &F,
                                          double *sm, int bx, int bz, R (&acc)[1])
 {
@@ -1070,12 +1072,13 @@ __device__ __forceinline__ void ph_mg_up(const LevelT<R> &f, const R *res, const
         R z = ld(&f.wd[q]) *
               (r + faces4<R>(f, q, st[tk + 1][tj - 1 + s], st[tk + 1][tj + s], st[tk][tj], st[tk + 2][tj]));
         // the coarsest level keeps no down half: its one sweep is undamped
-        if (F.om_ne1 && ec)
+        rarely(F.om_ne1 && ec, [&] {
             z = fma((R)F.omega, z,
                     (R)(1.0 - F.omega) * (ld(&f.e[q]) + ld(&ec[((bz * BZ - 1 + tk) >> 1) * Pc + bx * BX - 1 + tj])));
+        });
         if (tk >= 1 && tk <= BZ && tj >= 1 && tj <= BX) {
             out[q] = z;
-            acc[0] = fma(r, z, acc[0]);
+            if (DOT) acc[0] = fma(r, z, acc[0]);
         }
         return z;
     });
@@ -1089,7 +1092,7 @@ __device__ __forceinline__ void ph_mg_up(const LevelT<R> &f, const R *res, const
             const R r = ld(&res[q]);
             const R z = ld(&f.wd[q]) * (r + faces4<R>(f, q, sz[y][x - s], sz[y][x + 1 - s], sz[y - 1][x], sz[y + 1][x]));
             out[q] = z;
-            acc[0] = fma(r, z, acc[0]);
+            if (DOT) acc[0] = fma(r, z, acc[0]);
         }
     }
     __syncthreads();
@@ -1113,7 +1116,7 @@ __device__ __forceinline__ void ph_rb_up(const LevelT<R> &f, const R *rb, const 
     const R *rs = ec + (max(k - 1, 0) >> 1) * Pc, *rn = ec + (min(k + 1, G.nz - 1) >> 1) * Pc;
     const R r = ld(&rb[c]), w = ld(&f.wd[q]);
     R zv = w * (r + faces4<R>(f, q, ld(&row[jw]), ld(&row[je]), ld(&rs[j]), ld(&rn[j])));
-    if (F.om_ne1) zv = fma((R)F.omega, zv, (R)(1.0 - F.omega) * fma((R)F.omega * w, r, ld(&row[j])));
+    rarely(F.om_ne1, [&] { zv = fma((R)F.omega, zv, (R)(1.0 - F.omega) * fma((R)F.omega * w, r, ld(&row[j]))); });
     z[c] = zv;
     acc[0] = fma(r, zv, acc[0]);
 }
@@ -1177,7 +1180,7 @@ __device__ __forceinline__ void ph_update_single(const LevelT<R> &L, const R *qv
     if (i >= G.nx) return;
     const int c = cidx(G, j, k);
     const R pq = ld(&p[c]);
-    x[c] = first ? alpha * pq : fma(alpha, pq, ld(&x[c]));
+    x[c] = fma(alpha, pq, first ? (R)0 : ld(&x[c]));
     const R rn = fma(-alpha, ld(&qv[c]), ld(&rb[c]));
     rb[c] = rn;
     const R zv = ld(&L.wd[cidx(G, i, k)]) * rn;
@@ -1206,7 +1209,7 @@ __device__ __forceinline__ void ph_update_down(const LevelT<R> &f, const LevelT<
         if (tk >= 1 && tk <= BZ && tj >= 1 && tj <= BX) {
             rout[cc] = rn;
             const R pq = ld(&p[cc]);
-            x[cc] = first ? alpha * pq : fma(alpha, pq, ld(&x[cc]));
+            x[cc] = fma(alpha, pq, first ? (R)0 : ld(&x[cc]));
             acc[0] = fma(rn, rn, acc[0]);
         }
         return ld(&f.wd[q]) * rn;
@@ -1218,7 +1221,8 @@ __device__ __forceinline__ void ph_update_down(const LevelT<R> &f, const LevelT<
         const int s = k & 1, q = cidx(G, 2 * j + 1 - s, k);
         const int y = threadIdx.y + 1, xx = threadIdx.x + 1;
         v = faces4<R>(f, q, se[y][xx - s], se[y][xx + 1 - s], se[y - 1][xx], se[y + 1][xx]);
-        if (F.om_ne1) v = fma((R)F.omega, v, (R)(1.0 - F.omega) * ld(&f.d[cidx(G, 2 * j + s, k)]) * se[y][xx]);
+        rarely(F.om_ne1,
+               [&] { v = fma((R)F.omega, v, (R)(1.0 - F.omega) * ld(&f.d[cidx(G, 2 * j + s, k)]) * se[y][xx]); });
     }
     restrict_pairs<R>(c, v, sres, bx, bz);
     __syncthreads();
@@ -1382,10 +1386,10 @@ __device__ __forceinline__ void ph_correct(const StepArgs &a, const LevelT<R> &L
         N.p[q] = pn;
         N.rho[q] = pn * psq;
         N.pold[q] = pnq;
-        if (F.k_lagged) {
+        rarely(F.k_lagged, [&] {
             const double un = ld(&a.S.u[q]), wn = ld(&a.S.w[q]);
-            N.Kold[q] = 0.5 * (un * un + wn * wn);   // K^{n-1} of the next step
-        }
+            N.Kold[q] = 0.5 * fma(un, un, wn * wn);   // K^{n-1} of the next step
+        });
     }
     __syncthreads();
 }
