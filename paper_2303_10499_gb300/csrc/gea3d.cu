@@ -45,6 +45,11 @@ struct Geo {
     double dx, dy, dz;
     double idx, idy, idz, idx2, idy2, idz2, ivol;   // 1/dx, ..., 1/dx^2, ..., 1/(dx dy dz)
     double ax, ay, az;                              // face areas dy dz, dx dz, dx dy
+    // products formed once on the host (in a kernel each would be an FP64
+    // instruction of every thread)
+    double hidx, hidy, hidz, tidx, tidy, tidz;      // 1/(2 dx), ..., 2/dx, ...
+    double hax, hay, haz;                           // half the face areas
+    double s12;                                     // 1/(12 dx dy dz)
 };
 
 __host__ __device__ inline int id3(const Geo &G, int i, int j, int k)
@@ -54,7 +59,9 @@ __host__ __device__ inline int id3(const Geo &G, int i, int j, int k)
 
 struct Phy {
     double R, cp, g, mu, nuh, dt, idt, omega;
-    double icp;      // 1/cp
+    double icp, icv; // 1/cp, 1/cv
+    double mux, muy, muz, mud, nud;   // mu/dx^2, ..., 2 mu (1/dx^2 + 1/dy^2 + 1/dz^2), the same with mu/Pr
+    int les, pr_ne1; // les_d2 > 0; mu/Pr != mu
     double les_d2;   // (cs Delta)^2 with Delta = (dx dy dz)^(1/3); 0: constant mu
 };
 
@@ -111,6 +118,7 @@ struct Args {
     double *kin;    // K1 = |u1|^2 / 2
     double *mueff;  // mu + mu_t (LES only)
     const double *gzc, *gzf;   // g z of the cell centres (layer k) and of the horizontal faces (k = 0..nz)
+    const double *gx2, *gy2, *gz2;   // 2 g z / dx, 2 g z / dy of the cell centres, 2 g z / dz of the horizontal faces
     Cf cf;
     Sc *sc;
     double *part;
@@ -129,19 +137,20 @@ __device__ __forceinline__ bool cell(const Geo &G, int &i, int &j, int &k)
     return i < G.nx && j < G.ny && k < G.nz;
 }
 
-// The CG kernels with a reduction (FP64 and FP32) and the finest
-// prolongation walk kLayers consecutive cell layers of their column tile
-// (one block reduction per kLayers cells a thread): (i, j) of the thread
-// and its layer range [k0, k1). The layer loop stays rolled: unrolled, its
-// interleaved loads took 56-79 registers a thread and the kernels ran
-// 30-40 % slower at the lower occupancy.
-constexpr int kLayers = 8;
+// The kernels with a reduction and the finest prolongation walk consecutive
+// cell layers of their column tile (one block reduction per column: a
+// reduction of three FP64 values costs a block 36 FP64 instructions of one
+// warp, 4.5 per cell at one cell a thread): (i, j) of the thread and its layer
+// range [k0, k1), from the launch shape (columns_of). The layer loop stays
+// rolled: unrolled, its interleaved loads took 56-79 registers a thread and the
+// kernels ran 30-40 % slower at the lower occupancy.
 __device__ __forceinline__ bool column(const Geo &G, int &i, int &j, int &k0, int &k1)
 {
+    const int layers = (G.nz + gridDim.z - 1) / gridDim.z;
     i = blockIdx.x * TX + threadIdx.x;
     j = blockIdx.y * TY + threadIdx.y;
-    k0 = blockIdx.z * kLayers;
-    k1 = min(G.nz, k0 + kLayers);
+    k0 = blockIdx.z * layers;
+    k1 = min(G.nz, k0 + layers);
     return i < G.nx && j < G.ny;
 }
 
@@ -176,11 +185,6 @@ __device__ __forceinline__ double nbr(const Geo &G, const Phy &F, const double *
     return at<BC>(G, F, X, i + di, j + dj, k + dk);
 }
 
-__device__ __forceinline__ double i4(double xm, double xa, double xb, double xp)
-{
-    return (-xm + 7.0 * xa + 7.0 * xb - xp) * (1.0 / 12.0);
-}
-
 // Compact 7-point Laplacian through the ghosts.
 template <int BC>
 __device__ double lap(const Args &a, const double *X, int i, int j, int k)
@@ -191,15 +195,6 @@ __device__ double lap(const Args &a, const double *X, int i, int j, int k)
     return (at<BC>(G, F, X, i + 1, j, k) - xc + at<BC>(G, F, X, i - 1, j, k) - xc) * G.idx2 +
            (at<BC>(G, F, X, i, j + 1, k) - xc + at<BC>(G, F, X, i, j - 1, k) - xc) * G.idy2 +
            (at<BC>(G, F, X, i, j, k + 1) - xc + at<BC>(G, F, X, i, j, k - 1) - xc) * G.idz2;
-}
-
-__device__ double divg(const Args &a, int i, int j, int k)
-{
-    const Geo &G = a.G;
-    return (ld(&a.S.phix[id3(G, i + 1, j, k)]) - ld(&a.S.phix[id3(G, i, j, k)]) +
-            ld(&a.S.phiy[id3(G, i, j + 1, k)]) - ld(&a.S.phiy[id3(G, i, j, k)]) +
-            ld(&a.S.phiz[id3(G, i, j, k + 1)]) - ld(&a.S.phiz[id3(G, i, j, k)])) *
-           G.ivol;
 }
 
 // Deterministic grid sum of NV values per thread (3D grid of 32 x 8 blocks)
@@ -271,52 +266,49 @@ namespace g3 {
 // ---- set-up from conservative fields (dense nz x ny x nx arrays) ----
 
 __global__ void k_derive(Geo G, Phy F, const double *rho, const double *ru, const double *rv,
-                         const double *rw, const double *re, St S, Sc *sc)
+                         const double *rw, const double *re, const double *gzc, St S, Sc *sc)
 {
     int i, j, k;
     if (!cell(G, i, j, k)) return;
     const int n = (k * G.ny + j) * G.nx + i, q = id3(G, i, j, k);
-    const double z = (k + 0.5) * G.dz, cv = F.cp - F.R;
-    const double r = rho[n], u = ru[n] / r, v = rv[n] / r, w = rw[n] / r;
-    const double T = (re[n] / r - 0.5 * (u * u + v * v + w * w) - F.g * z) / cv;
+    const double gz = gzc[k];
+    const double r = rho[n], ir = gea::recip(r);
+    const double ru0 = ru[n], rv0 = rv[n], rw0 = rw[n], e1 = re[n];
+    const double u = ru0 * ir, v = rv0 * ir, w = rw0 * ir;
+    // e = re / r rounded as a division would: T and with it p = rho R T carry
+    // the hydrostatic balance
+    const double e0 = e1 * ir, e = fma(fma(-r, e0, e1), ir, e0);
+    const double T = ((e - 0.5 * fma(u, u, fma(v, v, w * w))) - gz) * F.icv;
     if (!(r > 0.0) || !(T > 0.0)) atomicAdd(&sc->bad_cells, 1);
     S.rho[q] = r; S.u[q] = u; S.v[q] = v; S.w[q] = w; S.T[q] = T; S.h[q] = F.cp * T;
     const double p = r * F.R * T;
-    S.p[q] = p; S.pp[q] = p + r * F.g * z; S.pold[q] = p;
+    S.p[q] = p; S.pp[q] = fma(r, gz, p); S.pold[q] = p;
     const int sx = 1, sy = G.nx, sz = G.nx * G.ny;
-    S.phix[q] = i > 0 ? 0.5 * (ru[n - sx] + ru[n]) * G.dy * G.dz : 0.0;
-    S.phiy[q] = j > 0 ? 0.5 * (rv[n - sy] + rv[n]) * G.dx * G.dz : 0.0;
-    S.phiz[q] = k > 0 ? 0.5 * (rw[n - sz] + rw[n]) * G.dx * G.dy : 0.0;
+    S.phix[q] = i > 0 ? (ru[n - sx] + ru0) * G.hax : 0.0;
+    S.phiy[q] = j > 0 ? (rv[n - sy] + rv0) * G.hay : 0.0;
+    S.phiz[q] = k > 0 ? (rw[n - sz] + rw0) * G.haz : 0.0;
     if (i == G.nx - 1) S.phix[id3(G, G.nx, j, k)] = 0.0;
     if (j == G.ny - 1) S.phiy[id3(G, i, G.ny, k)] = 0.0;
     if (k == G.nz - 1) S.phiz[id3(G, i, j, G.nz)] = 0.0;
 }
 
-// Face force G_f = (p'_b - p'_a)/Delta - g z_f (rho_b - rho_a)/Delta of the
-// face between cell q - s (a) and q (b) in direction d; zero on walls.
-__device__ __forceinline__ double fforce(const double *pp, const double *rho, int q, int s,
-                                         double inv, double gz)
+// Differences of p' and rho between two cells: p'_b - p'_a - gz (rho_b - rho_a),
+// the face force times the spacing when a and b share the face of height gz.
+// On a wall the cell stands for its missing neighbour, which gives zero.
+__device__ __forceinline__ double fdiff(const double *pp, const double *rho, int b, int a, double gz)
 {
-    return fma(-gz, ld(&rho[q]) - ld(&rho[q - s]), ld(&pp[q]) - ld(&pp[q - s])) * inv;
+    return fma(-gz, ld(&rho[b]) - ld(&rho[a]), ld(&pp[b]) - ld(&pp[a]));
 }
 
-// The face forces of cell (i,j,k): its west, south and bottom faces in fl
-// (zero on walls) and the cell averages of the two faces per direction in g.
-__device__ void cell_forces(const Args &a, const double *pp, const double *rho, int i, int j, int k,
-                            double (&fl)[3], double (&g)[3])
+// Neighbour indices of cell q at (i, j, k), the cell itself beyond a wall.
+struct Nb {
+    int w, e, s, n, b, t;
+};
+__device__ __forceinline__ Nb neighbours(const Geo &G, int q, int i, int j, int k)
 {
-    const Geo &G = a.G;
-    const int q = id3(G, i, j, k), sx = 1, sy = G.P, sz = G.P * (G.ny + 1);
-    const double gzc = ld(&a.gzc[k]);
-    fl[0] = i > 0 ? fforce(pp, rho, q, sx, G.idx, gzc) : 0.0;
-    const double fe = i + 1 < G.nx ? fforce(pp, rho, q + sx, sx, G.idx, gzc) : 0.0;
-    fl[1] = j > 0 ? fforce(pp, rho, q, sy, G.idy, gzc) : 0.0;
-    const double fn = j + 1 < G.ny ? fforce(pp, rho, q + sy, sy, G.idy, gzc) : 0.0;
-    fl[2] = k > 0 ? fforce(pp, rho, q, sz, G.idz, ld(&a.gzf[k])) : 0.0;
-    const double ft = k + 1 < G.nz ? fforce(pp, rho, q + sz, sz, G.idz, ld(&a.gzf[k + 1])) : 0.0;
-    g[0] = 0.5 * (fl[0] + fe);
-    g[1] = 0.5 * (fl[1] + fn);
-    g[2] = 0.5 * (fl[2] + ft);
+    const int sy = G.P, sz = G.P * (G.ny + 1);
+    return Nb{i > 0 ? q - 1 : q,  i + 1 < G.nx ? q + 1 : q,  j > 0 ? q - sy : q,
+              j + 1 < G.ny ? q + sy : q, k > 0 ? q - sz : q, k + 1 < G.nz ? q + sz : q};
 }
 
 __device__ __forceinline__ void fin_pred(Sc *sc, const double (&t)[3])
@@ -338,7 +330,7 @@ __global__ void k_les(Args a)
     if (!cell(a.G, i, j, k)) return;
     const Geo &G = a.G;
     const Phy &F = a.F;
-    const double hx = 0.5 * G.idx, hy = 0.5 * G.idy, hz = 0.5 * G.idz;
+    const double hx = G.hidx, hy = G.hidy, hz = G.hidz;
     const double *u = a.S.u, *v = a.S.v, *w = a.S.w;
     const int q = id3(G, i, j, k);
     const bool in = i >= 1 && i + 1 < G.nx && j >= 1 && j + 1 < G.ny && k >= 1 && k + 1 < G.nz;
@@ -355,8 +347,8 @@ __global__ void k_les(Args a)
     const double wy = (Wv(0, 1, 0) - Wv(0, -1, 0)) * hy;
     const double wz = (Wv(0, 0, 1) - Wv(0, 0, -1)) * hz;
     const double sxy = uy + vx, sxz = uz + wx, syz = vz + wy;
-    const double S = sqrt(2.0 * (ux * ux + vy * vy + wz * wz) + sxy * sxy + sxz * sxz + syz * syz);
-    a.mueff[q] = F.mu + ld(&a.S.rho[q]) * F.les_d2 * S;
+    const double S = sqrt(fma(2.0, fma(ux, ux, fma(vy, vy, wz * wz)), fma(sxy, sxy, fma(sxz, sxz, syz * syz))));
+    a.mueff[q] = fma(ld(&a.S.rho[q]) * F.les_d2, S, F.mu);
 }
 
 // rho1, the Jacobi reciprocals, b = rho^n u^n / dt - G_cell, initial guesses
@@ -366,67 +358,75 @@ __global__ void k_pred(Args a)
     if (a.sc->status) return;
     __shared__ double red[3 * NT];
     double acc[3] = {0.0, 0.0, 0.0}, tot[3];
-    int i, j, k;
-    if (cell(a.G, i, j, k)) {
-        const Geo &G = a.G;
-        const Phy &F = a.F;
-        const int q = id3(G, i, j, k), sy = G.P, sz = G.P * (G.ny + 1);
-        const double dv = divg(a, i, j, k), r = ld(&a.S.rho[q]);
-        const double rho1 = r - F.dt * dv;
-        a.rho1[q] = rho1;
-        // diffusion weights per face: mu/Delta^2, or with LES the face mean of
-        // mu_eff over Delta^2 (a wall face takes the cell's own, the even ghost)
-        double mw, me, ms, mn, mb, mt;
-        if (F.les_d2 > 0.0) {
-            const double mc = ld(&a.mueff[q]);
-            // (mu_c + mu_N)/2 / Delta^2, the halves folded into the factors
-            const double hx = 0.5 * G.idx2, hy = 0.5 * G.idy2, hz = 0.5 * G.idz2;
-            auto face = [&](int ii, int jj, int kk, double h) { return (mc + at<E3>(G, F, a.mueff, ii, jj, kk)) * h; };
-            mw = face(i - 1, j, k, hx); me = face(i + 1, j, k, hx);
-            ms = face(i, j - 1, k, hy); mn = face(i, j + 1, k, hy);
-            mb = face(i, j, k - 1, hz); mt = face(i, j, k + 1, hz);
-        } else {
-            mw = me = F.mu * G.idx2;
-            ms = mn = F.mu * G.idy2;
-            mb = mt = F.mu * G.idz2;
+    const Geo &G = a.G;
+    const Phy &F = a.F;
+    int i, j, k0, k1;
+    if (column(G, i, j, k0, k1))
+#pragma unroll 1
+        for (int k = k0; k < k1; ++k) {
+            const int q = id3(G, i, j, k), sy = G.P, sz = G.P * (G.ny + 1);
+            const Nb nb = neighbours(G, q, i, j, k);
+            const double pw = ld(&a.S.phix[q]), pe = ld(&a.S.phix[q + 1]);
+            const double ps = ld(&a.S.phiy[q]), pn = ld(&a.S.phiy[q + sy]);
+            const double pb = ld(&a.S.phiz[q]), pt = ld(&a.S.phiz[q + sz]);
+            const double dv = ((pe - pw) + (pn - ps) + (pt - pb)) * G.ivol, r = ld(&a.S.rho[q]);
+            const double rho1 = fma(-F.dt, dv, r);
+            a.rho1[q] = rho1;
+            // diffusion weights per face: mu/Delta^2, or with LES the face mean of
+            // mu_eff over Delta^2 (a wall face takes the cell's own, the even ghost)
+            double mw, me, ms, mn, mb, mt, md;
+            if (F.les) {
+                const double mc = ld(&a.mueff[q]);
+                // (mu_c + mu_N)/2 / Delta^2, the halves folded into the factors
+                const double hx = 0.5 * G.idx2, hy = 0.5 * G.idy2, hz = 0.5 * G.idz2;
+                mw = (mc + ld(&a.mueff[nb.w])) * hx; me = (mc + ld(&a.mueff[nb.e])) * hx;
+                ms = (mc + ld(&a.mueff[nb.s])) * hy; mn = (mc + ld(&a.mueff[nb.n])) * hy;
+                mb = (mc + ld(&a.mueff[nb.b])) * hz; mt = (mc + ld(&a.mueff[nb.t])) * hz;
+                md = (mw + me) + (ms + mn) + (mb + mt);
+            } else {
+                mw = me = F.mux;
+                ms = mn = F.muy;
+                mb = mt = F.muz;
+                md = F.mud;
+            }
+            const double c0 = fma(rho1, F.idt, (7.0 / 12.0) * dv);
+            const double cu = c0 + md, icu = gea::recip(cu);
+            a.dinvu[q] = icu;
+            // the enthalpy diagonal: the diffusion scaled by 1/Pr (LES requires Pr = 1)
+            double ich = icu;
+            gea::rarely(F.pr_ne1, [&] { ich = gea::recip(c0 + F.nud); });
+            a.dinvh[q] = ich;
+            // T as a stencil: the outgoing flux of a face times its fourth-order
+            // value (-X_m + 7 X_a + 7 X_b - X_p)/12, minus the diffusion
+            const double fw = pw * G.s12, fe = pe * G.s12, fs = ps * G.s12, fn = pn * G.s12, fb = pb * G.s12, ft = pt * G.s12;
+            const Cf &cf = a.cf;
+            cf.c[0][q] = cu;
+            cf.c[1][q] = fw;
+            cf.c[2][q] = -fma(7.0, fw, fe) - mw;
+            cf.c[3][q] = fma(7.0, fe, fw) - me;
+            cf.c[4][q] = -fe;
+            cf.c[5][q] = fs;
+            cf.c[6][q] = -fma(7.0, fs, fn) - ms;
+            cf.c[7][q] = fma(7.0, fn, fs) - mn;
+            cf.c[8][q] = -fn;
+            cf.c[9][q] = fb;
+            cf.c[10][q] = -fma(7.0, fb, ft) - mb;
+            cf.c[11][q] = fma(7.0, ft, fb) - mt;
+            cf.c[12][q] = -ft;
+            // sums of the two face forces of each direction (over the spacing); in x
+            // and y both faces have the cell's height
+            const double gc = ld(&a.gzc[k]);
+            const double sxf = fdiff(a.S.pp, a.S.rho, nb.e, nb.w, gc), syf = fdiff(a.S.pp, a.S.rho, nb.n, nb.s, gc);
+            const double szf = fdiff(a.S.pp, a.S.rho, nb.t, q, ld(&a.gzf[k + 1])) + fdiff(a.S.pp, a.S.rho, q, nb.b, ld(&a.gzf[k]));
+            a.dtr1[q] = F.dt * gea::recip(rho1);
+            const double u = ld(&a.S.u[q]), v = ld(&a.S.v[q]), w = ld(&a.S.w[q]), rdt = r * F.idt;
+            const double bu = fma(-G.hidx, sxf, rdt * u), bv = fma(-G.hidy, syf, rdt * v), bw = fma(-G.hidz, szf, rdt * w);
+            a.bu[q] = bu; a.bv[q] = bv; a.bw[q] = bw;
+            a.ua[q] = u; a.va[q] = v; a.wa[q] = w;
+            acc[0] = fma(bu, bu, acc[0]);
+            acc[1] = fma(bv, bv, acc[1]);
+            acc[2] = fma(bw, bw, acc[2]);
         }
-        const double cu = rho1 * F.idt + (7.0 / 12.0) * dv + ((mw + me) + (ms + mn) + (mb + mt));
-        const double icu = 1.0 / cu;
-        a.dinvu[q] = icu;
-        // the enthalpy diagonal: the diffusion scaled by 1/Pr (LES requires Pr = 1)
-        a.dinvh[q] = F.les_d2 > 0.0 ? icu
-                                    : 1.0 / (rho1 * F.idt + (7.0 / 12.0) * dv +
-                                             F.nuh * 2.0 * (G.idx2 + G.idy2 + G.idz2));
-        // T as a stencil: the outgoing flux of a face times its fourth-order
-        // value (-X_m + 7 X_a + 7 X_b - X_p)/12, minus the diffusion
-        const double i12 = G.ivol * (1.0 / 12.0);
-        const double pw = ld(&a.S.phix[q]), pe = ld(&a.S.phix[q + 1]);
-        const double ps = ld(&a.S.phiy[q]), pn = ld(&a.S.phiy[q + sy]);
-        const double pb = ld(&a.S.phiz[q]), pt = ld(&a.S.phiz[q + sz]);
-        const Cf &cf = a.cf;
-        cf.c[0][q] = cu;
-        cf.c[1][q] = pw * i12;
-        cf.c[2][q] = -(pe + 7.0 * pw) * i12 - mw;
-        cf.c[3][q] = (7.0 * pe + pw) * i12 - me;
-        cf.c[4][q] = -pe * i12;
-        cf.c[5][q] = ps * i12;
-        cf.c[6][q] = -(pn + 7.0 * ps) * i12 - ms;
-        cf.c[7][q] = (7.0 * pn + ps) * i12 - mn;
-        cf.c[8][q] = -pn * i12;
-        cf.c[9][q] = pb * i12;
-        cf.c[10][q] = -(pt + 7.0 * pb) * i12 - mb;
-        cf.c[11][q] = (7.0 * pt + pb) * i12 - mt;
-        cf.c[12][q] = -pt * i12;
-        double fl[3], gc[3];
-        cell_forces(a, a.S.pp, a.S.rho, i, j, k, fl, gc);
-        const double gx = gc[0], gy = gc[1], gz = gc[2];
-        a.dtr1[q] = F.dt / rho1;
-        const double u = ld(&a.S.u[q]), v = ld(&a.S.v[q]), w = ld(&a.S.w[q]);
-        const double bu = r * u * F.idt - gx, bv = r * v * F.idt - gy, bw = r * w * F.idt - gz;
-        a.bu[q] = bu; a.bv[q] = bv; a.bw[q] = bw;
-        a.ua[q] = u; a.va[q] = v; a.wa[q] = w;
-        acc[0] = bu * bu; acc[1] = bv * bv; acc[2] = bw * bw;
-    }
     if (gsum<3>(acc, red, a.part, &a.sc->counters[C_PRED], tot)) fin_pred(a.sc, tot);
 }
 
@@ -443,10 +443,11 @@ __device__ __forceinline__ W13 weights(const Args &a, int q)
     return c;
 }
 
-// Off-centre part of T(X): sum over the 12 neighbour slots of weight times
-// value (ghosts by rule BC; slots two cells beyond a wall carry weight 0).
+// b minus the off-centre part of T(X), the sum over the 12 neighbour slots of
+// weight times value (ghosts by rule BC; slots two cells beyond a wall carry
+// weight 0), as one chain of FMAs.
 template <int BC>
-__device__ __forceinline__ double toff(const Args &a, const W13 &c, const double *X, int i, int j, int k)
+__device__ __forceinline__ double toff(const Args &a, double b, const W13 &c, const double *X, int i, int j, int k)
 {
     const Geo &G = a.G;
     const Phy &F = a.F;
@@ -454,39 +455,40 @@ __device__ __forceinline__ double toff(const Args &a, const W13 &c, const double
         // away from the walls: the neighbours at fixed offsets (same order)
         const int sy = G.P, sz = G.P * (G.ny + 1);
         const double *x = X + id3(G, i, j, k);
-        double t = c.w[1] * ld(x - 2);
-        t = fma(c.w[2], ld(x - 1), t);
-        t = fma(c.w[3], ld(x + 1), t);
-        t = fma(c.w[4], ld(x + 2), t);
-        t = fma(c.w[5], ld(x - 2 * sy), t);
-        t = fma(c.w[6], ld(x - sy), t);
-        t = fma(c.w[7], ld(x + sy), t);
-        t = fma(c.w[8], ld(x + 2 * sy), t);
-        t = fma(c.w[9], ld(x - 2 * sz), t);
-        t = fma(c.w[10], ld(x - sz), t);
-        t = fma(c.w[11], ld(x + sz), t);
-        t = fma(c.w[12], ld(x + 2 * sz), t);
+        double t = fma(-c.w[1], ld(x - 2), b);
+        t = fma(-c.w[2], ld(x - 1), t);
+        t = fma(-c.w[3], ld(x + 1), t);
+        t = fma(-c.w[4], ld(x + 2), t);
+        t = fma(-c.w[5], ld(x - 2 * sy), t);
+        t = fma(-c.w[6], ld(x - sy), t);
+        t = fma(-c.w[7], ld(x + sy), t);
+        t = fma(-c.w[8], ld(x + 2 * sy), t);
+        t = fma(-c.w[9], ld(x - 2 * sz), t);
+        t = fma(-c.w[10], ld(x - sz), t);
+        t = fma(-c.w[11], ld(x + sz), t);
+        t = fma(-c.w[12], ld(x + 2 * sz), t);
         return t;
     }
-    double t = c.w[1] * at<BC>(G, F, X, i - 2, j, k);
-    t = fma(c.w[2], at<BC>(G, F, X, i - 1, j, k), t);
-    t = fma(c.w[3], at<BC>(G, F, X, i + 1, j, k), t);
-    t = fma(c.w[4], at<BC>(G, F, X, i + 2, j, k), t);
-    t = fma(c.w[5], at<BC>(G, F, X, i, j - 2, k), t);
-    t = fma(c.w[6], at<BC>(G, F, X, i, j - 1, k), t);
-    t = fma(c.w[7], at<BC>(G, F, X, i, j + 1, k), t);
-    t = fma(c.w[8], at<BC>(G, F, X, i, j + 2, k), t);
-    t = fma(c.w[9], at<BC>(G, F, X, i, j, k - 2), t);
-    t = fma(c.w[10], at<BC>(G, F, X, i, j, k - 1), t);
-    t = fma(c.w[11], at<BC>(G, F, X, i, j, k + 1), t);
-    t = fma(c.w[12], at<BC>(G, F, X, i, j, k + 2), t);
+    double t = fma(-c.w[1], at<BC>(G, F, X, i - 2, j, k), b);
+    t = fma(-c.w[2], at<BC>(G, F, X, i - 1, j, k), t);
+    t = fma(-c.w[3], at<BC>(G, F, X, i + 1, j, k), t);
+    t = fma(-c.w[4], at<BC>(G, F, X, i + 2, j, k), t);
+    t = fma(-c.w[5], at<BC>(G, F, X, i, j - 2, k), t);
+    t = fma(-c.w[6], at<BC>(G, F, X, i, j - 1, k), t);
+    t = fma(-c.w[7], at<BC>(G, F, X, i, j + 1, k), t);
+    t = fma(-c.w[8], at<BC>(G, F, X, i, j + 2, k), t);
+    t = fma(-c.w[9], at<BC>(G, F, X, i, j, k - 2), t);
+    t = fma(-c.w[10], at<BC>(G, F, X, i, j, k - 1), t);
+    t = fma(-c.w[11], at<BC>(G, F, X, i, j, k + 1), t);
+    t = fma(-c.w[12], at<BC>(G, F, X, i, j, k + 2), t);
     return t;
 }
 
-__device__ __forceinline__ void copy_cell(const Geo &G, const double *x, double *y)
+__device__ __forceinline__ void copy_column(const Geo &G, const double *x, double *y)
 {
-    int i, j, k;
-    if (cell(G, i, j, k)) y[id3(G, i, j, k)] = ld(&x[id3(G, i, j, k)]);
+    int i, j, k0, k1;
+    if (column(G, i, j, k0, k1))
+        for (int k = k0; k < k1; ++k) y[id3(G, i, j, k)] = ld(&x[id3(G, i, j, k)]);
 }
 
 // One Jacobi sweep of the three momentum components (pairs of sweeps; the
@@ -498,33 +500,37 @@ __global__ void __launch_bounds__(NT, 5) k_mom(Args a, const double *ui, const d
     Sc *sc = a.sc;
     if (sc->status) return;
     if (second && sc->done[L_MOM]) {
-        copy_cell(a.G, ui, uo);
-        copy_cell(a.G, vi, vo);
-        copy_cell(a.G, wi, wo);
+        copy_column(a.G, ui, uo);
+        copy_column(a.G, vi, vo);
+        copy_column(a.G, wi, wo);
         return;
     }
     __shared__ double red[3 * NT];
     double acc[3] = {0.0, 0.0, 0.0}, tot[3];
-    int i, j, k;
-    if (cell(a.G, i, j, k)) {
-        const int q = id3(a.G, i, j, k);
-        const double di = ld(&a.dinvu[q]);
-        const W13 c = weights(a, q);
-        // one component after the other (the empty asm keeps the compiler
-        // from interleaving their loads, which would cost registers)
-        const double u0 = ld(&ui[q]);
-        const double ru = ld(&a.bu[q]) - fma(c.w[0], u0, toff<U3>(a, c, ui, i, j, k));
-        uo[q] = fma(ru, di, u0);
-        asm volatile("" ::: "memory");
-        const double v0 = ld(&vi[q]);
-        const double rv = ld(&a.bv[q]) - fma(c.w[0], v0, toff<V3>(a, c, vi, i, j, k));
-        vo[q] = fma(rv, di, v0);
-        asm volatile("" ::: "memory");
-        const double w0 = ld(&wi[q]);
-        const double rw = ld(&a.bw[q]) - fma(c.w[0], w0, toff<W3>(a, c, wi, i, j, k));
-        wo[q] = fma(rw, di, w0);
-        acc[0] = ru * ru; acc[1] = rv * rv; acc[2] = rw * rw;
-    }
+    int i, j, k0, k1;
+    if (column(a.G, i, j, k0, k1))
+#pragma unroll 1
+        for (int k = k0; k < k1; ++k) {
+            const int q = id3(a.G, i, j, k);
+            const double di = ld(&a.dinvu[q]);
+            const W13 c = weights(a, q);
+            // one component after the other (the empty asm keeps the compiler
+            // from interleaving their loads, which would cost registers)
+            const double u0 = ld(&ui[q]);
+            const double ru = toff<U3>(a, fma(-c.w[0], u0, ld(&a.bu[q])), c, ui, i, j, k);
+            uo[q] = fma(ru, di, u0);
+            acc[0] = fma(ru, ru, acc[0]);
+            asm volatile("" ::: "memory");
+            const double v0 = ld(&vi[q]);
+            const double rv = toff<V3>(a, fma(-c.w[0], v0, ld(&a.bv[q])), c, vi, i, j, k);
+            vo[q] = fma(rv, di, v0);
+            acc[1] = fma(rv, rv, acc[1]);
+            asm volatile("" ::: "memory");
+            const double w0 = ld(&wi[q]);
+            const double rw = toff<W3>(a, fma(-c.w[0], w0, ld(&a.bw[q])), c, wi, i, j, k);
+            wo[q] = fma(rw, di, w0);
+            acc[2] = fma(rw, rw, acc[2]);
+        }
     if (gsum<3>(acc, red, a.part, &sc->counters[C_MOM], tot)) {
         sc->sweeps[0] += 1;
         if (!isfinite(tot[0]) || !isfinite(tot[1]) || !isfinite(tot[2])) sc->status = GEA_ERR_NONFINITE;
@@ -544,7 +550,7 @@ __global__ void k_kin(Args a, const double *u1, const double *v1, const double *
     if (!cell(a.G, i, j, k)) return;
     const int q = id3(a.G, i, j, k);
     const double u = ld(&u1[q]), v = ld(&v1[q]), w = ld(&w1[q]);
-    a.kin[q] = 0.5 * (u * u + v * v + w * w);
+    a.kin[q] = 0.5 * fma(u, u, fma(v, v, w * w));
 }
 
 // Right-hand side of the enthalpy equation and its initial guess h^n:
@@ -554,36 +560,37 @@ __global__ void k_enth_rhs(Args a, const double *w1)
     if (a.sc->status) return;
     __shared__ double red[NT];
     double acc[1] = {0.0}, tot[1];
-    int i, j, k;
-    if (cell(a.G, i, j, k)) {
-        const Geo &G = a.G;
-        const Phy &F = a.F;
-        const int q = id3(G, i, j, k);
-        // C(K1), fourth-order face values of K1 with even ghosts; the 1/12 of
-        // the face values is applied once to the sum: 12 X_f = 7 (X_a + X_b) - (X_m + X_p)
-        double s = 0.0;
-        const double Kc = ld(&a.kin[q]);
-        const bool in = i >= 2 && i + 2 < G.nx && j >= 2 && j + 2 < G.ny && k >= 2 && k + 2 < G.nz;
-        auto K = [&](int ii, int jj, int kk) {
-            return nbr<E3>(G, F, a.kin, q, in, i, j, k, ii - i, jj - j, kk - k);
-        };
-        auto f12 = [](double xm, double xa, double xb, double xp) { return fma(7.0, xa + xb, -(xm + xp)); };
-        if (i + 1 < G.nx) s = fma(ld(&a.S.phix[id3(G, i + 1, j, k)]), f12(K(i - 1, j, k), Kc, K(i + 1, j, k), K(i + 2, j, k)), s);
-        if (i > 0) s = fma(-ld(&a.S.phix[q]), f12(K(i - 2, j, k), K(i - 1, j, k), Kc, K(i + 1, j, k)), s);
-        if (j + 1 < G.ny) s = fma(ld(&a.S.phiy[id3(G, i, j + 1, k)]), f12(K(i, j - 1, k), Kc, K(i, j + 1, k), K(i, j + 2, k)), s);
-        if (j > 0) s = fma(-ld(&a.S.phiy[q]), f12(K(i, j - 2, k), K(i, j - 1, k), Kc, K(i, j + 1, k)), s);
-        if (k + 1 < G.nz) s = fma(ld(&a.S.phiz[id3(G, i, j, k + 1)]), f12(K(i, j, k - 1), Kc, K(i, j, k + 1), K(i, j, k + 2)), s);
-        if (k > 0) s = fma(-ld(&a.S.phiz[q]), f12(K(i, j, k - 2), K(i, j, k - 1), Kc, K(i, j, k + 1)), s);
-        s *= G.ivol * (1.0 / 12.0);
-        const double r = ld(&a.S.rho[q]), u = ld(&a.S.u[q]), v = ld(&a.S.v[q]), w = ld(&a.S.w[q]);
-        const double h = ld(&a.S.h[q]), rho1 = ld(&a.rho1[q]);
-        const double Kn = 0.5 * (u * u + v * v + w * w);
-        const double be = (r * h + r * Kn - ld(&a.S.pold[q])) * F.idt;
-        const double bh = be - rho1 * Kc * F.idt - s + ld(&a.S.p[q]) * F.idt - rho1 * F.g * ld(&w1[q]);
-        a.bh[q] = bh;
-        a.ha[q] = h;
-        acc[0] = bh * bh;
-    }
+    const Geo &G = a.G;
+    const Phy &F = a.F;
+    int i, j, k0, k1;
+    if (column(G, i, j, k0, k1))
+#pragma unroll 1
+        for (int k = k0; k < k1; ++k) {
+            const int q = id3(G, i, j, k);
+            // C(K1), fourth-order face values of K1 with even ghosts; the 1/12 of
+            // the face values is applied once to the sum: 12 X_f = 7 (X_a + X_b) - (X_m + X_p)
+            double s = 0.0;
+            const double Kc = ld(&a.kin[q]);
+            const bool in = i >= 2 && i + 2 < G.nx && j >= 2 && j + 2 < G.ny && k >= 2 && k + 2 < G.nz;
+            auto K = [&](int ii, int jj, int kk) {
+                return nbr<E3>(G, F, a.kin, q, in, i, j, k, ii - i, jj - j, kk - k);
+            };
+            auto f12 = [](double xm, double xa, double xb, double xp) { return fma(7.0, xa + xb, -(xm + xp)); };
+            if (i + 1 < G.nx) s = fma(ld(&a.S.phix[id3(G, i + 1, j, k)]), f12(K(i - 1, j, k), Kc, K(i + 1, j, k), K(i + 2, j, k)), s);
+            if (i > 0) s = fma(-ld(&a.S.phix[q]), f12(K(i - 2, j, k), K(i - 1, j, k), Kc, K(i + 1, j, k)), s);
+            if (j + 1 < G.ny) s = fma(ld(&a.S.phiy[id3(G, i, j + 1, k)]), f12(K(i, j - 1, k), Kc, K(i, j + 1, k), K(i, j + 2, k)), s);
+            if (j > 0) s = fma(-ld(&a.S.phiy[q]), f12(K(i, j - 2, k), K(i, j - 1, k), Kc, K(i, j + 1, k)), s);
+            if (k + 1 < G.nz) s = fma(ld(&a.S.phiz[id3(G, i, j, k + 1)]), f12(K(i, j, k - 1), Kc, K(i, j, k + 1), K(i, j, k + 2)), s);
+            if (k > 0) s = fma(-ld(&a.S.phiz[q]), f12(K(i, j, k - 2), K(i, j, k - 1), Kc, K(i, j, k + 1)), s);
+            const double r = ld(&a.S.rho[q]), u = ld(&a.S.u[q]), v = ld(&a.S.v[q]), w = ld(&a.S.w[q]);
+            const double h = ld(&a.S.h[q]), rho1 = ld(&a.rho1[q]);
+            const double Kn = 0.5 * fma(u, u, fma(v, v, w * w));
+            const double te = fma(r, h + Kn, -ld(&a.S.pold[q])) + ld(&a.S.p[q]);
+            const double bh = fma(-rho1 * F.g, ld(&w1[q]), fma(F.idt, fma(-rho1, Kc, te), -(G.s12 * s)));
+            a.bh[q] = bh;
+            a.ha[q] = h;
+            acc[0] = fma(bh, bh, acc[0]);
+        }
     if (gsum<1>(acc, red, a.part, &a.sc->counters[C_ERHS], tot)) {
         a.sc->bn2[3] = tot[0];
         a.sc->done[L_ENTH] = 0;
@@ -599,23 +606,24 @@ __global__ void __launch_bounds__(NT, 5) k_enth(Args a, const double *hi, double
     Sc *sc = a.sc;
     if (sc->status) return;
     if (second && sc->done[L_ENTH]) {
-        copy_cell(a.G, hi, ho);
+        copy_column(a.G, hi, ho);
         return;
     }
     __shared__ double red[NT];
     double acc[1] = {0.0}, tot[1];
-    int i, j, k;
-    if (cell(a.G, i, j, k)) {
-        const int q = id3(a.G, i, j, k);
-        const W13 c = weights(a, q);
-        const double h0 = ld(&hi[q]);
-        // T with nu_h = mu/Pr: the mu-stencil plus (mu - nu_h) L(h)
-        double t = fma(c.w[0], h0, toff<H3>(a, c, hi, i, j, k));
-        if (a.F.nuh != a.F.mu) t = fma(a.F.mu - a.F.nuh, lap<H3>(a, hi, i, j, k), t);
-        const double r = ld(&a.bh[q]) - t;
-        ho[q] = fma(r, ld(&a.dinvh[q]), h0);
-        acc[0] = r * r;
-    }
+    int i, j, k0, k1;
+    if (column(a.G, i, j, k0, k1))
+#pragma unroll 1
+        for (int k = k0; k < k1; ++k) {
+            const int q = id3(a.G, i, j, k);
+            const W13 c = weights(a, q);
+            const double h0 = ld(&hi[q]);
+            // T with nu_h = mu/Pr: the mu-stencil plus (mu - nu_h) L(h)
+            double r = toff<H3>(a, fma(-c.w[0], h0, ld(&a.bh[q])), c, hi, i, j, k);
+            gea::rarely(a.F.pr_ne1, [&] { r = fma(a.F.nuh - a.F.mu, lap<H3>(a, hi, i, j, k), r); });
+            ho[q] = fma(r, ld(&a.dinvh[q]), h0);
+            acc[0] = fma(r, r, acc[0]);
+        }
     if (gsum<1>(acc, red, a.part, &sc->counters[C_ENTH], tot)) {
         sc->sweeps[1] += 1;
         if (!isfinite(tot[0])) sc->status = GEA_ERR_NONFINITE;
@@ -634,7 +642,7 @@ __global__ void k_eos(Args a, Lev L, Lev32 m, const double *h1)
     const int q = id3(a.G, i, j, k);
     const double hq = ld(&h1[q]);
     const double T1 = fma(hq - ld(&a.S.h[q]), F.icp, ld(&a.S.T[q]));
-    const double psi = 1.0 / (F.R * T1);
+    const double psi = gea::recip(F.R * T1);
     a.N.T[q] = T1;
     a.N.h[q] = hq;
     a.rho2[q] = ld(&a.S.p[q]) * psi;
@@ -657,7 +665,7 @@ __global__ void k_faces(Args a, Lev L, Lev32 m)
     const int q = id3(G, i, j, k), sx = 1, sy = G.P, sz = G.P * (G.ny + 1);
     const double r2 = ld(&a.rho2[q]), r1 = ld(&a.rho1[q]), dt = a.F.dt;
     // the halves of the two face means cancel exactly
-    auto D = [&](int qn) { return dt * (r2 + ld(&a.rho2[qn])) / (r1 + ld(&a.rho1[qn])); };
+    auto D = [&](int qn) { return dt * (r2 + ld(&a.rho2[qn])) * gea::recip(r1 + ld(&a.rho1[qn])); };
     const double Dw = i > 0 ? D(q - sx) : 0.0;
     const double Ds = j > 0 ? D(q - sy) : 0.0;
     const double Db = k > 0 ? D(q - sz) : 0.0;
@@ -701,10 +709,10 @@ __global__ void k_H(Args a, const double *U, const double *V, const double *W)
     const double r = ld(&a.S.rho[q]) * a.F.idt;
     // C(X) - mu L(X) = T(X) - (rho1/dt) X
     const W13 c = weights(a, q);
-    const double c0 = c.w[0] - ld(&a.rho1[q]) * a.F.idt;
-    a.Hx[q] = r * ld(&a.S.u[q]) - fma(c0, ld(&U[q]), toff<U3>(a, c, U, i, j, k));
-    a.Hy[q] = r * ld(&a.S.v[q]) - fma(c0, ld(&V[q]), toff<V3>(a, c, V, i, j, k));
-    a.Hz[q] = r * ld(&a.S.w[q]) - fma(c0, ld(&W[q]), toff<W3>(a, c, W, i, j, k));
+    const double c0 = fma(-ld(&a.rho1[q]), a.F.idt, c.w[0]);
+    a.Hx[q] = toff<U3>(a, fma(-c0, ld(&U[q]), r * ld(&a.S.u[q])), c, U, i, j, k);
+    a.Hy[q] = toff<V3>(a, fma(-c0, ld(&V[q]), r * ld(&a.S.v[q])), c, V, i, j, k);
+    a.Hz[q] = toff<W3>(a, fma(-c0, ld(&W[q]), r * ld(&a.S.w[q])), c, W, i, j, k);
 }
 
 // A x at cell (i,j,k) of level L for x given cellwise by xf(q, i, j, k) (interior
@@ -767,41 +775,47 @@ __global__ void k_helm_rhs(Args a, Lev L, const double *xin, double *xout, int c
     if (a.sc->status) return;
     __shared__ double red[2 * NT];
     double acc[2] = {0.0, 0.0}, tot[2];
-    int i, j, k;
-    if (cell(a.G, i, j, k)) {
-        const Geo &G = a.G;
-        const Phy &F = a.F;
-        const int q = id3(G, i, j, k), sx = 1, sy = G.P, sz = G.P * (G.ny + 1);
-        const double gc = ld(&a.gzc[k]), r2 = ld(&a.rho2[q]);
-        // a face's D_f/Delta (s (H_c + H_N)/2 + g z_f (rho2_N - rho2_c)/Delta):
-        // hs = s/2 with s the sign of the outward normal, gzi = g z_f/Delta
-        auto face = [&](const double *D, const double *H, int fq, int nq, double hs, double gzi,
-                        double idl) {
-            return ld(&D[fq]) * idl * fma(gzi, ld(&a.rho2[nq]) - r2, hs * (ld(&H[q]) + ld(&H[nq])));
-        };
-        const double gx = gc * G.idx, gy = gc * G.idy;
-        double fl = 0.0;
-        if (i + 1 < G.nx) fl += face(a.Dx, a.Hx, q + sx, q + sx, 0.5, gx, G.idx);
-        if (i > 0) fl += face(a.Dx, a.Hx, q, q - sx, -0.5, gx, G.idx);
-        if (j + 1 < G.ny) fl += face(a.Dy, a.Hy, q + sy, q + sy, 0.5, gy, G.idy);
-        if (j > 0) fl += face(a.Dy, a.Hy, q, q - sy, -0.5, gy, G.idy);
-        if (k + 1 < G.nz) fl += face(a.Dz, a.Hz, q + sz, q + sz, 0.5, ld(&a.gzf[k + 1]) * G.idz, G.idz);
-        if (k > 0) fl += face(a.Dz, a.Hz, q, q - sz, -0.5, ld(&a.gzf[k]) * G.idz, G.idz);
-        const double b = fma(ld(&a.psi[q]) * r2, gc, ld(&a.S.rho[q])) * F.idt - fl;
-        const double r = b - helm(L, [&](int qq, int, int, int) { return ld(&xin[qq]); }, i, j, k);
-        a.b[q] = b;
-        L.r[q] = r;
-        xout[q] = ld(&xin[q]);
-        a.p0[q] = 0.0;
-        if (mr) {
-            mr[q] = (float)r;
-            mx[q] = 0.0f;
-            mp0[q] = 0.0f;
+    const Geo &G = a.G;
+    const Phy &F = a.F;
+    int i, j, k0, k1;
+    if (column(G, i, j, k0, k1))
+#pragma unroll 1
+        for (int k = k0; k < k1; ++k) {
+            const int q = id3(G, i, j, k), sy = G.P, sz = G.P * (G.ny + 1);
+            const Nb nb = neighbours(G, q, i, j, k);
+            const double r2 = ld(&a.rho2[q]);
+            // twice the outgoing flux of a direction over its spacing, from
+            // D_f (H_a + H_b + 2 g z_f (rho2_b - rho2_a) / Delta); D_f = 0 on walls
+            auto pair = [&](const double *D, int up, const double *H, int ql, int qu, double gl, double gu) {
+                const double h = ld(&H[q]);
+                const double f = ld(&D[q + up]) * fma(gu, ld(&a.rho2[qu]) - r2, h + ld(&H[qu]));
+                return fma(-ld(&D[q]), fma(gl, r2 - ld(&a.rho2[ql]), h + ld(&H[ql])), f);
+            };
+            const double gx = ld(&a.gx2[k]), gy = ld(&a.gy2[k]);
+            double fl = G.hidx * pair(a.Dx, 1, a.Hx, nb.w, nb.e, gx, gx);
+            fl = fma(G.hidy, pair(a.Dy, sy, a.Hy, nb.s, nb.n, gy, gy), fl);
+            fl = fma(G.hidz, pair(a.Dz, sz, a.Hz, nb.b, nb.t, ld(&a.gz2[k]), ld(&a.gz2[k + 1])), fl);
+            const double b = fma(fma(ld(&a.psi[q]) * r2, ld(&a.gzc[k]), ld(&a.S.rho[q])), F.idt, -fl);
+            double r = fma(-ld(&L.d[q]), ld(&xin[q]), b);
+            r = fma(ld(&L.ax[q]), ld(&xin[nb.w]), r);
+            r = fma(ld(&L.ax[q + 1]), ld(&xin[nb.e]), r);
+            r = fma(ld(&L.ay[q]), ld(&xin[nb.s]), r);
+            r = fma(ld(&L.ay[q + sy]), ld(&xin[nb.n]), r);
+            r = fma(ld(&L.az[q]), ld(&xin[nb.b]), r);
+            r = fma(ld(&L.az[q + sz]), ld(&xin[nb.t]), r);
+            a.b[q] = b;
+            L.r[q] = r;
+            xout[q] = ld(&xin[q]);
+            a.p0[q] = 0.0;
+            if (mr) {
+                mr[q] = (float)r;
+                mx[q] = 0.0f;
+                mp0[q] = 0.0f;
+            }
+            if (rf) rf[q] = (float)r;
+            acc[0] = fma(b, b, acc[0]);
+            acc[1] = fma(r, r, acc[1]);
         }
-        if (rf) rf[q] = (float)r;
-        acc[0] = b * b;
-        acc[1] = r * r;
-    }
     if (gsum<2>(acc, red, a.part, &a.sc->counters[C_HELM], tot)) {
         if (mr) fin_helm_mixed(a.sc, tot, a.ctol2, corr);
         else fin_helm(a.sc, tot, a.ctol2, corr);
@@ -1070,21 +1084,27 @@ __global__ void k_correct(Args a)
     if (!cell(a.G, i, j, k)) return;
     const Geo &G = a.G;
     const int q = id3(G, i, j, k), sx = 1, sy = G.P, sz = G.P * (G.ny + 1);
-    double fl[3], gc[3];
-    cell_forces(a, a.N.pp, a.rho2, i, j, k, fl, gc);
+    const Nb nb = neighbours(G, q, i, j, k);
+    const double gc = ld(&a.gzc[k]);
+    // Delta G_f of the west, south and bottom faces, and the sum over both
+    // faces of each direction
+    const double fw = fdiff(a.N.pp, a.rho2, q, nb.w, gc), fs = fdiff(a.N.pp, a.rho2, q, nb.s, gc);
+    const double fb = fdiff(a.N.pp, a.rho2, q, nb.b, ld(&a.gzf[k]));
+    const double sxf = fdiff(a.N.pp, a.rho2, nb.e, nb.w, gc), syf = fdiff(a.N.pp, a.rho2, nb.n, nb.s, gc);
+    const double szf = fdiff(a.N.pp, a.rho2, nb.t, q, ld(&a.gzf[k + 1])) + fb;
     const double c1 = ld(&a.dtr1[q]);
     const double hx = ld(&a.Hx[q]), hy = ld(&a.Hy[q]), hz = ld(&a.Hz[q]);
-    a.N.u[q] = c1 * (hx - gc[0]);
-    a.N.v[q] = c1 * (hy - gc[1]);
-    a.N.w[q] = c1 * (hz - gc[2]);
-    const double pn = fma(-ld(&a.rho2[q]), ld(&a.gzc[k]), ld(&a.N.pp[q]));
+    a.N.u[q] = c1 * fma(-G.hidx, sxf, hx);
+    a.N.v[q] = c1 * fma(-G.hidy, syf, hy);
+    a.N.w[q] = c1 * fma(-G.hidz, szf, hz);
+    const double pn = fma(-ld(&a.rho2[q]), gc, ld(&a.N.pp[q]));
     a.N.p[q] = pn;
     a.N.rho[q] = pn * ld(&a.psi[q]);
     a.N.pold[q] = ld(&a.S.p[q]);
-    // F_f = D_f (H_f - G_f) |A_f| on the west, south and bottom faces
-    a.N.phix[q] = i > 0 ? ld(&a.Dx[q]) * fma(0.5, hx + ld(&a.Hx[q - sx]), -fl[0]) * G.ax : 0.0;
-    a.N.phiy[q] = j > 0 ? ld(&a.Dy[q]) * fma(0.5, hy + ld(&a.Hy[q - sy]), -fl[1]) * G.ay : 0.0;
-    a.N.phiz[q] = k > 0 ? ld(&a.Dz[q]) * fma(0.5, hz + ld(&a.Hz[q - sz]), -fl[2]) * G.az : 0.0;
+    // F_f |A_f| = D_f (|A_f| / 2) (H_a + H_b - 2 G_f) (D_f = 0 on walls)
+    a.N.phix[q] = (ld(&a.Dx[q]) * G.hax) * fma(-G.tidx, fw, hx + ld(&a.Hx[nb.w]));
+    a.N.phiy[q] = (ld(&a.Dy[q]) * G.hay) * fma(-G.tidy, fs, hy + ld(&a.Hy[nb.s]));
+    a.N.phiz[q] = (ld(&a.Dz[q]) * G.haz) * fma(-G.tidz, fb, hz + ld(&a.Hz[nb.b]));
     if (i == G.nx - 1) a.N.phix[q + sx] = 0.0;
     if (j == G.ny - 1) a.N.phiy[q + sy] = 0.0;
     if (k == G.nz - 1) a.N.phiz[q + sz] = 0.0;
@@ -1199,28 +1219,29 @@ __global__ void k_mx_r0mom(Args a, Mx m)
     if (sc->status) return;
     __shared__ double red[3 * NT];
     double acc[3] = {0.0, 0.0, 0.0}, tot[3];
-    int i, j, k;
-    if (cell(a.G, i, j, k)) {
-        const int q = id3(a.G, i, j, k);
-        const W13 c = weights(a, q);
-        const double u0 = ld(&a.S.u[q]);
-        const double ru = ld(&a.bu[q]) - fma(c.w[0], u0, toff<U3>(a, c, a.S.u, i, j, k));
-        asm volatile("" ::: "memory");
-        const double v0 = ld(&a.S.v[q]);
-        const double rv = ld(&a.bv[q]) - fma(c.w[0], v0, toff<V3>(a, c, a.S.v, i, j, k));
-        asm volatile("" ::: "memory");
-        const double w0 = ld(&a.S.w[q]);
-        const double rw = ld(&a.bw[q]) - fma(c.w[0], w0, toff<W3>(a, c, a.S.w, i, j, k));
+    int i, j, k0, k1;
+    if (column(a.G, i, j, k0, k1))
+#pragma unroll 1
+        for (int k = k0; k < k1; ++k) {
+            const int q = id3(a.G, i, j, k);
+            const W13 c = weights(a, q);
+            const double ru = toff<U3>(a, fma(-c.w[0], ld(&a.S.u[q]), ld(&a.bu[q])), c, a.S.u, i, j, k);
+            asm volatile("" ::: "memory");
+            const double rv = toff<V3>(a, fma(-c.w[0], ld(&a.S.v[q]), ld(&a.bv[q])), c, a.S.v, i, j, k);
+            asm volatile("" ::: "memory");
+            const double rw = toff<W3>(a, fma(-c.w[0], ld(&a.S.w[q]), ld(&a.bw[q])), c, a.S.w, i, j, k);
 #pragma unroll
-        for (int s = 0; s < NCF; ++s) m.c[s][q] = (float)c.w[s];
-        const float di = (float)ld(&a.dinvu[q]);
-        m.dinvu[q] = di;
-        m.dinvh[q] = (float)ld(&a.dinvh[q]);
-        const float fu = (float)ru, fv = (float)rv, fw = (float)rw;
-        m.r0u[q] = fu; m.r0v[q] = fv; m.r0w[q] = fw;
-        m.du[0][q] = fu * di; m.dv[0][q] = fv * di; m.dw[0][q] = fw * di;
-        acc[0] = ru * ru; acc[1] = rv * rv; acc[2] = rw * rw;
-    }
+            for (int s = 0; s < NCF; ++s) m.c[s][q] = (float)c.w[s];
+            const float di = (float)ld(&a.dinvu[q]);
+            m.dinvu[q] = di;
+            m.dinvh[q] = (float)ld(&a.dinvh[q]);
+            const float fu = (float)ru, fv = (float)rv, fw = (float)rw;
+            m.r0u[q] = fu; m.r0v[q] = fv; m.r0w[q] = fw;
+            m.du[0][q] = fu * di; m.dv[0][q] = fv * di; m.dw[0][q] = fw * di;
+            acc[0] = fma(ru, ru, acc[0]);
+            acc[1] = fma(rv, rv, acc[1]);
+            acc[2] = fma(rw, rw, acc[2]);
+        }
     if (gsum<3>(acc, red, a.part, &sc->counters[C_MOM], tot)) {
         for (int s = 0; s < 3; ++s) sc->bn2[s] = tot[s];
         sc->done[L_MOM] = 0;
@@ -1289,19 +1310,19 @@ __global__ void k_mx_r0h(Args a, Mx m)
     if (sc->status) return;
     __shared__ double red[NT];
     double acc[1] = {0.0}, tot[1];
-    int i, j, k;
-    if (cell(a.G, i, j, k)) {
-        const int q = id3(a.G, i, j, k);
-        const W13 c = weights(a, q);
-        const double h0 = ld(&a.S.h[q]);
-        double t = fma(c.w[0], h0, toff<H3>(a, c, a.S.h, i, j, k));
-        if (a.F.nuh != a.F.mu) t = fma(a.F.mu - a.F.nuh, lap<H3>(a, a.S.h, i, j, k), t);
-        const double r0 = ld(&a.bh[q]) - t;
-        const float f = (float)r0;
-        m.r0h[q] = f;
-        m.dh[0][q] = f * ldf(&m.dinvh[q]);
-        acc[0] = r0 * r0;
-    }
+    int i, j, k0, k1;
+    if (column(a.G, i, j, k0, k1))
+#pragma unroll 1
+        for (int k = k0; k < k1; ++k) {
+            const int q = id3(a.G, i, j, k);
+            const W13 c = weights(a, q);
+            double r0 = toff<H3>(a, fma(-c.w[0], ld(&a.S.h[q]), ld(&a.bh[q])), c, a.S.h, i, j, k);
+            gea::rarely(a.F.pr_ne1, [&] { r0 = fma(a.F.nuh - a.F.mu, lap<H3>(a, a.S.h, i, j, k), r0); });
+            const float f = (float)r0;
+            m.r0h[q] = f;
+            m.dh[0][q] = f * ldf(&m.dinvh[q]);
+            acc[0] = fma(r0, r0, acc[0]);
+        }
     if (gsum<1>(acc, red, a.part, &sc->counters[C_ENTH], tot)) {
         sc->bn2[3] = tot[0];
         sc->done[L_ENTH] = 0;
@@ -1330,7 +1351,7 @@ __global__ void k_mx_enth(Args a, Mx m, const float *hi, float *ho, int second)
         const W13f c = weightsf(m, q);
         const float h0 = ldf(&hi[q]);
         float t = fmaf(c.w[0], h0, tofff<E3>(G, c, hi, i, j, k));
-        if (a.F.nuh != a.F.mu) t = fmaf((float)(a.F.mu - a.F.nuh), lapf(G, hi, i, j, k), t);
+        gea::rarely(a.F.pr_ne1, [&] { t = fmaf((float)(a.F.mu - a.F.nuh), lapf(G, hi, i, j, k), t); });
         const float r = ldf(&m.r0h[q]) - t;
         ho[q] = fmaf(r, ldf(&m.dinvh[q]), h0);
         acc[0] = r * r;
@@ -1530,6 +1551,10 @@ Geo make_geo(int nx, int ny, int nz, double lx, double ly, double lz)
     G.idx2 = 1.0 / (G.dx * G.dx); G.idy2 = 1.0 / (G.dy * G.dy); G.idz2 = 1.0 / (G.dz * G.dz);
     G.ivol = 1.0 / (G.dx * G.dy * G.dz);
     G.ax = G.dy * G.dz; G.ay = G.dx * G.dz; G.az = G.dx * G.dy;
+    G.hidx = 0.5 * G.idx; G.hidy = 0.5 * G.idy; G.hidz = 0.5 * G.idz;
+    G.tidx = 2.0 * G.idx; G.tidy = 2.0 * G.idy; G.tidz = 2.0 * G.idz;
+    G.hax = 0.5 * G.ax; G.hay = 0.5 * G.ay; G.haz = 0.5 * G.az;
+    G.s12 = G.ivol / 12.0;
     return G;
 }
 
@@ -1564,8 +1589,19 @@ __global__ void k_diag3(Geo G, Phy F, double p0, St S, const double *thbar, cons
 }
 
 dim3 grid_of(const Geo &G) { return dim3((G.nx + TX - 1) / TX, (G.ny + TY - 1) / TY, G.nz); }
-// the grid of the column kernels (kLayers cell layers per block)
-dim3 gridc_of(const Geo &G) { return dim3((G.nx + TX - 1) / TX, (G.ny + TY - 1) / TY, (G.nz + kLayers - 1) / kLayers); }
+// The grid of the column kernels: up to `most` layers per block, fewer where
+// that would leave less than about three waves of five blocks an SM (a grid of
+// 33 x 33 x 24 has 240 one-layer tiles in all). The light CG kernels walk up to
+// eight layers, the stencil kernels up to four.
+constexpr int kLayers = 8, kLayersHeavy = 4, kMinBlocks = 2400;
+dim3 columns_of(const Geo &G, int most)
+{
+    const dim3 g = grid_of(G);
+    int layers = most;
+    while (layers > 1 && (size_t)g.x * g.y * ((G.nz + layers - 1) / layers) < (size_t)kMinBlocks) layers /= 2;
+    return dim3(g.x, g.y, (G.nz + layers - 1) / layers);
+}
+dim3 gridc_of(const Geo &G) { return columns_of(G, kLayers); }
 const dim3 kBlk(TX, TY);
 size_t nblocks(const Geo &G)
 {
@@ -1590,6 +1626,9 @@ Args args_of(gea3d_ctx *c, int from)
     a.mueff = c->mueff;
     a.gzc = c->gz;
     a.gzf = c->gz + c->G.nz;
+    a.gx2 = a.gzf + c->G.nz + 1;
+    a.gy2 = a.gx2 + c->G.nz;
+    a.gz2 = a.gy2 + c->G.nz;
     a.sc = c->sc; a.part = c->part;
     a.jtol2 = c->C.jac_rtol * c->C.jac_rtol;
     a.ctol2 = c->C.cg_rtol * c->C.cg_rtol;
@@ -1784,7 +1823,7 @@ int record3(gea3d_ctx *ctx, int from, cudaStream_t s, bool graph, Trace3 *tr)
     const int nlev = (int)ctx->M.size();
     const Geo &G = ctx->G;
     const dim3 grid = grid_of(G);
-    const dim3 gridc(grid.x, grid.y, (G.nz + kLayers - 1) / kLayers);   // column kernels
+    const dim3 gridc = gridc_of(G), gridh = columns_of(G, kLayersHeavy);   // column kernels
     const int jtrips = (ctx->C.jac_maxit + 1) / 2;
     const int gr = graph ? 1 : 0;
     int fixed = 0, rc;
@@ -1793,11 +1832,11 @@ int record3(gea3d_ctx *ctx, int from, cudaStream_t s, bool graph, Trace3 *tr)
     };
     k_begin<<<1, 1, 0, s>>>(a.sc); ++fixed;
     if (ctx->mueff) { traced(tr, "g3_les", G, s, [&] { k_les<<<grid, kBlk, 0, s>>>(a); }); ++fixed; }
-    traced(tr, "g3_pred", G, s, [&] { k_pred<<<grid, kBlk, 0, s>>>(a); }); ++fixed;
+    traced(tr, "g3_pred", G, s, [&] { k_pred<<<gridh, kBlk, 0, s>>>(a); }); ++fixed;
     const Mx &m = ctx->mx;
     if (ctx->mixed) {
         // FP64 residuals, FP32 Jacobi on the increments (pairs end in du[0]), FP64 update
-        traced(tr, "g3_mx_r0mom", G, s, [&] { k_mx_r0mom<<<grid, kBlk, 0, s>>>(a, m); }); ++fixed;
+        traced(tr, "g3_mx_r0mom", G, s, [&] { k_mx_r0mom<<<gridh, kBlk, 0, s>>>(a, m); }); ++fixed;
         rc = loop(L_MOM, jtrips, [&](cudaStream_t bs, cudaGraphConditionalHandle h) {
             traced(tr, "g3_mx_mom", G, bs, [&] {
                 k_mx_mom<<<grid, kBlk, 0, bs>>>(a, m, m.du[0], m.dv[0], m.dw[0], m.du[1], m.dv[1], m.dw[1], 0);
@@ -1811,16 +1850,16 @@ int record3(gea3d_ctx *ctx, int from, cudaStream_t s, bool graph, Trace3 *tr)
         traced(tr, "g3_mx_u1", G, s, [&] { k_mx_u1<<<grid, kBlk, 0, s>>>(a, m.du[0], m.dv[0], m.dw[0]); }); ++fixed;
     } else {
         rc = loop(L_MOM, jtrips, [&](cudaStream_t bs, cudaGraphConditionalHandle h) {
-            traced(tr, "g3_mom", G, bs, [&] { k_mom<<<grid, kBlk, 0, bs>>>(a, a.ua, a.va, a.wa, a.ub, a.vb, a.wb, 0); });
-            traced(tr, "g3_mom", G, bs, [&] { k_mom<<<grid, kBlk, 0, bs>>>(a, a.ub, a.vb, a.wb, a.ua, a.va, a.wa, 1); });
+            traced(tr, "g3_mom", G, bs, [&] { k_mom<<<gridh, kBlk, 0, bs>>>(a, a.ua, a.va, a.wa, a.ub, a.vb, a.wb, 0); });
+            traced(tr, "g3_mom", G, bs, [&] { k_mom<<<gridh, kBlk, 0, bs>>>(a, a.ub, a.vb, a.wb, a.ua, a.va, a.wa, 1); });
             k_ctl<<<1, 1, 0, bs>>>(a.sc, h, gr, L_MOM, jtrips, 3);
         });
         if (rc) return rc;
     }
     traced(tr, "g3_kin", G, s, [&] { k_kin<<<grid, kBlk, 0, s>>>(a, a.ua, a.va, a.wa); }); ++fixed;
-    traced(tr, "g3_enth_rhs", G, s, [&] { k_enth_rhs<<<grid, kBlk, 0, s>>>(a, a.wa); }); ++fixed;
+    traced(tr, "g3_enth_rhs", G, s, [&] { k_enth_rhs<<<gridh, kBlk, 0, s>>>(a, a.wa); }); ++fixed;
     if (ctx->mixed) {
-        traced(tr, "g3_mx_r0h", G, s, [&] { k_mx_r0h<<<grid, kBlk, 0, s>>>(a, m); }); ++fixed;
+        traced(tr, "g3_mx_r0h", G, s, [&] { k_mx_r0h<<<gridh, kBlk, 0, s>>>(a, m); }); ++fixed;
         rc = loop(L_ENTH, jtrips, [&](cudaStream_t bs, cudaGraphConditionalHandle h) {
             traced(tr, "g3_mx_enth", G, bs, [&] { k_mx_enth<<<grid, kBlk, 0, bs>>>(a, m, m.dh[0], m.dh[1], 0); });
             traced(tr, "g3_mx_enth", G, bs, [&] { k_mx_enth<<<grid, kBlk, 0, bs>>>(a, m, m.dh[1], m.dh[0], 1); });
@@ -1830,8 +1869,8 @@ int record3(gea3d_ctx *ctx, int from, cudaStream_t s, bool graph, Trace3 *tr)
         traced(tr, "g3_mx_h1", G, s, [&] { k_mx_h1<<<grid, kBlk, 0, s>>>(a, m.dh[0]); }); ++fixed;
     } else {
         rc = loop(L_ENTH, jtrips, [&](cudaStream_t bs, cudaGraphConditionalHandle h) {
-            traced(tr, "g3_enth", G, bs, [&] { k_enth<<<grid, kBlk, 0, bs>>>(a, a.ha, a.hb, 0); });
-            traced(tr, "g3_enth", G, bs, [&] { k_enth<<<grid, kBlk, 0, bs>>>(a, a.hb, a.ha, 1); });
+            traced(tr, "g3_enth", G, bs, [&] { k_enth<<<gridh, kBlk, 0, bs>>>(a, a.ha, a.hb, 0); });
+            traced(tr, "g3_enth", G, bs, [&] { k_enth<<<gridh, kBlk, 0, bs>>>(a, a.hb, a.ha, 1); });
             k_ctl<<<1, 1, 0, bs>>>(a.sc, h, gr, L_ENTH, jtrips, 3);
         });
         if (rc) return rc;
@@ -1849,9 +1888,9 @@ int record3(gea3d_ctx *ctx, int from, cudaStream_t s, bool graph, Trace3 *tr)
         traced(tr, "g3_H", G, s, [&] { k_H<<<grid, kBlk, 0, s>>>(a, U, V, W); }); ++fixed;
         traced(tr, "g3_helm_rhs", G, s, [&] {
             if (ctx->mixed)
-                k_helm_rhs<<<grid, kBlk, 0, s>>>(a, L[0], c == 0 ? a.S.pp : a.N.pp, a.N.pp, c, m.r, m.x, m.p0);
+                k_helm_rhs<<<gridh, kBlk, 0, s>>>(a, L[0], c == 0 ? a.S.pp : a.N.pp, a.N.pp, c, m.r, m.x, m.p0);
             else
-                k_helm_rhs<<<grid, kBlk, 0, s>>>(a, L[0], c == 0 ? a.S.pp : a.N.pp, a.N.pp, c, nullptr, nullptr,
+                k_helm_rhs<<<gridh, kBlk, 0, s>>>(a, L[0], c == 0 ? a.S.pp : a.N.pp, a.N.pp, c, nullptr, nullptr,
                                                  nullptr, ctx->M[0].r);
         });
         ++fixed;
@@ -1928,6 +1967,14 @@ int gea3d_create(const gea3d_grid *grid, const gea_constants *c, gea3d_ctx **out
     {
         const double delta = cbrt(ctx->G.dx * ctx->G.dy * ctx->G.dz);
         ctx->F.les_d2 = c->cs * c->cs * delta * delta;
+        Phy &F = ctx->F;
+        const Geo &g = ctx->G;
+        F.icv = 1.0 / (c->cp - c->R);
+        F.mux = F.mu * g.idx2; F.muy = F.mu * g.idy2; F.muz = F.mu * g.idz2;
+        F.mud = 2.0 * (F.mux + F.muy + F.muz);
+        F.nud = 2.0 * F.nuh * (g.idx2 + g.idy2 + g.idz2);
+        F.les = F.les_d2 > 0.0 ? 1 : 0;
+        F.pr_ne1 = F.nuh != F.mu ? 1 : 0;
     }
     // multigrid levels: halve all three sizes while they are even and >= 8
     // and (unless mg_min_cells is given) the Laplacian-to-diagonal estimate
@@ -1976,9 +2023,14 @@ int gea3d_create(const gea3d_grid *grid, const gea_constants *c, gea3d_ctx **out
         // the heights g z of the cell centres and of the horizontal faces,
         // rounded as the expressions g ((k + 1/2) dz) and g (k dz)
         const int nz = ctx->G.nz;
-        std::vector<double> h(2 * (size_t)nz + 1);
+        std::vector<double> h(5 * (size_t)nz + 2);
         for (int k = 0; k < nz; ++k) h[k] = c->g * ((k + 0.5) * ctx->G.dz);
         for (int k = 0; k <= nz; ++k) h[nz + k] = c->g * (k * ctx->G.dz);
+        // and twice these over the spacings (Args::gx2, gy2, gz2)
+        double *t = h.data() + 2 * nz + 1;
+        for (int k = 0; k < nz; ++k) t[k] = h[k] * ctx->G.tidx;
+        for (int k = 0; k < nz; ++k) t[nz + k] = h[k] * ctx->G.tidy;
+        for (int k = 0; k <= nz; ++k) t[2 * nz + k] = h[nz + k] * ctx->G.tidz;
         ctx->gz = take(h.size());
         if (ctx->gz && cudaMemcpy(ctx->gz, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
             ok = false;
@@ -2063,7 +2115,7 @@ int gea3d_set_conservative(gea3d_ctx *ctx, const double *rho, const double *rhou
     for (int f = 0; f < 5; ++f)
         CK3(cudaMemcpyAsync(ctx->stage + f * n, src[f], n * sizeof(double), cudaMemcpyDefault, ctx->stream));
     k_derive<<<grid_of(G), kBlk, 0, ctx->stream>>>(G, ctx->F, ctx->stage, ctx->stage + n, ctx->stage + 2 * n,
-                                                   ctx->stage + 3 * n, ctx->stage + 4 * n, ctx->S[0], ctx->sc);
+                                                   ctx->stage + 3 * n, ctx->stage + 4 * n, ctx->gz, ctx->S[0], ctx->sc);
     CK3(cudaGetLastError());
     Sc h;
     CK3(cudaMemcpyAsync(&h, ctx->sc, sizeof(Sc), cudaMemcpyDeviceToHost, ctx->stream));
