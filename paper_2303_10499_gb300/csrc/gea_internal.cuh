@@ -150,7 +150,7 @@ struct Scal {
     int cg_it;                  // CG iterations of the running solve
     int corr;                   // running corrector
     int cg_iters[4];
-    double cg_relres[4];
+    double cg_r2[4], cg_b2[4];  // squared residual of each solve and what it is relative to
     int status;                 // first device-side error of the running step
     int bad_cells;              // set_state validation
     long long steps_done;
@@ -162,9 +162,10 @@ struct Scal {
     double mass, energy;        // diagnostics
     long long launches;         // kernel launches of completed and running steps
     unsigned counters[32];      // reduction arrival counters, one per kernel kind
-    // persistent step kernels: grid barrier (a monotone arrival counter,
-    // zero at the start of every launch, and the count of blocks that left
-    // the launch, each on a cache line of its own) and per-step results
+    // persistent step kernels: grid barrier (a monotone arrival counter in
+    // steps of two, its lowest bit a block's request to stop, zero at the start
+    // of every launch, and the count of blocks that left the launch, each on a
+    // cache line of its own) and per-step results
     alignas(128) unsigned bar_count;
     alignas(128) unsigned bar_exit;
     alignas(128) int u1_slot;   // 1 if u^{n+1/3} / h^{n+1} ended in the b buffers
@@ -172,6 +173,14 @@ struct Scal {
     unsigned long long press_ns; // globaltimer nanoseconds of the pressure solves, last step
     double galpha;              // step length of the learned initial guess
 };
+
+// Relative residual of corrector c's solve, formed at the end of a step only:
+// its division and square root take about 900 cycles, which at the end of every
+// CG iteration all blocks would wait for.
+__device__ __forceinline__ double cg_relres(const Scal &s, int c)
+{
+    return s.cg_b2[c] > 0.0 ? sqrt(s.cg_r2[c] / s.cg_b2[c]) : 0.0;
+}
 
 // Optional per-launch hook (profiled eager steps only; never during graph
 // capture): begin/end bracket every kernel launch on stream st.
@@ -284,28 +293,34 @@ __device__ __forceinline__ T warp_sum(T v)
 }
 
 // Block totals of NV per-thread values, valid in thread 0. The values pass
-// through shared memory (red: NV * NTHREADS doubles) and one warp adds them,
-// 8 per lane and then a shuffle tree: about 1.5 FP64 additions per value per
-// thread instead of 5 for a full-block shuffle tree (FP64 issue is the
-// scarce resource on this GPU).
+// through shared memory (red: NV * NTHREADS values) and warp j adds value j, 8 per
+// lane and then a shuffle tree: about 1.5 FP64 additions per value per thread
+// instead of 5 for a full-block shuffle tree (FP64 issue is the scarce resource
+// on this GPU). An FP64 instruction takes a warp 64 cycles of its quarter of
+// the SM whether or not it depends on the one before (measured), so a value
+// takes 12 x 64 cycles and the shuffles; one warp per value keeps them from
+// adding up (two values: 0.8 -> 0.5 us).
 template <int NV, class T = double>
 __device__ __forceinline__ void block_sum(const T (&v)[NV], T *red, T (&out)[NV])
 {
+    static_assert(32 * NV <= NTHREADS, "a warp per value");
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
 #pragma unroll
     for (int j = 0; j < NV; ++j) red[j * NTHREADS + tid] = v[j];
     __syncthreads();
-    if (tid < 32) {
+    if (tid < 32 * NV) {
+        T *p = red + (tid / 32) * NTHREADS + (tid & 31);
+        T s = p[0];
 #pragma unroll
-        for (int j = 0; j < NV; ++j) {
-            T s = red[j * NTHREADS + tid];
-#pragma unroll
-            for (int q = 1; q < NTHREADS / 32; ++q) s += red[j * NTHREADS + tid + 32 * q];
-            s = warp_sum(s);
-            if (tid == 0) out[j] = s;
-        }
+        for (int q = 1; q < NTHREADS / 32; ++q) s += p[32 * q];
+        s = warp_sum(s);
+        if ((tid & 31) == 0) p[0] = s;
     }
     __syncthreads();
+    if (tid == 0) {
+#pragma unroll
+        for (int j = 0; j < NV; ++j) out[j] = red[j * NTHREADS];
+    }
 }
 
 // The partials buffer of a context: kGcntDoubles doubles of group counters

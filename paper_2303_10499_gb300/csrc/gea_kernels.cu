@@ -353,7 +353,7 @@ __global__ void k_loop_gate(Scal *sc, cudaGraphConditionalHandle h, int which)
 __global__ void k_step_begin(Scal *sc)
 {
     sc->u1_slot = sc->h1_slot = 0;
-    for (int c = 0; c < 4; ++c) { sc->cg_iters[c] = 0; sc->cg_relres[c] = 0.0; }
+    for (int c = 0; c < 4; ++c) { sc->cg_iters[c] = 0; sc->cg_b2[c] = 0.0; }
     sc->sweeps[0] = sc->sweeps[1] = 0;
 }
 
@@ -369,7 +369,7 @@ __global__ void k_step_end(Scal *sc, int fixed_launches)
     sc->last_sweeps[1] = sc->sweeps[1];
     for (int c = 0; c < 4; ++c) {
         sc->last_cg_iters[c] = sc->cg_iters[c];
-        sc->last_cg_relres[c] = sc->cg_relres[c];
+        sc->last_cg_relres[c] = cg_relres(*sc, c);
     }
     sc->last_status = 0;
 }

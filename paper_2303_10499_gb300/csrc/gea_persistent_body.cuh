@@ -29,6 +29,8 @@ namespace {
 // values per thread a grid reduction may carry: the block-sum scratch after
 // the tile area holds kRedVals x NTHREADS doubles
 constexpr int kRedVals = 4;
+// blocks up to which one warp per value adds a grid reduction's partials
+constexpr int kDirectPartials = 128;
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
 {
@@ -110,7 +112,7 @@ __device__ __forceinline__ void load_ctl(const Scal *gs)
 }
 
 // Grid barrier on a monotone arrival counter: barrier k of a launch is
-// passed once the counter reaches k x (blocks), so the last block to arrive
+// passed once the counter reaches 2 k x (blocks), so the last block to arrive
 // releases the others by its arrival alone. A block arrives with one
 // acquire-release add (thread 0, after the block barrier: it publishes the
 // block's writes of the phase) and polls the counter with acquire loads
@@ -118,28 +120,33 @@ __device__ __forceinline__ void load_ctl(const Scal *gs)
 // every block's writes). Every data read across blocks goes through L2
 // (ld.global.cg), ordered after the acquire by the block barrier. The count
 // wraps modulo 2^32; the comparison is of the signed difference.
+// A block that gives up sets the context's status and the counter's lowest
+// bit; the others see the bit in the word they poll anyway, at this barrier or
+// the next (a read of the status word after every barrier cost 0.2 us).
 __device__ __forceinline__ void gbar(const Grp &g)
 {
     Scal *gs = g.gs;
     __syncthreads();
     if (tid_of() == 0) {
         const unsigned k = *g.gen + 1u;
-        const unsigned target = k * (unsigned)g.nb;
+        const unsigned target = 2u * k * (unsigned)g.nb;
         unsigned long long *tr =
             (g.trace && k <= (unsigned)g.trace_bars) ? g.trace + 2 * ((size_t)k * g.nb + g.rank) : nullptr;
         if (tr) tr[0] = globaltimer();
-        unsigned c = atom_add_acq_rel(&gs->bar_count, 1u) + 1u;
+        unsigned c = atom_add_acq_rel(&gs->bar_count, 2u) + 2u;
         unsigned long long spins = 0;
-        while ((int)(c - target) < 0) {
+        while ((int)((c & ~1u) - target) < 0 && !(c & 1u)) {
             if (spins++ >= g.spin_limit) {
                 atomicCAS(&gs->status, 0, GEA_ERR_TIMEOUT);
+                atomicOr(&gs->bar_count, 1u);
+                c |= 1u;
                 break;
             }
             c = ld_acquire(&gs->bar_count);
         }
         if (tr) tr[1] = globaltimer();
         *g.gen = k;
-        s_stop = rdi(&gs->status) != 0 || s_ctl.status != 0;
+        s_stop = (c & 1u) != 0 || s_ctl.status != 0;
     }
     __syncthreads();
 }
@@ -178,13 +185,37 @@ __device__ __forceinline__ void rbar(const Grp &g, const T (&v)[NV], double *red
         for (int j = 0; j < NV; ++j) pb[(size_t)j * nb + g.rank] = (double)bt[j];
     }
     gbar(g);
-    double s[NV], tot[NV];
+    double tot[NV];
+    if (nb <= kDirectPartials) {
+        // few blocks: warp j adds the partials of value j at once, without the
+        // pass through shared memory (four per lane and the shuffle tree)
+        const int lane = tid & 31;
+        for (int j = tid / 32; j < NV; j += NTHREADS / 32) {
+            double s = 0.0;
+            for (int b = lane; b < nb; b += 32) {
+                const double v = __ldcg(&pb[(size_t)j * nb + b]);
+                s = b == lane ? v : s + v;
+            }
+            s = warp_sum(s);
+            if (lane == 0) red[j] = s;
+        }
+        if (NV > 1) __syncthreads();
+        if (tid == 0) {
 #pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        s[j] = 0.0;
-        for (int b = tid; b < nb; b += NTHREADS) s[j] += __ldcg(&pb[(size_t)j * nb + b]);
+            for (int j = 0; j < NV; ++j) tot[j] = red[j];
+        }
+    } else {
+        double s[NV];
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+            s[j] = 0.0;
+            for (int b = tid; b < nb; b += NTHREADS) {
+                const double v = __ldcg(&pb[(size_t)j * nb + b]);
+                s[j] = b == tid ? v : s[j] + v;
+            }
+        }
+        block_sum<NV>(s, red, tot);
     }
-    block_sum<NV>(s, red, tot);
     if (tid == 0) {
         fin(tot);
         if (s_ctl.status) {
@@ -226,7 +257,7 @@ __device__ __forceinline__ void end_step(const Grp &g)
         c.last_sweeps[1] = c.sweeps[1];
         for (int k = 0; k < 4; ++k) {
             c.last_cg_iters[k] = c.cg_iters[k];
-            c.last_cg_relres[k] = c.cg_relres[k];
+            if (g.rank == 0) c.last_cg_relres[k] = cg_relres(c, k);
         }
         c.last_status = 0;
         if (g.rank == 0) {
@@ -356,7 +387,7 @@ __device__ bool run_step(const PersistArgs &P, const StepArgs &a, const Grp &g, 
         rbar<4>(g, acc, red, a.partials, [&](const double (&t)[4]) {
             const double tb[2] = {t[0], t[1]}, tr[2] = {t[2], t[3]};
             fin_pred(sc, tb);
-            for (int c = 0; c < 4; ++c) { sc->cg_iters[c] = 0; sc->cg_relres[c] = 0.0; }
+            for (int c = 0; c < 4; ++c) { sc->cg_iters[c] = 0; sc->cg_b2[c] = 0.0; }
             sc->sweeps[1] = 0;
             sc->press_ns = 0ull;
             fin_mom(sc, tr, a.jac_rtol2);
@@ -481,7 +512,7 @@ __device__ bool run_step_mixed(const PersistArgs &P, const MixedPersist &X, cons
         for_tiles(g, G, [&](int bx, int bz) { ph_pred_t<true>(a, m, sm, bx, bz, acc); });
         rbar<2>(g, acc, red, a.partials, [&](const double (&t)[2]) {
             fin_pred(sc, t);
-            for (int c = 0; c < 4; ++c) { sc->cg_iters[c] = 0; sc->cg_relres[c] = 0.0; }
+            for (int c = 0; c < 4; ++c) { sc->cg_iters[c] = 0; sc->cg_b2[c] = 0.0; }
             sc->sweeps[1] = 0;
             sc->press_ns = 0ull;
         });

@@ -1438,7 +1438,8 @@ __device__ __forceinline__ void fin_helm(Scal *sc, const double (&t)[2], double 
     sc->beta = 0.0;
     sc->done[LOOP_CG] = t[1] <= tol2 * t[0];
     sc->cg_iters[corr] = 0;
-    sc->cg_relres[corr] = t[0] > 0.0 ? sqrt(t[1] / t[0]) : 0.0;
+    sc->cg_r2[corr] = t[1];
+    sc->cg_b2[corr] = t[0];
     if (!isfinite(t[0]) || !isfinite(t[1])) sc->status = 5;
 }
 
@@ -1456,7 +1457,7 @@ __device__ __forceinline__ void fin_helm_mixed(Scal *sc, const double (&t)[2], d
     sc->beta = 0.0;
     sc->done[LOOP_CG] = t[1] <= tol2_fp64 * t[0];
     sc->cg_iters[corr] = 0;
-    sc->cg_relres[corr] = 1.0;
+    sc->cg_r2[corr] = sc->cg_b2[corr] = t[1] > 0.0 ? t[1] : 1.0;
     if (!isfinite(t[0]) || !isfinite(t[1])) sc->status = GEA_ERR_NONFINITE;
 }
 
@@ -1480,7 +1481,8 @@ __device__ __forceinline__ void fin_update(Scal *sc, const double (&t)[1], doubl
     sc->r2 = t[0];
     const int c = sc->corr;
     sc->cg_iters[c] = it;
-    sc->cg_relres[c] = sc->b2 > 0.0 ? sqrt(t[0] / sc->b2) : 0.0;
+    sc->cg_r2[c] = t[0];
+    sc->cg_b2[c] = sc->b2;
     if (!isfinite(t[0])) sc->status = 5;
     else if (t[0] <= tol2 * sc->b2) sc->done[LOOP_CG] = 1;
 }
@@ -1495,7 +1497,8 @@ __device__ __forceinline__ void fin_guess_dots(Scal *sc, const double (&t)[2])
 __device__ __forceinline__ void fin_guess_apply(Scal *sc, const double (&t)[1], double tol2)
 {
     sc->r2 = t[0];
-    sc->cg_relres[sc->corr] = sc->b2 > 0.0 ? sqrt(t[0] / sc->b2) : 0.0;
+    sc->cg_r2[sc->corr] = t[0];
+    sc->cg_b2[sc->corr] = sc->b2;
     if (!isfinite(t[0])) sc->status = GEA_ERR_NONFINITE;
     else if (t[0] <= tol2 * sc->b2) sc->done[LOOP_CG] = 1;
 }
