@@ -620,14 +620,38 @@ __device__ bool run_step_mixed(const PersistArgs &P, const MixedPersist &X, cons
 // with five levels: 2070 -> 1844 us a step, 200 x 200 (175 blocks) 1100 -> 1076.
 __device__ __forceinline__ int single_rank() { return (int)(gridDim.x - 1 - blockIdx.x); }
 
-__global__ void __launch_bounds__(NTHREADS, 3) k_persistent(PersistArgs P)
+// The argument block `src` copied to shared memory (whole words).
+template <class T>
+__device__ __forceinline__ const T &args_to_shared(void *dst, const T &src)
+{
+    static_assert(sizeof(T) % 4 == 0, "copied by words");
+    const uint32_t *s = reinterpret_cast<const uint32_t *>(&src);
+    uint32_t *d = reinterpret_cast<uint32_t *>(dst);
+    for (int w = tid_of(); w < (int)(sizeof(T) / 4); w += NTHREADS) d[w] = s[w];
+    return *reinterpret_cast<const T *>(dst);
+}
+
+// The step kernels read their arguments (pointers and sizes of the state, the
+// work arrays and every level, several kB) from a copy in shared memory, as an
+// ensemble's blocks do. Kernel parameters indexed by slot or level at run time
+// come through the small constant cache, which the phases in turn overflow. Per
+// pass: 640 x 320 2005 -> 1938 us, 160 x 80 267 -> 259, the multi-level grids 1 %.
+constexpr size_t kArgsFp64 = sizeof(PersistArgs);
+constexpr size_t kArgsMixed = sizeof(PersistArgs) + sizeof(MixedPersist);
+constexpr size_t kPersistSmem =
+    (size_t)(kTileSmem + kRedVals * NTHREADS) * sizeof(double) + (kArgsFp64 + 15) / 16 * 16;
+constexpr size_t kPersistSmemMixed =
+    (size_t)(kTileSmem + kRedVals * NTHREADS) * sizeof(double) + (kArgsMixed + 15) / 16 * 16;
+
+__global__ void __launch_bounds__(NTHREADS, 3) k_persistent(const __grid_constant__ PersistArgs Pk)
 {
     extern __shared__ double dsm[];
     double *sm = dsm;
     double *red = dsm + kTileSmem;
+    const PersistArgs &P = args_to_shared(red + kRedVals * NTHREADS, Pk);
     // an error status is sticky until the next set_state, which clears it
     __shared__ unsigned gen;
-    Scal *gs = P.a[0].sc;
+    Scal *gs = Pk.a[0].sc;
     if (tid_of() == 0) {
         s_stop = rdi(&gs->status) != 0;
         gen = 0u;
@@ -647,16 +671,18 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_persistent(PersistArgs P)
     leave(g);
 }
 
-constexpr size_t kPersistSmem = (size_t)(kTileSmem + kRedVals * NTHREADS) * sizeof(double);
-
 // The mixed-precision step as one cooperative launch (small grids).
-__global__ void __launch_bounds__(NTHREADS, 3) k_persistent_mixed(PersistArgs P, MixedPersist X)
+__global__ void __launch_bounds__(NTHREADS, 3)
+    k_persistent_mixed(const __grid_constant__ PersistArgs Pk, const __grid_constant__ MixedPersist Xk)
 {
     extern __shared__ double dsm[];
     double *sm = dsm;
     double *red = dsm + kTileSmem;
+    char *args = reinterpret_cast<char *>(red + kRedVals * NTHREADS);
+    const PersistArgs &P = args_to_shared(args, Pk);
+    const MixedPersist &X = args_to_shared(args + sizeof(PersistArgs), Xk);
     __shared__ unsigned gen;
-    Scal *gs = P.a[0].sc;
+    Scal *gs = Pk.a[0].sc;
     if (tid_of() == 0) {
         s_stop = rdi(&gs->status) != 0;
         gen = 0u;
@@ -738,17 +764,11 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_ensemble(const char *Pm, int st
     }
 }
 
-// bytes of one member's argument block and the ensemble kernels' shared memory
-constexpr size_t kArgsFp64 = sizeof(PersistArgs);
-constexpr size_t kArgsMixed = sizeof(PersistArgs) + sizeof(MixedPersist);
-constexpr size_t kEnsembleSmem = kPersistSmem + (kArgsFp64 + 15) / 16 * 16;
-constexpr size_t kEnsembleSmemMixed = kPersistSmem + (kArgsMixed + 15) / 16 * 16;
-
 int ensemble_max_blocks(int mixed)
 {
     int dev = 0, sms = 0, per_sm = 0;
     const void *k = mixed ? (const void *)k_ensemble<true> : (const void *)k_ensemble<false>;
-    const size_t smem = mixed ? kEnsembleSmemMixed : kEnsembleSmem;
+    const size_t smem = mixed ? kPersistSmemMixed : kPersistSmem;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
@@ -763,7 +783,7 @@ cudaError_t launch_ensemble(const void *Pm, int mixed, const int *groups, int ng
     void *args[] = {&P, &stride, &groups, &ngroups};
     const void *k = mixed ? (const void *)k_ensemble<true> : (const void *)k_ensemble<false>;
     return cudaLaunchCooperativeKernel(k, dim3(blocks), dim3(BX, BZ), args,
-                                       mixed ? kEnsembleSmemMixed : kEnsembleSmem, st);
+                                       mixed ? kPersistSmemMixed : kPersistSmem, st);
 }
 
 int persistent_max_blocks()
@@ -808,9 +828,9 @@ int persistent_mixed_max_blocks()
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     if (cudaFuncSetAttribute(k_persistent_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kPersistSmem) != cudaSuccess)
+                             (int)kPersistSmemMixed) != cudaSuccess)
         return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persistent_mixed, NTHREADS, kPersistSmem) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persistent_mixed, NTHREADS, kPersistSmemMixed) !=
         cudaSuccess)
         return 0;
     return per_sm * sms;
@@ -841,7 +861,7 @@ cudaError_t launch_persistent_mixed(const StepArgs a[2], const Level &L0, const 
     X.nlev = nlev;
     void *args[] = {&P, &X};
     return cudaLaunchCooperativeKernel((const void *)k_persistent_mixed, dim3(blocks), dim3(BX, BZ), args,
-                                       kPersistSmem, st);
+                                       kPersistSmemMixed, st);
 }
 
 }  // namespace
