@@ -720,10 +720,13 @@ KERNEL_MODEL_3D = {
     "g3_mx_r0h": (16.5, 31, "f64"),
     "g3_mx_enth": (8.5, 31, "f32"),
     "g3_mx_h1": (2.5, 1, "f64"),
-    "g3_mx_pupd": (1.5, 2, "f32"),
-    "g3_mx_spmv": (3, 15, "f32"),
-    "g3_mx_update": (3, 6, "f32"),
-    "g3_mx_papply": (2.5, 1, "f64"),
+    "g3_mx_rb_start": (2.8, 7, "f32"),
+    "g3_mx_pupd": (0.75, 1, "f32"),
+    "g3_mx_spmv_red": (2.25, 6.5, "f32"),
+    "g3_mx_spmv_black": (2.5, 8, "f32"),
+    "g3_mx_update": (1.9, 3.5, "f32"),
+    "g3_mx_mg_up": (2.6, 8, "f32"),
+    "g3_mx_solution": (4.25, 8, "f32"),
     "g3_pred": (31, 102, "f64"),
     "g3_mom": (23, 93, "f64"),
     "g3_kin": (4, 6, "f64"),
@@ -731,17 +734,20 @@ KERNEL_MODEL_3D = {
     "g3_enth": (17, 31, "f64"),
     "g3_eos": (9, 7, "f64"),
     "g3_faces": (8, 15, "f64"),
-    "g3_diag": (6, 7, "f64"),
+    "g3_diag": (7, 13, "f64"),
     "g3_coarsen": (38, 32, "f64"),
     "g3_H": (24, 87, "f64"),
-    "g3_helm_rhs": (18, 70, "f64"),
-    "g3_mg_down": (49, 137, "f64"),
-    "g3_mg_coarse": (7, 17, "f64"),
-    "g3_mg_up": (7.125, 20, "f64"),
-    "g3_mg_single": (6, 20, "f64"),
-    "g3_pupd": (3, 2, "f64"),
-    "g3_spmv": (6, 15, "f64"),
-    "g3_update": (6, 6, "f64"),
+    "g3_helm_rhs": (16.5, 71, "f64"),
+    "g3_rb_start": (5.5, 7, "f64"),
+    "g3_mg_down": (14.5, 49, "f32"),
+    "g3_mg_black": (2.8, 14, "f32"),
+    "g3_mg_red": (2.5, 7, "f32"),
+    "g3_mg_up": (2.8, 8, "f32"),
+    "g3_pupd": (1.25, 1, "f64"),
+    "g3_spmv_red": (4.5, 6.5, "f64"),
+    "g3_spmv_black": (5, 8, "f64"),
+    "g3_update": (3.5, 3.5, "f64"),
+    "g3_solution": (6.5, 8, "f64"),
     "g3_correct": (20, 61, "f64"),
 }
 

@@ -8,10 +8,10 @@
 // scalars even, h with dh/dz = -g). The transport operator
 // T(X) = (rho1/dt) X + C(X) - nu L(X) (fourth-order face values, 13-point
 // cross stencil) is evaluated from the face fluxes in every sweep. The
-// pressure equation is solved by CG preconditioned with a Galerkin V(1,1)
-// cycle (piecewise-constant transfer over 2 x 2 x 2 cells, damped Jacobi
-// smoothing), the loops as conditional WHILE nodes of a CUDA graph ended by
-// a one-thread control kernel. Reductions are deterministic (block partials
+// pressure equation is solved by CG on the black half of a red-black colouring,
+// preconditioned with a V-cycle (piecewise-constant transfer over 2 x 2 x 2
+// cells, red-black smoothing), the loops as conditional WHILE nodes of a CUDA
+// graph ended by a one-thread control kernel. Reductions are deterministic (block partials
 // summed in a fixed order by the last block).
 //
 // Layout: every array (cells and faces) is indexed (k (ny+1) + j) P + i with
@@ -25,6 +25,7 @@
 #include <string.h>
 
 #include <climits>
+#include <type_traits>
 #include <vector>
 
 namespace g3 {
@@ -32,8 +33,6 @@ namespace g3 {
 constexpr int TX = 32, TY = 8, NT = TX * TY;
 static_assert(NT == gea::NTHREADS, "block_sum reduces NTHREADS values");
 constexpr int kMaxLev = 12;
-constexpr int kCoarseSweeps = 2;
-constexpr double kOmega = 0.8;
 constexpr double kCoarsestRatio = 1.0;
 constexpr double kRefT = 300.0;
 enum { E3 = 0, U3 = 1, V3 = 2, W3 = 3, H3 = 4 };
@@ -58,7 +57,7 @@ __host__ __device__ inline int id3(const Geo &G, int i, int j, int k)
 }
 
 struct Phy {
-    double R, cp, g, mu, nuh, dt, idt, omega;
+    double R, cp, g, mu, nuh, dt, idt;
     double icp, icv; // 1/cp, 1/cv
     double mux, muy, muz, mud, nud;   // mu/dx^2, ..., 2 mu (1/dx^2 + 1/dy^2 + 1/dz^2), the same with mu/Pr
     int les, pr_ne1; // les_d2 > 0; mu/Pr != mu
@@ -69,19 +68,37 @@ struct St {
     double *rho, *u, *v, *w, *T, *h, *p, *pp, *pold, *phix, *phiy, *phiz;
 };
 
-// Helmholtz level: (A x)_i = c_i x_i + sum_f a_f (x_i - x_N), d = c + sum a,
-// a on the x-, y- and z-faces (zero on walls).
+// The FP64 Helmholtz operator: (A x)_i = c_i x_i + sum_f a_f (x_i - x_N),
+// d = c + sum a, wd = 1/d, a on the x-, y- and z-faces (zero on walls); r the
+// residual of a solve's start.
 struct Lev {
     Geo G;
-    double *c, *d, *ax, *ay, *az, *r, *e2;   // e2: the preconditioned residual z
+    double *c, *d, *ax, *ay, *az, *r, *wd;
 };
 
 // FP32 level of the multigrid preconditioner (on the finest level the twin
-// of the FP64 operator, r the FP32 copy of the FP64 step's CG residual and
-// e2 unused): w = omega/d, e and e2 the smoothed corrections.
+// of the FP64 operator; r, e and e2 unused there): w = 1/d, r the restricted
+// residual, e the smoothed correction of the down half, e2 the correction.
 struct Lev32 {
     Geo G;
     float *c, *d, *ax, *ay, *az, *w, *r, *e, *e2;
+};
+
+// The operator of a solve in its own precision.
+template <class R>
+struct Op {
+    Geo G;
+    const R *d, *ax, *ay, *az, *wd;
+};
+
+// The vectors of a solve: one value per pair of cells of a row, of its black
+// cell or (w) of its red one. p the direction, w the red part of A p over d
+// with the sign turned, q = S p, rb the residual, xb the solution, ef = rb / d
+// and z the preconditioned residual (z = ef on a hierarchy of one level).
+template <class R>
+struct Rb {
+    R *p, *w, *q, *rb, *xb;
+    float *ef, *z;
 };
 
 // The transport operator T(X) = (rho1/dt) X + C(X) - mu L(X) of the step as
@@ -113,7 +130,7 @@ struct Args {
     Phy F;
     St S, N;
     double *rho1, *dinvu, *dinvh, *bu, *bv, *bw, *ua, *va, *wa, *ub, *vb, *wb, *bh, *ha, *hb;
-    double *rho2, *psi, *Dx, *Dy, *Dz, *Hx, *Hy, *Hz, *b, *p0, *p1, *q;
+    double *rho2, *psi, *Dx, *Dy, *Dz, *Hx, *Hy, *Hz;
     double *dtr1;   // dt / rho1
     double *kin;    // K1 = |u1|^2 / 2
     double *mueff;  // mu + mu_t (LES only)
@@ -126,6 +143,7 @@ struct Args {
 };
 
 __device__ __forceinline__ double ld(const double *p) { return __ldg(p); }
+__device__ __forceinline__ float ld(const float *p) { return __ldg(p); }
 __device__ __forceinline__ float ldf(const float *p) { return __ldg(p); }
 
 // Cell (i,j,k) of the thread, or false beyond the box.
@@ -678,7 +696,9 @@ __global__ void k_faces(Args a, Lev L, Lev32 m)
     if (k == G.nz - 1) { a.Dz[q + sz] = 0.0; L.az[q + sz] = 0.0; m.az[q + sz] = 0.0f; }
 }
 
-// Diagonal d = c + the six face coefficients, and the Jacobi weight omega/d.
+// Diagonal d = c + the six face coefficients, and 1/d (in FP64 where the solve
+// is: RECIP).
+template <bool RECIP>
 __global__ void k_diag(Lev L, Lev32 m, Sc *sc)
 {
     if (sc->status) return;
@@ -689,8 +709,9 @@ __global__ void k_diag(Lev L, Lev32 m, Sc *sc)
     const double d = ld(&L.c[q]) + (ld(&L.ax[q]) + ld(&L.ax[q + 1])) + (ld(&L.ay[q]) + ld(&L.ay[q + sy])) +
                      (ld(&L.az[q]) + ld(&L.az[q + sz]));
     L.d[q] = d;
+    if (RECIP) L.wd[q] = gea::recip(d);
     m.d[q] = (float)d;
-    m.w[q] = (float)kOmega / (float)d;   // FP32 smoother weight: an FP32 division
+    m.w[q] = 1.0f / (float)d;
 }
 
 }  // namespace g3
@@ -715,21 +736,73 @@ __global__ void k_H(Args a, const double *U, const double *V, const double *W)
     a.Hz[q] = toff<W3>(a, fma(-c0, ld(&W[q]), r * ld(&a.S.w[q])), c, W, i, j, k);
 }
 
-// A x at cell (i,j,k) of level L for x given cellwise by xf(q, i, j, k) (interior
-// neighbours only; wall faces have zero coefficients).
-template <class XF>
-__device__ __forceinline__ double helm(const Lev &L, XF xf, int i, int j, int k)
+// ---- the pressure solve: red-black multigrid CG ----
+//
+// Cells are coloured by the parity of i + j + k (even: black). A couples the
+// two colours only, so the red unknowns follow from the black ones and CG runs
+// on the black half with S = A_bb - A_br A_rr^-1 A_rb: half the vector traffic,
+// as many coefficient reads as A, and fewer iterations with the red-black
+// V-cycle than with damped Jacobi on all cells. One FP64 step of
+// 512 x 512 x 256 (two levels): 11 + 5 -> 10 + 5 iterations of 2.9 -> 1.95 ms,
+// 139 -> 117 ms; the mixed step of 192 x 192 x 96 (one level): 4 + 4 -> 3 + 3
+// iterations, 5.8 -> 5.1 ms. The products are at the FP64 rate (7.5 instructions
+// a cell, 0.97 ms together), the vector steps and the cycle at memory's.
+//
+// The vectors hold one value per pair of cells (2 m, 2 m + 1) of a row, at
+// (k (ny+1) + j) P/2 + m. With s = (j + k) & 1 the pair's black cell is 2 m + s,
+// its red one 2 m + 1 - s; the black cell's red neighbours are those of the
+// pairs m - 1 + s (west), m + s (east) and m of the rows beside, above and
+// below, the red cell's black neighbours those of m - s, m + 1 - s and m: all
+// reads are contiguous.
+
+// Pair m of a row (j, k) and its layer range, as column().
+__device__ __forceinline__ bool pair_column(const Geo &G, int &m, int &j, int &k0, int &k1)
 {
-    const Geo &G = L.G;
-    const int q = id3(G, i, j, k), sy = G.P, sz = G.P * (G.ny + 1);
-    double t = ld(&L.d[q]) * xf(q, i, j, k);
-    if (i > 0) t -= ld(&L.ax[q]) * xf(q - 1, i - 1, j, k);
-    if (i + 1 < G.nx) t -= ld(&L.ax[q + 1]) * xf(q + 1, i + 1, j, k);
-    if (j > 0) t -= ld(&L.ay[q]) * xf(q - sy, i, j - 1, k);
-    if (j + 1 < G.ny) t -= ld(&L.ay[q + sy]) * xf(q + sy, i, j + 1, k);
-    if (k > 0) t -= ld(&L.az[q]) * xf(q - sz, i, j, k - 1);
-    if (k + 1 < G.nz) t -= ld(&L.az[q + sz]) * xf(q + sz, i, j, k + 1);
-    return t;
+    const int layers = (G.nz + gridDim.z - 1) / gridDim.z;
+    m = blockIdx.x * TX + threadIdx.x;
+    j = blockIdx.y * TY + threadIdx.y;
+    k0 = blockIdx.z * layers;
+    k1 = min(G.nz, k0 + layers);
+    return 2 * m < G.nx && j < G.ny;
+}
+
+__device__ __forceinline__ int pair_id(const Geo &G, int m, int j, int k)
+{
+    return (k * (G.ny + 1) + j) * (G.P / 2) + m;
+}
+
+// Indices of the six neighbours of cell i of pair index c (RED: the pair's
+// red cell). A neighbour beyond a wall is replaced by the opposite one: its
+// coefficient is zero and the opposite cell always exists.
+template <bool RED>
+__device__ __forceinline__ Nb pair_neighbours(const Geo &G, int c, int i, int j, int k)
+{
+    const int s = (j + k) & 1, cw = c + (RED ? -s : s - 1), ce = cw + 1;
+    const int cy = G.P / 2, cz = cy * (G.ny + 1);
+    return Nb{i > 0 ? cw : ce,          i + 1 < G.nx ? ce : cw,     j > 0 ? c - cy : c + cy,
+              j + 1 < G.ny ? c + cy : c - cy, k > 0 ? c - cz : c + cz, k + 1 < G.nz ? c + cz : c - cz};
+}
+
+// The same on a field of cells.
+__device__ __forceinline__ Nb other_colour(const Geo &G, int q, int i, int j, int k)
+{
+    const int sy = G.P, sz = G.P * (G.ny + 1);
+    return Nb{i > 0 ? q - 1 : q + 1,          i + 1 < G.nx ? q + 1 : q - 1,  j > 0 ? q - sy : q + sy,
+              j + 1 < G.ny ? q + sy : q - sy, k > 0 ? q - sz : q + sz, k + 1 < G.nz ? q + sz : q - sz};
+}
+
+// t + the six face coefficients of cell q times x at its neighbours.
+template <class R, class XF>
+__device__ __forceinline__ R add_faces(R t, const Geo &G, const R *ax, const R *ay, const R *az, int q, const Nb &n,
+                                       XF x)
+{
+    const int sy = G.P, sz = G.P * (G.ny + 1);
+    t = fma(ld(&ax[q]), x(n.w), t);
+    t = fma(ld(&ax[q + 1]), x(n.e), t);
+    t = fma(ld(&ay[q]), x(n.s), t);
+    t = fma(ld(&ay[q + sy]), x(n.n), t);
+    t = fma(ld(&az[q]), x(n.b), t);
+    return fma(ld(&az[q + sz]), x(n.t), t);
 }
 
 __device__ __forceinline__ void fin_helm(Sc *sc, const double (&t)[2], double tol2, int corr)
@@ -766,11 +839,10 @@ __device__ __forceinline__ void fin_helm_mixed(Sc *sc, const double (&t)[2], dou
 }
 
 // b_i = (rho^n_i + psi_i rho2_i g z_i)/dt - sum_f D_f/Delta_f [H_f . n + g z_f (rho2_N - rho2_i)/Delta_f],
-// r = b - A x with x = xin (copied to xout), p0 = 0; acc += (b^2, r^2).
-// Mixed step (mr given): r0 rounded to FP32 into mr, and a zero FP32
-// increment mx and first direction mp0.
-__global__ void k_helm_rhs(Args a, Lev L, const double *xin, double *xout, int corr, float *mr = nullptr,
-                           float *mx = nullptr, float *mp0 = nullptr, float *rf = nullptr)
+// r = b - A x with x = xin, and r/d on the red cells into w; acc += (b^2, r^2).
+// Mixed step (R = float): r rounded to FP32.
+template <class R>
+__global__ void k_helm_rhs(Args a, Lev L, const double *xin, int corr, R *rout, const R *wd, R *w)
 {
     if (a.sc->status) return;
     __shared__ double red[2 * NT];
@@ -803,54 +875,30 @@ __global__ void k_helm_rhs(Args a, Lev L, const double *xin, double *xout, int c
             r = fma(ld(&L.ay[q + sy]), ld(&xin[nb.n]), r);
             r = fma(ld(&L.az[q]), ld(&xin[nb.b]), r);
             r = fma(ld(&L.az[q + sz]), ld(&xin[nb.t]), r);
-            a.b[q] = b;
-            L.r[q] = r;
-            xout[q] = ld(&xin[q]);
-            a.p0[q] = 0.0;
-            if (mr) {
-                mr[q] = (float)r;
-                mx[q] = 0.0f;
-                mp0[q] = 0.0f;
-            }
-            if (rf) rf[q] = (float)r;
+            rout[q] = (R)r;
+            if ((i + j + k) & 1) w[pair_id(G, i >> 1, j, k)] = ld(&wd[q]) * (R)r;
             acc[0] = fma(b, b, acc[0]);
             acc[1] = fma(r, r, acc[1]);
         }
     if (gsum<2>(acc, red, a.part, &a.sc->counters[C_HELM], tot)) {
-        if (mr) fin_helm_mixed(a.sc, tot, a.ctol2, corr);
+        if (sizeof(R) == sizeof(float)) fin_helm_mixed(a.sc, tot, a.ctol2, corr);
         else fin_helm(a.sc, tot, a.ctol2, corr);
     }
 }
 
-// ---- multigrid V(1,1) cycle in FP32 (the preconditioner of the FP64 CG) ----
+// ---- red-black V-cycle in FP32 (the preconditioner of the CG) ----
 //
 // The preconditioner only shapes the search directions: the CG residual and
-// its stopping test stay FP64, so the converged pressure is that of the FP64
-// system. Every level's operator, weights and vectors are FP32 twins (Lev32);
-// the finest level reads the FP64 residual and writes z in FP64.
+// its stopping test keep the solve's precision, so the converged pressure is
+// that of the solve's system. On the black half of the finest level the cycle
+// starts with e = rb / d on black (the red residual is zero), restricts what
+// that leaves on red, and ends with one black relaxation.
 
-template <class XF>
-__device__ __forceinline__ float helm32(const Lev32 &L, XF xf, int i, int j, int k)
-{
-    const Geo &G = L.G;
-    const int q = id3(G, i, j, k), sy = G.P, sz = G.P * (G.ny + 1);
-    float t = ldf(&L.d[q]) * xf(q, i, j, k);
-    if (i > 0) t -= ldf(&L.ax[q]) * xf(q - 1, i - 1, j, k);
-    if (i + 1 < G.nx) t -= ldf(&L.ax[q + 1]) * xf(q + 1, i + 1, j, k);
-    if (j > 0) t -= ldf(&L.ay[q]) * xf(q - sy, i, j - 1, k);
-    if (j + 1 < G.ny) t -= ldf(&L.ay[q + sy]) * xf(q + sy, i, j + 1, k);
-    if (k > 0) t -= ldf(&L.az[q]) * xf(q - sz, i, j, k - 1);
-    if (k + 1 < G.nz) t -= ldf(&L.az[q + sz]) * xf(q + sz, i, j, k + 1);
-    return t;
-}
-
-__device__ __forceinline__ float tof(double v) { return (float)v; }
-__device__ __forceinline__ float tof(float v) { return v; }
-
-// Galerkin coarsening (restriction = mean over the 8 children, piecewise-
-// constant prolongation): c_C = mean of the children's c, a coarse face =
-// (1/8) sum of its 4 fine faces, d_C = c_C + sum of its faces. One thread
-// per coarse cell; sums in FP64, stored FP32.
+// Coarse level: c_C = mean of the 8 children's c, a coarse face = (1/16) sum
+// of its 4 fine faces, d_C = c_C + sum of its faces. Piecewise-constant
+// transfer with the Galerkin value 1/8 makes the coarse operator of smooth
+// fields twice too stiff; half of it is the operator of the coarse grid. One
+// thread per coarse cell; sums in FP64, stored FP32.
 __global__ void k_coarsen(Lev32 f, Lev32 c)
 {
     int I, J, K;
@@ -868,52 +916,93 @@ __global__ void k_coarsen(Lev32 f, Lev32 c)
                 if (dj == 0) fy0 += ldf(&f.ay[q]); else fy1 += ldf(&f.ay[q + G.P]);
                 if (dk == 0) fz0 += ldf(&f.az[q]); else fz1 += ldf(&f.az[q + G.P * (G.ny + 1)]);
             }
-    const double cc = 0.125 * cs;
+    const double cc = 0.125 * cs, h = 0.0625;
     c.c[Q] = (float)cc;
-    c.ax[Q] = (float)(0.125 * fx0); c.ay[Q] = (float)(0.125 * fy0); c.az[Q] = (float)(0.125 * fz0);
-    if (I == H.nx - 1) c.ax[Q + 1] = (float)(0.125 * fx1);
-    if (J == H.ny - 1) c.ay[Q + H.P] = (float)(0.125 * fy1);
-    if (K == H.nz - 1) c.az[Q + H.P * (H.ny + 1)] = (float)(0.125 * fz1);
-    const double d = cc + 0.125 * (fx0 + fx1 + fy0 + fy1 + fz0 + fz1);
+    c.ax[Q] = (float)(h * fx0); c.ay[Q] = (float)(h * fy0); c.az[Q] = (float)(h * fz0);
+    if (I == H.nx - 1) c.ax[Q + 1] = (float)(h * fx1);
+    if (J == H.ny - 1) c.ay[Q + H.P] = (float)(h * fy1);
+    if (K == H.nz - 1) c.az[Q + H.P * (H.ny + 1)] = (float)(h * fz1);
+    const double d = cc + h * (fx0 + fx1 + fy0 + fy1 + fz0 + fz1);
     c.d[Q] = (float)d;
-    c.w[Q] = (float)(kOmega / d);
+    c.w[Q] = (float)(1.0 / d);
 }
 
-// Pre-smoothing from zero, e = (omega/d) r, and restriction of r - A e to
-// the coarse level (mean of the 8 children). One thread per coarse cell.
-template <class RT>
-__global__ void k_mg_down(Lev32 f, const RT *r, Lev32 c, Sc *sc)
+// Restriction of the residual sum a e_b on the red cells to the coarse level
+// (mean of the 8 children; zero on black). e_b is ef pair by pair on the
+// finest level (FINE), f.e on the others. One thread per coarse cell.
+template <bool FINE>
+__global__ void k_mg_down(Lev32 f, const float *ef, Lev32 c, Sc *sc)
 {
     if (over(sc, L_CG)) return;
     int I, J, K;
     if (!cell(c.G, I, J, K)) return;
     const Geo &G = f.G;
-    auto e = [&](int q, int, int, int) { return ldf(&f.w[q]) * tof(__ldg(&r[q])); };
-    float s = 0.0f;
+    float t = 0.0f;
+#pragma unroll
     for (int dk = 0; dk < 2; ++dk)
-        for (int dj = 0; dj < 2; ++dj)
-            for (int di = 0; di < 2; ++di) {
-                const int i = 2 * I + di, j = 2 * J + dj, k = 2 * K + dk;
-                const int q = id3(G, i, j, k);
-                f.e[q] = e(q, i, j, k);
-                s += tof(__ldg(&r[q])) - helm32(f, e, i, j, k);
-            }
-    c.r[id3(c.G, I, J, K)] = 0.125f * s;
+#pragma unroll
+        for (int dj = 0; dj < 2; ++dj) {
+            const int j = 2 * J + dj, k = 2 * K + dk, i = 2 * I + 1 - ((dj + dk) & 1);
+            const int q = id3(G, i, j, k);
+            const Nb n = FINE ? pair_neighbours<true>(G, pair_id(G, I, j, k), i, j, k) : other_colour(G, q, i, j, k);
+            t = add_faces<float>(t, G, f.ax, f.ay, f.az, q, n, [&](int x) { return ldf(&ef[x]); });
+        }
+    c.r[id3(c.G, I, J, K)] = 0.125f * t;
 }
 
-// Coarsest level: damped Jacobi sweep (first: from zero).
-__global__ void k_mg_coarse(Lev32 L, const float *ein, float *eout, int first, Sc *sc)
+// The cell of one colour in pair m of a row.
+template <bool RED>
+__device__ __forceinline__ bool coloured(const Geo &G, int &i, int &j, int &k)
+{
+    const int m = blockIdx.x * TX + threadIdx.x;
+    j = blockIdx.y * TY + threadIdx.y;
+    k = blockIdx.z;
+    const int s = (j + k) & 1;
+    i = 2 * m + (RED ? 1 - s : s);
+    return i < G.nx && j < G.ny && k < G.nz;
+}
+
+// Black half of a red-black sweep on a level below the finest: the red cells
+// hold r / d plus (up half) the coarse correction ec, and black gets
+// (r + sum a e_red) / d, into out.
+__global__ void k_mg_black(Lev32 f, const float *ec, Geo cg, float *out, Sc *sc)
 {
     if (over(sc, L_CG)) return;
     int i, j, k;
-    if (!cell(L.G, i, j, k)) return;
-    const int q = id3(L.G, i, j, k);
-    const float w = ldf(&L.w[q]);
-    if (first) {
-        eout[q] = w * ldf(&L.r[q]);
-        return;
-    }
-    eout[q] = ldf(&ein[q]) + w * (ldf(&L.r[q]) - helm32(L, [&](int qq, int, int, int) { return ldf(&ein[qq]); }, i, j, k));
+    if (!coloured<false>(f.G, i, j, k)) return;
+    const Geo &G = f.G;
+    const int q = id3(G, i, j, k);
+    const Nb n = other_colour(G, q, i, j, k);
+    // the pair's other cell has the same coarse parent, the neighbours beyond
+    // the 2 x 2 x 2 block the adjacent one
+    const int Q = ec ? id3(cg, i >> 1, j >> 1, k >> 1) : 0, cy = cg.P, cz = cg.P * (cg.ny + 1);
+    const int up = (n.e - q) * ((i & 1) ? 1 : 0), dn = (n.w - q) * ((i & 1) ? 0 : 1);
+    auto e = [&](int x, int Qx) {
+        const float v = ldf(&f.w[x]) * ldf(&f.r[x]);
+        return ec ? v + ldf(&ec[Qx]) : v;
+    };
+    const int jn = n.n > q ? 1 : -1, js = n.s > q ? 1 : -1, kt = n.t > q ? 1 : -1, kb = n.b > q ? 1 : -1;
+    float t = ldf(&f.r[q]);
+    const int sy = G.P, sz = G.P * (G.ny + 1);
+    t = fmaf(ldf(&f.ax[q]), e(n.w, Q + (dn < 0 ? -1 : 0)), t);
+    t = fmaf(ldf(&f.ax[q + 1]), e(n.e, Q + (up > 0 ? 1 : 0)), t);
+    t = fmaf(ldf(&f.ay[q]), e(n.s, Q + (((j + js) >> 1) - (j >> 1)) * cy), t);
+    t = fmaf(ldf(&f.ay[q + sy]), e(n.n, Q + (((j + jn) >> 1) - (j >> 1)) * cy), t);
+    t = fmaf(ldf(&f.az[q]), e(n.b, Q + (((k + kb) >> 1) - (k >> 1)) * cz), t);
+    t = fmaf(ldf(&f.az[q + sz]), e(n.t, Q + (((k + kt) >> 1) - (k >> 1)) * cz), t);
+    out[q] = ldf(&f.w[q]) * t;
+}
+
+// Red half of the sweep that ends a level: (r + sum a out_black) / d.
+__global__ void k_mg_red(Lev32 f, float *out, Sc *sc)
+{
+    if (over(sc, L_CG)) return;
+    int i, j, k;
+    if (!coloured<true>(f.G, i, j, k)) return;
+    const int q = id3(f.G, i, j, k);
+    const Nb n = other_colour(f.G, q, i, j, k);
+    const float t = add_faces<float>(ldf(&f.r[q]), f.G, f.ax, f.ay, f.az, q, n, [&](int x) { return out[x]; });
+    out[q] = ldf(&f.w[q]) * t;
 }
 
 __device__ __forceinline__ void fin_rz(Sc *sc, double t)
@@ -922,154 +1011,183 @@ __device__ __forceinline__ void fin_rz(Sc *sc, double t)
     sc->rz = t;
 }
 
-// z = e + w (r - A e) at cell (i,j,k) of level f, with e the cell's own
-// smoothed correction plus its coarse parent's (prolongation and one
-// damped-Jacobi post-smoothing sweep); the residual value in rq.
-template <class RT>
-__device__ __forceinline__ float mg_up_cell(const Lev32 &f, const RT *r, const float *ec, const Geo &cg, int i,
-                                            int j, int k, RT &rq)
+// Up half on the finest level: z = (rb + sum a P ec) / d = ef + w sum a P ec on
+// black; acc += rb z (FP64 for the FP64 CG, FP32 for the mixed step's).
+template <class R>
+__global__ void k_mg_up(Lev32 f, Rb<R> v, const float *ec, Geo cg, Sc *sc, double *part)
 {
+    if (over(sc, L_CG)) return;
+    __shared__ double red[NT];
+    R acc[1] = {(R)0};
+    double tot[1];
     const Geo &G = f.G;
-    const int q = id3(G, i, j, k);
-    // coarse parent of the cell, and of a neighbour one cell away: the
-    // same parent or the adjacent one, by the parity of the cell's index
-    const int Q = id3(cg, i >> 1, j >> 1, k >> 1), cy = cg.P, cz = cg.P * (cg.ny + 1);
-    auto step = [](int d, int idx, int s) -> int {
-        return d > 0 ? ((idx & 1) ? s : 0) : d < 0 ? ((idx & 1) ? 0 : -s) : 0;
-    };
-    auto ef = [&](int qq, int ii, int jj, int kk) {
-        const int Qn = Q + step(ii - i, i, 1) + step(jj - j, j, cy) + step(kk - k, k, cz);
-        return ldf(&f.e[qq]) + ldf(&ec[Qn]);
-    };
-    rq = __ldg(&r[q]);
-    return ef(q, i, j, k) + ldf(&f.w[q]) * (tof(rq) - helm32(f, ef, i, j, k));
-}
-
-// Intermediate levels: one thread per cell, no reduction.
-template <class RT, class OT>
-__global__ void k_mg_up(Lev32 f, const RT *r, const float *ec, Geo cg, OT *out, Sc *sc)
-{
-    if (over(sc, L_CG)) return;
-    int i, j, k;
-    if (!cell(f.G, i, j, k)) return;
-    RT rq;
-    out[id3(f.G, i, j, k)] = (OT)mg_up_cell(f, r, ec, cg, i, j, k, rq);
-}
-
-// Finest level: column tiles of kLayers cells a thread (one block reduction
-// per column), with the r.z reduction of CG in OT (FP64 for the FP64 CG,
-// FP32 for the mixed step's).
-template <class RT, class OT>
-__global__ void k_mg_up_fin(Lev32 f, const RT *r, const float *ec, Geo cg, OT *out, Sc *sc, double *part)
-{
-    if (over(sc, L_CG)) return;
-    __shared__ double red[NT];
-    OT acc[1] = {(OT)0};
-    double tot[1];
-    int i, j, k0, k1;
-    if (column(f.G, i, j, k0, k1))
+    int m, j, k0, k1;
+    if (pair_column(G, m, j, k0, k1))
 #pragma unroll 1
         for (int k = k0; k < k1; ++k) {
-            RT rq;
-            const float z = mg_up_cell(f, r, ec, cg, i, j, k, rq);
-            out[id3(f.G, i, j, k)] = (OT)z;
-            acc[0] = fma((OT)rq, (OT)z, acc[0]);
+            const int s = (j + k) & 1, i = 2 * m + s;
+            if (i >= G.nx) continue;
+            const int q = id3(G, i, j, k), c = pair_id(G, m, j, k);
+            // parents of the neighbours: of the black cell's own pair m, and the
+            // pairs, rows and layers beside it
+            auto parent = [&](int mm, int jj, int kk) { return id3(cg, mm, jj >> 1, kk >> 1); };
+            const int mw = s ? m : max(m - 1, 0), me = s && i + 1 < G.nx ? m + 1 : m;
+            const Nb n{parent(mw, j, k), parent(me, j, k), parent(m, j > 0 ? j - 1 : j, k),
+                       parent(m, j + 1 < G.ny ? j + 1 : j, k), parent(m, j, k > 0 ? k - 1 : k),
+                       parent(m, j, k + 1 < G.nz ? k + 1 : k)};
+            const float t =
+                add_faces<float>(0.0f, G, f.ax, f.ay, f.az, q, n, [&](int x) { return ldf(&ec[x]); });
+            const float z = fmaf(ldf(&f.w[q]), t, ldf(&v.ef[c]));
+            v.z[c] = z;
+            acc[0] = fma(ld(&v.rb[c]), (R)z, acc[0]);
         }
-    if (gsum<1, OT>(acc, red, part, &sc->counters[C_RZ], tot)) fin_rz(sc, tot[0]);
+    if (gsum<1, R>(acc, red, part, &sc->counters[C_RZ], tot)) fin_rz(sc, tot[0]);
 }
 
-// One level only: z = e + (omega/d)(r - A e), e = (omega/d) r; acc += r.z
-// (T = double: the FP64 CG; T = float: the mixed step's FP32 CG).
-template <class T>
-__global__ void k_mg_single(Lev32 f, const T *r, T *out, Sc *sc, double *part)
+// ---- CG on the black half ----
+
+// Start of a solve: the black residual that the relaxed red cells (v.w = r/d)
+// leave, rb = r + sum a w, and ef. SINGLE (one level): z = ef; acc += rb z.
+template <class R, bool SINGLE>
+__global__ void k_rb_start(Op<R> A, const R *r, const float *wf, Rb<R> v, Sc *sc, double *part)
 {
     if (over(sc, L_CG)) return;
     __shared__ double red[NT];
-    T acc[1] = {(T)0};
+    R acc[1] = {(R)0};
     double tot[1];
-    int i, j, k;
-    if (cell(f.G, i, j, k)) {
-        const int q = id3(f.G, i, j, k);
-        auto e = [&](int qq, int, int, int) { return ldf(&f.w[qq]) * (float)__ldg(&r[qq]); };
-        const T rq = __ldg(&r[q]);
-        const float z = e(q, i, j, k) + ldf(&f.w[q]) * ((float)rq - helm32(f, e, i, j, k));
-        out[q] = (T)z;
-        acc[0] = rq * (T)z;
-    }
-    if (gsum<1, T>(acc, red, part, &sc->counters[C_RZ], tot)) fin_rz(sc, tot[0]);
-}
-
-// ---- CG steps (directions alternate between p0 and p1 by parity) ----
-
-// p = z + beta p_old (the new direction into the other buffer)
-__global__ void k_pupd(Args a, Lev L)
-{
-    Sc *sc = a.sc;
-    if (over(sc, L_CG)) return;
-    int i, j, k;
-    if (!cell(L.G, i, j, k)) return;
-    const int it = sc->cg_it;
-    const double *pold = (it & 1) ? a.p1 : a.p0;
-    double *pnew = (it & 1) ? a.p0 : a.p1;
-    const int q = id3(L.G, i, j, k);
-    pnew[q] = fma(sc->beta, ld(&pold[q]), ld(&L.e2[q]));
-}
-
-// q = A p, acc += p.q; alpha = rz / p.q
-__global__ void k_spmv(Args a, Lev L)
-{
-    Sc *sc = a.sc;
-    if (over(sc, L_CG)) return;
-    __shared__ double red[NT];
-    double acc[1] = {0.0}, tot[1];
-    const double *p = (sc->cg_it & 1) ? a.p0 : a.p1;
-    int i, j, k0, k1;
-    if (column(L.G, i, j, k0, k1))
+    const Geo &G = A.G;
+    int m, j, k0, k1;
+    if (pair_column(G, m, j, k0, k1))
 #pragma unroll 1
         for (int k = k0; k < k1; ++k) {
-            const int q = id3(L.G, i, j, k);
-            const double pq = ld(&p[q]);
-            const double Ap = helm(L, [&](int qq, int, int, int) { return ld(&p[qq]); }, i, j, k);
-            a.q[q] = Ap;
-            acc[0] = fma(pq, Ap, acc[0]);
+            const int i = 2 * m + ((j + k) & 1);
+            if (i >= G.nx) continue;
+            const int q = id3(G, i, j, k), c = pair_id(G, m, j, k);
+            const R g = add_faces<R>(ld(&r[q]), G, A.ax, A.ay, A.az, q, pair_neighbours<false>(G, c, i, j, k),
+                                     [&](int x) { return ld(&v.w[x]); });
+            const float e = ldf(&wf[q]) * (float)g;
+            v.rb[c] = g;
+            v.ef[c] = e;
+            if (SINGLE) acc[0] = fma(g, (R)e, acc[0]);
         }
-    if (gsum<1>(acc, red, a.part, &sc->counters[C_PQ], tot)) {
+    if (SINGLE)
+        if (gsum<1, R>(acc, red, part, &sc->counters[C_RZ], tot)) fin_rz(sc, tot[0]);
+}
+
+// p = z + beta p (the first direction: z), pair by pair.
+template <class R>
+__global__ void k_pupd(Geo G, Rb<R> v, Sc *sc)
+{
+    if (over(sc, L_CG)) return;
+    int i, j, k;
+    if (!coloured<false>(G, i, j, k)) return;
+    const int c = pair_id(G, i >> 1, j, k);
+    const R z = (R)ldf(&v.z[c]);
+    v.p[c] = sc->cg_it == 0 ? z : fma((R)sc->beta, v.p[c], z);
+}
+
+// w = (sum a p) / d on red
+template <class R>
+__global__ void k_spmv_red(Op<R> A, Rb<R> v, Sc *sc)
+{
+    if (over(sc, L_CG)) return;
+    int i, j, k;
+    if (!coloured<true>(A.G, i, j, k)) return;
+    const Geo &G = A.G;
+    const int q = id3(G, i, j, k), c = pair_id(G, i >> 1, j, k);
+    const R t = add_faces<R>((R)0, G, A.ax, A.ay, A.az, q, pair_neighbours<true>(G, c, i, j, k),
+                             [&](int x) { return ld(&v.p[x]); });
+    v.w[c] = ld(&A.wd[q]) * t;
+}
+
+// q = S p = d p - sum a w on black, acc += p.q; alpha = rz / p.q
+template <class R>
+__global__ void k_spmv_black(Op<R> A, Rb<R> v, Sc *sc, double *part)
+{
+    if (over(sc, L_CG)) return;
+    __shared__ double red[NT];
+    R acc[1] = {(R)0};
+    double tot[1];
+    const Geo &G = A.G;
+    int m, j, k0, k1;
+    if (pair_column(G, m, j, k0, k1))
+#pragma unroll 1
+        for (int k = k0; k < k1; ++k) {
+            const int i = 2 * m + ((j + k) & 1);
+            if (i >= G.nx) continue;
+            const int q = id3(G, i, j, k), c = pair_id(G, m, j, k);
+            const R p = ld(&v.p[c]);
+            const R t = add_faces<R>(-ld(&A.d[q]) * p, G, A.ax, A.ay, A.az, q, pair_neighbours<false>(G, c, i, j, k),
+                                     [&](int x) { return ld(&v.w[x]); });
+            v.q[c] = -t;
+            acc[0] = fma(p, -t, acc[0]);
+        }
+    if (gsum<1, R>(acc, red, part, &sc->counters[C_PQ], tot)) {
         sc->pq = tot[0];
         sc->alpha = tot[0] != 0.0 ? sc->rz / tot[0] : 0.0;
         if (!isfinite(tot[0])) sc->status = GEA_ERR_NONFINITE;
     }
 }
 
-// x += alpha p, r -= alpha q (in place, each cell its own) with an FP32 copy
-// of r for the multigrid restriction; acc += r^2.
-__global__ void k_update(Args a, Lev L, double *x, float *rf, int maxit)
+// xb += alpha p, rb -= alpha q, ef = rb / d; acc += rb^2 and (SINGLE) rb z.
+template <class R, bool SINGLE>
+__global__ void k_update(Geo G, const float *wf, Rb<R> v, double tol2, Sc *sc, double *part)
 {
-    Sc *sc = a.sc;
     if (over(sc, L_CG)) return;
-    __shared__ double red[NT];
-    double acc[1] = {0.0}, tot[1];
-    const int it = sc->cg_it;
-    const double *p = (it & 1) ? a.p0 : a.p1;
-    const double alpha = sc->alpha;
-    int i, j, k0, k1;
-    if (column(L.G, i, j, k0, k1))
+    constexpr int NV = SINGLE ? 2 : 1;
+    __shared__ double red[NV * NT];
+    R acc[NV] = {};
+    double tot[NV];
+    const R alpha = (R)sc->alpha;
+    const bool first = sc->cg_it == 0;
+    int m, j, k0, k1;
+    if (pair_column(G, m, j, k0, k1))
 #pragma unroll 1
         for (int k = k0; k < k1; ++k) {
-            const int q = id3(L.G, i, j, k);
-            x[q] = fma(alpha, ld(&p[q]), x[q]);
-            const double rn = fma(-alpha, ld(&a.q[q]), L.r[q]);
-            L.r[q] = rn;
-            rf[q] = (float)rn;
+            const int i = 2 * m + ((j + k) & 1);
+            if (i >= G.nx) continue;
+            const int q = id3(G, i, j, k), c = pair_id(G, m, j, k);
+            v.xb[c] = fma(alpha, ld(&v.p[c]), first ? (R)0 : v.xb[c]);
+            const R rn = fma(-alpha, ld(&v.q[c]), v.rb[c]);
+            const float e = ldf(&wf[q]) * (float)rn;
+            v.rb[c] = rn;
+            v.ef[c] = e;
             acc[0] = fma(rn, rn, acc[0]);
+            if (SINGLE) acc[NV - 1] = fma(rn, (R)e, acc[NV - 1]);
         }
-    if (gsum<1>(acc, red, a.part, &sc->counters[C_UPD], tot)) {
+    if (gsum<NV, R>(acc, red, part, &sc->counters[C_UPD], tot)) {
         const int n = sc->cg_it + 1;
         sc->cg_it = n;
         sc->r2 = tot[0];
         sc->cg_iters[sc->corr] = n;
         sc->cg_relres[sc->corr] = sc->b2 > 0.0 ? sqrt(tot[0] / sc->b2) : 0.0;
         if (!isfinite(tot[0])) sc->status = GEA_ERR_NONFINITE;
-        else if (tot[0] <= a.ctol2 * sc->b2) sc->done[L_CG] = 1;
+        else if (tot[0] <= tol2 * sc->b2) sc->done[L_CG] = 1;
+        else if (SINGLE) fin_rz(sc, tot[NV - 1]);
+    }
+}
+
+// The solution: xout = xin + xb on black, xin + (r + sum a xb) / d on red (xin
+// alone if there was nothing to solve).
+template <class R>
+__global__ void k_solution(Op<R> A, const R *r, Rb<R> v, const double *xin, double *xout, const Sc *sc)
+{
+    if (sc->status) return;
+    const Geo &G = A.G;
+    const bool dx = sc->cg_it > 0;
+    const int m = blockIdx.x * TX + threadIdx.x, j = blockIdx.y * TY + threadIdx.y, k = blockIdx.z;
+    if (2 * m >= G.nx || j >= G.ny) return;
+    const int s = (j + k) & 1, c = pair_id(G, m, j, k), q = id3(G, 2 * m, j, k);
+    if (2 * m + s < G.nx) xout[q + s] = dx ? xin[q + s] + (double)ld(&v.xb[c]) : xin[q + s];
+    const int i = 2 * m + 1 - s, qr = q + 1 - s;
+    if (i < G.nx) {
+        double x = xin[qr];
+        if (dx) {
+            const R t = add_faces<R>(ld(&r[qr]), G, A.ax, A.ay, A.az, qr, pair_neighbours<true>(G, c, i, j, k),
+                                     [&](int y) { return ld(&v.xb[y]); });
+            x += (double)(ld(&A.wd[qr]) * t);
+        }
+        xout[qr] = x;
     }
 }
 
@@ -1121,13 +1239,12 @@ __global__ void k_correct(Args a)
 
 // FP32 data of the mixed step: the stencil weights and reciprocals, the
 // FP64 residuals rounded to FP32, the increments (Jacobi ping-pong), and the
-// pressure increment with its CG vectors (r the FP32 residual, z the
-// preconditioned residual).
+// start residual of the pressure solve.
 struct Mx {
     float *c[NCF];
     float *dinvu, *dinvh, *r0u, *r0v, *r0w, *r0h;
     float *du[2], *dv[2], *dw[2], *dh[2];
-    float *x, *p0, *p1, *q, *r, *z;
+    float *r;            // the pressure residual
     double tol2;
 };
 
@@ -1373,88 +1490,6 @@ __global__ void k_mx_h1(Args a, const float *dh)
     a.ha[q] = ld(&a.S.h[q]) + (double)ldf(&dh[q]);
 }
 
-// FP32 CG on the pressure increment with the FP32 finest operator M0.
-
-// p = z + beta p_old
-__global__ void k_mx_pupd(Args a, Mx m, Lev32 M0)
-{
-    Sc *sc = a.sc;
-    if (over(sc, L_CG)) return;
-    int i, j, k;
-    if (!cell(M0.G, i, j, k)) return;
-    const int it = sc->cg_it;
-    const float *pold = (it & 1) ? m.p1 : m.p0;
-    float *pnew = (it & 1) ? m.p0 : m.p1;
-    const int q = id3(M0.G, i, j, k);
-    pnew[q] = fmaf((float)sc->beta, ldf(&pold[q]), ldf(&m.z[q]));
-}
-
-// q = A p, acc += p.q; alpha = rz / p.q
-__global__ void k_mx_spmv(Args a, Mx m, Lev32 M0)
-{
-    Sc *sc = a.sc;
-    if (over(sc, L_CG)) return;
-    __shared__ double red[NT];
-    float acc[1] = {0.0f};
-    double tot[1];
-    const float *p = (sc->cg_it & 1) ? m.p0 : m.p1;
-    int i, j, k0, k1;
-    if (column(M0.G, i, j, k0, k1))
-#pragma unroll 1
-        for (int k = k0; k < k1; ++k) {
-            const int q = id3(M0.G, i, j, k);
-            const float Ap = helm32(M0, [&](int qq, int, int, int) { return ldf(&p[qq]); }, i, j, k);
-            m.q[q] = Ap;
-            acc[0] = fmaf(ldf(&p[q]), Ap, acc[0]);
-        }
-    if (gsum<1, float>(acc, red, a.part, &sc->counters[C_PQ], tot)) {
-        sc->pq = tot[0];
-        sc->alpha = tot[0] != 0.0 ? sc->rz / tot[0] : 0.0;
-        if (!isfinite(tot[0])) sc->status = GEA_ERR_NONFINITE;
-    }
-}
-
-// x += alpha p, r -= alpha q; acc += r^2, relative to ||r0||^2 with mp_rtol.
-__global__ void k_mx_update(Args a, Mx m, Lev32 M0)
-{
-    Sc *sc = a.sc;
-    if (over(sc, L_CG)) return;
-    __shared__ double red[NT];
-    float acc[1] = {0.0f};
-    double tot[1];
-    const float *p = (sc->cg_it & 1) ? m.p0 : m.p1;
-    const float alpha = (float)sc->alpha;
-    int i, j, k0, k1;
-    if (column(M0.G, i, j, k0, k1))
-#pragma unroll 1
-        for (int k = k0; k < k1; ++k) {
-            const int q = id3(M0.G, i, j, k);
-            m.x[q] = fmaf(alpha, ldf(&p[q]), m.x[q]);
-            const float rn = fmaf(-alpha, ldf(&m.q[q]), m.r[q]);
-            m.r[q] = rn;
-            acc[0] = fmaf(rn, rn, acc[0]);
-        }
-    if (gsum<1, float>(acc, red, a.part, &sc->counters[C_UPD], tot)) {
-        const int n = sc->cg_it + 1;
-        sc->cg_it = n;
-        sc->r2 = tot[0];
-        sc->cg_iters[sc->corr] = n;
-        sc->cg_relres[sc->corr] = sc->b2 > 0.0 ? sqrt(tot[0] / sc->b2) : 0.0;
-        if (!isfinite(tot[0])) sc->status = GEA_ERR_NONFINITE;
-        else if (tot[0] <= m.tol2 * sc->b2) sc->done[L_CG] = 1;
-    }
-}
-
-// p' += dp (FP64).
-__global__ void k_mx_papply(Args a, Mx m)
-{
-    if (a.sc->status) return;
-    int i, j, k;
-    if (!cell(a.G, i, j, k)) return;
-    const int q = id3(a.G, i, j, k);
-    a.N.pp[q] = ld(&a.N.pp[q]) + (double)ldf(&m.x[q]);
-}
-
 // ---- loop control and step bookkeeping (one thread) ----
 
 __global__ void k_ctl(Sc *sc, cudaGraphConditionalHandle h, int graph, int which, int maxtrips, int body)
@@ -1500,7 +1535,9 @@ struct gea3d_ctx {
     std::vector<void *> allocs;
     St S[2];
     double *rho1, *dinvu, *dinvh, *bu, *bv, *bw, *ua, *va, *wa, *ub, *vb, *wb, *bh, *ha, *hb;
-    double *rho2, *psi, *Dx, *Dy, *Dz, *Hx, *Hy, *Hz, *b, *p0, *p1, *q;
+    double *rho2, *psi, *Dx, *Dy, *Dz, *Hx, *Hy, *Hz;
+    Rb<double> rb{};                      // the pressure solve's vectors (FP64 step)
+    Rb<float> rbf{};                      // (mixed step)
     double *dtr1;                         // dt / rho1
     double *kin;                          // K1
     double *mueff = nullptr;              // LES eddy viscosity field
@@ -1594,14 +1631,14 @@ dim3 grid_of(const Geo &G) { return dim3((G.nx + TX - 1) / TX, (G.ny + TY - 1) /
 // 33 x 33 x 24 has 240 one-layer tiles in all). The light CG kernels walk up to
 // eight layers, the stencil kernels up to four.
 constexpr int kLayers = 8, kLayersHeavy = 4, kMinBlocks = 2400;
-dim3 columns_of(const Geo &G, int most)
+dim3 columns_of(const Geo &G, const dim3 &g, int most)
 {
-    const dim3 g = grid_of(G);
     int layers = most;
     while (layers > 1 && (size_t)g.x * g.y * ((G.nz + layers - 1) / layers) < (size_t)kMinBlocks) layers /= 2;
     return dim3(g.x, g.y, (G.nz + layers - 1) / layers);
 }
-dim3 gridc_of(const Geo &G) { return columns_of(G, kLayers); }
+// The grids over pairs of cells: one layer a block, and columns.
+dim3 grid_pairs(const Geo &G) { return dim3(((G.nx + 1) / 2 + TX - 1) / TX, (G.ny + TY - 1) / TY, G.nz); }
 const dim3 kBlk(TX, TY);
 size_t nblocks(const Geo &G)
 {
@@ -1619,7 +1656,7 @@ Args args_of(gea3d_ctx *c, int from)
     a.ua = c->ua; a.va = c->va; a.wa = c->wa; a.ub = c->ub; a.vb = c->vb; a.wb = c->wb;
     a.bh = c->bh; a.ha = c->ha; a.hb = c->hb;
     a.rho2 = c->rho2; a.psi = c->psi; a.Dx = c->Dx; a.Dy = c->Dy; a.Dz = c->Dz;
-    a.Hx = c->Hx; a.Hy = c->Hy; a.Hz = c->Hz; a.b = c->b; a.p0 = c->p0; a.p1 = c->p1; a.q = c->q;
+    a.Hx = c->Hx; a.Hy = c->Hy; a.Hz = c->Hz;
     a.cf = c->cf;
     a.dtr1 = c->dtr1;
     a.kin = c->kin;
@@ -1678,8 +1715,10 @@ struct Trace3 {
     // the loop whose finished flag makes the kernel return, or -1
     static int gate(const char *name)
     {
-        static const char *cg[] = {"g3_mg_coarse", "g3_mg_down", "g3_mg_single", "g3_mg_up", "g3_pupd", "g3_spmv",
-                                   "g3_update", "g3_mx_pupd", "g3_mx_spmv", "g3_mx_update"};
+        static const char *cg[] = {"g3_rb_start",  "g3_mg_down",     "g3_mg_black",      "g3_mg_red",
+                                   "g3_mg_up",     "g3_pupd",        "g3_spmv_red",      "g3_spmv_black",
+                                   "g3_update",    "g3_mx_rb_start", "g3_mx_mg_up",      "g3_mx_pupd",
+                                   "g3_mx_spmv_red", "g3_mx_spmv_black", "g3_mx_update"};
         for (const char *c : cg)
             if (!strcmp(name, c)) return L_CG;
         if (!strcmp(name, "g3_mom") || !strcmp(name, "g3_mx_mom")) return L_MOM;
@@ -1733,82 +1772,85 @@ int eager_while3(gea3d_ctx *ctx, cudaStream_t s, int which, int maxtrips, Body b
     return GEA_OK;
 }
 
-// z = M^-1 r on the finest level (one FP32 V(1,1) cycle); returns launches
-int vcycle(gea3d_ctx *ctx, const Args &a, cudaStream_t st, Trace3 *tr)
+// z = M^-1 rb (one FP32 V-cycle; nothing to do on one level); returns launches
+template <class R>
+int vcycle(gea3d_ctx *ctx, const Args &a, const Rb<R> &v, cudaStream_t st, Trace3 *tr)
 {
     Lev32 *M = ctx->M.data();
-    Lev &F = ctx->L[0];
     const int nlev = (int)ctx->M.size();
-    if (ctx->mixed) {
-        // the mixed step's FP32 CG: from the FP32 residual r to z, both FP32
-        const Mx &m = ctx->mx;
-        if (nlev == 1) {
-            traced(tr, "g3_mg_single", F.G, st, [&] {
-                k_mg_single<float><<<grid_of(F.G), kBlk, 0, st>>>(M[0], m.r, m.z, a.sc, a.part);
-            });
-            return 1;
-        }
-        int n = 0;
-        traced(tr, "g3_mg_down", M[1].G, st, [&] {
-            k_mg_down<float><<<grid_of(M[1].G), kBlk, 0, st>>>(M[0], m.r, M[1], a.sc);
-        });
-        ++n;
-        for (int l = 1; l + 1 < nlev; ++l, ++n)
-            traced(tr, "g3_mg_down", M[l + 1].G, st, [&] {
-                k_mg_down<float><<<grid_of(M[l + 1].G), kBlk, 0, st>>>(M[l], M[l].r, M[l + 1], a.sc);
-            });
-        Lev32 &C = M[nlev - 1];
-        for (int s = 0; s < kCoarseSweeps; ++s, ++n) {
-            float *out = ((kCoarseSweeps - 1 - s) % 2 == 0) ? C.e2 : C.e;
-            const float *in = (out == C.e2) ? C.e : C.e2;
-            traced(tr, "g3_mg_coarse", C.G, st, [&] {
-                k_mg_coarse<<<grid_of(C.G), kBlk, 0, st>>>(C, in, out, s == 0, a.sc);
-            });
-        }
-        for (int l = nlev - 2; l >= 1; --l, ++n)
-            traced(tr, "g3_mg_up", M[l].G, st, [&] {
-                k_mg_up<float, float><<<grid_of(M[l].G), kBlk, 0, st>>>(M[l], M[l].r, M[l + 1].e2, M[l + 1].G,
-                                                                         M[l].e2, a.sc);
-            });
-        traced(tr, "g3_mg_up", F.G, st, [&] {
-            k_mg_up_fin<float, float><<<gridc_of(F.G), kBlk, 0, st>>>(M[0], m.r, M[1].e2, M[1].G, m.z, a.sc,
-                                                                      a.part);
-        });
-        return n + 1;
-    }
-    if (nlev == 1) {
-        traced(tr, "g3_mg_single", F.G, st, [&] {
-            k_mg_single<double><<<grid_of(F.G), kBlk, 0, st>>>(M[0], F.r, F.e2, a.sc, a.part);
-        });
-        return 1;
-    }
+    if (nlev == 1) return 0;
     int n = 0;
+    auto black = [&](const Lev32 &f, const float *ec, const Geo &cg, float *out) {
+        traced(tr, "g3_mg_black", f.G, st, [&] { k_mg_black<<<grid_pairs(f.G), kBlk, 0, st>>>(f, ec, cg, out, a.sc); });
+        ++n;
+    };
+    auto red = [&](const Lev32 &f) {
+        traced(tr, "g3_mg_red", f.G, st, [&] { k_mg_red<<<grid_pairs(f.G), kBlk, 0, st>>>(f, f.e2, a.sc); });
+        ++n;
+    };
     traced(tr, "g3_mg_down", M[1].G, st, [&] {
-        k_mg_down<float><<<grid_of(M[1].G), kBlk, 0, st>>>(M[0], M[0].r, M[1], a.sc);
+        k_mg_down<true><<<grid_of(M[1].G), kBlk, 0, st>>>(M[0], v.ef, M[1], a.sc);
     });
     ++n;
-    for (int l = 1; l + 1 < nlev; ++l, ++n)
+    for (int l = 1; l + 1 < nlev; ++l) {
+        black(M[l], nullptr, M[l].G, M[l].e);
         traced(tr, "g3_mg_down", M[l + 1].G, st, [&] {
-            k_mg_down<float><<<grid_of(M[l + 1].G), kBlk, 0, st>>>(M[l], M[l].r, M[l + 1], a.sc);
+            k_mg_down<false><<<grid_of(M[l + 1].G), kBlk, 0, st>>>(M[l], M[l].e, M[l + 1], a.sc);
         });
-    Lev32 &C = M[nlev - 1];
-    for (int s = 0; s < kCoarseSweeps; ++s, ++n) {
-        float *out = ((kCoarseSweeps - 1 - s) % 2 == 0) ? C.e2 : C.e;
-        const float *in = (out == C.e2) ? C.e : C.e2;
-        traced(tr, "g3_mg_coarse", C.G, st, [&] {
-            k_mg_coarse<<<grid_of(C.G), kBlk, 0, st>>>(C, in, out, s == 0, a.sc);
-        });
+        ++n;
     }
-    for (int l = nlev - 2; l >= 1; --l, ++n)
-        traced(tr, "g3_mg_up", M[l].G, st, [&] {
-            k_mg_up<float, float><<<grid_of(M[l].G), kBlk, 0, st>>>(M[l], M[l].r, M[l + 1].e2, M[l + 1].G,
-                                                                     M[l].e2, a.sc);
-        });
-    traced(tr, "g3_mg_up", F.G, st, [&] {
-        k_mg_up_fin<double, double><<<gridc_of(F.G), kBlk, 0, st>>>(M[0], F.r, M[1].e2, M[1].G, F.e2, a.sc,
-                                                                    a.part);
+    // the coarsest level: one symmetric red-black sweep
+    for (int l = nlev - 1; l >= 1; --l) {
+        black(M[l], l == nlev - 1 ? nullptr : M[l + 1].e2, l == nlev - 1 ? M[l].G : M[l + 1].G, M[l].e2);
+        red(M[l]);
+    }
+    const Geo &G = ctx->G;
+    traced(tr, ctx->mixed ? "g3_mx_mg_up" : "g3_mg_up", G, st, [&] {
+        k_mg_up<R><<<columns_of(G, grid_pairs(G), kLayers), kBlk, 0, st>>>(M[0], v, M[1].e2, M[1].G, a.sc, a.part);
     });
     return n + 1;
+}
+
+// One pressure solve of corrector c from x = xin into N.pp: residual, CG on
+// the black half to the relative residual tol2 (squared) and the solution.
+// A: the operator in the solve's precision, r its start residual.
+template <class R, class Loop>
+int solve_pressure(gea3d_ctx *ctx, const Args &a, const Op<R> &A, R *r, const Rb<R> &v, double tol2, const double *xin,
+                   int c, cudaStream_t s, bool graph, Trace3 *tr, Loop loop, int &fixed)
+{
+    const Geo &G = ctx->G;
+    const bool mx = ctx->mixed, single = ctx->M.size() == 1;
+    const float *wf = ctx->M[0].w;
+    const dim3 pairs = grid_pairs(G), cols = columns_of(G, pairs, kLayers);
+    const int nlev = (int)ctx->M.size(), gr = graph ? 1 : 0;
+    traced(tr, "g3_helm_rhs", G, s, [&] {
+        k_helm_rhs<R><<<columns_of(G, grid_of(G), kLayersHeavy), kBlk, 0, s>>>(a, ctx->L[0], xin, c, r, A.wd, v.w);
+    });
+    traced(tr, mx ? "g3_mx_rb_start" : "g3_rb_start", G, s, [&] {
+        if (single) k_rb_start<R, true><<<cols, kBlk, 0, s>>>(A, r, wf, v, a.sc, a.part);
+        else k_rb_start<R, false><<<cols, kBlk, 0, s>>>(A, r, wf, v, a.sc, a.part);
+    });
+    fixed += 2 + vcycle<R>(ctx, a, v, s, tr);
+    const int body = 4 + (nlev == 1 ? 0 : 4 * (nlev - 1)) + 1;
+    const int rc = loop(L_CG, ctx->C.cg_maxit, [&](cudaStream_t bs, cudaGraphConditionalHandle h) {
+        traced(tr, mx ? "g3_mx_pupd" : "g3_pupd", G, bs, [&] { k_pupd<R><<<pairs, kBlk, 0, bs>>>(G, v, a.sc); });
+        traced(tr, mx ? "g3_mx_spmv_red" : "g3_spmv_red", G, bs,
+               [&] { k_spmv_red<R><<<pairs, kBlk, 0, bs>>>(A, v, a.sc); });
+        traced(tr, mx ? "g3_mx_spmv_black" : "g3_spmv_black", G, bs,
+               [&] { k_spmv_black<R><<<cols, kBlk, 0, bs>>>(A, v, a.sc, a.part); });
+        traced(tr, mx ? "g3_mx_update" : "g3_update", G, bs, [&] {
+            if (single) k_update<R, true><<<cols, kBlk, 0, bs>>>(G, wf, v, tol2, a.sc, a.part);
+            else k_update<R, false><<<cols, kBlk, 0, bs>>>(G, wf, v, tol2, a.sc, a.part);
+        });
+        vcycle<R>(ctx, a, v, bs, tr);
+        k_ctl<<<1, 1, 0, bs>>>(a.sc, h, gr, L_CG, ctx->C.cg_maxit, body);
+    });
+    if (rc) return rc;
+    traced(tr, mx ? "g3_mx_solution" : "g3_solution", G, s, [&] {
+        k_solution<R><<<pairs, kBlk, 0, s>>>(A, r, v, xin, a.N.pp, a.sc);
+    });
+    ++fixed;
+    return GEA_OK;
 }
 
 // The kernel sequence of one step reading slot `from` (Section 3: Step 1,
@@ -1823,7 +1865,7 @@ int record3(gea3d_ctx *ctx, int from, cudaStream_t s, bool graph, Trace3 *tr)
     const int nlev = (int)ctx->M.size();
     const Geo &G = ctx->G;
     const dim3 grid = grid_of(G);
-    const dim3 gridc = gridc_of(G), gridh = columns_of(G, kLayersHeavy);   // column kernels
+    const dim3 gridh = columns_of(G, grid, kLayersHeavy);   // column kernels
     const int jtrips = (ctx->C.jac_maxit + 1) / 2;
     const int gr = graph ? 1 : 0;
     int fixed = 0, rc;
@@ -1877,42 +1919,24 @@ int record3(gea3d_ctx *ctx, int from, cudaStream_t s, bool graph, Trace3 *tr)
     }
     traced(tr, "g3_eos", G, s, [&] { k_eos<<<grid, kBlk, 0, s>>>(a, L[0], M[0], a.ha); }); ++fixed;
     traced(tr, "g3_faces", G, s, [&] { k_faces<<<grid, kBlk, 0, s>>>(a, L[0], M[0]); }); ++fixed;
-    traced(tr, "g3_diag", G, s, [&] { k_diag<<<grid, kBlk, 0, s>>>(L[0], M[0], a.sc); }); ++fixed;
+    traced(tr, "g3_diag", G, s, [&] {
+        if (ctx->mixed) k_diag<false><<<grid, kBlk, 0, s>>>(L[0], M[0], a.sc);
+        else k_diag<true><<<grid, kBlk, 0, s>>>(L[0], M[0], a.sc);
+    });
+    ++fixed;
     for (int l = 0; l + 1 < nlev; ++l, ++fixed)
         traced(tr, "g3_coarsen", M[l + 1].G, s, [&] {
             k_coarsen<<<grid_of(M[l + 1].G), kBlk, 0, s>>>(M[l], M[l + 1]);
         });
-    const int body_cg = (nlev == 1 ? 4 : 3 + (nlev - 1) + kCoarseSweeps + (nlev - 1)) + 1;
+    const Op<double> A{G, L[0].d, L[0].ax, L[0].ay, L[0].az, L[0].wd};
+    const Op<float> Af{G, M[0].d, M[0].ax, M[0].ay, M[0].az, M[0].w};
     for (int c = 0; c < ctx->C.n_corr; ++c) {
         const double *U = c == 0 ? a.ua : a.N.u, *V = c == 0 ? a.va : a.N.v, *W = c == 0 ? a.wa : a.N.w;
         traced(tr, "g3_H", G, s, [&] { k_H<<<grid, kBlk, 0, s>>>(a, U, V, W); }); ++fixed;
-        traced(tr, "g3_helm_rhs", G, s, [&] {
-            if (ctx->mixed)
-                k_helm_rhs<<<gridh, kBlk, 0, s>>>(a, L[0], c == 0 ? a.S.pp : a.N.pp, a.N.pp, c, m.r, m.x, m.p0);
-            else
-                k_helm_rhs<<<gridh, kBlk, 0, s>>>(a, L[0], c == 0 ? a.S.pp : a.N.pp, a.N.pp, c, nullptr, nullptr,
-                                                 nullptr, ctx->M[0].r);
-        });
-        ++fixed;
-        fixed += vcycle(ctx, a, s, tr);
-        rc = loop(L_CG, ctx->C.cg_maxit, [&](cudaStream_t bs, cudaGraphConditionalHandle h) {
-            if (ctx->mixed) {
-                traced(tr, "g3_mx_pupd", G, bs, [&] { k_mx_pupd<<<grid, kBlk, 0, bs>>>(a, m, M[0]); });
-                traced(tr, "g3_mx_spmv", G, bs, [&] { k_mx_spmv<<<gridc, kBlk, 0, bs>>>(a, m, M[0]); });
-                traced(tr, "g3_mx_update", G, bs, [&] { k_mx_update<<<gridc, kBlk, 0, bs>>>(a, m, M[0]); });
-            } else {
-                traced(tr, "g3_pupd", G, bs, [&] { k_pupd<<<grid, kBlk, 0, bs>>>(a, L[0]); });
-                traced(tr, "g3_spmv", G, bs, [&] { k_spmv<<<gridc, kBlk, 0, bs>>>(a, L[0]); });
-                traced(tr, "g3_update", G, bs, [&] { k_update<<<gridc, kBlk, 0, bs>>>(a, L[0], a.N.pp, ctx->M[0].r, ctx->C.cg_maxit); });
-            }
-            vcycle(ctx, a, bs, tr);
-            k_ctl<<<1, 1, 0, bs>>>(a.sc, h, gr, L_CG, ctx->C.cg_maxit, body_cg);
-        });
+        const double *xin = c == 0 ? a.S.pp : a.N.pp;
+        rc = ctx->mixed ? solve_pressure<float>(ctx, a, Af, m.r, ctx->rbf, m.tol2, xin, c, s, graph, tr, loop, fixed)
+                        : solve_pressure<double>(ctx, a, A, L[0].r, ctx->rb, a.ctol2, xin, c, s, graph, tr, loop, fixed);
         if (rc) return rc;
-        if (ctx->mixed) {
-            traced(tr, "g3_mx_papply", G, s, [&] { k_mx_papply<<<grid, kBlk, 0, s>>>(a, m); });
-            ++fixed;
-        }
         traced(tr, "g3_correct", G, s, [&] { k_correct<<<grid, kBlk, 0, s>>>(a); }); ++fixed;
     }
     ++fixed;
@@ -1963,7 +1987,7 @@ int gea3d_create(const gea3d_grid *grid, const gea_constants *c, gea3d_ctx **out
     ctx->C = *c;
     ctx->G = make_geo(grid->nx, grid->ny, grid->nz, grid->lx, grid->ly, grid->lz);
     ctx->F.R = c->R; ctx->F.cp = c->cp; ctx->F.g = c->g; ctx->F.mu = c->mu; ctx->F.nuh = c->mu / c->Pr;
-    ctx->F.dt = c->dt; ctx->F.idt = 1.0 / c->dt; ctx->F.omega = kOmega; ctx->F.icp = 1.0 / c->cp;
+    ctx->F.dt = c->dt; ctx->F.idt = 1.0 / c->dt; ctx->F.icp = 1.0 / c->cp;
     {
         const double delta = cbrt(ctx->G.dx * ctx->G.dy * ctx->G.dz);
         ctx->F.les_d2 = c->cs * c->cs * delta * delta;
@@ -2012,8 +2036,7 @@ int gea3d_create(const gea3d_grid *grid, const gea_constants *c, gea3d_ctx **out
     }
     double **sc[] = {&ctx->rho1, &ctx->dinvu, &ctx->dinvh, &ctx->bu, &ctx->bv, &ctx->bw, &ctx->ua, &ctx->va,
                      &ctx->wa, &ctx->ub, &ctx->vb, &ctx->wb, &ctx->bh, &ctx->ha, &ctx->hb, &ctx->rho2,
-                     &ctx->psi, &ctx->Dx, &ctx->Dy, &ctx->Dz, &ctx->Hx, &ctx->Hy, &ctx->Hz, &ctx->b, &ctx->p0,
-                     &ctx->p1, &ctx->q};
+                     &ctx->psi, &ctx->Dx, &ctx->Dy, &ctx->Dz, &ctx->Hx, &ctx->Hy, &ctx->Hz};
     for (auto pp : sc) *pp = take(E);
     for (int m = 0; m < NCF; ++m) ctx->cf.c[m] = take(E);
     ctx->dtr1 = take(E);
@@ -2042,7 +2065,7 @@ int gea3d_create(const gea3d_grid *grid, const gea_constants *c, gea3d_ctx **out
         for (int s = 0; s < NCF; ++s) m.c[s] = tf();
         m.dinvu = tf(); m.dinvh = tf(); m.r0u = tf(); m.r0v = tf(); m.r0w = tf(); m.r0h = tf();
         for (int b = 0; b < 2; ++b) { m.du[b] = tf(); m.dv[b] = tf(); m.dw[b] = tf(); m.dh[b] = tf(); }
-        m.x = tf(); m.p0 = tf(); m.p1 = tf(); m.q = tf(); m.r = tf(); m.z = tf();
+        m.r = tf();
         const double rt = c->mp_rtol != 0.0 ? c->mp_rtol : 1e-5;
         m.tol2 = rt * rt;
     }
@@ -2051,7 +2074,7 @@ int gea3d_create(const gea3d_grid *grid, const gea_constants *c, gea3d_ctx **out
         Lev l;
         l.G = ctx->G;
         l.c = take(E); l.d = take(E); l.ax = take(E); l.ay = take(E); l.az = take(E);
-        l.r = take(E); l.e2 = take(E);
+        l.r = take(E); l.wd = take(E);
         ctx->L.push_back(l);
     }
     auto takef = [&](size_t n) -> float * {
@@ -2063,12 +2086,23 @@ int gea3d_create(const gea3d_grid *grid, const gea_constants *c, gea3d_ctx **out
         m.G = lg[lv];
         const size_t e = elems(lg[lv]);
         m.c = takef(e); m.d = takef(e); m.ax = takef(e); m.ay = takef(e); m.az = takef(e);
-        m.w = takef(e); m.e = takef(e);
-        // the FP64 step keeps an FP32 copy of the CG residual on the finest
-        // level for the restriction (the mixed step's residual is FP32)
-        m.r = (lv || !ctx->mixed) ? takef(e) : nullptr;
+        m.w = takef(e);
+        m.e = lv ? takef(e) : nullptr;
+        m.r = lv ? takef(e) : nullptr;
         m.e2 = lv ? takef(e) : nullptr;
         ctx->M.push_back(m);
+    }
+    {
+        // the pressure solve's vectors, a value per pair of cells (P is even)
+        auto half = [&](auto &v) {
+            using R = std::remove_reference_t<decltype(*v.p)>;
+            const size_t n = E / 2, d = (n * sizeof(R) + sizeof(double) - 1) / sizeof(double);
+            for (R **x : {&v.p, &v.w, &v.q, &v.rb, &v.xb}) *x = reinterpret_cast<R *>(take(d));
+            v.ef = takef(n);
+            v.z = ctx->M.size() > 1 ? takef(n) : v.ef;
+        };
+        if (ctx->mixed) half(ctx->rbf);
+        else half(ctx->rb);
     }
     {
         const size_t nb = nblocks(ctx->G), ng = (nb + kGroup - 1) / kGroup;
