@@ -915,11 +915,13 @@ __device__ __forceinline__ PairTile<H, R> &pair_tile(double *sm, int at)
 }
 
 // The thread's pair (j, k); false outside the rows and pairs of the level.
-__device__ __forceinline__ bool pair_of(const Geom &G, int bx, int bz, int &j, int &k)
+// Tiles of fewer rows than BZ (an even number) keep all threads on the halo's
+// elements and the first rows of threads on the own ones.
+__device__ __forceinline__ bool pair_of(const Geom &G, int bx, int bz, int &j, int &k, int rows = BZ)
 {
     j = bx * BX + threadIdx.x;
-    k = bz * BZ + threadIdx.y;
-    return j < pairs_of(G) && k < G.nz;
+    k = bz * rows + threadIdx.y;
+    return j < pairs_of(G) && k < G.nz && (int)threadIdx.y < rows;
 }
 
 // sum of the face coefficients of cell q times its four neighbours' values
@@ -932,16 +934,16 @@ __device__ __forceinline__ R faces4(const LevelT<R> &L, int q, R w, R e, R s, R 
     return fma(ld(&L.az[q + L.G.P]), n, t);
 }
 
-// Fills rows -H .. BZ + H - 1 and pairs -1 .. BX of a pair tile with
+// Fills rows -H .. rows + H - 1 and pairs -1 .. BX of a pair tile with
 // f(q, c) at the cells of one colour (RED: the red ones) inside the box
 // (q: cell index, c: pair index), zero elsewhere.
 template <int H, bool RED, class R, class Fn>
-__device__ __forceinline__ void fill_pairs(PairTile<H, R> &t, const Geom &G, int bx, int bz, Fn f)
+__device__ __forceinline__ void fill_pairs(PairTile<H, R> &t, const Geom &G, int bx, int bz, Fn f, int rows = BZ)
 {
     const int tid = threadIdx.x + threadIdx.y * BX;
-    for (int e = tid; e < (BZ + 2 * H) * kPW; e += NTHREADS) {
+    for (int e = tid; e < (rows + 2 * H) * kPW; e += NTHREADS) {
         const int tk = e / kPW, tj = e - tk * kPW;
-        const int j = bx * BX - 1 + tj, k = bz * BZ - H + tk;
+        const int j = bx * BX - 1 + tj, k = bz * rows - H + tk;
         const int i = 2 * j + (RED ? 1 - (k & 1) : (k & 1));
         t[tk][tj] = (j >= 0 && i < G.nx && k >= 0 && k < G.nz) ? (R)f(k * G.P + i, k * G.P + j, j, k) : (R)0;
     }
@@ -952,12 +954,12 @@ __device__ __forceinline__ void fill_pairs(PairTile<H, R> &t, const Geom &G, int
 // pairs next to the black pairs 0 .. BX - 1 of a row are -1 + s .. BX - 1 + s,
 // the black ones next to the red pairs -s .. BX - s (tile columns one more).
 template <bool RED, class R, class Fn>
-__device__ __forceinline__ void fill_next(PairTile<1, R> &t, const Geom &G, int bx, int bz, Fn f)
+__device__ __forceinline__ void fill_next(PairTile<1, R> &t, const Geom &G, int bx, int bz, Fn f, int rows = BZ)
 {
     const int tid = threadIdx.x + threadIdx.y * BX;
-    for (int e = tid; e < (BZ + 2) * (BX + 1); e += NTHREADS) {
+    for (int e = tid; e < (rows + 2) * (BX + 1); e += NTHREADS) {
         const int tk = e / (BX + 1);
-        const int k = bz * BZ - 1 + tk, s = k & 1;
+        const int k = bz * rows - 1 + tk, s = k & 1;
         const int tj = e - tk * (BX + 1) + (RED ? s : 1 - s);
         const int j = bx * BX - 1 + tj;
         const int i = 2 * j + (RED ? 1 - s : s);
@@ -969,13 +971,13 @@ __device__ __forceinline__ void fill_next(PairTile<1, R> &t, const Geom &G, int 
 // residual of the pair's two cells after pre-smoothing): a quarter of the sum
 // over the two pairs of a coarse cell, which has the pair's index.
 template <class R>
-__device__ __forceinline__ void restrict_pairs(const LevelT<R> &c, R v, R *sres, int bx, int bz)
+__device__ __forceinline__ void restrict_pairs(const LevelT<R> &c, R v, R *sres, int bx, int bz, int rows = BZ)
 {
     const int tx = threadIdx.x, ty = threadIdx.y;
     sres[ty * BX + tx] = v;
     __syncthreads();
-    if (ty < BZ / 2) {
-        const int I = bx * BX + tx, K = bz * (BZ / 2) + ty;
+    if (ty < rows / 2) {
+        const int I = bx * BX + tx, K = bz * (rows / 2) + ty;
         if (I < c.G.nx && K < c.G.nz)
             c.r[cidx(c.G, I, K)] = (R)0.25 * (sres[2 * ty * BX + tx] + sres[(2 * ty + 1) * BX + tx]);
     }
@@ -1015,29 +1017,29 @@ __device__ __forceinline__ void ph_rb_start(const LevelT<R> &L, R *rb, R *z, dou
 // iteration it follows from rb).
 template <bool FINE, class R>
 __device__ __forceinline__ void ph_mg_down(const LevelT<R> &f, const LevelT<R> &c, R *rb, const Phys &F, double *sm,
-                                           int bx, int bz)
+                                           int bx, int bz, int rows = BZ)
 {
     const Geom &G = f.G;
     PairTile<2, R> &st = pair_tile<2, R>(sm, 0);
     PairTile<1, R> &se = pair_tile<1, R>(sm, kPH2);
     R *sres = reinterpret_cast<R *>(sm) + kPH2 + kPH1;
-    fill_pairs<2, true, R>(st, G, bx, bz, [&](int q, int, int, int) { return ld(&f.wd[q]) * ld(&f.r[q]); });
+    fill_pairs<2, true, R>(st, G, bx, bz, [&](int q, int, int, int) { return ld(&f.wd[q]) * ld(&f.r[q]); }, rows);
     __syncthreads();
     fill_next<false, R>(se, G, bx, bz, [&](int q, int cc, int tk, int tj, int s) {
         const R g = ld(&f.r[q]) + faces4<R>(f, q, st[tk + 1][tj - 1 + s], st[tk + 1][tj + s], st[tk][tj], st[tk + 2][tj]);
         R e = ld(&f.wd[q]) * g;
-        const bool own = tk >= 1 && tk <= BZ && tj >= 1 && tj <= BX;
+        const bool own = tk >= 1 && tk <= rows && tj >= 1 && tj <= BX;
         if (FINE && own) rb[cc] = g;
         rarely(F.om_ne1, [&] {
             e *= (R)F.omega;
             if (own && !FINE) f.e[q] = e;
         });
         return e;
-    });
+    }, rows);
     __syncthreads();
     int j, k;
     R v = 0;
-    if (pair_of(G, bx, bz, j, k)) {
+    if (pair_of(G, bx, bz, j, k, rows)) {
         const int s = k & 1, q = cidx(G, 2 * j + 1 - s, k);
         const int y = threadIdx.y + 1, x = threadIdx.x + 1;
         v = faces4<R>(f, q, se[y][x - s], se[y][x + 1 - s], se[y - 1][x], se[y + 1][x]);
@@ -1046,7 +1048,7 @@ __device__ __forceinline__ void ph_mg_down(const LevelT<R> &f, const LevelT<R> &
             v = fma((R)((1.0 - F.omega) / F.omega), gb, v);
         });
     }
-    restrict_pairs<R>(c, v, sres, bx, bz);
+    restrict_pairs<R>(c, v, sres, bx, bz, rows);
     __syncthreads();
 }
 
@@ -1057,7 +1059,7 @@ __device__ __forceinline__ void ph_mg_down(const LevelT<R> &f, const LevelT<R> &
 // correction. DOT (on the finest level): acc += r z.
 template <bool DOT, class R>
 __device__ __forceinline__ void ph_mg_up(const LevelT<R> &f, const R *res, const R *ec, int Pc, R *out, const Phys &F,
-                                         double *sm, int bx, int bz, R (&acc)[1])
+                                         double *sm, int bx, int bz, R (&acc)[1], int rows = BZ)
 {
     const Geom &G = f.G;
     PairTile<2, R> &st = pair_tile<2, R>(sm, 0);
@@ -1065,7 +1067,7 @@ __device__ __forceinline__ void ph_mg_up(const LevelT<R> &f, const R *res, const
     fill_pairs<2, true, R>(st, G, bx, bz, [&](int q, int, int jj, int kk) {
         const R r = ld(&res[q]), w = ld(&f.wd[q]);
         return ec ? fma(w, r, ld(&ec[(kk >> 1) * Pc + jj])) : w * r;
-    });
+    }, rows);
     __syncthreads();
     fill_next<false, R>(sz, G, bx, bz, [&](int q, int, int tk, int tj, int s) {
         const R r = ld(&res[q]);
@@ -1074,17 +1076,17 @@ __device__ __forceinline__ void ph_mg_up(const LevelT<R> &f, const R *res, const
         // the coarsest level keeps no down half: its one sweep is undamped
         rarely(F.om_ne1 && ec, [&] {
             z = fma((R)F.omega, z,
-                    (R)(1.0 - F.omega) * (ld(&f.e[q]) + ld(&ec[((bz * BZ - 1 + tk) >> 1) * Pc + bx * BX - 1 + tj])));
+                    (R)(1.0 - F.omega) * (ld(&f.e[q]) + ld(&ec[((bz * rows - 1 + tk) >> 1) * Pc + bx * BX - 1 + tj])));
         });
-        if (tk >= 1 && tk <= BZ && tj >= 1 && tj <= BX) {
+        if (tk >= 1 && tk <= rows && tj >= 1 && tj <= BX) {
             out[q] = z;
             if (DOT) acc[0] = fma(r, z, acc[0]);
         }
         return z;
-    });
+    }, rows);
     __syncthreads();
     int j, k;
-    if (pair_of(G, bx, bz, j, k)) {
+    if (pair_of(G, bx, bz, j, k, rows)) {
         const int s = k & 1, i = 2 * j + 1 - s;
         if (i < G.nx) {
             const int q = cidx(G, i, k);
