@@ -7,9 +7,10 @@
  * equation) on a uniform Cartesian x-y-z grid: x and y horizontal, z up,
  * free-slip walls on all six sides, constant viscosity mu (Remark 1) or a
  * Smagorinsky eddy viscosity, FP64.
- * The pressure equation is solved by conjugate gradients preconditioned by a
- * Galerkin geometric multigrid V(1,1) cycle (coarsening 2 x 2 x 2); the
- * solver loops run on the device inside a CUDA graph.
+ * The pressure equation is solved by conjugate gradients on the black half of a
+ * red-black colouring, preconditioned by a geometric multigrid V-cycle
+ * (coarsening 2 x 2 x 2); the solver loops run on the device inside a CUDA
+ * graph.
  *
  * Conventions
  *  - Cell fields are dense nz x ny x nx arrays, x fastest: cell (i,j,k)
