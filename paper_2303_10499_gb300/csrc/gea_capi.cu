@@ -155,7 +155,15 @@ StepArgs step_args(gea_ctx *c, int from)
 // it by 4. Coarsening continues while the ratio exceeds this bound.
 constexpr double kCoarsestRatio = 1.0;
 constexpr double kRefT = 300.0;    // reference temperature of that estimate (K)
-constexpr int kPersistTilesPerBlock = 4;
+// Tiles per resident block (456 blocks) up to which a step runs as one
+// persistent launch. Graph / persistent, us a step: FP64 1001 x 503 (4.4 tiles a
+// block) 2287 / 1783, 1280 x 720 (7.9) 2058 / 1801, 1440 x 900 (11) 3335 / 3154,
+// 1701 x 1001 (15) 5354 / 4515, 2048 x 1024 (18) 4946 / 4903, 2560 x 1280 (28)
+// 7900 / 8120; mixed 1001 x 503 1075 / 959, 1280 x 720 1202 / 1144, 1440 x 900
+// 1661 / 1743, 1701 x 1001 2508 / 2420, 2048 x 1024 2473 / 2676. The graph's kernels
+// keep more blocks an SM in flight, the persistent step has no launches and
+// gaps between its phases; FP32 phases are short, so their line lies lower.
+constexpr int kPersistTilesPerBlock = 16, kPersistTilesPerBlockMixed = 8;
 constexpr double kMixedRtol = 1e-5;  // default tolerance of the FP32 solves (relative to ||r0||)
 
 // Append a WHILE conditional node to the graph being captured on `s`; its
@@ -850,14 +858,14 @@ int gea_create(const gea_grid *grid, const gea_constants *c, gea_ctx **out)
     }
     for (int e = 0; e < 8; ++e) cudaEventCreate(&ctx->ev[e]);
     ctx->nev = 8;
-    // step driver: the persistent kernel pays off while a phase is a few
-    // tiles per resident block (its phases are latency-bound); on larger
-    // grids the per-phase kernels keep more blocks resident per SM
+    // step driver: the persistent kernel pays off up to some tiles per resident
+    // block; on larger grids the per-phase kernels keep more blocks resident per SM
     if (!(c->flags & (GEA_FLAG_GRAPH | GEA_FLAG_KEEP_R0))) {
         const PersistOps &o = persist_ops(ctx->shape);
         const int pmax = ctx->mixed ? o.mixed_max_blocks() : o.max_blocks();
         cudaGetLastError();
-        if (pmax > 0 && (long long)nb <= (long long)kPersistTilesPerBlock * pmax)
+        const int most = ctx->mixed ? kPersistTilesPerBlockMixed : kPersistTilesPerBlock;
+        if (pmax > 0 && (long long)nb <= (long long)most * pmax)
             ctx->pers_blocks = pmax < (int)nb ? pmax : (int)nb;
     }
     if (cudaStreamCreateWithFlags(&ctx->cap, cudaStreamNonBlocking) != cudaSuccess ||
