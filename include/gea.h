@@ -86,9 +86,9 @@ typedef struct gea_grid {
  *            at most this many cells (a value >= nx*nz gives one level).
  *  flags     GEA_FLAG_GRAPH: always run steps as a CUDA graph of per-phase
  *            kernels. By default the library picks the persistent
- *            cooperative kernel when the grid has at most 4 tiles (32 x 8
- *            cells) per block that fits on the GPU at once, where a phase is
- *            latency-bound, and the graph otherwise.
+ *            cooperative kernel when the grid has at most 16 tiles (32 x 8
+ *            cells; mixed precision 8) per block that fits on the GPU at
+ *            once, and the graph otherwise.
  *            GEA_FLAG_MIXED: mixed-precision step (the driver is chosen as
  *            for the FP64 step; with GEA_FLAG_GRAPH the graph). The
  *            state, the hydrostatic split p' = p + rho g z, the face forces,
