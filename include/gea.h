@@ -211,10 +211,14 @@ int gea_set_state(gea_ctx *ctx, const gea_state_view *v);
  * are enqueued and the status of the finished steps has been read back,
  * i.e. it synchronises the stream once at the end. On GEA_ERR_NOCONV,
  * GEA_ERR_NONFINITE or GEA_ERR_TIMEOUT the state stays at the last completed
- * step. With the persistent driver all n steps run in one cooperative kernel
+ * step. With the persistent driver the n steps run in one cooperative kernel
  * launch whose blocks stay resident (grid barriers between phases, solver
- * loops on the device); with the graph driver each step is one CUDA graph
- * launch (see gea_constants.flags). */
+ * loops on the device), on grids of more than 4 tiles per resident block each
+ * step in a launch of its own; with the graph driver each step is one CUDA
+ * graph launch (see gea_constants.flags). A persistent launch holds the SMs:
+ * work of other streams that does not fit beside its blocks waits for its end,
+ * where the graph's kernels let it in between; GEA_FLAG_GRAPH is for programs
+ * that need that. */
 int gea_step(gea_ctx *ctx, int32_t n);
 
 /* Enqueue n steps without waiting; gea_sync reports their status. */

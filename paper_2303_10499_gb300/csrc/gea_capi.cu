@@ -66,6 +66,7 @@ struct gea_ctx {
     bool have_state = false;
     int base = 0;                         // state slot loaded by the last set_state
     int pers_blocks = 0;                  // persistent-kernel grid (0: graph path only)
+    int pers_steps = INT_MAX;             // steps of one persistent launch at most
     long long wait_polls = -1;            // grid-barrier poll limit of the persistent kernels (< 0: default)
     unsigned long long *trace = nullptr;  // phase trace of the persistent kernels (gea_set_trace; not owned)
     int trace_bars = 0;
@@ -164,6 +165,13 @@ constexpr double kRefT = 300.0;    // reference temperature of that estimate (K)
 // keep more blocks an SM in flight, the persistent step has no launches and
 // gaps between its phases; FP32 phases are short, so their line lies lower.
 constexpr int kPersistTilesPerBlock = 16, kPersistTilesPerBlockMixed = 8;
+// A persistent launch holds the SMs until it ends, so work of other streams
+// that does not fit beside its blocks waits. Up to this many tiles a block
+// (steps of up to about 1 ms) all steps of a call are one launch; above it each
+// step is one, and the others get their turn between two steps. A step of
+// 160 x 80 beside a call of 20 steps on another stream: at 1001 x 503 1374 us
+// (all steps one launch 22564, graph 614), at 1280 x 720 2080 (36779, graph 647).
+constexpr int kPersistTilesAllSteps = 4;
 constexpr double kMixedRtol = 1e-5;  // default tolerance of the FP32 solves (relative to ||r0||)
 
 // Append a WHILE conditional node to the graph being captured on `s`; its
@@ -867,6 +875,7 @@ int gea_create(const gea_grid *grid, const gea_constants *c, gea_ctx **out)
         const int most = ctx->mixed ? kPersistTilesPerBlockMixed : kPersistTilesPerBlock;
         if (pmax > 0 && (long long)nb <= (long long)most * pmax)
             ctx->pers_blocks = pmax < (int)nb ? pmax : (int)nb;
+        if ((long long)nb > (long long)kPersistTilesAllSteps * pmax) ctx->pers_steps = 1;
     }
     if (cudaStreamCreateWithFlags(&ctx->cap, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&ctx->cap2, cudaStreamNonBlocking) != cudaSuccess ||
@@ -971,16 +980,19 @@ int gea_step_async(gea_ctx *ctx, int32_t n)
     if (n == 0) return GEA_OK;
     if (ctx->pers_blocks > 0 && !ctx->net) {
         StepArgs a[2] = {step_args(ctx, 0), step_args(ctx, 1)};
-        const int first = (int)((ctx->base + ctx->steps_at_sync) & 1);
         const PersistOps &o = persist_ops(ctx->shape);
-        if (ctx->mixed)
-            CK(o.launch_mixed(a, ctx->L[0], ctx->mx, ctx->Lf.data(), (int)ctx->Lf.size(), ctx->C.n_corr, ctx->C.jac_maxit, ctx->C.cg_maxit, first, n,
-                                       ctx->pers_blocks, ctx->wait_polls, ctx->stream));
-        else
-            CK(o.launch(a, ctx->L.data(), (int)ctx->L.size(), ctx->C.n_corr,
-                                 ctx->C.jac_maxit, ctx->C.cg_maxit, first, n, ctx->pers_blocks,
-                                 ctx->wait_polls, ctx->stream));
-        ctx->steps_at_sync += n;
+        for (int done = 0, k; done < n; done += k) {
+            k = std::min(n - done, ctx->pers_steps);
+            const int first = (int)((ctx->base + ctx->steps_at_sync) & 1);
+            if (ctx->mixed)
+                CK(o.launch_mixed(a, ctx->L[0], ctx->mx, ctx->Lf.data(), (int)ctx->Lf.size(), ctx->C.n_corr,
+                                  ctx->C.jac_maxit, ctx->C.cg_maxit, first, k, ctx->pers_blocks, ctx->wait_polls,
+                                  ctx->stream));
+            else
+                CK(o.launch(a, ctx->L.data(), (int)ctx->L.size(), ctx->C.n_corr, ctx->C.jac_maxit, ctx->C.cg_maxit,
+                            first, k, ctx->pers_blocks, ctx->wait_polls, ctx->stream));
+            ctx->steps_at_sync += k;
+        }
         return GEA_OK;
     }
     int rc = ensure_graphs(ctx);
