@@ -14,6 +14,8 @@
 #include "../../include/gea.h"
 #include "../../include/gea_net.h"
 
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <nvtx3/nvToolsExt.h>
 #include <limits.h>
 #include <stdarg.h>
@@ -96,9 +98,11 @@ int fail(gea_ctx *c, int code, const char *fmt, ...)
 #define CK(call)                                                                           \
     do {                                                                                   \
         cudaError_t e_ = (call);                                                           \
-        if (e_ != cudaSuccess)                                                             \
+        if (e_ != cudaSuccess) {                                                           \
+            cudaGetLastError();   /* reported here, not by the next call's launch check */ \
             return fail(ctx, GEA_ERR_CUDA, "%s: %s (%s:%d)", #call, cudaGetErrorString(e_), \
                         __FILE__, __LINE__);                                               \
+        }                                                                                  \
     } while (0)
 
 size_t round_up(size_t x, size_t m) { return (x + m - 1) / m * m; }
@@ -580,20 +584,55 @@ DenseFields dense_fields(const gea_state_view *v, int nf)
     return d;
 }
 
-// Whether the non-null pointers are plain device memory of the context's
-// device, which a kernel may access directly (managed and host pointers, and
-// another device's, go through the runtime's copies whatever the caller's mem).
-bool on_device(const gea_ctx *ctx, double *const *p, int n)
+// Columns, rows and values of a full view's arrays.
+struct FieldShape {
+    int cols[NFIELDS], rows[NFIELDS];
+    size_t count[NFIELDS];
+    explicit FieldShape(const Geom &G)
+    {
+        for (int f = 0; f < NFIELDS; ++f) {
+            cols[f] = f == FIELD_PHIX ? G.nx + 1 : G.nx;
+            rows[f] = f == FIELD_PHIZ ? G.nz + 1 : G.nz;
+            count[f] = (size_t)cols[f] * rows[f];
+        }
+    }
+};
+
+// Whether the non-null arrays (count[f] values each) are plain device memory of
+// the context's device from end to end, which a kernel may access directly.
+// Managed and host pointers, another device's, and arrays that run past their
+// allocation go through the runtime's copies whatever the caller's mem: the
+// runtime serves the first and refuses the last, which a kernel would access
+// out of bounds. (An array over several mappings of one virtual range takes
+// the copies too.)
+bool on_device(const gea_ctx *ctx, double *const *p, const size_t *count, int n)
 {
+    static const PFN_cuPointerGetAttributes_v7000 query = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 7000, cudaEnableDefault, &found) !=
+                cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<PFN_cuPointerGetAttributes_v7000>(f);
+    }();
+    if (!query) return false;
     for (int f = 0; f < n; ++f) {
         if (!p[f]) continue;
-        cudaPointerAttributes at;
-        if (cudaPointerGetAttributes(&at, p[f]) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        if (at.type != cudaMemoryTypeDevice || at.device != ctx->device ||
-            reinterpret_cast<uintptr_t>(p[f]) % sizeof(double))
+        unsigned type = 0, managed = 0;
+        int device = -1;
+        unsigned long long start = 0;
+        size_t size = 0;
+        CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                      CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                      CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+        void *into[] = {&type, &managed, &device, &start, &size};
+        const unsigned long long a = reinterpret_cast<uintptr_t>(p[f]);
+        if (query(5, what, into, a) != CUDA_SUCCESS) return false;
+        if (type != CU_MEMORYTYPE_DEVICE || managed || device != ctx->device || a % sizeof(double) || a < start ||
+            count[f] * sizeof(double) > size - (a - start))
             return false;
     }
     return true;
@@ -906,6 +945,7 @@ int gea_set_state(gea_ctx *ctx, const gea_state_view *v)
     double *dst[11] = {S.rho, S.u, S.w, S.T, S.h, S.p, S.pp, S.pold, S.phix, S.phiz, S.Kold};
     // K^{n-1} belongs to the state only in the literal reading of eq. step3_sd
     const int nf = ctx->F.k_lagged ? 11 : 10;
+    const FieldShape shape(G);
     // arguments are checked before the context is touched
     if (v->kind == GEA_STATE_CONSERVATIVE) {
         if (!v->rhou || !v->rhow || !v->rhoe) return fail(ctx, GEA_ERR_INVAL, "null conservative field");
@@ -925,7 +965,8 @@ int gea_set_state(gea_ctx *ctx, const gea_state_view *v)
         const size_t cellw = ctx->stage_stride;
         double *st = ctx->stage;
         int rc;
-        if (v->mem == GEA_MEM_DEVICE && on_device(ctx, in, 4)) {
+        const size_t cells = (size_t)nx * nz, count[4] = {cells, cells, cells, cells};
+        if (v->mem == GEA_MEM_DEVICE && on_device(ctx, in, count, 4)) {
             launch_derive(G, ctx->F, v->rho, v->rhou, v->rhow, v->rhoe, nx, ctx->gzc, S, ctx->sc, ctx->stream);
         } else {
             for (int f = 0; f < 4; ++f)
@@ -933,15 +974,12 @@ int gea_set_state(gea_ctx *ctx, const gea_state_view *v)
             launch_derive(G, ctx->F, st, st + cellw, st + 2 * cellw, st + 3 * cellw, G.P, ctx->gzc, S, ctx->sc, ctx->stream);
         }
         CK(cudaGetLastError());
-    } else if (DenseFields d = dense_fields(v, nf); v->mem == GEA_MEM_DEVICE && on_device(ctx, d.p, nf)) {
+    } else if (DenseFields d = dense_fields(v, nf); v->mem == GEA_MEM_DEVICE && on_device(ctx, d.p, shape.count, nf)) {
         launch_fields_in(G, S, d, ctx->stream);
         CK(cudaGetLastError());
     } else {
-        for (int f = 0; f < nf; ++f) {
-            const int cols = f == 8 ? nx + 1 : nx, rows = f == 9 ? nz + 1 : nz;
-            int rc = copy_in(ctx, dst[f], src[f], cols, rows);
-            if (rc) return rc;
-        }
+        for (int f = 0; f < nf; ++f)
+            if (int rc = copy_in(ctx, dst[f], src[f], shape.cols[f], shape.rows[f])) return rc;
     }
     if (v->kind == GEA_STATE_FULL) {
         // a full state is taken as given (only the derivation from the
@@ -1041,14 +1079,8 @@ int gea_get_state(gea_ctx *ctx, gea_state_view *v)
     if (v->kind == GEA_STATE_FULL) {
         const int nf = ctx->F.k_lagged ? 11 : 10;
         const DenseFields d = dense_fields(v, nf);
-        int cols[NFIELDS], rows[NFIELDS];
-        size_t count[NFIELDS];
-        for (int f = 0; f < nf; ++f) {
-            cols[f] = f == FIELD_PHIX ? nx + 1 : nx;
-            rows[f] = f == FIELD_PHIZ ? nz + 1 : nz;
-            count[f] = (size_t)cols[f] * rows[f];
-        }
-        if (v->mem == GEA_MEM_DEVICE && on_device(ctx, d.p, nf) && disjoint(d.p, count, nf)) {
+        const FieldShape shape(G);
+        if (v->mem == GEA_MEM_DEVICE && on_device(ctx, d.p, shape.count, nf) && disjoint(d.p, shape.count, nf)) {
             launch_fields_out(G, ctx->S, ctx->base, ctx->sc, d, ctx->stream);
             CK(cudaGetLastError());
         } else {
@@ -1056,12 +1088,12 @@ int gea_get_state(gea_ctx *ctx, gea_state_view *v)
             if ((rc = read_scal(ctx, &h))) return rc;
             const FieldPtrs src = state_fields(ctx->S[current_slot(ctx, h)]);
             for (int f = 0; f < nf; ++f)
-                if (d.p[f] && (rc = copy_out(ctx, d.p[f], src.p[f], cols[f], rows[f]))) return rc;
+                if (d.p[f] && (rc = copy_out(ctx, d.p[f], src.p[f], shape.cols[f], shape.rows[f]))) return rc;
         }
     } else {
         double *const dst[4] = {v->rho, v->rhou, v->rhow, v->rhoe};
         const size_t cells = (size_t)nx * nz, count[4] = {cells, cells, cells, cells};
-        if (v->mem == GEA_MEM_DEVICE && on_device(ctx, dst, 4) && disjoint(dst, count, 4)) {
+        if (v->mem == GEA_MEM_DEVICE && on_device(ctx, dst, count, 4) && disjoint(dst, count, 4)) {
             launch_conserve(G, ctx->F, ctx->S, ctx->base, ctx->sc, v->rho, v->rhou, v->rhow, v->rhoe, nx, ctx->stream);
             CK(cudaGetLastError());
         } else {
