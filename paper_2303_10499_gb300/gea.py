@@ -487,8 +487,11 @@ class Solver:
         each candidate number of tiles a block walks, one untimed step (which
         records the step graph) and `steps` timed steps (gea_step
         synchronises, so host time brackets the device work); keeps the
-        fastest. The state advances by len(candidates) x (steps + 1) steps."""
+        fastest. The state advances by len(candidates) x (steps + 1) steps.
+        Steps of the persistent kernel have no tile columns: their times say
+        nothing about the candidates, and the size rule (0) stays."""
         import time
+        persistent = self.stats()["driver"].endswith("persistent")
         times = {}
         for n in candidates:
             self.set_tiles_per_block(n)
@@ -496,7 +499,7 @@ class Solver:
             t0 = time.perf_counter()
             self.step(steps)
             times[int(n)] = (time.perf_counter() - t0) / steps * 1e3
-        best = min(times, key=times.get)
+        best = 0 if persistent else min(times, key=times.get)
         self.set_tiles_per_block(best)
         return {"ms_per_step": times, "tiles_per_block": best}
 
