@@ -57,6 +57,7 @@ constexpr LayerDef kL[L] = {
 constexpr int kOut = L - 1;
 constexpr int kThreads = 256;
 constexpr int kWgPix = 64;       // pixels of a weight-gradient row segment at most
+constexpr int kWgChain = 256;    // terms of one thread's running weight-gradient sum at most (k_wgrad)
 
 __device__ __forceinline__ float bf2f(uint16_t u) { return __uint_as_float((uint32_t)u << 16); }
 __device__ __forceinline__ uint16_t f2bf(float f)
@@ -373,6 +374,16 @@ __global__ void k_form_input(int n, int h, int w, int c4, const uint2 *x0, const
 // (64 -> 64, a quarter of the size), 33 TFLOP/s; with the sums over the blocks
 // in parallel and first gradients written in place the backward pass went
 // from 6.46 to 1.2 ms.
+//
+// A thread's running sums end after kWgChain terms, so that a larger batch
+// does not lose bits: sums of equal terms, the worst case, are off by 2.4e-6 at
+// 12 x 256 x 256 and 3.2e-6 at 64 x 512 x 512 (running through all of a
+// block's items 4.1e-6 and 7.0e-5; one accumulator per thread and tap with
+// 128-pixel partial sums 2.9e-6 and 1.4e-5). Of 64 / 128 / 256 / 512 terms, 256 is
+// the longest that is no further off at any size than those partial sums. The
+// split is by launches: the sums added to the block's partial inside the
+// kernel took 1 to 2 % more at 8 x 256 x 256, where one launch holds all items
+// (1300 us before and 1292 after; 4 x 1024 x 1024: 6763 -> 7284).
 
 struct WgArgs {
     int n, h, w;            // the layer's size
@@ -383,6 +394,7 @@ struct WgArgs {
     int strips, pt;         // row segments per row and their pixels
     int rb, chunks;         // rows of a work item and items per column of segments
     int items;              // n x strips x chunks
+    int first, last, add;   // the launch's items; add: to the partials of the launches before
 };
 
 // First pixel, rows and sample of item t.
@@ -432,7 +444,7 @@ __global__ void __launch_bounds__(WgShape<CIN, COUT, GR>::THREADS, 768 / WgShape
         for (int c = 0; c < 4; ++c)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[t][c][i] = 0.0f;
-    for (int t = blockIdx.x; t < a.items; t += gridDim.x) {
+    for (int t = a.first + blockIdx.x; t < a.last; t += gridDim.x) {
         int b, x0, y0, y1;
         wg_item(a, t, b, x0, y0, y1);
         // input row y into slot (y - y0 + 1) & 3, pixels x0 - 1 .. x0 + pt, zero outside the image
@@ -519,12 +531,17 @@ __global__ void __launch_bounds__(WgShape<CIN, COUT, GR>::THREADS, 768 / WgShape
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-            *reinterpret_cast<float4 *>(out + ((size_t)(dy * 3 + k) * COUT + co + c) * CIN + ci) =
-                make_float4(acc[k][c][0], acc[k][c][1], acc[k][c][2], acc[k][c][3]);
+        for (int c = 0; c < 4; ++c) {
+            float4 *p = reinterpret_cast<float4 *>(out + ((size_t)(dy * 3 + k) * COUT + co + c) * CIN + ci);
+            const float4 u = a.add ? *p : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            *p = make_float4(u.x + acc[k][c][0], u.y + acc[k][c][1], u.z + acc[k][c][2], u.w + acc[k][c][3]);
+        }
     if (bias)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) a.partb[(size_t)blockIdx.x * COUT + co + c] = accb[c];
+        for (int c = 0; c < 4; ++c) {
+            float *p = a.partb + (size_t)blockIdx.x * COUT + co + c;
+            *p = (a.add ? *p : 0.0f) + accb[c];
+        }
 }
 
 // The first layer (one input channel, 16 outputs): a thread keeps the 9 taps
@@ -538,7 +555,7 @@ __global__ void __launch_bounds__(kThreads) k_wgrad_first(WgArgs a)
     float acc[40];   // 9 taps x 4 outputs, then db
 #pragma unroll
     for (int k = 0; k < 40; ++k) acc[k] = 0.0f;
-    for (int t = blockIdx.x; t < a.items; t += gridDim.x) {
+    for (int t = a.first + blockIdx.x; t < a.last; t += gridDim.x) {
         int b, x0, y0, y1;
         wg_item(a, t, b, x0, y0, y1);
         const int xx = x0 + px;
@@ -584,8 +601,8 @@ __global__ void __launch_bounds__(kThreads) k_wgrad_first(WgArgs a)
     if (j < 160) {
         float s = 0.0f;
         for (int q = 0; q < kThreads / 32; ++q) s += red[q][j];
-        if (j < 144) a.part[(size_t)blockIdx.x * 144 + j] = s;
-        else a.partb[(size_t)blockIdx.x * 16 + j - 144] = s;
+        float *p = j < 144 ? a.part + (size_t)blockIdx.x * 144 + j : a.partb + (size_t)blockIdx.x * 16 + j - 144;
+        *p = (a.add ? *p : 0.0f) + s;
     }
 }
 
@@ -700,12 +717,12 @@ inline unsigned blocks(long long cnt) { return (unsigned)((cnt + kThreads - 1) /
 // Weight-gradient kernel of a layer: its function, threads and shared memory.
 struct WgKernel {
     void (*f)(WgArgs);
-    int threads, smem;
+    int threads, smem, groups;   // groups: of a segment's pixels, each summed by threads of its own
 };
 template <int CIN, int COUT, int GR>
 constexpr WgKernel wg_of()
 {
-    return WgKernel{k_wgrad<CIN, COUT, GR>, WgShape<CIN, COUT, GR>::THREADS, WgShape<CIN, COUT, GR>::SMEM};
+    return WgKernel{k_wgrad<CIN, COUT, GR>, WgShape<CIN, COUT, GR>::THREADS, WgShape<CIN, COUT, GR>::SMEM, GR};
 }
 // Pixel groups: a block of 192 threads (48 or 96 per group) keeps several
 // blocks on an SM; from 32 x 32 on one group fills it.
@@ -719,7 +736,7 @@ inline WgKernel wg_kernel(int cin, int cout)
     case 3264: return wg_of<32, 64, 1>();
     case 6432: return wg_of<64, 32, 1>();
     case 6464: return wg_of<64, 64, 1>();
-    default: return WgKernel{k_wgrad_first, kThreads, 0};
+    default: return WgKernel{k_wgrad_first, kThreads, 0, kWgPix};
     }
 }
 
@@ -835,17 +852,20 @@ int forward(gea_net *net, int n, int h, int w, const float *r, float *y)
     return GEA_OK;
 }
 
-// Split of a weight gradient over `slots` resident blocks: row segments of at
-// most kWgPix pixels, and as many rows per work item as make the longest
-// block's rows (plus the item's two extra input rows) fewest. Returns the
-// blocks to launch.
-int wgrad_split(WgArgs &a, int n, int h, int w, int slots)
+// Weight gradient of a layer into block partials, on at most `slots` resident
+// blocks: row segments of at most kWgPix pixels, and as many rows per work item as
+// make the longest block's rows (an item costs one more, for its first rows'
+// loads, which nothing overlaps) fewest, within a thread's kWgChain terms. Items
+// beyond those terms go to further launches, which add to the same partials.
+// Returns the number of partials.
+int wgrad(WgArgs &a, const WgKernel &k, int n, int h, int w, int slots, cudaStream_t st)
 {
     a.n = n; a.h = h; a.w = w;
     a.strips = (w + kWgPix - 1) / kWgPix;
     a.pt = (w + a.strips - 1) / a.strips;
+    const int pg = (a.pt + k.groups - 1) / k.groups;   // pixels of a row that one thread walks
     long long best = -1;
-    for (int rb = 1; rb <= h; ++rb) {
+    for (int rb = 1; rb <= std::min(h, kWgChain / pg); ++rb) {
         const int chunks = (h + rb - 1) / rb;
         const long long items = (long long)n * a.strips * chunks;
         const long long cost = (items + slots - 1) / slots * (rb + 1);
@@ -856,7 +876,12 @@ int wgrad_split(WgArgs &a, int n, int h, int w, int slots)
             a.items = (int)items;
         }
     }
-    return a.items < slots ? a.items : slots;
+    const int ns = std::min(a.items, slots), step = ns * (kWgChain / (a.rb * pg));
+    for (a.first = 0, a.add = 0; a.first < a.items; a.first = a.last, a.add = 1) {
+        a.last = std::min(a.first + step, a.items);
+        k.f<<<std::min(ns, a.last - a.first), k.threads, k.smem, st>>>(a);
+    }
+    return ns;
 }
 
 int backward(gea_net *net, const float *dy, float *grad)
@@ -899,9 +924,7 @@ int backward(gea_net *net, const float *dy, float *grad)
         }
         a.g = net->gact[l];
         a.part = net->part; a.partb = net->partb;
-        const int ns = wgrad_split(a, n, hl, wl, net->wg_blocks[l]);
-        const WgKernel k = wg_kernel(d.cin, d.cout);
-        k.f<<<ns, k.threads, k.smem, st>>>(a);
+        const int ns = wgrad(a, wg_kernel(d.cin, d.cout), n, hl, wl, net->wg_blocks[l], st);
         k_wgrad_reduce<<<(9 * d.cin * d.cout + d.cout + 31) / 32, dim3(32, 8), 0, st>>>(
             net->part, net->partb, ns, d.cin, d.cout, grad + net->offw[l], grad + net->offb[l]);
         if (l == 0) break;
