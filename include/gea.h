@@ -344,11 +344,12 @@ int gea_set_trace(gea_ctx *ctx, uint64_t *trace, int32_t max_barriers, int64_t c
 int gea_get_field(gea_ctx *ctx, int32_t which, double *host);
 
 /* Apply the pressure solve's preconditioner to r: z = M r with M one
- * V(1,1)-cycle of the multigrid hierarchy of the last completed step, with a
- * red-black Gauss-Seidel smoother (red then black before the coarse
- * correction, black then red after it)
- * (the operator of eq. p_prime_sd in its Helmholtz form, as the CG of Step 3
- * uses it; one symmetric red-black sweep when the hierarchy has one level). r, z:
+ * V(1,1)-cycle of the multigrid hierarchy of the last completed step (the
+ * operator of eq. p_prime_sd in its Helmholtz form), with a red-black
+ * Gauss-Seidel smoother (red then black before the coarse correction, black
+ * then red after it); one symmetric red-black sweep when the hierarchy has one
+ * level. The CG of Step 3 works on the black cells (i + k even) with the black
+ * half of M: its z is the black part of M r for r with zero red part. r, z:
  * nz*nx doubles, host or device. Lets a caller check what CG needs of M: it
  * is linear, symmetric and positive definite. FP64 contexts only.
  * Synchronises. Errors: GEA_ERR_INVAL (null pointers, a mixed-precision
