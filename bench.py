@@ -35,17 +35,21 @@ UNIT = "cell-steps/s"
 # once plus written once (an FP32 value is half a word), and operations (add,
 # mul, div, sqrt each 1; an FMA counts 2) in the precision named last.
 # Coarse-level multigrid kernels are per cell of the level they run on.
-# Derivations are in the design notes. The mx_ kernels are the
-# mixed-precision step.
+# A value that several threads form (halos, the other colour's cells) counts
+# once, a reciprocal as one operation; LES and Pr != 1 terms are not counted.
+# Rows of kernels that serve both steps count what both do ("correct": the FP64
+# operations of the mixed one). The counts lie at or below the instructions
+# that ncu counted (profiles/executed_ops.json, tests/test_flop_model.py). The
+# mx_ kernels are the mixed-precision step.
 KERNEL_MODEL = {
-    "pred_setup": (22, 66, "f64"),
+    "pred_setup": (22, 51, "f64"),
     "mom_jacobi": (16, 44, "f64"),
-    "enth_rhs": (13, 41, "f64"),
+    "enth_rhs": (13, 45, "f64"),
     "enth_jacobi": (13, 22, "f64"),
-    "eos_coef": (16, 33, "f64"),
-    "mg_coarsen": (17, 18, "f64"),
-    "H": (17, 44, "f64"),
-    "helm_rhs": (13, 51, "f64"),
+    "eos_coef": (16, 25, "f64"),
+    "mg_coarsen": (17, 17, "f64"),
+    "H": (17, 41, "f64"),
+    "helm_rhs": (13, 44, "f64"),
     "mg_down": (4.25, 9, "f64"),
     "mg_coarse": (5, 9.5, "f64"),
     "mg_up": (5.25, 10, "f64"),
@@ -54,14 +58,14 @@ KERNEL_MODEL = {
     "cg_pspmv": (5, 10.5, "f64"),
     "cg_update_single": (4, 4.5, "f64"),
     "cg_update_down": (5.75, 7.5, "f64"),
-    "correct": (20.5, 43.5, "f64"),
-    "mx_pred": (23.5, 104, "f64"),
-    "mx_mom": (8, 46, "f32"),
-    "mx_enth_rhs": (23.5, 70, "f64"),
-    "mx_enth": (6.5, 31, "f32"),
-    "mx_eos": (18, 33, "f64"),
-    "mx_coarsen": (8.5, 18, "f32"),
-    "mx_helm_rhs": (12.5, 51, "f64"),
+    "correct": (20.5, 30, "f64"),
+    "mx_pred": (23.5, 87, "f64"),
+    "mx_mom": (8, 44, "f32"),
+    "mx_enth_rhs": (23.5, 65, "f64"),
+    "mx_enth": (6.5, 22, "f32"),
+    "mx_eos": (18, 26, "f64"),
+    "mx_coarsen": (8.5, 17, "f32"),
+    "mx_helm_rhs": (12.5, 44, "f64"),
     "mx_mg_down": (2.125, 9, "f32"),
     "mx_mg_coarse": (2.5, 9.5, "f32"),
     "mx_mg_up": (2.625, 10, "f32"),
@@ -713,42 +717,42 @@ def run_ensemble(args):
 # Per-cell model of the three-dimensional kernels (same conventions as
 # KERNEL_MODEL; coarsening and restriction per coarse cell).
 KERNEL_MODEL_3D = {
-    "g3_les": (5, 60, "f64"),
-    "g3_mx_r0mom": (31.5, 87, "f64"),
-    "g3_mx_mom": (11.5, 93, "f32"),
+    "g3_les": (5, 37, "f64"),
+    "g3_mx_r0mom": (31.5, 84, "f64"),
+    "g3_mx_mom": (11.5, 87, "f32"),
     "g3_mx_u1": (7.5, 3, "f64"),
-    "g3_mx_r0h": (16.5, 31, "f64"),
-    "g3_mx_enth": (8.5, 31, "f32"),
+    "g3_mx_r0h": (16.5, 28, "f64"),
+    "g3_mx_enth": (8.5, 29, "f32"),
     "g3_mx_h1": (2.5, 1, "f64"),
-    "g3_mx_rb_start": (2.8, 7, "f32"),
-    "g3_mx_pupd": (0.75, 1, "f32"),
+    "g3_mx_rb_start": (2.8, 6.5, "f32"),
+    "g3_mx_pupd": (0.75, 0.75, "f32"),
     "g3_mx_spmv_red": (2.25, 6.5, "f32"),
-    "g3_mx_spmv_black": (2.5, 8, "f32"),
+    "g3_mx_spmv_black": (2.5, 7.5, "f32"),
     "g3_mx_update": (1.9, 3.5, "f32"),
     "g3_mx_mg_up": (2.6, 8, "f32"),
-    "g3_mx_solution": (4.25, 8, "f32"),
-    "g3_pred": (31, 102, "f64"),
-    "g3_mom": (23, 93, "f64"),
+    "g3_mx_solution": (4.25, 6.5, "f32"),
+    "g3_pred": (31, 72, "f64"),
+    "g3_mom": (23, 90, "f64"),
     "g3_kin": (4, 6, "f64"),
-    "g3_enth_rhs": (15, 45, "f64"),
-    "g3_enth": (17, 31, "f64"),
+    "g3_enth_rhs": (15, 56, "f64"),
+    "g3_enth": (17, 30, "f64"),
     "g3_eos": (9, 7, "f64"),
-    "g3_faces": (8, 15, "f64"),
-    "g3_diag": (7, 13, "f64"),
-    "g3_coarsen": (38, 32, "f64"),
-    "g3_H": (24, 87, "f64"),
-    "g3_helm_rhs": (16.5, 71, "f64"),
-    "g3_rb_start": (5.5, 7, "f64"),
+    "g3_faces": (8, 18, "f64"),
+    "g3_diag": (7, 6, "f64"),
+    "g3_coarsen": (38, 44, "f64"),
+    "g3_H": (24, 84, "f64"),
+    "g3_helm_rhs": (16.5, 61.5, "f64"),
+    "g3_rb_start": (5.5, 6, "f64"),
     "g3_mg_down": (14.5, 49, "f32"),
-    "g3_mg_black": (2.8, 14, "f32"),
-    "g3_mg_red": (2.5, 7, "f32"),
-    "g3_mg_up": (2.8, 8, "f32"),
+    "g3_mg_black": (2.8, 7.5, "f32"),
+    "g3_mg_red": (2.5, 6.5, "f32"),
+    "g3_mg_up": (2.8, 7, "f32"),
     "g3_pupd": (1.25, 1, "f64"),
     "g3_spmv_red": (4.5, 6.5, "f64"),
-    "g3_spmv_black": (5, 8, "f64"),
+    "g3_spmv_black": (5, 7.5, "f64"),
     "g3_update": (3.5, 3.5, "f64"),
-    "g3_solution": (6.5, 8, "f64"),
-    "g3_correct": (20, 61, "f64"),
+    "g3_solution": (6.5, 7.5, "f64"),
+    "g3_correct": (20, 52, "f64"),
 }
 
 
