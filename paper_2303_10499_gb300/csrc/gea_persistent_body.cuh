@@ -29,8 +29,12 @@ namespace {
 // values per thread a grid reduction may carry: the block-sum scratch after
 // the tile area holds kRedVals x NTHREADS doubles
 constexpr int kRedVals = 4;
-// blocks up to which one warp per value adds a grid reduction's partials
-constexpr int kDirectPartials = 128;
+// Blocks up to which one warp per value adds a grid reduction's partials. FP64 us
+// a step, one warp / all threads: 32 blocks 587 / 608, 50 blocks 562 / 576, 64 blocks
+// 593 / 606, 80 blocks 588 / 586, 100 blocks 615 / 590, 120 blocks 614 / 584 (128, where
+// no lane has a partial more than another, 581 / 592): with two partials a
+// lane and fewer the pass through shared memory costs more than the loads.
+constexpr int kDirectPartials = 64;
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
 {
@@ -189,7 +193,7 @@ __device__ __forceinline__ void rbar(const Grp &g, const T (&v)[NV], double *red
     double tot[NV];
     if (nb <= kDirectPartials) {
         // few blocks: warp j adds the partials of value j at once, without the
-        // pass through shared memory (four per lane and the shuffle tree)
+        // pass through shared memory (two per lane and the shuffle tree)
         const int lane = tid & 31;
         for (int j = tid / 32; j < NV; j += NTHREADS / 32) {
             double s = 0.0;
