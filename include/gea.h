@@ -89,10 +89,9 @@ typedef struct gea_grid {
  *            cooperative kernel when the grid has at most 16 tiles (32 x 8
  *            cells; mixed precision 8) per block that fits on the GPU at
  *            once, and the graph otherwise.
- *            GEA_FLAG_MIXED: mixed-precision step (the driver is chosen as
- *            for the FP64 step; with GEA_FLAG_GRAPH the graph). The
- *            state, the hydrostatic split p' = p + rho g z, the face forces,
- *            every right-hand side and H(u) stay FP64; each of the three
+ *            GEA_FLAG_MIXED: mixed-precision step. The state, the
+ *            hydrostatic split p' = p + rho g z, the face forces, every
+ *            right-hand side and H(u) stay FP64; each of the three
  *            linear solves becomes one defect correction: an FP64 residual
  *            r0 = b - A x_old, an FP32 solve A dx = r0 (Jacobi, or multigrid
  *            CG for the pressure) to ||r|| <= mp_rtol ||r0||, and the FP64
@@ -288,10 +287,11 @@ int gea_set_tiles_per_block(gea_ctx *ctx, int32_t n);
 
 /* Weight omega of the relaxations of the black cells in the red-black
  * Gauss-Seidel smoother of the pressure solve's multigrid V-cycle (default 1;
- * the red cells are always relaxed exactly). A one-level preconditioner only
- * scales by it, which conjugate gradients do not see. Takes effect from the
- * next step; the converged pressure does not depend on it, the CG iterations
- * do. Synchronises the stream; the step graphs are recorded anew. Errors:
+ * the red cells are always relaxed exactly). A one-level hierarchy does not use
+ * it: its preconditioner is one undamped sweep, which the weight would only
+ * scale, and conjugate gradients do not see that. Takes effect from the next
+ * step; the converged pressure does not depend on it, the CG iterations of a
+ * multi-level hierarchy do. Synchronises the stream; the step graphs are recorded anew. Errors:
  * GEA_ERR_INVAL (omega outside (0, 2)). */
 int gea_set_smoother_weight(gea_ctx *ctx, double omega);
 
@@ -358,7 +358,9 @@ int gea_get_field(gea_ctx *ctx, int32_t which, double *host);
 int gea_apply_precond(gea_ctx *ctx, const double *r, double *z);
 
 /* Event-timed duration (ms) of the pressure solves (all correctors) of the
- * last step launched by gea_step/gea_step_async, or -1 if unavailable. */
+ * last step launched by gea_step/gea_step_async, or -1 if unavailable: from
+ * the right-hand side and residual to the last iteration. The correction adds the
+ * increment and forms the red half of it on its tiles, which is not included. */
 double gea_last_pressure_ms(gea_ctx *ctx);
 
 /* Per-kernel timing of one step. */
@@ -420,11 +422,12 @@ int gea_probe_fma(int32_t bits, int32_t blocks, int32_t iters, void *out, void *
 
 /* Grid-barrier latency probe (the paper has no counterpart): one cooperative
  * launch of `blocks` blocks of 256 threads (all resident at once) that pass
- * `iters` grid barriers of the protocol the persistent step kernels use
+ * `iters` grid barriers in the manner of the persistent step kernels
  * (one acquire-release arrival per block on a monotone counter, acquire
  * polls until it reaches the barrier's count), with nothing between them;
- * read_status != 0 adds the read of a status word after each barrier, as
- * those kernels do. scratch: caller-owned device memory of at least 16
+ * read_status != 0 adds the read of a status word after each barrier (the
+ * step kernels read none: a request to stop is a bit of the counter they
+ * poll). scratch: caller-owned device memory of at least 16
  * bytes, zeroed by the call; its third 32-bit word is nonzero afterwards if a
  * bounded wait (2^22 polls) gave up. Enqueued on `stream`; the caller times
  * it with CUDA events (time / iters = one barrier). Errors: GEA_ERR_INVAL

@@ -2,12 +2,14 @@
 // (Girfoglio, Quaini & Rozza, arXiv 2303.10499, Section 3) on a uniform
 // Cartesian x-y-z grid, FP64, and the C ABI of include/gea3d.h.
 //
-// One thread per cell on 32 x 8 x 1 blocks (grid z = the cell layer);
-// neighbour values are read through the read-only cache with the one-layer
+// Blocks of 32 x 8 threads: one thread per cell of a layer, or per column of a
+// few layers in the kernels with a reduction and the finest prolongation
+// (columns_of); the solve's kernels take one pair of cells of a row per thread.
+// Neighbour values are read through the read-only cache with the one-layer
 // wall ghosts applied on the fly (wall-normal velocity odd, tangential and
 // scalars even, h with dh/dz = -g). The transport operator
-// T(X) = (rho1/dt) X + C(X) - nu L(X) (fourth-order face values, 13-point
-// cross stencil) is evaluated from the face fluxes in every sweep. The
+// T(X) = (rho1/dt) X + C(X) - nu L(X) (fourth-order face values) is assembled
+// once a step as a 13-point cross stencil. The
 // pressure equation is solved by CG on the black half of a red-black colouring,
 // preconditioned with a V-cycle (piecewise-constant transfer over 2 x 2 x 2
 // cells, red-black smoothing), the loops as conditional WHILE nodes of a CUDA
@@ -1627,9 +1629,14 @@ __global__ void k_diag3(Geo G, Phy F, double p0, St S, const double *thbar, cons
 
 dim3 grid_of(const Geo &G) { return dim3((G.nx + TX - 1) / TX, (G.ny + TY - 1) / TY, G.nz); }
 // The grid of the column kernels: up to `most` layers per block, fewer where
-// that would leave less than about three waves of five blocks an SM (a grid of
-// 33 x 33 x 24 has 240 one-layer tiles in all). The light CG kernels walk up to
-// eight layers, the stencil kernels up to four.
+// that would leave less than kMinBlocks blocks, about three waves of five
+// blocks on each of 152 SMs (a grid of 33 x 33 x 24 has 240 one-layer tiles in
+// all). Lines measured in us a step, FP64 / mixed. kMinBlocks 1200, 2400, 4800:
+// 96 x 96 x 96 2274, 2237, 2237 / 1533, 1519, 1512; 192 x 192 x 96 6632, 6670,
+// 6809 / 4644, 4660, 4745; without columns 6926 / 4813. kLayersHeavy (the stencil
+// kernels) 1, 2, 4, 8 at 256 x 256 x 128: 15126, 14723, 14668, 14827 / 10740,
+// 10530, 10455, 10489. kLayers (the light CG kernels) 4, 8 and 16 differ by less
+// than 0.2 % there.
 constexpr int kLayers = 8, kLayersHeavy = 4, kMinBlocks = 2400;
 dim3 columns_of(const Geo &G, const dim3 &g, int most)
 {

@@ -223,37 +223,6 @@ struct StepArgs {
 
 __device__ __forceinline__ int cidx(const Geom &G, int i, int k) { return k * G.P + i; }
 
-// Cell value at (i,k), i in [-1, nx] and k in [-1, nz]; outside the box the
-// one-layer ghost of the wall condition: wall-normal velocity odd (zero on
-// the wall), tangential velocity and scalars even (zero gradient), h with
-// dh/dz = -g on the bottom and top walls.
-template <int BC>
-__device__ __forceinline__ double ldc(const Geom &G, const Phys &F, const double *__restrict__ X,
-                                      int i, int k)
-{
-    if (i < 0) {
-        double v = X[k * G.P];
-        return BC == BC_U ? -v : v;
-    }
-    if (i >= G.nx) {
-        double v = X[k * G.P + G.nx - 1];
-        return BC == BC_U ? -v : v;
-    }
-    if (k < 0) {
-        double v = X[i];
-        if (BC == BC_W) return -v;
-        if (BC == BC_H) return v + F.g * G.dz;
-        return v;
-    }
-    if (k >= G.nz) {
-        double v = X[(G.nz - 1) * G.P + i];
-        if (BC == BC_W) return -v;
-        if (BC == BC_H) return v - F.g * G.dz;
-        return v;
-    }
-    return X[k * G.P + i];
-}
-
 // 1 / a for a normal a (densities, temperatures, diagonals) by one step of
 // Chebyshev's third-order iteration for the reciprocal, x0 (1 + e + e^2) with
 // e = 1 - a x0, from the hardware's seed (about 20 bits, so e^3 is below the

@@ -8,7 +8,7 @@
 // forces, the right-hand sides, H(u), the flux correction -- and moves the
 // iterative solves to FP32 by defect correction: each implicit problem
 // T x = b gets one FP64 residual r0 = b - T x_old, an FP32 solve T dx = r0 to a
-// relative residual of 1e-6 (Jacobi for the predictors, multigrid-
+// relative residual of mp_rtol, 1e-5 by default (Jacobi for the predictors, multigrid-
 // preconditioned CG for the pressure equation) and the FP64 update
 // x = x_old + dx. Increments have homogeneous wall conditions (the h ghost
 // offset g dz cancels). FP32 reductions are summed per block in FP32 and

@@ -725,7 +725,10 @@ constexpr WgKernel wg_of()
     return WgKernel{k_wgrad<CIN, COUT, GR>, WgShape<CIN, COUT, GR>::THREADS, WgShape<CIN, COUT, GR>::SMEM, GR};
 }
 // Pixel groups: a block of 192 threads (48 or 96 per group) keeps several
-// blocks on an SM; from 32 x 32 on one group fills it.
+// blocks on an SM; from 32 x 32 on one group fills it. Backward pass at
+// 8 x 256 x 256, us: 16 x 16 with 1, 2, 4 groups 1622, 1301, 1295; 16 x 32 and
+// 32 x 16 with 1, 2, 4 1292, 1295, 1285; 32 x 32 with 1, 2 1295, 1290 (12 x 256 x 256:
+// 1757, 1797); 32 x 64 and 64 x 32 with 1, 2 1295, 1301.
 inline WgKernel wg_kernel(int cin, int cout)
 {
     switch (cin * 100 + cout) {
@@ -854,8 +857,10 @@ int forward(gea_net *net, int n, int h, int w, const float *r, float *y)
 
 // Weight gradient of a layer into block partials, on at most `slots` resident
 // blocks: row segments of at most kWgPix pixels, and as many rows per work item as
-// make the longest block's rows (an item costs one more, for its first rows'
-// loads, which nothing overlaps) fewest, within a thread's kWgChain terms. Items
+// make the longest block's rows fewest, within a thread's kWgChain terms. An
+// item counts one row more than it has, for its first rows' loads, which nothing
+// overlaps (8 x 256 x 256: 1295 us, without it 1351, with two rows 1295; its two
+// extra input rows cost loads only). Items
 // beyond those terms go to further launches, which add to the same partials.
 // Returns the number of partials.
 int wgrad(WgArgs &a, const WgKernel &k, int n, int h, int w, int slots, cudaStream_t st)

@@ -2,9 +2,11 @@
 // solver (Girfoglio, Quaini & Rozza, arXiv 2303.10499, Section 3) as one
 // cooperative kernel.
 //
-// On grids of up to a few hundred thousand cells a step is a chain of ~90
-// short phases, and launching each as its own kernel leaves the GPU waiting
-// on launch latency. Here the blocks stay resident for the whole step: each
+// A step is a chain of 30 to several hundred phases. On small grids launching
+// each as its own kernel leaves the GPU waiting on launch latency, and up to
+// nearly two million cells (16 tiles a block; FP32 phases half of that) the
+// launches and the gaps between them still cost more than the blocks in flight
+// that this kernel gives up. Here the blocks stay resident for the whole step: each
 // phase is a block-stride loop over tiles running the tile functions of
 // gea_tiles_body.cuh, phases are separated by a grid barrier, and every
 // residual norm or CG dot product rides on the barrier: each block writes its

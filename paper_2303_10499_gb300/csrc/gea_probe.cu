@@ -34,8 +34,7 @@ __global__ void __launch_bounds__(kProbeThreads) k_fma_chains(int iters, R a, R 
 }
 
 // Words of the barrier probe's scratch: the arrival counter, a status word
-// (read after every barrier when asked, as the persistent step kernels do),
-// and the give-up flag.
+// (read after every barrier when asked) and the give-up flag.
 struct BarScratch {
     unsigned count;
     int status;
@@ -44,10 +43,12 @@ struct BarScratch {
 
 constexpr unsigned long long kBarPolls = 1ull << 22;
 
-// `iters` grid barriers of the persistent step kernels' protocol: thread 0
+// `iters` grid barriers in the manner of the persistent step kernels: thread 0
 // of each block arrives with one acquire-release add on a monotone counter
 // and polls it with acquire loads until it reaches k x blocks; the block's
-// threads meet at __syncthreads on both sides. A poll limit bounds every
+// threads meet at __syncthreads on both sides. (The step kernels count in
+// steps of two and keep a block's request to stop in the lowest bit of the word
+// they poll, so they read nothing else.) A poll limit bounds every
 // wait: a block that gives up sets the flag, and every block leaves at its
 // next barrier once the flag is set.
 __global__ void __launch_bounds__(kProbeThreads) k_grid_barriers(BarScratch *w, int iters, int read_status)

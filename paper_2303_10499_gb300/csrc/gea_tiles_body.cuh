@@ -21,8 +21,8 @@
 //    filled while loading, so the arithmetic has no boundary branches;
 //  - the implicit transport operator of Steps 1-2 is assembled once per step
 //    as a 9-point stencil; a Jacobi sweep and H(u) are 9 FMAs per component;
-//  - the Helmholtz operator is kept as d x - sum a x_N with omega/d stored;
-//    values needed at neighbours are computed once per tile cell;
+//  - the Helmholtz operator is kept as d x - sum a x_N with 1/d stored; values
+//    needed at neighbours are computed once per tile cell;
 //  - divisions are done once per step into stored reciprocals.
 // Global reads go through L2 (ld.global.cg): within one persistent launch a
 // buffer is rewritten by other blocks between phases, and L1 is not coherent

@@ -474,7 +474,8 @@ class Solver:
         self._net = net if mode else None   # keep it alive while attached
 
     def set_smoother_weight(self, omega: float):
-        """Weight of the preconditioner's Jacobi sweeps (gea_set_smoother_weight)."""
+        """Weight of the black relaxations of the multigrid smoother
+        (gea_set_smoother_weight; a one-level hierarchy does not use it)."""
         self._check(self.lib.gea_set_smoother_weight(self.h, float(omega)))
 
     def set_tiles_per_block(self, n: int):
@@ -599,10 +600,10 @@ def probe_fma(bits: int = 64, blocks: int = 608, iters: int = 16384, stream=None
 
 def probe_barrier(blocks: int = 456, iters: int = 20000, read_status: bool = True, stream=None,
                   repeats: int = 3) -> Dict:
-    """Measured cost of one grid barrier of the persistent kernels' protocol
-    (gea_probe_barrier): the best of `repeats` CUDA-event timed launches of
-    `iters` barriers on `blocks` co-resident blocks, in microseconds per
-    barrier."""
+    """Measured cost of one grid barrier in the manner of the persistent
+    kernels (gea_probe_barrier; read_status adds a read that they do without):
+    the best of `repeats` CUDA-event timed launches of `iters` barriers on
+    `blocks` co-resident blocks, in microseconds per barrier."""
     import torch
     lib = library()
     stream = stream or torch.cuda.current_stream()
