@@ -26,6 +26,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <climits>
 #include <type_traits>
 #include <vector>
@@ -84,6 +85,7 @@ struct Lev {
 struct Lev32 {
     Geo G;
     float *c, *d, *ax, *ay, *az, *w, *r, *e, *e2;
+    double fx, fy, fz;   // coarse-face factors 1/8 coarse_scale (k_coarsen)
 };
 
 // The operator of a solve in its own precision.
@@ -896,11 +898,11 @@ __global__ void k_helm_rhs(Args a, Lev L, const double *xin, int corr, R *rout, 
 // starts with e = rb / d on black (the red residual is zero), restricts what
 // that leaves on red, and ends with one black relaxation.
 
-// Coarse level: c_C = mean of the 8 children's c, a coarse face = (1/16) sum
-// of its 4 fine faces, d_C = c_C + sum of its faces. Piecewise-constant
-// transfer with the Galerkin value 1/8 makes the coarse operator of smooth
-// fields twice too stiff; half of it is the operator of the coarse grid. One
-// thread per coarse cell; sums in FP64, stored FP32.
+// Coarse level: c_C = mean of the 8 children's c, a coarse face = c.fx, c.fy or
+// c.fz times the sum of its 4 fine faces (an eighth, the Galerkin value, times
+// coarse_scale of its direction; a sixteenth where the spacings are equal),
+// d_C = c_C + sum of its faces. One thread per coarse cell; sums in FP64,
+// stored FP32.
 __global__ void k_coarsen(Lev32 f, Lev32 c)
 {
     int I, J, K;
@@ -918,13 +920,13 @@ __global__ void k_coarsen(Lev32 f, Lev32 c)
                 if (dj == 0) fy0 += ldf(&f.ay[q]); else fy1 += ldf(&f.ay[q + G.P]);
                 if (dk == 0) fz0 += ldf(&f.az[q]); else fz1 += ldf(&f.az[q + G.P * (G.ny + 1)]);
             }
-    const double cc = 0.125 * cs, h = 0.0625;
+    const double cc = 0.125 * cs;
     c.c[Q] = (float)cc;
-    c.ax[Q] = (float)(h * fx0); c.ay[Q] = (float)(h * fy0); c.az[Q] = (float)(h * fz0);
-    if (I == H.nx - 1) c.ax[Q + 1] = (float)(h * fx1);
-    if (J == H.ny - 1) c.ay[Q + H.P] = (float)(h * fy1);
-    if (K == H.nz - 1) c.az[Q + H.P * (H.ny + 1)] = (float)(h * fz1);
-    const double d = cc + h * (fx0 + fx1 + fy0 + fy1 + fz0 + fz1);
+    c.ax[Q] = (float)(c.fx * fx0); c.ay[Q] = (float)(c.fy * fy0); c.az[Q] = (float)(c.fz * fz0);
+    if (I == H.nx - 1) c.ax[Q + 1] = (float)(c.fx * fx1);
+    if (J == H.ny - 1) c.ay[Q + H.P] = (float)(c.fy * fy1);
+    if (K == H.nz - 1) c.az[Q + H.P * (H.ny + 1)] = (float)(c.fz * fz1);
+    const double d = cc + c.fx * (fx0 + fx1) + c.fy * (fy0 + fy1) + c.fz * (fz0 + fz1);
     c.d[Q] = (float)d;
     c.w[Q] = (float)(1.0 / d);
 }
@@ -2088,9 +2090,13 @@ int gea3d_create(const gea3d_grid *grid, const gea_constants *c, gea3d_ctx **out
         // FP32 arrays: half as many doubles, rounded up
         return reinterpret_cast<float *>(take((n + 1) / 2));
     };
+    const double hmin = std::min({ctx->G.dx, ctx->G.dy, ctx->G.dz});
     for (size_t lv = 0; lv < lg.size(); ++lv) {
         Lev32 m;
         m.G = lg[lv];
+        m.fx = 0.125 * gea::coarse_scale(ctx->G.dx, hmin);
+        m.fy = 0.125 * gea::coarse_scale(ctx->G.dy, hmin);
+        m.fz = 0.125 * gea::coarse_scale(ctx->G.dz, hmin);
         const size_t e = elems(lg[lv]);
         m.c = takef(e); m.d = takef(e); m.ax = takef(e); m.ay = takef(e); m.az = takef(e);
         m.w = takef(e);

@@ -322,7 +322,8 @@ int record_step(gea_ctx *ctx, int from, cudaStream_t s, bool graph, Tracer *tr)
     });
     if (rc) return rc;
     launch_eos_coef(a, L[0], s, tr); ++fixed;
-    for (int l = 0; l + 1 < nlev; ++l) { launch_mg_coarsen<double>(L[l], L[l + 1], s, tr); ++fixed; }
+    for (int l = 0; l + 1 < nlev; ++l, ++fixed)
+        launch_mg_coarsen<double>(L[l], L[l + 1], ctx->F.cfx, ctx->F.cfz, s, tr);
     // Step 3: PISO correctors
     for (int c = 0; c < ctx->C.n_corr; ++c) {
         const double *U = c == 0 ? a.ua : a.N.u;
@@ -414,7 +415,8 @@ int record_step_mixed(gea_ctx *ctx, int from, cudaStream_t s, bool graph, Tracer
     });
     if (rc) return rc;
     launch_mx_eos(a, L0, Lf[0], m.dh[0], s, tr); ++fixed;
-    for (int l = 0; l + 1 < nlev; ++l) { launch_mg_coarsen<float>(Lf[l], Lf[l + 1], s, tr); ++fixed; }
+    for (int l = 0; l + 1 < nlev; ++l, ++fixed)
+        launch_mg_coarsen<float>(Lf[l], Lf[l + 1], ctx->F.cfx, ctx->F.cfz, s, tr);
     for (int c = 0; c < ctx->C.n_corr; ++c) {
         const double *U = c == 0 ? a.ua : a.N.u;
         const double *W = c == 0 ? a.wa : a.N.w;
@@ -822,6 +824,9 @@ int gea_create(const gea_grid *grid, const gea_constants *c, gea_ctx **out)
     ctx->thbar = vec(nz, "thbar");
     if (c->flags & GEA_FLAG_KEEP_R0) ctx->r0keep = cellA("r0keep", 0);
     if (c->cs > 0.0) ctx->mueff = cellA("mueff", 0);
+    const double hmin = std::min(G.dx, G.dz);
+    ctx->F.cfx = 0.25 * coarse_scale(G.dx, hmin);
+    ctx->F.cfz = 0.25 * coarse_scale(G.dz, hmin);
     for (size_t lv = 0; lv < nlev64; ++lv) {
         const Geom &g = lg[lv];
         const int l_ = (int)lv;

@@ -10,6 +10,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "../../include/gea.h"
@@ -50,6 +51,7 @@ struct Phys {
     double hdx, hdz;                         // dx / 2, dz / 2
     double s12, s24;                         // 1 / (12 dx dz), 1 / (24 dx dz)
     double icp, icv;                         // 1 / cp, 1 / cv
+    double cfx, cfz;                         // coarse-face factors, 1/4 coarse_scale (ph_coarsen)
     // uniform branch flags as integers (an FP64 compare issues on the FP64 pipe)
     int les;                                 // les_d2 > 0
     int pr_ne1;                              // nuh != mu (Pr != 1): the enthalpy stencil differs
@@ -75,6 +77,25 @@ struct DenseFields {
 inline FieldPtrs state_fields(const State &S)
 {
     return FieldPtrs{{S.rho, S.u, S.w, S.T, S.h, S.p, S.pp, S.pold, S.phix, S.phiz, S.Kold}};
+}
+
+// Coarse faces across spacing h over their Galerkin value (a coarse operator of
+// piecewise-constant transfer), hmin the smallest spacing. The jump of a
+// piecewise-constant function over one fine spacing stands for a slope over a
+// coarse one, so the Galerkin value makes the coarse Laplacian of smooth fields
+// twice too stiff: the direction of the smallest spacing takes half, with equal
+// spacings all do. A direction coupled rho = (h / hmin)^2 times weaker is
+// smoothed by the relaxations as good as nothing, its rough errors reach the
+// coarse level too, and for those the Galerkin value is the right one: it takes
+// rho^(1/4) / 2, at most 1. First corrector's iterations and time of a step, FP64,
+// half in every direction -> this: 640x64 cells of 40 x 5 m, dt 0.5, 120 -> 95,
+// 8.15 -> 6.43 ms; 640x32 of them, dt 0.2, 77 -> 72, 4.49 -> 4.19 ms; 1024x32
+// of 80 x 5 m, dt 0.2, 102 -> 103, 6.01 -> 6.02 ms; 96x96x48 of 40 x 40 x 10 m,
+// dt 0.5, 78 -> 53, 11.2 -> 7.8 ms.
+inline double coarse_scale(double h, double hmin)
+{
+    const double s = 0.5 * sqrt(h / hmin);
+    return s < 1.0 ? s : 1.0;
 }
 
 // One multigrid level of the Helmholtz operator
@@ -460,7 +481,8 @@ void launch_enth_jacobi(const StepArgs &a, const double *hin, double *hout, int 
                         cudaStream_t st, Tracer *tr);
 void launch_eos_coef(const StepArgs &a, const Level &L0, cudaStream_t st, Tracer *tr);
 template <class R>
-void launch_mg_coarsen(const LevelT<R> &f, const LevelT<R> &c, cudaStream_t st, Tracer *tr);
+void launch_mg_coarsen(const LevelT<R> &f, const LevelT<R> &c, double cfx, double cfz, cudaStream_t st,
+                       Tracer *tr);
 void launch_H(const StepArgs &a, const double *U, const double *W, cudaStream_t st, Tracer *tr);
 void launch_helm_rhs(const StepArgs &a, const Level &L0, const double *xin, double *xout,
                      int corr, cudaStream_t st, Tracer *tr);

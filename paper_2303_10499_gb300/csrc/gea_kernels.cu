@@ -188,9 +188,9 @@ __global__ void k_eos_coef(StepArgs a, Level L)
 }
 
 template <class R>
-__global__ void k_mg_coarsen(LevelT<R> f, LevelT<R> c)
+__global__ void k_mg_coarsen(LevelT<R> f, LevelT<R> c, double cfx, double cfz)
 {
-    ph_coarsen<R>(f, c, blockIdx.x, blockIdx.y);
+    ph_coarsen<R>(f, c, cfx, cfz, blockIdx.x, blockIdx.y);
 }
 
 // ---- Step 3 ----
@@ -490,10 +490,11 @@ const char *name_of(const char *f64, const char *f32)
 }
 
 template <class R>
-void launch_mg_coarsen(const LevelT<R> &f, const LevelT<R> &c, cudaStream_t st, Tracer *tr)
+void launch_mg_coarsen(const LevelT<R> &f, const LevelT<R> &c, double cfx, double cfz, cudaStream_t st,
+                       Tracer *tr)
 {
     TRACED(tr, name_of<R>("mg_coarsen", "mx_coarsen"), ncell(c.G),
-           (k_mg_coarsen<R><<<grid_of(c.G), kBlock, 0, st>>>(f, c)));
+           (k_mg_coarsen<R><<<grid_of(c.G), kBlock, 0, st>>>(f, c, cfx, cfz)));
 }
 
 void launch_H(const StepArgs &a, const double *U, const double *W, cudaStream_t st, Tracer *tr)
@@ -598,7 +599,8 @@ void launch_correct(const StepArgs &a, const LevelT<R> &L, const SolveT<R> &v, d
 }
 
 #define INSTANTIATE(R)                                                                                              \
-    template void launch_mg_coarsen<R>(const LevelT<R> &, const LevelT<R> &, cudaStream_t, Tracer *);               \
+    template void launch_mg_coarsen<R>(const LevelT<R> &, const LevelT<R> &, double, double, cudaStream_t,          \
+                                       Tracer *);                                                                   \
     template int launch_vcycle<R>(const StepArgs &, const LevelT<R> *, int, cudaStream_t, Tracer *);                \
     template int launch_cg_start<R>(const StepArgs &, const LevelT<R> *, int, cudaStream_t, Tracer *);              \
     template int launch_cg_iter<R>(const StepArgs &, const LevelT<R> *, int, const CgVecT<R> &, double,             \

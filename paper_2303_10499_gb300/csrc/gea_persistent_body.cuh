@@ -517,7 +517,7 @@ __device__ bool run_step(const PersistArgs &P, const StepArgs &a, const Grp &g, 
     for_tiles(g, G, [&](int bx, int bz) { ph_H(a, u1, w1, sm, bx, bz); });
     gbar(g);
     for (int l = 0; l + 1 < nlev; ++l) {
-        for_tiles(g, L[l + 1].G, [&](int bx, int bz) { ph_coarsen(L[l], L[l + 1], bx, bz); });
+        for_tiles(g, L[l + 1].G, [&](int bx, int bz) { ph_coarsen(L[l], L[l + 1], a.F.cfx, a.F.cfz, bx, bz); });
         gbar(g);
     }
     if (stop(sc)) return false;
@@ -645,7 +645,7 @@ __device__ bool run_step_mixed(const PersistArgs &P, const MixedPersist &X, cons
     for_tiles(g, G, [&](int bx, int bz) { ph_H(a, a.ua, a.wa, sm, bx, bz); });
     gbar(g);
     for (int l = 0; l + 1 < nlev; ++l) {
-        for_tiles(g, L[l + 1].G, [&](int bx, int bz) { ph_coarsen<float>(L[l], L[l + 1], bx, bz); });
+        for_tiles(g, L[l + 1].G, [&](int bx, int bz) { ph_coarsen<float>(L[l], L[l + 1], a.F.cfx, a.F.cfz, bx, bz); });
         gbar(g);
     }
     if (stop(sc)) return false;
